@@ -17,9 +17,10 @@
 // that, and a floor of 1/4 loses its gain).  Training minimises
 // sum_i (w(f_i) a_i - b_i)^2 for given targets a, b (a = 1 and b a wanted
 // factor fits the factor itself); the gradient is taken by a hand-written backward
-// pass whose weight gradients are fixed-order chunked sums.
+// pass whose sums run in a fixed order.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -105,84 +106,255 @@ __device__ __forceinline__ void stage_params(const float *params, float *P) {
 }
 
 // ---------------------------------------------------------------- training
-// Per sample: loss (w a - b)^2, and the deltas needed by the weight gradients.
-__global__ void mlp_fwd_bwd_kernel(const float *__restrict__ params, const float *__restrict__ feats,
-                                   const float *__restrict__ ta, const float *__restrict__ tb, int64_t n,
-                                   float *__restrict__ H1, float *__restrict__ D1, float *__restrict__ H2,
-                                   float *__restrict__ D2, float *__restrict__ DO, float *__restrict__ loss) {
-    __shared__ float P[MLP_NPARAM];
-    stage_params(params, P);
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float f[MLP_IN], h1[MLP_W], h2[MLP_W];
+// Loss and gradient in one persistent kernel.  A block takes tiles of kTile
+// samples and keeps everything of a tile in shared memory: activations and
+// deltas as [unit][sample] (row stride kLd, 4 mod 32 banks, so that the 128-bit
+// reads of eight consecutive rows hit different banks).  The three 64 x 64
+// products of a sample (forward, input gradient, weight gradient) are register
+// tiles (8 samples x 4 units, or 4 x 4 weights), so the kernel runs on the FP32
+// pipe: 8.7 kFMA a sample, 23 us for 65536 samples at the full rate.  The
+// gradient sums stay in registers over all tiles of a block; each block then
+// writes one row of partial sums, and a second kernel adds the rows in order.
+// Measured at 65536 samples: 76 us + 6 us, against 172 + 2375 us when the
+// activations went through memory and each parameter walked the samples alone.
+constexpr int kTile = 128, kLd = kTile + 4, kTrainThreads = 256;
+constexpr int kTrainSmem = (3 * MLP_W * kLd + MLP_IN * kLd + 2 * MLP_W * MLP_W + MLP_W * MLP_IN + 3 * MLP_W + 2 * kTile) *
+                           (int)sizeof(float);
+
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// A thread's eight samples are s0 .. s0 + 3 and s0 + 64 .. s0 + 67, so that the
+// 16 threads of a unit group read and write whole rows without bank conflicts.
+constexpr int kHalf = kTile / 2;
+
+__device__ __forceinline__ void put8(float *row, int s0, const float (&v)[8]) {
+    *reinterpret_cast<float4 *>(row + s0) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4 *>(row + s0 + kHalf) = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+__device__ __forceinline__ void get8(const float *row, int s0, float (&v)[8]) {
+    const float4 x = ld4(row + s0), y = ld4(row + s0 + kHalf);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+}
+
+// acc[j][i] += sum_k A[k][sample i] B[k][u0 + j] over k < 64 (4 units x 8 samples)
+__device__ __forceinline__ void tile_product(const float *A, const float *B, int s0, int u0, float (&acc)[4][8]) {
+#pragma unroll 4
+    for (int k = 0; k < MLP_W; ++k) {
+        float a[8];
+        get8(A + k * kLd, s0, a);
+        const float4 w = ld4(B + k * MLP_W + u0);
+        const float b[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-    for (int c = 0; c < MLP_IN; ++c) f[c] = feats[i * MLP_IN + c];
-    const float o = mlp_forward(P, f, h1, h2);
-    const float th = tanhf(o);
-    const float w = expf(kLogR * th);
-    const float a = ta[i], b = tb[i];
-    const float err = w * a - b;
-    loss[i] = err * err;
-    const float dout = 2.0f * err * a * w * kLogR * (1.0f - th * th);   // dL/do
-    DO[i] = dout;
-    float d2[MLP_W];
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int c = 0; c < MLP_W; ++c) d2[c] = h2[c] > 0.0f ? dout * P[OFF_W3 + c] : 0.0f;
-#pragma unroll 2
-    for (int c = 0; c < MLP_W; ++c) {
-        float s = 0.0f;
-#pragma unroll
-        for (int a2 = 0; a2 < MLP_W; ++a2) s = fmaf(P[OFF_W2 + a2 * MLP_W + c], d2[a2], s);
-        D1[i * MLP_W + c] = h1[c] > 0.0f ? s : 0.0f;
-    }
-#pragma unroll
-    for (int c = 0; c < MLP_W; ++c) {
-        H1[i * MLP_W + c] = h1[c];
-        H2[i * MLP_W + c] = h2[c];
-        D2[i * MLP_W + c] = d2[c];
+            for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(a[i], b[j], acc[j][i]);
     }
 }
 
-// partial[c][t] for parameter t over samples of chunk c (fixed order)
-constexpr int kMlpChunk = 1024;
-__global__ void mlp_grad_partial_kernel(const float *__restrict__ feats, const float *__restrict__ H1,
-                                        const float *__restrict__ D1, const float *__restrict__ H2,
-                                        const float *__restrict__ D2, const float *__restrict__ DO,
-                                        const float *__restrict__ loss, int64_t n, float *__restrict__ partial) {
-    const int c = blockIdx.x;
-    const int64_t i0 = (int64_t)c * kMlpChunk, i1 = (n < i0 + kMlpChunk) ? n : i0 + kMlpChunk;
-    for (int t = threadIdx.x; t <= MLP_NPARAM; t += blockDim.x) {
-        float s = 0.0f;
-        if (t == MLP_NPARAM) {                         // the loss itself
-            for (int64_t i = i0; i < i1; ++i) s += loss[i];
-        } else if (t < OFF_B1) {                       // W1[a][c] = sum D1[a] f[c]
-            const int a = t / MLP_IN, cc = t % MLP_IN;
-            for (int64_t i = i0; i < i1; ++i) s = fmaf(D1[i * MLP_W + a], feats[i * MLP_IN + cc], s);
-        } else if (t < OFF_W2) {                       // b1
-            const int a = t - OFF_B1;
-            for (int64_t i = i0; i < i1; ++i) s += D1[i * MLP_W + a];
-        } else if (t < OFF_B2) {                       // W2[a][c] = sum D2[a] H1[c]
-            const int a = (t - OFF_W2) / MLP_W, cc = (t - OFF_W2) % MLP_W;
-            for (int64_t i = i0; i < i1; ++i) s = fmaf(D2[i * MLP_W + a], H1[i * MLP_W + cc], s);
-        } else if (t < OFF_W3) {                       // b2
-            const int a = t - OFF_B2;
-            for (int64_t i = i0; i < i1; ++i) s += D2[i * MLP_W + a];
-        } else if (t < OFF_B3) {                       // w3[c] = sum DO H2[c]
-            const int cc = t - OFF_W3;
-            for (int64_t i = i0; i < i1; ++i) s = fmaf(DO[i], H2[i * MLP_W + cc], s);
-        } else {                                       // b3
-            for (int64_t i = i0; i < i1; ++i) s += DO[i];
+__global__ void __launch_bounds__(kTrainThreads, 1)
+mlp_train_kernel(const float *__restrict__ params, const float *__restrict__ feats, const float *__restrict__ ta,
+                 const float *__restrict__ tb, int64_t n, int64_t tiles, float *__restrict__ partial) {
+    extern __shared__ __align__(16) float sm[];
+    float *H1 = sm, *H2 = H1 + MLP_W * kLd, *D1 = H2 + MLP_W * kLd, *F = D1 + MLP_W * kLd;
+    float *W2 = F + MLP_IN * kLd, *W2T = W2 + MLP_W * MLP_W, *W1 = W2T + MLP_W * MLP_W;
+    float *B1 = W1 + MLP_W * MLP_IN, *B2 = B1 + MLP_W, *W3 = B2 + MLP_W, *DO = W3 + MLP_W, *ER = DO + kTile;
+    const int t = threadIdx.x;
+    for (int e = t; e < MLP_W * MLP_W; e += kTrainThreads) {
+        const float v = q16(params[OFF_W2 + e]);
+        W2[e] = v;
+        W2T[(e % MLP_W) * MLP_W + e / MLP_W] = v;
+    }
+    for (int e = t; e < MLP_W * MLP_IN; e += kTrainThreads) W1[e] = q16(params[OFF_W1 + e]);
+    if (t < MLP_W) {
+        B1[t] = params[OFF_B1 + t];
+        B2[t] = params[OFF_B2 + t];
+        W3[t] = q16(params[OFF_W3 + t]);
+    }
+    const float b3 = params[OFF_B3];
+    // register tile of the sample products: 16 unit groups x 16 sample groups
+    const int u0 = 4 * (t / 16), s0 = 4 * (t % 16);
+    // gradient sums of this thread: W2[ga + 16 i][gc + 16 j]; W1[wa][wc, wc + 1];
+    // b1, b2, w3 of unit wa over samples 32 (t % 4) ..; b3 and the loss on thread t < kTile
+    const int ga = t / 16, gc = t % 16, wa = t / 4, wq = t % 4;
+    float g2[4][4] = {}, g1[2] = {0.0f, 0.0f}, gb1 = 0.0f, gb2 = 0.0f, gw3 = 0.0f, gb3 = 0.0f, gl = 0.0f;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t i0 = tile * kTile;
+        const int valid = (int)min((int64_t)kTile, n - i0);
+        __syncthreads();
+        for (int e = t; e < kTile * MLP_IN; e += kTrainThreads) {
+            const int s = e / MLP_IN, c = e % MLP_IN;
+            F[c * kLd + s] = s < valid ? feats[i0 * MLP_IN + e] : 0.0f;
         }
-        partial[(int64_t)c * (MLP_NPARAM + 1) + t] = s;
+        __syncthreads();
+        {
+            float acc[4][8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[j][i] = B1[u0 + j];
+#pragma unroll
+            for (int c = 0; c < MLP_IN; ++c) {
+                float f[8];
+                get8(F + c * kLd, s0, f);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) acc[j][i] = fmaf(W1[(u0 + j) * MLP_IN + c], f[i], acc[j][i]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[j][i] = fmaxf(acc[j][i], 0.0f);
+                put8(H1 + (u0 + j) * kLd, s0, acc[j]);
+            }
+        }
+        __syncthreads();
+        {
+            float acc[4][8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[j][i] = B2[u0 + j];
+            tile_product(H1, W2T, s0, u0, acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[j][i] = fmaxf(acc[j][i], 0.0f);
+                put8(H2 + (u0 + j) * kLd, s0, acc[j]);
+            }
+        }
+        __syncthreads();
+        if (t < kTile) {
+            float o = b3;
+#pragma unroll 8
+            for (int c = 0; c < MLP_W; ++c) o = fmaf(W3[c], H2[c * kLd + t], o);
+            float dout = 0.0f;
+            if (t < valid) {
+                const float th = tanhf(o);
+                const float w = expf(kLogR * th);
+                const float a = ta[i0 + t], b = tb[i0 + t];
+                const float err = w * a - b;
+                gl = fmaf(err, err, gl);
+                dout = 2.0f * err * a * w * kLogR * (1.0f - th * th);   // dL/do
+                gb3 += dout;
+            }
+            DO[t] = dout;
+        }
+        __syncthreads();
+        // w3's sums, and H2 becomes D2 in place
+        {
+            const float w3 = W3[wa];
+#pragma unroll 4
+            for (int k = 0; k < 8; ++k) {
+                const int s = 4 * (wq + 4 * k);
+                float4 h = ld4(H2 + wa * kLd + s);
+                const float4 d = ld4(DO + s);
+                gw3 = fmaf(d.x, h.x, fmaf(d.y, h.y, fmaf(d.z, h.z, fmaf(d.w, h.w, gw3))));
+                h.x = (s < valid && h.x > 0.0f) ? d.x * w3 : 0.0f;
+                h.y = (s + 1 < valid && h.y > 0.0f) ? d.y * w3 : 0.0f;
+                h.z = (s + 2 < valid && h.z > 0.0f) ? d.z * w3 : 0.0f;
+                h.w = (s + 3 < valid && h.w > 0.0f) ? d.w * w3 : 0.0f;
+                gb2 += (h.x + h.y) + (h.z + h.w);
+                *reinterpret_cast<float4 *>(H2 + wa * kLd + s) = h;
+            }
+        }
+        __syncthreads();
+        {
+            float acc[4][8] = {};
+            tile_product(H2, W2, s0, u0, acc);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float h[8];
+                get8(H1 + (u0 + j) * kLd, s0, h);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int smp = s0 + (i & 3) + kHalf * (i >> 2);
+                    acc[j][i] = (smp < valid && h[i] > 0.0f) ? acc[j][i] : 0.0f;
+                }
+                put8(D1 + (u0 + j) * kLd, s0, acc[j]);
+            }
+        }
+        // W2[a][c] += sum D2[a] H1[c]
+#pragma unroll 2
+        for (int s = 0; s < kTile; s += 4) {
+            float4 d[4], h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[i] = ld4(H2 + (ga + 16 * i) * kLd + s);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) h[j] = ld4(H1 + (gc + 16 * j) * kLd + s);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    g2[i][j] = fmaf(d[i].w, h[j].w, fmaf(d[i].z, h[j].z, fmaf(d[i].y, h[j].y, fmaf(d[i].x, h[j].x,
+                                                                                                 g2[i][j]))));
+        }
+        __syncthreads();
+        // W1[a][c] += sum D1[a] f[c]: columns 2 wq and 2 wq + 1
+#pragma unroll 2
+        for (int s = 0; s < kTile; s += 4) {
+            const float4 d = ld4(D1 + wa * kLd + s), f0 = ld4(F + (2 * wq) * kLd + s), f1 = ld4(F + (2 * wq + 1) * kLd + s);
+            g1[0] = fmaf(d.w, f0.w, fmaf(d.z, f0.z, fmaf(d.y, f0.y, fmaf(d.x, f0.x, g1[0]))));
+            g1[1] = fmaf(d.w, f1.w, fmaf(d.z, f1.z, fmaf(d.y, f1.y, fmaf(d.x, f1.x, g1[1]))));
+            if (((s >> 2) & 3) == wq) gb1 += (d.x + d.y) + (d.z + d.w);
+        }
+    }
+    float *out = partial + (int64_t)blockIdx.x * (MLP_NPARAM + 1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[OFF_W2 + (ga + 16 * i) * MLP_W + gc + 16 * j] = g2[i][j];
+    out[OFF_W1 + wa * MLP_IN + 2 * wq] = g1[0];
+    out[OFF_W1 + wa * MLP_IN + 2 * wq + 1] = g1[1];
+#pragma unroll
+    for (int h = 1; h < 4; h <<= 1) {
+        gb1 += __shfl_xor_sync(0xffffffffu, gb1, h);
+        gb2 += __shfl_xor_sync(0xffffffffu, gb2, h);
+        gw3 += __shfl_xor_sync(0xffffffffu, gw3, h);
+    }
+    if (wq == 0) {
+        out[OFF_B1 + wa] = gb1;
+        out[OFF_B2 + wa] = gb2;
+        out[OFF_W3 + wa] = gw3;
+    }
+    __syncthreads();
+    if (t < kTile) {
+        DO[t] = gb3;
+        ER[t] = gl;
+    }
+    __syncthreads();
+    for (int h = kTile / 2; h > 0; h >>= 1) {
+        if (t < h) {
+            DO[t] += DO[t + h];
+            ER[t] += ER[t + h];
+        }
+        __syncthreads();
+    }
+    if (t == 0) {
+        out[OFF_B3] = DO[0];
+        out[MLP_NPARAM] = ER[0];
     }
 }
 
-__global__ void mlp_grad_reduce_kernel(const float *__restrict__ partial, int chunks, float scale,
-                                       float *__restrict__ grads, float *__restrict__ loss_out) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t > MLP_NPARAM) return;
+// One warp per 32 parameters x 8 rows at a time: thread (x, y) adds rows y,
+// y + 8, ... in order, then the eight sums are added in order.
+__global__ void __launch_bounds__(256)
+mlp_grad_reduce_kernel(const float *__restrict__ partial, int rows, float scale, float *__restrict__ grads,
+                       float *__restrict__ loss_out) {
+    __shared__ float sums[8][32];
+    const int x = threadIdx.x % 32, y = threadIdx.x / 32;
+    const int t = blockIdx.x * 32 + x;
     float s = 0.0f;
-    for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * (MLP_NPARAM + 1) + t];
+    if (t <= MLP_NPARAM)
+#pragma unroll 8
+        for (int c = y; c < rows; c += 8) s += partial[(int64_t)c * (MLP_NPARAM + 1) + t];
+    sums[y][x] = s;
+    __syncthreads();
+    if (y != 0 || t > MLP_NPARAM) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += sums[k][x];
     if (t == MLP_NPARAM) *loss_out = s * scale;
     else grads[t] = s * scale;
 }
@@ -356,21 +528,30 @@ extern "C" int hb_mlp_set(hb_ctx *ctx, const hb_mlp_weights *wt) {
     return HB_OK;
 }
 
+// One row of partial sums per block of the training kernel: a block per SM, and
+// no more than there are tiles.
+static int64_t train_tiles(int64_t n) { return (n + kTile - 1) / kTile; }
+constexpr int kTrainMaxBlocks = 256;
+
 extern "C" int64_t hb_mlp_workspace_bytes(int64_t n) {
-    const int64_t chunks = (n + kMlpChunk - 1) / kMlpChunk;
-    return (int64_t)sizeof(float) * (n * (4 * MLP_W + 2) + chunks * (MLP_NPARAM + 1) + 64);
+    return (int64_t)sizeof(float) * std::min<int64_t>(std::max<int64_t>(train_tiles(n), 1), kTrainMaxBlocks) *
+           (MLP_NPARAM + 1);
 }
 
 extern "C" int hb_mlp_loss_grad(const float *params, const float *feats, const float *a, const float *b, int64_t n,
                                 float *grads, float *loss, void *work, void *stream) {
     if (!params || !feats || !a || !b || !grads || !loss || !work || n <= 0) return HB_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    float *H1 = (float *)work, *D1 = H1 + n * MLP_W, *H2 = D1 + n * MLP_W, *D2 = H2 + n * MLP_W;
-    float *DO = D2 + n * MLP_W, *L = DO + n, *partial = L + n;
-    mlp_fwd_bwd_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(params, feats, a, b, n, H1, D1, H2, D2, DO, L);
-    const int chunks = (int)((n + kMlpChunk - 1) / kMlpChunk);
-    mlp_grad_partial_kernel<<<chunks, 256, 0, s>>>(feats, H1, D1, H2, D2, DO, L, n, partial);
-    mlp_grad_reduce_kernel<<<(MLP_NPARAM + 1 + 255) / 256, 256, 0, s>>>(partial, chunks, 1.0f / (float)n, grads, loss);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem) != cudaSuccess)
+        return HB_ERR_CUDA;
+    const int64_t tiles = train_tiles(n);
+    const int blocks = (int)std::min<int64_t>(tiles, std::min(sms, kTrainMaxBlocks));
+    float *partial = (float *)work;
+    mlp_train_kernel<<<blocks, kTrainThreads, kTrainSmem, s>>>(params, feats, a, b, n, tiles, partial);
+    mlp_grad_reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, s>>>(partial, blocks, 1.0f / (float)n, grads, loss);
     return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ERR_CUDA;
 }
 
