@@ -144,8 +144,7 @@ static int l2_mirror_prepare(hb_ctx *ctx, int n, int W, cudaStream_t s) {
     if (below <= 0 || below % 2) return HB_OK;
     const int64_t nl = below / 2;
     // one allocation (each cudaMalloc costs tens of microseconds): the int64
-    // lists, then every entry's column (for this search only), the lower
-    // entries' columns and the flag
+    // lists, then every entry's column, the lower entries' columns and the flag
     uint8_t *buf = nullptr;
     const size_t n8 = (size_t)n + 1 + 2 * (size_t)nl, n4 = (size_t)ctx->l2_nnz + (size_t)nl + 1;
     int rc = dalloc(ctx, &buf, 8 * n8 + 4 * n4);
@@ -168,6 +167,7 @@ static int l2_mirror_prepare(hb_ctx *ctx, int n, int W, cudaStream_t s) {
         ctx->l2_mdst = dst;
         ctx->l2_msrc = src;
         ctx->l2_mcol = mcol;
+        ctx->l2_cols = col_all;
         ctx->l2_nlow = nl;
     }
     return HB_OK;

@@ -155,7 +155,7 @@ struct hb_ctx {
     int64_t l2_nnz = 0, tt_pairs = 0, tl2_pairs = 0;
     // the L2 x L2 entries below the diagonal and their mirrors (null: none found)
     int64_t *l2_low_ptr = nullptr, *l2_mdst = nullptr, *l2_msrc = nullptr;
-    int32_t *l2_mcol = nullptr;
+    int32_t *l2_mcol = nullptr, *l2_cols = nullptr;   // l2_cols: the column of every L2 x L2 entry
     int64_t l2_nlow = 0;
     hb::MixedState *mixed = nullptr;
     hb::DevPool pool;        // device memory beyond the staged problem

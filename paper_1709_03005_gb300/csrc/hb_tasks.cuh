@@ -223,7 +223,7 @@ struct C4Item {         // one work item of the tensor-core class-4 kernel
     int ti, l, jt, nkb;       // task, L2 row, orbital tile, K blocks of 32 terms
 };
 
-struct L2Task {         // classes 2 and 8: L2-L2 CSR of one Hamiltonian
+struct L2Task {         // classes 2 and 8 without the staged columns (no couplings, or an asymmetric list)
     Ints I;
     const uint64_t *dets;
     int n, nseg;
@@ -233,10 +233,21 @@ struct L2Task {         // classes 2 and 8: L2-L2 CSR of one Hamiltonian
     int32_t *col;
     double *val;
     double e_core;
-    // non-null: entries below the diagonal of row r are [row_ptr[r], row_ptr[r] +
-    // low_ptr[r + 1] - low_ptr[r]) and come from g_l2_mirror; only col >= row here
-    const int64_t *low_ptr;
     int row_lo, row_hi;       // the rows evaluated (all of them unless sharded)
+};
+
+struct L2VTask {        // classes 2 and 8 where hb_init listed every entry's column: the entries with col >= row
+    Ints I;
+    const uint64_t *dets;
+    int n, steps;              // steps of 32 consecutive entries a warp takes
+    int64_t n_up, diag_blocks; // entries with col >= row; blocks of the task that evaluate diagonals
+    const int64_t *row_ptr, *low_ptr;   // low_ptr: prefix of the entries below the diagonal per row
+    const int32_t *cols;       // column of every entry
+    int64_t *row_ptr_out;
+    int32_t *col;
+    double *val;
+    double e_core;
+    int row_lo, row_hi;        // the rows evaluated (all of them unless sharded)
 };
 
 struct L2MTask {        // classes 2 and 8: the entries below the diagonal from their mirrors
@@ -255,7 +266,11 @@ int g_pair_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s);
 // the diagonal records (m, m) of same-group tasks, one thread per row
 int g_diag_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s);
 int64_t blocks_diag_values(int n_rows);
-int g_l2_csr(const Grouped<L2Task> &g, int W, int dfloat, cudaStream_t s);
+int g_l2_csr(const Grouped<L2Task> &g, int W, cudaStream_t s);
+int g_l2_values(const Grouped<L2VTask> &g, int W, cudaStream_t s);
+int64_t l2_diag_blocks(int n);
+int l2_value_steps(int64_t n_up);
+int64_t blocks_l2_values(int n, int64_t n_up);
 int g_l2_mirror(const Grouped<L2MTask> &g, cudaStream_t s);
 constexpr int kL2MirrorThreads = 256;
 // width: states per pass of the double-float kernel (16, 24 or 32; the

@@ -115,6 +115,7 @@ struct Plan {
     Stage<C4FTask> c4f;                // class 4 on the tensor cores: term lists, then the GEMMs
     Stage<C4TTask> c4t;
     Stage<L2Task> l2;
+    Stage<L2VTask> l2v;          // the L2 x L2 entries from their staged columns
     Stage<L2MTask> l2m;          // the L2 x L2 entries below the diagonal, after l2
     std::vector<ExpCol> cols;          // columns of the merged expansion blocks
     size_t off_cols = 0;
@@ -203,7 +204,7 @@ void stage_bind(Stage<T> &st, uint8_t *dev) {
 void fill_tasks(Plan &p) {
     p.cls_tt.clear(); p.cls_tl2.clear(); p.pv.clear(); p.pvd.clear(); p.sw.clear(); p.sws.clear(); p.sw_width = 16; p.gamw.clear(); p.gdp.clear(); p.gdr.clear(); p.tn.clear(); p.tnr.clear();
     p.itf.clear(); p.zero.clear(); p.sort.clear(); p.scan.clear(); p.gam.clear(); p.asmb.clear();
-    p.x64.clear(); p.slc.clear(); p.drows.clear(); p.l2.clear(); p.l2m.clear();
+    p.x64.clear(); p.slc.clear(); p.drows.clear(); p.l2.clear(); p.l2v.clear(); p.l2m.clear();
     for (auto &v : p.c4v) v.st.clear();
     p.c4f.clear(); p.c4t.clear();
     for (auto &sg : p.split) sg.st.clear();
@@ -396,10 +397,18 @@ void fill_tasks(Plan &p) {
             var->st.add(c4t, blocks_class4(nl, G.cn, jt));
             if (p.precision == HB_MIXED) p.tune_c4.push_back(TuneC4{c4t});
         }
-        if (ctx->n_l2 > 0) {
+        if (ctx->n_l2 > 0 && ctx->l2_low_ptr) {
+            const int64_t n_up = ctx->l2_nnz - ctx->l2_nlow;
+            p.l2v.add(L2VTask{I, ctx->l2, ctx->n_l2, l2_value_steps(n_up), n_up, l2_diag_blocks(ctx->n_l2),
+                              ctx->l2_rowptr, ctx->l2_low_ptr, ctx->l2_cols, out.l2_row_ptr, out.l2_col, out.l2_val,
+                              ctx->e_core, l0, l0 + nl},
+                      blocks_l2_values(ctx->n_l2, n_up));
+        } else if (ctx->n_l2 > 0) {
             p.l2.add(L2Task{I, ctx->l2, ctx->n_l2, seg_count(ctx->n_l2), ctx->l2_rowptr, ctx->l2_seg_off, out.l2_row_ptr,
-                            out.l2_col, out.l2_val, ctx->e_core, ctx->l2_low_ptr, l0, l0 + nl},
+                            out.l2_col, out.l2_val, ctx->e_core, l0, l0 + nl},
                      blocks_seg_rows8(ctx->n_l2, ctx->n_l2));
+        }
+        if (ctx->n_l2 > 0) {
             // an entry below the diagonal is copied by the rank that evaluates its
             // mirror, whose row is the entry's column
             if (ctx->l2_low_ptr && ctx->l2_nlow > 0)
@@ -491,7 +500,7 @@ void pack_all(Plan &p) {
     stage_pack(p.zero, p.host); stage_pack(p.sort, p.host); stage_pack(p.scan, p.host); stage_pack(p.gam, p.host);
     stage_pack(p.asmb, p.host); stage_pack(p.x64, p.host); stage_pack(p.slc, p.host);
     for (auto &sg : p.split) stage_pack(sg.st, p.host);
-    stage_pack(p.drows, p.host); stage_pack(p.l2, p.host); stage_pack(p.l2m, p.host);
+    stage_pack(p.drows, p.host); stage_pack(p.l2, p.host); stage_pack(p.l2v, p.host); stage_pack(p.l2m, p.host);
     for (auto &v : p.c4v) stage_pack(v.st, p.host);
     stage_pack(p.c4f, p.host); stage_pack(p.c4t, p.host);
     p.off_cols = align256(p.host.size());
@@ -510,7 +519,7 @@ void bind_all(Plan &p) {
     stage_bind(p.zero, p.dev); stage_bind(p.sort, p.dev); stage_bind(p.scan, p.dev); stage_bind(p.gam, p.dev);
     stage_bind(p.asmb, p.dev); stage_bind(p.x64, p.dev); stage_bind(p.slc, p.dev);
     for (auto &sg : p.split) stage_bind(sg.st, p.dev);
-    stage_bind(p.drows, p.dev); stage_bind(p.l2, p.dev); stage_bind(p.l2m, p.dev);
+    stage_bind(p.drows, p.dev); stage_bind(p.l2, p.dev); stage_bind(p.l2v, p.dev); stage_bind(p.l2m, p.dev);
     for (auto &v : p.c4v) stage_bind(v.st, p.dev);
     stage_bind(p.c4f, p.dev); stage_bind(p.c4t, p.dev);
     p.d_cols = (const ExpCol *)(p.dev + p.off_cols);
@@ -887,8 +896,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     cudaStreamWaitEvent(p->main, p->fork, 0);
     cudaStreamWaitEvent(s2, p->fork, 0);
     // class 4 (Eq. 5) and classes 2 and 8
-    // the L2 rows stay FP64: their sums are short and the kernel is bound by the
-    // pair scan, where the longer double-float sums cost more than FP64 adds
+    // the L2 rows stay FP64: their sums are short, and double-float sums cost
+    // more than the FP64 adds they replace
     rec_on(p->ev[5], s2);
     // a sharded build runs in two phases: the contraction (1), then, with the
     // reduced coefficient rows in place, classes 4, 2, 8 and the expansion (2)
@@ -905,7 +914,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         // fit beside either: the L2 rows run beside the target side, then
         // class 4, and the expansion starts once both are done
         rec_on(p->ev[7], s2);
-        L += g_l2_csr(p->l2.g, W, 0, s2);
+        L += g_l2_csr(p->l2.g, W, s2);
+        L += g_l2_values(p->l2v.g, W, s2);
         L += g_l2_mirror(p->l2m.g, s2);
         rec_on(p->ev[4], s2);
         cudaMemsetAsync(p->err + 1, 0, sizeof(int), s2);
@@ -918,7 +928,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         for (auto &v : p->c4v) L += g_class4(v.st.g, W, p->precision == HB_MIXED ? 1 : 0, v.ns_tile, v.jt, s2);
         rec_on(p->ev[3], s2);
         rec_on(p->ev[7], s2);
-        L += g_l2_csr(p->l2.g, W, 0, s2);
+        L += g_l2_csr(p->l2.g, W, s2);
+        L += g_l2_values(p->l2v.g, W, s2);
         L += g_l2_mirror(p->l2m.g, s2);
         rec_on(p->ev[4], s2);
     }

@@ -8,6 +8,8 @@
 // (the standard rules for an orthonormal spin-orbital basis; the paper
 // evaluates them symbolically, Eq. 6).  (pp|qq) and (pq|qp) come from a small
 // n_to x n_to table that stays in L1/L2; other (tt|tt) integrals are gathered.
+#include <algorithm>
+
 #include "hb_df.cuh"
 #include "hb_tasks.cuh"
 
@@ -148,9 +150,10 @@ constexpr int kWarps = 8;
 // Block = 8 rows (one warp each) x one segment of kSegCols columns, staged
 // through shared memory word-major (conflict-free lane reads); the segment's
 // output offset within each row comes from the staging-time segment counts.
+// For L2 lists whose columns are not staged (no two functions couple).
 // Matches are queued per warp in column order and evaluated 32 at a time,
 // one per lane.
-template <int W, class Acc>
+template <int W>
 __global__ void __launch_bounds__(32 * kWarps)
 l2_csr_kernel(const L2Task *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     constexpr int TC = kSegCols;
@@ -183,23 +186,12 @@ l2_csr_kernel(const L2Task *__restrict__ tasks, const int64_t *__restrict__ blk,
     const int t0 = sg * TC;
     if (t0 >= n) return;
     const int tn = min(TC, n - t0);
-    // upper triangle only: a segment below the diagonal of every row of the block has nothing to do
-    if (T.low_ptr && t0 + tn <= rb * kWarps) return;
     for (int i = threadIdx.x; i < tn * 2 * W; i += blockDim.x) {
         const int c = i / (2 * W), w = i % (2 * W);
         tile[w * TC + c] = __ldg(D + (int64_t)t0 * 2 * W + i);
     }
     __syncthreads();
     if (!active) return;
-    int cmin = 0;             // first column of the segment evaluated in this row
-    if (T.low_ptr) {
-        if (t0 + tn <= row) return;
-        if (t0 <= row) {
-            // the diagonal's segment: the entries of this row from the diagonal on
-            cmin = row - t0;
-            pos = T.row_ptr[row] + (T.low_ptr[row + 1] - T.low_ptr[row]);
-        }
-    }
     auto drain = [&](int cnt) {
         if (lane < cnt) {
             const int cl = q[lane];
@@ -213,7 +205,7 @@ l2_csr_kernel(const L2Task *__restrict__ tasks, const int64_t *__restrict__ blk,
             const int deg = x >> 1;
             const int64_t at = pos + lane;
             if (at < end) {
-                Acc v = element<W, Acc>(I, a, b, deg);
+                AccD v = element<W, AccD>(I, a, b, deg);
                 if (deg == 0) v.add_const(T.e_core);
                 T.col[at] = t0 + cl;
                 T.val[at] = v.value();
@@ -225,7 +217,7 @@ l2_csr_kernel(const L2Task *__restrict__ tasks, const int64_t *__restrict__ blk,
     for (int c0 = 0; c0 < tn; c0 += 32) {
         const int cl = c0 + lane;
         bool ok = false;
-        if (cl < tn && cl >= cmin) {
+        if (cl < tn) {
             int x = 0;
 #pragma unroll
             for (int i = 0; i < 2 * W; ++i) x += __popcll(a[i] ^ tile[i * TC + cl]);
@@ -242,6 +234,227 @@ l2_csr_kernel(const L2Task *__restrict__ tasks, const int64_t *__restrict__ blk,
             const int mv = lane < rest ? q[32 + lane] : 0;
             __syncwarp();
             if (lane < rest) q[lane] = mv;
+            qn = rest;
+            __syncwarp();
+        }
+    }
+    if (qn > 0) drain(qn);
+}
+
+// ------------------------------------------- the L2 rows from their columns
+// hb_init finds the sparsity pattern, so a build need not search for the pairs
+// again: one lane per entry with col > row, in CSR order.  With the pair search
+// the kernel was bound by its 2 W popcounts for each of n^2 / 2 pairs (of which
+// 2 % couple) and by warps whose 32 matches mixed singles, doubles and a
+// diagonal: 28.9 ms at 122103 functions (1.8e8 entries above the diagonal),
+// against 5.1 ms here.
+// What is left are two gathered integrals per double (the (tt|tt) table lies
+// in L2), the singles' sums of N + N_sigma integrals, and 12 bytes written per
+// entry.  A warp takes 32 steps consecutive entries, evaluates the doubles as
+// they come and queues the singles until 32 of them fill its lanes.  The
+// diagonal entries, each a sum over all electron pairs, take a warp per row
+// (blocks diag_blocks of the task, before the others).
+
+// Parity of the number of set bits of X below the four positions together.
+template <int W>
+__device__ __forceinline__ int parity4(const uint64_t (&x)[2 * W], int a, int b, int c, int d) {
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) {
+        auto below = [&](int pos) -> uint64_t {
+            const int k = pos - 64 * w;
+            return k <= 0 ? 0ull : (k >= 64 ? ~0ull : (1ull << k) - 1ull);
+        };
+        n ^= __popcll(x[w] & (below(a) ^ below(b) ^ below(c) ^ below(d)));
+    }
+    return n & 1;
+}
+
+// sum of a double: an FP64 operation only where both integrals survive
+template <int W>
+__device__ __forceinline__ double double_element(const Ints &I, const uint64_t (&a)[2 * W], const uint64_t (&b)[2 * W]) {
+    int h[2], p[2];
+    diff_bits<W>(b, a, h);
+    diff_bits<W>(a, b, p);
+    constexpr int sb = 64 * W;
+    const int odd = parity4<W>(b, h[0], h[1], p[0], p[1]) ^
+                    ((1 + (h[0] < p[1]) + (h[1] < p[1]) + (h[0] < p[0]) + (h[1] < p[0])) & 1);
+    const int hs0 = h[0] >= sb, hs1 = h[1] >= sb, ps0 = p[0] >= sb, ps1 = p[1] >= sb;
+    const int h0 = h[0] - hs0 * sb, h1 = h[1] - hs1 * sb, p0 = p[0] - ps0 * sb, p1 = p[1] - ps1 * sb;
+    const bool direct = ps0 == hs0 && ps1 == hs1, cross = ps0 == hs1 && ps1 == hs0;
+    const double x = direct ? __ldg(I.tttt + eri_idx(I, p0, h0, p1, h1)) : 0.0;
+    const double y = cross ? __ldg(I.tttt + eri_idx(I, p0, h1, p1, h0)) : 0.0;
+    const double v = cross ? (direct ? x - y : -y) : x;
+    return odd ? -v : v;
+}
+
+// sum of a single: the integrals of up to eight electrons in flight at a time,
+// added in the order of single_value
+template <int W>
+__device__ __forceinline__ double single_element(const Ints &I, const uint64_t (&a)[2 * W], const uint64_t (&b)[2 * W]) {
+    int hh[2], pp[2];
+    diff_bits<W>(b, a, hh);
+    diff_bits<W>(a, b, pp);
+    constexpr int sb = 64 * W;
+    const int odd = parity4<W>(b, hh[0], pp[0], 0, 0) ^ (hh[0] < pp[0]);
+    const int hs = hh[0] >= sb, h = hh[0] - hs * sb, p = pp[0] - (pp[0] >= sb) * sb;
+    double v = __ldg(I.h + (int64_t)p * I.n_orb + h);
+    const double *ph = I.tttt + pair_idx(p, h) * I.Pt;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            uint64_t x = a[s * W + w] & b[s * W + w];
+            while (x) {
+                double J[8], K[8];
+                int cnt = 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (!x) { J[u] = K[u] = 0.0; continue; }
+                    const int k = 64 * w + __ffsll((long long)x) - 1;
+                    x &= x - 1;
+                    J[u] = __ldg(ph + pair_idx(k, k));
+                    K[u] = s == hs ? __ldg(I.tttt + eri_idx(I, p, k, k, h)) : 0.0;
+                    cnt = u + 1;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u < cnt) {
+                        v += J[u];
+                        if (s == hs) v -= K[u];
+                    }
+            }
+        }
+    return odd ? -v : v;
+}
+
+// <a|H|a> by a warp: lane j holds the j-th electron's orbital, electron i
+// meets the electrons after it; the lanes' sums are added in a fixed tree.
+template <int W>
+__device__ __forceinline__ double diag_element_warp(const Ints &I, const uint64_t (&a)[2 * W], uint16_t *occ) {
+    const int lane = threadIdx.x & 31;
+    const int n = I.n_to;
+    constexpr int sb = 64 * W;
+    int ne = 0;
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t bits = (uint32_t)(a[w] >> (32 * half));
+            if ((bits >> lane) & 1u)
+                occ[ne + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(64 * w + 32 * half + lane);
+            ne += __popc(bits);
+        }
+    __syncwarp();
+    double v = 0.0;
+    for (int j = lane; j < ne; j += 32) {
+        const int q = occ[j], sq = q >= sb, oq = q - sq * sb;
+        v += __ldg(I.h + (int64_t)oq * (I.n_orb + 1));
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) {
+            const int p = occ[i], sp = p >= sb, op = p - sp * sb;
+            v += __ldg(I.jk + (int64_t)op * n + oq);
+            if (sp == sq) v -= __ldg(I.jk + (int64_t)n * n + (int64_t)op * n + oq);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncwarp();
+    return v;
+}
+
+template <int W>
+__global__ void __launch_bounds__(32 * kWarps)
+l2_values_kernel(const L2VTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+    __shared__ int2 queue[kWarps][64];         // (row, column) of the singles
+    __shared__ int64_t where[kWarps][64];      // and their positions
+    __shared__ uint16_t occupied[kWarps][128 * W];
+    const int ti = task_of(blk, n_tasks, blockIdx.x);
+    const L2VTask &T = tasks[ti];
+    const Ints I = T.I;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t lb = blockIdx.x - blk[ti];
+    const int64_t *__restrict__ rp = T.row_ptr, *__restrict__ low = T.low_ptr;
+    if (lb < T.diag_blocks) {
+        const int row = (int)(lb * kWarps) + warp;
+        if (row >= T.n || row < T.row_lo || row >= T.row_hi) return;
+        uint64_t a[2 * W];
+        load_det<W>(T.dets + (int64_t)row * 2 * W, a);
+        const double v = diag_element_warp<W>(I, a, occupied[warp]);
+        if (lane == 0) {
+            const int64_t at = __ldg(rp + row) + (__ldg(low + row + 1) - __ldg(low + row));
+            T.col[at] = row;
+            T.val[at] = v + T.e_core;
+            T.row_ptr_out[row] = __ldg(rp + row);
+            if (row == T.n - 1) T.row_ptr_out[T.n] = __ldg(rp + T.n);
+        }
+        return;
+    }
+    // the upper entries of row r are numbered from row_ptr[r] - low_ptr[r]
+    auto first = [&](int r) -> int64_t { return __ldg(rp + r) - __ldg(low + r); };
+    const int64_t u0 = ((lb - T.diag_blocks) * kWarps + warp) * 32 * (int64_t)T.steps;
+    if (u0 >= T.n_up) return;
+    int row = 0;
+    {
+        const int64_t u = u0 + lane < T.n_up ? u0 + lane : T.n_up - 1;
+        int hi = T.n;
+        while (hi - row > 1) {
+            const int mid = row + ((hi - row) >> 1);
+            if (first(mid) <= u) row = mid;
+            else hi = mid;
+        }
+    }
+    int2 *q = queue[warp];
+    int64_t *qw = where[warp];
+    int qn = 0;
+    auto drain = [&](int cnt) {
+        if (lane < cnt) {
+            const int2 rc = q[lane];
+            uint64_t a[2 * W], b[2 * W];
+            load_det<W>(T.dets + (int64_t)rc.x * 2 * W, a);
+            load_det<W>(T.dets + (int64_t)rc.y * 2 * W, b);
+            T.val[qw[lane]] = single_element<W>(I, a, b);
+        }
+    };
+    int64_t next = first(row + 1);
+    for (int st = 0; st < T.steps; ++st) {
+        const int64_t u = u0 + 32 * st + lane;
+        bool single = false;
+        int c = 0;
+        int64_t at = 0;
+        if (u < T.n_up) {
+            while (next <= u) next = first(++row + 1);
+            at = u + __ldg(low + row + 1);
+            c = __ldg(T.cols + at);
+            if (c != row && row >= T.row_lo && row < T.row_hi) {
+                uint64_t a[2 * W], b[2 * W];
+                load_det<W>(T.dets + (int64_t)row * 2 * W, a);
+                load_det<W>(T.dets + (int64_t)c * 2 * W, b);
+                int x = 0;
+#pragma unroll
+                for (int i = 0; i < 2 * W; ++i) x += __popcll(a[i] ^ b[i]);
+                T.col[at] = c;
+                if (x > 2) T.val[at] = double_element<W>(I, a, b);
+                else single = true;
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, single);
+        if (single) {
+            const int k = qn + __popc(m & ((1u << lane) - 1u));
+            q[k] = make_int2(row, c);
+            qw[k] = at;
+        }
+        qn += __popc(m);
+        __syncwarp();
+        if (qn >= 32) {
+            drain(32);
+            __syncwarp();
+            const int rest = qn - 32;
+            int2 mv = make_int2(0, 0);
+            int64_t mw = 0;
+            if (lane < rest) { mv = q[32 + lane]; mw = qw[32 + lane]; }
+            __syncwarp();
+            if (lane < rest) { q[lane] = mv; qw[lane] = mw; }
             qn = rest;
             __syncwarp();
         }
@@ -431,11 +644,10 @@ int g_diag_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s) {
     return 1;
 }
 
-int g_l2_csr(const Grouped<L2Task> &g, int W, int dfloat, cudaStream_t s) {
+int g_l2_csr(const Grouped<L2Task> &g, int W, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
     const dim3 grid((unsigned)g.blocks), block(32 * kWarps);
-#define HB_L2(WW) (dfloat ? l2_csr_kernel<WW, AccF><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n) \
-                          : l2_csr_kernel<WW, AccD><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n))
+#define HB_L2(WW) l2_csr_kernel<WW><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n)
     switch (W) {
         case 1: HB_L2(1); break;
         case 2: HB_L2(2); break;
@@ -443,6 +655,28 @@ int g_l2_csr(const Grouped<L2Task> &g, int W, int dfloat, cudaStream_t s) {
         default: HB_L2(4); break;
     }
 #undef HB_L2
+    return 1;
+}
+
+// Blocks of the rows' diagonals, and of the entries above them: 32 steps
+// entries a warp.  Long runs fill the singles' queue; short ones keep at least
+// 24 warps on each of 152 SMs where there are that many entries.
+int64_t l2_diag_blocks(int n) { return (n + kWarps - 1) / kWarps; }
+int l2_value_steps(int64_t n_up) { return (int)std::min<int64_t>(16, std::max<int64_t>(1, n_up / (32 * 24 * 152))); }
+int64_t blocks_l2_values(int n, int64_t n_up) {
+    const int64_t per = 32 * kWarps * (int64_t)l2_value_steps(n_up);
+    return l2_diag_blocks(n) + (n_up + per - 1) / per;
+}
+
+int g_l2_values(const Grouped<L2VTask> &g, int W, cudaStream_t s) {
+    if (g.blocks <= 0) return 0;
+    const dim3 grid((unsigned)g.blocks), block(32 * kWarps);
+    switch (W) {
+        case 1: l2_values_kernel<1><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n); break;
+        case 2: l2_values_kernel<2><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n); break;
+        case 3: l2_values_kernel<3><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n); break;
+        default: l2_values_kernel<4><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n); break;
+    }
     return 1;
 }
 
