@@ -18,6 +18,7 @@ struct DiagWork {
     double *proj = nullptr;       // projection coefficients kept on the device
     int32_t *idx = nullptr;
     double *HlcT = nullptr;       // class-4 block transposed (Dc x n_l2)
+    double *prod = nullptr;      // slice sums of the FP64 products
     double *XT = nullptr;         // the L2 part of a block of vectors, [n_l2][q] (vectors interleaved)
     int64_t XT_rows = 0;
     const double *HlcT_src = nullptr;

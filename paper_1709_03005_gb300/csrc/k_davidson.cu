@@ -5,7 +5,7 @@
 //   Rayleigh-Ritz: T = V^T AV, T s = theta s, Ritz vectors x = V s, Ax = AV s
 //   residuals r = Ax - theta x; stop when ||r_i|| <= tol for i < k
 //   correction t_i = r_i / (H_ii - theta_i) (optionally times a learned factor)
-//   t orthogonalised against V twice, then among itself (SVQB), appended
+//   t orthogonalised against V and among itself (SVQB), both twice, appended
 //   thick restart to the 2b lowest Ritz vectors when the basis is full.
 // The products H V, the projection V^T AV, the Ritz combinations, residuals
 // and the orthogonalisation run on the GPU in FP64 with fixed-order sums; only
@@ -27,56 +27,104 @@ using namespace hb;
 
 namespace {
 
-// out[j][i] = beta * out[j][i] + sum_k A[i][k] B[j][k]  (i < M, j < N)
-constexpr int GM = 64, GN = 32, GK = 16;
-__global__ void __launch_bounds__(256)
-gemm_nt_kernel(const double *__restrict__ A, int64_t lda, const double *__restrict__ B, int64_t ldb, int M, int N,
-               int K, double *__restrict__ out, int64_t ldo, int beta) {
-    __shared__ double As[GK][GM + 1];
-    __shared__ double Bs[GK][GN + 1];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int m0 = blockIdx.x * GM, n0 = blockIdx.y * GN;
-    double acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    for (int k0 = 0; k0 < K; k0 += GK) {
+// The vector kernels below run on the FP64 pipe, 2 FMAs a cycle and SM, so a
+// warp's FMA holds it for 16 cycles whatever its lanes do: their time is the
+// work per SM.  Each is cut so that a matrix of a few thousand rows still
+// reaches every SM, and so that columns beyond the q of the block cost whole
+// idle warps and not lanes.
+
+// Y = H X in FP64 without the L2 block: rows i < Dc are [Hcc | Hlc^T] X, rows
+// from Dc on Hlc X_c.  A block takes 16 rows x 16 vectors x one slice of kslice
+// terms (the slices are summed in order by product_reduce_kernel), a thread 4
+// vectors of one row.  With 64 x 32 tiles over whole rows, 24 blocks of a
+// 1980-row matrix with 12 vectors took 474 us a product (three a matrix), each
+// computing 32 columns; one launch of 90 us now.
+constexpr int kPT = 16, kPK = 32, kPThreads = 64;
+struct ProductArgs {
+    const double *Hcc, *HlcT, *Hlc;
+    int64_t Dc, nl;
+    const double *X;
+    int64_t ldx;
+    int q, kslice, up_tiles, up_slices, lo_slices;
+    double *out;             // [slice][q][ldo]
+    int64_t ldo, slice_ld;
+};
+__global__ void __launch_bounds__(kPThreads)
+product_kernel(const ProductArgs P) {
+    __shared__ double As[kPT][kPK + 1], Bs[kPK][kPT + 2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t lb = blockIdx.x;
+    const bool upper = lb < (int64_t)P.up_tiles * P.up_slices;
+    if (!upper) lb -= (int64_t)P.up_tiles * P.up_slices;
+    const int ns = upper ? P.up_slices : P.lo_slices;
+    const int64_t i0 = (lb / ns) * kPT, rows = upper ? P.Dc : P.nl;
+    const int sl = (int)(lb % ns), j0 = blockIdx.y * kPT;
+    const int64_t K = upper ? P.Dc + P.nl : P.Dc;
+    const int64_t k0 = (int64_t)sl * P.kslice, k1 = min(K, k0 + P.kslice);
+    double ra[8], rb[8];
+    auto fetch = [&](int64_t kb) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = tid + u * 256, r = e / GK, kk = e % GK;
-            const int gm = m0 + r, gk = k0 + kk;
-            As[kk][r] = (gm < M && gk < K) ? __ldg(A + (int64_t)gm * lda + gk) : 0.0;
+        for (int u = 0; u < 8; ++u) {
+            const int e = tid + u * kPThreads, r = e / kPK;
+            const int64_t k = kb + e % kPK, i = i0 + r;
+            ra[u] = 0.0;
+            rb[u] = 0.0;
+            if (k < k1) {
+                if (i < rows)
+                    ra[u] = !upper ? __ldg(P.Hlc + i * P.Dc + k)
+                                   : (k < P.Dc ? __ldg(P.Hcc + i * P.Dc + k) : __ldg(P.HlcT + i * P.nl + k - P.Dc));
+                if (j0 + r < P.q) rb[u] = __ldg(P.X + (int64_t)(j0 + r) * P.ldx + k);
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = tid + u * 256, r = e / GK, kk = e % GK;
-            const int gn = n0 + r, gk = k0 + kk;
-            Bs[kk][r] = (gn < N && gk < K) ? __ldg(B + (int64_t)gn * ldb + gk) : 0.0;
-        }
+    };
+    const int row = lane & 15, c0 = 8 * warp + 4 * (lane >> 4);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    fetch(k0);
+    for (int64_t kb = k0; kb < k1; kb += kPK) {
         __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            double a[4], b[2];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) b[j] = Bs[kk][tx * 2 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int u = 0; u < 8; ++u) {
+            const int e = tid + u * kPThreads;
+            As[e / kPK][e % kPK] = ra[u];
+            Bs[e % kPK][e / kPK] = rb[u];
         }
         __syncthreads();
-    }
+        if (kb + kPK < k1) fetch(kb + kPK);
+        if (j0 + 8 * warp < P.q) {
+#pragma unroll 8
+            for (int k = 0; k < kPK; ++k) {
+                const double a = As[row][k];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int gn = n0 + tx * 2 + j;
-        if (gn >= N) continue;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int gm = m0 + ty * 4 + i;
-            if (gm >= M) continue;
-            double *o = out + (int64_t)gn * ldo + gm;
-            *o = beta ? *o + acc[i][j] : acc[i][j];
+                for (int c = 0; c < 4; ++c) acc[c] = fma(a, Bs[k][c0 + c], acc[c]);
+            }
         }
     }
+    const int64_t i = i0 + row;
+    if (i >= rows) return;
+    double *o = P.out + (int64_t)sl * P.slice_ld + (upper ? 0 : P.Dc) + i;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (j0 + c0 + c < P.q) o[(int64_t)(j0 + c0 + c) * P.ldo] = acc[c];
+}
+
+// Y[j][i] = sum over slices, in order
+__global__ void product_reduce_kernel(const double *__restrict__ part, int64_t n, int64_t Dc, int q, int up_slices,
+                                      int lo_slices, double *__restrict__ Y, int64_t ldy) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y;
+    if (i >= n) return;
+    const int ns = i < Dc ? up_slices : lo_slices;
+    double v = 0.0;
+    for (int s = 0; s < ns; ++s) v += __ldg(part + ((int64_t)s * q + j) * n + i);
+    Y[(int64_t)j * ldy + i] = v;
+}
+
+// Terms per slice of a product with n rows and q vectors: as many slices as
+// give four blocks on each of 152 SMs, none under 64 terms.
+int product_slice(int64_t n, int q) {
+    const int64_t tiles = ((n + kPT - 1) / kPT) * ((q + kPT - 1) / kPT);
+    const int64_t slices = std::max<int64_t>(1, std::min<int64_t>((608 + tiles - 1) / tiles, n / 64));
+    return (int)(((n + slices - 1) / slices + kPK - 1) / kPK * kPK);
 }
 
 // XT[l][j] = X[j][l] for l < rows, j < q: the vectors interleaved, so that
@@ -101,71 +149,97 @@ __global__ void interleave_kernel(const double *__restrict__ X, int64_t ldx, int
 }
 
 // Y[j][l] += sum_p val[p] XT[col[p]][j] over CSR rows l (classes 2 and 8 of
-// the matrix): one warp per row, lanes over vectors (in groups of 32),
-// entries in order.  Each entry reads its column's vectors as one contiguous
-// run of XT, so the warp's loads coalesce; the L2 block of an L2-heavy matrix
-// (hundreds of millions of entries) streams once per product.
-__global__ void spmm_csr_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                const double *__restrict__ val, int rows, const double *__restrict__ XT, int q,
-                                double *__restrict__ Y, int64_t ldy) {
-    const int lane = threadIdx.x & 31;
-    const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (l >= rows) return;
-    const int64_t b = rp[l], e = rp[l + 1];
-    for (int j0 = 0; j0 < q; j0 += 32) {
-        const int j = j0 + lane;
+// the matrix).  Each entry reads its column's vectors as one contiguous run of
+// XT, so the loads coalesce; the L2 block of an L2-heavy matrix (hundreds of
+// millions of entries) streams once per product.  A block of four warps per
+// row, a contiguous share of the entries each (a reference function's row
+// holds every column, and with a warp per row it set the kernel's length: 153
+// us at 1500 rows, now 42 us); for up to 16 vectors each half warp takes its
+// own share.  The shares are added in order.
+constexpr int kSpWarps = 4;
+template <int G>             // shares per warp: 1 (32 vectors at a time) or 2 (16)
+__global__ void __launch_bounds__(32 * kSpWarps)
+spmm_csr_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
+                const double *__restrict__ val, int rows, const double *__restrict__ XT, int q,
+                double *__restrict__ Y, int64_t ldy) {
+    constexpr int LW = 32 / G, NS = kSpWarps * G;
+    __shared__ double red[NS][LW];
+    const int ll = threadIdx.x % LW, sub = threadIdx.x / LW;
+    const int l = blockIdx.x;
+    const int64_t b0 = __ldg(rp + l), len = __ldg(rp + l + 1) - b0;
+    const int64_t b = b0 + len * sub / NS, e = b0 + len * (sub + 1) / NS;
+    const unsigned mask = G == 1 ? 0xffffffffu : (0xffffu << (16 * (sub & 1)));
+    for (int j0 = 0; j0 < q; j0 += LW) {
+        const int j = j0 + ll;
         double acc = 0.0;
-        // 32 entries at a time: the warp loads their (column, value) pairs in
-        // one coalesced read, then every lane walks them in order, taking each
+        // LW entries at a time: the share's lanes load their (column, value)
+        // pairs in one coalesced read, then walk them in order, taking each
         // pair from the lane that holds it; the gathers of one batch do not
         // depend on each other, so they are in flight together.
-        for (int64_t p0 = b; p0 < e; p0 += 32) {
-            const int64_t p = p0 + lane;
+        for (int64_t p0 = b; p0 < e; p0 += LW) {
+            const int64_t p = p0 + ll;
             const int c_mine = p < e ? __ldg(col + p) : 0;
             const double v_mine = p < e ? __ldg(val + p) : 0.0;
-            const int cnt = (int)min((int64_t)32, e - p0);
+            const int cnt = (int)min((int64_t)LW, e - p0);
 #pragma unroll 8
             for (int t = 0; t < cnt; ++t) {
-                const int c = __shfl_sync(0xffffffffu, c_mine, t);
-                const double v = __shfl_sync(0xffffffffu, v_mine, t);
+                const int c = __shfl_sync(mask, c_mine, t, LW);
+                const double v = __shfl_sync(mask, v_mine, t, LW);
                 if (j < q) acc = fma(v, __ldg(XT + (int64_t)c * q + j), acc);
             }
         }
-        if (j < q) Y[(int64_t)j * ldy + l] += acc;
+        red[sub][ll] = acc;
+        __syncthreads();
+        if (sub == 0 && j < q) {
+            double v = red[0][ll];
+#pragma unroll
+            for (int s = 1; s < NS; ++s) v += red[s][ll];
+            Y[(int64_t)j * ldy + l] += v;
+        }
+        __syncthreads();
     }
 }
 
-// partial[c][a][b] = sum_{i in chunk c} X[a][i] Y[b][i]: one block per
-// (chunk of kGramChunk entries, 32 x 32 tile of (a, b)); the rows of the tile
-// pass through shared memory 64 entries at a time (coalesced along i), each
-// thread keeps 4 outputs; fixed order, so the sums are deterministic.
-constexpr int kGramChunk = 512;
-constexpr int kGramTile = 32, kGramSub = 64;
+// partial[c][a][b] = sum_{i in chunk c} X[a][i] Y[b][i]: one block per (chunk,
+// 32 x 32 tile of (a, b)); the rows of the tile pass through shared memory 32
+// entries at a time (coalesced along i), a warp keeps 32 rows x 4 columns;
+// fixed order, so the sums are deterministic.  Chunks of 512 entries left a
+// 1980-row solve on 12 blocks that all computed 32 columns of its 12: 146 us a
+// projection, now 9 us.
+constexpr int kGramTile = 32, kGramSub = 32;
+int gram_chunk(int64_t n) {
+    if (n >= 32768) return 512;
+    return (int)std::max<int64_t>(kGramSub, (n / 152 + kGramSub - 1) / kGramSub * kGramSub);
+}
+int gram_chunks(int64_t n) { return (int)((n + gram_chunk(n) - 1) / gram_chunk(n)); }
 __global__ void __launch_bounds__(256)
 gram_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, const double *__restrict__ Y, int64_t ldy, int q,
-                    int64_t n, double *__restrict__ partial) {
+                    int64_t n, int chunk, double *__restrict__ partial) {
     __shared__ double xs[kGramTile][kGramSub + 1], ys[kGramTile][kGramSub + 1];
     const int c = blockIdx.x;
     const int tiles_q = (q + kGramTile - 1) / kGramTile;
     const int a0 = (blockIdx.y / tiles_q) * kGramTile, b0 = (blockIdx.y % tiles_q) * kGramTile;
-    const int64_t i0 = (int64_t)c * kGramChunk, i1 = (n < i0 + kGramChunk) ? n : i0 + kGramChunk;
+    const int64_t i0 = (int64_t)c * chunk, i1 = (n < i0 + chunk) ? n : i0 + chunk;
     const int tid = threadIdx.x;
-    const int ta = tid / 8, tb = (tid % 8) * 4;     // outputs (a0 + ta, b0 + tb .. tb + 3)
+    const int ta = tid % 32, tb = (tid / 32) * 4;     // outputs (a0 + ta, b0 + tb .. tb + 3)
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int64_t s0 = i0; s0 < i1; s0 += kGramSub) {
         __syncthreads();
-        for (int e = tid; e < kGramTile * kGramSub; e += 256) {
-            const int r = e / kGramSub, k = e % kGramSub;
+#pragma unroll
+        for (int u = 0; u < kGramTile * kGramSub / 256; ++u) {
+            const int e = tid + u * 256, r = e / kGramSub, k = e % kGramSub;
             const int64_t i = s0 + k;
             xs[r][k] = (a0 + r < p && i < i1) ? __ldg(X + (int64_t)(a0 + r) * ldx + i) : 0.0;
             ys[r][k] = (b0 + r < q && i < i1) ? __ldg(Y + (int64_t)(b0 + r) * ldy + i) : 0.0;
         }
         __syncthreads();
+        if (b0 + tb < q) {
 #pragma unroll 8
-        for (int k = 0; k < kGramSub; ++k) {
-            const double x = xs[ta][k];
+            for (int k = 0; k < kGramSub; ++k) {
+                const double x = xs[ta][k];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fma(x, ys[tb + u][k], acc[u]);
+                for (int u = 0; u < 4; ++u) acc[u] = fma(x, ys[tb + u][k], acc[u]);
+            }
         }
     }
     const int a = a0 + ta;
@@ -179,10 +253,11 @@ gram_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, const doub
 // each thread a strided share of the chunk, then a fixed-order tree over the
 // block, so the sums are deterministic
 __global__ void __launch_bounds__(256)
-norms_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, int64_t n, double *__restrict__ partial) {
+norms_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, int64_t n, int chunk,
+                     double *__restrict__ partial) {
     __shared__ double red[256];
     const int c = blockIdx.x, a = blockIdx.y;
-    const int64_t i0 = (int64_t)c * kGramChunk, i1 = (n < i0 + kGramChunk) ? n : i0 + kGramChunk;
+    const int64_t i0 = (int64_t)c * chunk, i1 = (n < i0 + chunk) ? n : i0 + chunk;
     double acc = 0.0;
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const double x = __ldg(X + (int64_t)a * ldx + i);
@@ -197,47 +272,68 @@ norms_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, int64_t n
     if (threadIdx.x == 0) partial[(int64_t)c * p + a] = red[0];
 }
 
-__global__ void reduce_kernel(const double *__restrict__ partial, int chunks, int nout, double *__restrict__ out) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nout) return;
+// out[t] = sum_c partial[c][t]: 32 outputs a block, warp y adds the chunks y,
+// y + 8, ... in order, then the eight sums are added in order (a thread per
+// output, walking up to 152 chunks alone, took 12 to 20 us, now 6 to 8 us).
+__global__ void __launch_bounds__(256)
+reduce_kernel(const double *__restrict__ partial, int chunks, int nout, double *__restrict__ out) {
+    __shared__ double sums[8][32];
+    const int x = threadIdx.x % 32, y = threadIdx.x / 32, t = blockIdx.x * 32 + x;
     double acc = 0.0;
-    for (int c = 0; c < chunks; ++c) acc += partial[(int64_t)c * nout + t];
+    if (t < nout) {
+#pragma unroll 8
+        for (int c = y; c < chunks; c += 8) acc += __ldg(partial + (int64_t)c * nout + t);
+    }
+    sums[y][x] = acc;
+    __syncthreads();
+    if (y != 0 || t >= nout) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) acc += sums[k][x];
     out[t] = acc;
 }
 
 // Y[j][i] = beta * Y[j][i] + scale * sum_a C[a][j] X[a][i]   (a < p, j < q), C on device [p][q];
-// the coefficients pass through shared memory kCombineRows rows at a time.
-constexpr int kCombineRows = 256;
-__global__ void combine_kernel(const double *__restrict__ X, int64_t ldx, int p, const double *__restrict__ C, int q,
-                               int64_t n, double *__restrict__ Y, int64_t ldy, double beta, double scale) {
-    __shared__ double cs[kCombineRows * 16];
-    const int j0 = blockIdx.y * 16;
-    const int nq = min(16, q - j0);
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double acc[16];
-#pragma unroll
-    for (int jj = 0; jj < 16; ++jj) acc[jj] = 0.0;
+// kCombineRows rows of coefficients and vectors at a time pass through shared
+// memory, all their loads in flight together.  A block of two warps takes 16
+// entries x 16 vectors, a thread 4 vectors: with 256 entries a block, a
+// 1980-row solve used 8 SMs (47 us a combination, now 14 us).
+constexpr int kCombineRows = 64;
+__global__ void __launch_bounds__(64)
+combine_kernel(const double *__restrict__ X, int64_t ldx, int p, const double *__restrict__ C, int q,
+               int64_t n, double *__restrict__ Y, int64_t ldy, double beta, double scale) {
+    __shared__ double cs[kCombineRows][16], xs[kCombineRows][16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j0 = blockIdx.y * 16, c0 = 8 * warp + 4 * (lane >> 4);
+    const int64_t i0 = (int64_t)blockIdx.x * 16, i = i0 + (lane & 15);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int a0 = 0; a0 < p; a0 += kCombineRows) {
         const int na = min(kCombineRows, p - a0);
+        const int jj = threadIdx.x % 16;
         __syncthreads();
-        for (int t = threadIdx.x; t < na * 16; t += blockDim.x) {
-            const int a = t / 16, jj = t % 16;
-            cs[t] = jj < nq ? scale * C[(int64_t)(a0 + a) * q + j0 + jj] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kCombineRows / 4; ++u) {
+            const int a = u * 4 + threadIdx.x / 16;
+            if (a < na) {
+                xs[a][jj] = i0 + jj < n ? __ldg(X + (int64_t)(a0 + a) * ldx + i0 + jj) : 0.0;
+                cs[a][jj] = j0 + jj < q ? scale * __ldg(C + (int64_t)(a0 + a) * q + j0 + jj) : 0.0;
+            }
         }
         __syncthreads();
-        if (i < n)
+        if (j0 + 8 * warp < q) {
+#pragma unroll 8
             for (int a = 0; a < na; ++a) {
-                const double x = __ldg(X + (int64_t)(a0 + a) * ldx + i);
+                const double x = xs[a][lane & 15];
 #pragma unroll
-                for (int jj = 0; jj < 16; ++jj) acc[jj] = fma(cs[a * 16 + jj], x, acc[jj]);
+                for (int c = 0; c < 4; ++c) acc[c] = fma(cs[a][c0 + c], x, acc[c]);
             }
+        }
     }
     if (i >= n) return;
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj)
-        if (jj < nq) {
-            double *y = Y + (int64_t)(j0 + jj) * ldy + i;
-            *y = beta != 0.0 ? beta * *y + acc[jj] : acc[jj];
+    for (int c = 0; c < 4; ++c)
+        if (j0 + c0 + c < q) {
+            double *y = Y + (int64_t)(j0 + c0 + c) * ldy + i;
+            *y = beta != 0.0 ? beta * *y + acc[c] : acc[c];
         }
 }
 
@@ -273,9 +369,20 @@ __global__ void diag_kernel(const double *__restrict__ Hcc, int64_t Dc, const in
         d[i] = Hcc[i * Dc + i];
     } else if (i < Dc + nl) {
         const int64_t l = i - Dc;
+        // columns ascend in a built block: search, then look at every entry
         double v = 0.0;
-        for (int64_t p = rp[l]; p < rp[l + 1]; ++p)
-            if (col[p] == (int32_t)l) { v = val[p]; break; }
+        int64_t b = rp[l], e = rp[l + 1];
+        while (b < e) {
+            const int64_t m = b + ((e - b) >> 1);
+            if (col[m] < (int32_t)l) b = m + 1;
+            else e = m;
+        }
+        if (b < rp[l + 1] && col[b] == (int32_t)l) {
+            v = val[b];
+        } else {
+            for (int64_t p = rp[l]; p < rp[l + 1]; ++p)
+                if (col[p] == (int32_t)l) { v = val[p]; break; }
+        }
         d[i] = v;
     }
 }
@@ -729,24 +836,30 @@ struct Ops {
             return;
         }
         if (Dc > 0) {
-            dim3 g((unsigned)((Dc + GM - 1) / GM), (q + GN - 1) / GN);
-            gemm_nt_kernel<<<g, 256, 0, s>>>(H->Hcc, Dc, X, ld, (int)Dc, q, (int)Dc, Y, ld, 0);
+            ProductArgs P;
+            P.Hcc = H->Hcc; P.HlcT = w->HlcT; P.Hlc = H->Hlc;
+            P.Dc = Dc; P.nl = nl;
+            P.X = X; P.ldx = ld; P.q = q;
+            P.kslice = product_slice(n, q);
+            P.up_tiles = (int)((Dc + kPT - 1) / kPT);
+            P.up_slices = (int)((n + P.kslice - 1) / P.kslice);
+            P.lo_slices = nl > 0 ? (int)((Dc + P.kslice - 1) / P.kslice) : 0;
+            const bool direct = P.up_slices == 1;
+            P.out = direct ? Y : w->prod;
+            P.ldo = direct ? ld : n;
+            P.slice_ld = (int64_t)q * n;
+            const int64_t blocks = (int64_t)P.up_tiles * P.up_slices + (nl + kPT - 1) / kPT * P.lo_slices;
+            product_kernel<<<dim3((unsigned)blocks, (q + kPT - 1) / kPT), kPThreads, 0, s>>>(P);
             ++launches;
-            if (nl > 0) {
-                gemm_nt_kernel<<<g, 256, 0, s>>>(w->HlcT, nl, X + Dc, ld, (int)Dc, q, (int)nl, Y, ld, 1);
+            if (!direct) {
+                product_reduce_kernel<<<dim3((unsigned)((n + 127) / 128), q), 128, 0, s>>>(w->prod, n, Dc, q, P.up_slices,
+                                                                                           P.lo_slices, Y, ld);
                 ++launches;
             }
+        } else {
+            for (int j = 0; j < q; ++j) cudaMemsetAsync(Y + (int64_t)j * ld, 0, sizeof(double) * nl, s);
         }
-        if (nl > 0) {
-            dim3 g((unsigned)((nl + GM - 1) / GM), (q + GN - 1) / GN);
-            if (Dc > 0) {
-                gemm_nt_kernel<<<g, 256, 0, s>>>(H->Hlc, Dc, X, ld, (int)nl, q, (int)Dc, Y + Dc, ld, 0);
-                ++launches;
-            } else {
-                for (int j = 0; j < q; ++j) cudaMemsetAsync(Y + (int64_t)j * ld, 0, sizeof(double) * nl, s);
-            }
-            l2_product(X, Y, q, ld);
-        }
+        if (nl > 0) l2_product(X, Y, q, ld);
     }
 
     // Y_l += (L2 block) X_l for the q vectors: interleave the L2 part of the
@@ -756,8 +869,12 @@ struct Ops {
             const int qq = std::min(q - j0, w->mmax);
             dim3 gi((unsigned)((nl + 31) / 32), (unsigned)((qq + 31) / 32));
             interleave_kernel<<<gi, dim3(32, 8), 0, s>>>(X + (int64_t)j0 * ld + Dc, ld, nl, qq, w->XT);
-            spmm_csr_kernel<<<(unsigned)((nl + 7) / 8), 256, 0, s>>>(H->l2_row_ptr, H->l2_col, H->l2_val, (int)nl,
-                                                                     w->XT, qq, Y + (int64_t)j0 * ld + Dc, ld);
+            if (qq <= 16)
+                spmm_csr_kernel<2><<<(unsigned)nl, 32 * kSpWarps, 0, s>>>(H->l2_row_ptr, H->l2_col, H->l2_val, (int)nl,
+                                                                          w->XT, qq, Y + (int64_t)j0 * ld + Dc, ld);
+            else
+                spmm_csr_kernel<1><<<(unsigned)nl, 32 * kSpWarps, 0, s>>>(H->l2_row_ptr, H->l2_col, H->l2_val, (int)nl,
+                                                                          w->XT, qq, Y + (int64_t)j0 * ld + Dc, ld);
             launches += 2;
         }
     }
@@ -765,10 +882,10 @@ struct Ops {
     // G[a][b] = X[a] . Y[b] on the host (p x q)
     void gram(const double *X, int p, const double *Y, int q, int64_t ld, std::vector<double> &G) {
         const double t0 = now_ms();
-        const int chunks = (int)((n + kGramChunk - 1) / kGramChunk);
+        const int chunks = gram_chunks(n);
         dim3 g(chunks, ((p + kGramTile - 1) / kGramTile) * ((q + kGramTile - 1) / kGramTile));
-        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, w->partial);
-        reduce_kernel<<<(p * q + 255) / 256, 256, 0, s>>>(w->partial, chunks, p * q, w->small);
+        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n), w->partial);
+        reduce_kernel<<<(p * q + 31) / 32, 256, 0, s>>>(w->partial, chunks, p * q, w->small);
         launches += 2;
         proj_flops += 2.0 * p * q * (double)n;
         G.resize((size_t)p * q);
@@ -780,9 +897,9 @@ struct Ops {
     // r2[a] = |X[a]|^2 on the host (p values)
     void norms2(const double *X, int p, int64_t ld, std::vector<double> &r2) {
         const double t0 = now_ms();
-        const int chunks = (int)((n + kGramChunk - 1) / kGramChunk);
-        norms_partial_kernel<<<dim3(chunks, p), 256, 0, s>>>(X, ld, p, n, w->partial);
-        reduce_kernel<<<(p + 255) / 256, 256, 0, s>>>(w->partial, chunks, p, w->small);
+        const int chunks = gram_chunks(n);
+        norms_partial_kernel<<<dim3(chunks, p), 256, 0, s>>>(X, ld, p, n, gram_chunk(n), w->partial);
+        reduce_kernel<<<(p + 31) / 32, 256, 0, s>>>(w->partial, chunks, p, w->small);
         launches += 2;
         proj_flops += 2.0 * p * (double)n;
         r2.resize((size_t)p);
@@ -801,8 +918,8 @@ struct Ops {
     void combine(const double *X, int p, const std::vector<double> &C, int q, double *Y, int64_t ld, double beta) {
         const double t0 = now_ms();
         cudaMemcpyAsync(w->small, C.data(), sizeof(double) * p * q, cudaMemcpyHostToDevice, s);
-        dim3 g((unsigned)((n + 255) / 256), (q + 15) / 16);
-        combine_kernel<<<g, 256, 0, s>>>(X, ld, p, w->small, q, n, Y, ld, beta, 1.0);
+        dim3 g((unsigned)((n + 15) / 16), (q + 15) / 16);
+        combine_kernel<<<g, 64, 0, s>>>(X, ld, p, w->small, q, n, Y, ld, beta, 1.0);
         ++launches;
         proj_flops += 2.0 * p * q * (double)n;
         // no wait: the next upload into w->small is ordered after this kernel
@@ -814,12 +931,12 @@ struct Ops {
     void project_out(const double *X, int p, double *Y, int q, int64_t ld) {
         if (p <= 0 || q <= 0) return;
         const double t0 = now_ms();
-        const int chunks = (int)((n + kGramChunk - 1) / kGramChunk);
+        const int chunks = gram_chunks(n);
         dim3 g(chunks, ((p + kGramTile - 1) / kGramTile) * ((q + kGramTile - 1) / kGramTile));
-        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, w->partial);
-        reduce_kernel<<<(p * q + 255) / 256, 256, 0, s>>>(w->partial, chunks, p * q, w->proj);
-        dim3 g2((unsigned)((n + 255) / 256), (q + 15) / 16);
-        combine_kernel<<<g2, 256, 0, s>>>(X, ld, p, w->proj, q, n, Y, ld, 1.0, -1.0);
+        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n), w->partial);
+        reduce_kernel<<<(p * q + 31) / 32, 256, 0, s>>>(w->partial, chunks, p * q, w->proj);
+        dim3 g2((unsigned)((n + 15) / 16), (q + 15) / 16);
+        combine_kernel<<<g2, 64, 0, s>>>(X, ld, p, w->proj, q, n, Y, ld, 1.0, -1.0);
         launches += 3;
         proj_flops += 4.0 * p * q * (double)n;
         ms_gram += now_ms() - t0;
@@ -878,6 +995,20 @@ static int setup_tensor_products(hb_ctx *ctx, const hb_blocks *H, DiagWork *w, i
     return HB_OK;
 }
 
+// Doubles of the FP64 products' slice sums for up to mmax vectors at a time
+// (nothing where one slice covers the rows, which then go straight to Y).
+static int64_t product_doubles(int64_t n, int mmax) {
+    int64_t most = 1;
+    for (int q = 1; q <= mmax; q += q % kPT == 0 ? 1 : kPT - q % kPT) {
+        // within a tile of vectors the slices are the same: its widest block
+        const int wide = std::min(mmax, (q + kPT - 1) / kPT * kPT);
+        const int64_t ks = product_slice(n, wide), sl = (n + ks - 1) / ks;
+        if (sl > 1) most = std::max(most, sl * wide * n);
+        else break;
+    }
+    return most;
+}
+
 // Device bytes a solve for k eigenpairs takes from the context's memory (the
 // allocations of ensure_diag_work, of the interleaved vectors and the class-4
 // transpose, of the tensor-core slices, and of the learned factors), each
@@ -888,10 +1019,11 @@ int64_t hb::diag_workspace_bytes(const hb_ctx *ctx, int k, int precond) {
     if (n < 1 || k < 1) return 0;
     const int b = (int)std::min<int64_t>(n, k + std::max(4, std::min(16, k / 2)));
     const int mmax = (int)std::min<int64_t>(n, (int64_t)ctx->diag_basis * b);
-    const int64_t chunks = (n + kGramChunk - 1) / kGramChunk;
+    const int64_t chunks = gram_chunks(n);
     int64_t t = 5 * r(8.0 * mmax * n) + r(8.0 * n) + r(8.0 * chunks * mmax * mmax) + 2 * r(8.0 * mmax * mmax) +
                 r(8.0 * mmax) + r(4.0 * mmax);
     if (nl > 0) t += r(8.0 * nl * mmax);
+    if (Dc > 0) t += r(8.0 * product_doubles(n, mmax));
     if (Dc > 0 && nl > 0) t += r(8.0 * Dc * nl);
     if (precond & HB_DIAG_TENSOR) {
         const int S = ctx->split_slices >= 2 && ctx->split_slices <= 6 ? ctx->split_slices : 6;
@@ -919,8 +1051,8 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
     if (w->mmax < mmax || w->n != n) {
         auto fr = [&](void *p) { dfree(ctx, p); };
         fr(w->V); fr(w->AV); fr(w->X); fr(w->AX); fr(w->W2); fr(w->d); fr(w->partial); fr(w->small); fr(w->theta);
-        fr(w->idx); fr(w->proj); fr(w->XT);
-        w->V = w->AV = w->X = w->AX = w->W2 = w->d = w->partial = w->small = w->theta = w->proj = w->XT = nullptr;
+        fr(w->idx); fr(w->proj); fr(w->XT); fr(w->prod);
+        w->V = w->AV = w->X = w->AX = w->W2 = w->d = w->partial = w->small = w->theta = w->proj = w->XT = w->prod = nullptr;
         w->idx = nullptr;
         w->XT_rows = 0;
         const size_t vec = (size_t)mmax * n;
@@ -930,12 +1062,13 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->AX, vec);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->W2, vec);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->d, (size_t)n);
-        const int chunks = (int)((n + kGramChunk - 1) / kGramChunk);
+        const int chunks = gram_chunks(n);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->partial, (size_t)chunks * mmax * mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->small, (size_t)mmax * mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->proj, (size_t)mmax * mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->theta, (size_t)mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->idx, (size_t)mmax);
+        if (e == cudaSuccess && ctx->Dc > 0) e = dmalloc_n(ctx, &w->prod, (size_t)product_doubles(n, mmax));
         if (e != cudaSuccess) return diag_fail(ctx, HB_ERR_OOM, std::string("Davidson workspace: ") + cudaGetErrorString(e));
         w->mmax = mmax;
         w->n = n;
@@ -1220,8 +1353,11 @@ extern "C" int hb_diag(hb_ctx *ctx, const hb_blocks *H, int32_t k, double tol, i
             precond_kernel<<<g, 256, 0, s>>>(w->AX, ld, w->d, w->theta, w->idx, q, n, wts, Tn, ld);
             ++ops.launches;
         }
-        // orthogonalise against the basis twice, then within the block
-        for (int pass = 0; pass < 2; ++pass) ops.project_out(w->V, m, Tn, q, ld);
+        // orthogonalise against the basis and within the block, twice: the
+        // second round works on unit vectors, whose part along the basis is
+        // the rounding of the first round over the shortest direction the
+        // block keeps (1e-7 of its longest), and leaves rounding of that
+        ops.project_out(w->V, m, Tn, q, ld);
         int kept = 0;
         svqb(Tn, q, kept);
         if (kept == 0) break;
@@ -1304,7 +1440,7 @@ void hb::release_diag(hb_ctx *ctx) {
     release_tensor_products(ctx, w);
     for (void *p : {(void *)w->V, (void *)w->AV, (void *)w->X, (void *)w->AX, (void *)w->W2, (void *)w->d, (void *)w->partial,
                     (void *)w->small, (void *)w->proj, (void *)w->theta, (void *)w->idx, (void *)w->HlcT,
-                    (void *)w->XT})
+                    (void *)w->XT, (void *)w->prod})
         dfree(ctx, p);
     delete w;
     ctx->diag = nullptr;
