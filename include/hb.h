@@ -140,7 +140,9 @@ typedef struct {
 } hb_problem;
 
 typedef struct {
-    int32_t split_slices;     /* mixed path: bf16 slices per operand (2..6), 0 = default (6) */
+    int32_t split_slices;     /* mixed path: bf16 slices per operand (2..6); 0 = default: 5 of 9 bits in the
+                                 expansion (at least as accurate as 6 of 7 bits), 6 in class 4 and in
+                                 hb_diag's products */
     int32_t validate;         /* 0 = skip the O(n^2) input checks */
     int32_t autotune;         /* 1 = time the launch-shape candidates on the first build
                                  (results are bit-identical for every candidate) */
@@ -276,7 +278,9 @@ int hb_set_workspace(hb_ctx *ctx, void *dev_ptr, size_t bytes);
 int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
 
 /* Build every class (1-8) into the caller's device buffers.  precision:
-   HB_FP64 (double arithmetic throughout) or HB_MIXED: the continuum-continuum
+   HB_FP64 (double arithmetic; the sums of Eq. 7 exact sums of 62-bit products
+   of the operands, rounded once, on the tensor cores where the operand slices
+   fit the memory) or HB_MIXED: the continuum-continuum
    contraction (Eq. 7), and class 4 (Eq. 5) of groups of 32..64 states (see
    hb_options.class4_path), on bf16 tensor cores with split operands, exact
    FP32 accumulation and double-float recovery; the target-side contraction

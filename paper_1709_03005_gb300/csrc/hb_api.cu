@@ -441,7 +441,7 @@ int stage_problem(hb_ctx *ctx, const hb_problem *p, const hb_options *o, cudaStr
     ctx->n_to = p->n_to; ctx->n_co = p->n_co; ctx->n_orb = p->n_to + p->n_co;
     ctx->n_elec = p->n_elec; ctx->W = p->n_words; ctx->cont_spin = p->cont_spin;
     ctx->n_groups = p->n_groups; ctx->n_l2 = p->n_l2; ctx->e_core = p->e_core;
-    ctx->split_slices = (o && o->split_slices > 0) ? o->split_slices : 6;
+    if (o && o->split_slices > 0) ctx->split_slices = ctx->expand_slices = o->split_slices;
     ctx->autotune = (o && o->autotune) ? 1 : 0;
     if (o) {
         ctx->force_tile = o->split_tile;
@@ -709,6 +709,8 @@ extern "C" int64_t hb_group_offset(const hb_ctx *ctx, int32_t g) {
     return g == ctx->n_groups ? ctx->Dc : ctx->groups[g].row_off;
 }
 
+static const char *const kF64Timeout = "a tensor-core kernel of an FP64 build gave up waiting";
+
 extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *out, hb_stats *st,
                                void *stream) {
     if (!ctx || !out) return fail(ctx, HB_ERR_INVALID_ARG, "NULL argument");
@@ -744,6 +746,9 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
         int rc = plan_set_outputs(plan, out, &err, s);
         if (rc != HB_OK) return fail(ctx, rc, err);
     }
+    // an FP64 build is left running; a wait that gave up in it is reported by
+    // the call that waits for it, or by the next one
+    if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
     int launches = 0;
     int rc = plan_run(plan, s, true, false, &launches, &err);
     if (rc != HB_OK) return fail(ctx, rc, err);
@@ -755,7 +760,10 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
         if (word != 0)
             return fail(ctx, HB_ERR_TIMEOUT, "a tensor-core kernel (split expansion, codes 1-6, or class 4, codes 21-26) gave up waiting (code " + std::to_string(word) + ")");
     }
-    if (st) plan_stats(plan, st);
+    if (st) {
+        plan_stats(plan, st);                    // waits for the build
+        if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
+    }
     return HB_OK;
 }
 
@@ -927,6 +935,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
         if (precision == HB_MIXED && P.A_df) split_df(P.A, (int64_t)n, P.A_df, s);
         off += (int64_t)n;
     }
+    if (plan_host_error(p)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
     plan_set_phase(p, 2);
     std::string err;
     int launches = 0;
@@ -977,6 +986,7 @@ extern "C" int hb_workspace_size(hb_ctx *ctx, int32_t precision, int32_t diag_k,
     // the autotuner's timing buffers and the allocator's alignment
     need += (16 << 20) + need / 64;
     ctx->pool.measured = need;
+    ctx->pool.measured_f64 = precision == HB_FP64;
     *bytes = need;
     return HB_OK;
 }

@@ -62,6 +62,7 @@ struct DevPool {
     size_t live_bytes = 0, peak_bytes = 0;
     size_t init_allocs = 0;                      // hb_ctx::allocs made by hb_init
     int64_t measured = 0;                        // the last hb_workspace_size result
+    bool measured_f64 = false;                   // and whether it was for an FP64 build
 };
 cudaError_t dmalloc(hb_ctx *ctx, void **p, size_t bytes);
 void dfree(hb_ctx *ctx, void *p);
@@ -105,7 +106,8 @@ struct hb_ctx {
     int device = 0;
     int n_to = 0, n_co = 0, n_orb = 0, n_elec = 0, W = 1, cont_spin = 0, n_groups = 0, n_l2 = 0;
     double e_core = 0.0;
-    int split_slices = 5;
+    int split_slices = 6;    // bf16 slices of the Davidson products and of class 4 (base-128 and -256 digits)
+    int expand_slices = 5;   // and of the mixed expansion (base-512 digits)
     int autotune = 0;
     int force_tile = 0, force_c4_states = 0, force_c4_threads = 0;   // 0: chosen by the plan
     int force_cols = 0;      // tensor-core expansion tile width (32, 64, 128); 0: chosen by the plan

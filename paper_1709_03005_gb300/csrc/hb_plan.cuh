@@ -24,6 +24,8 @@ bool plan_is_shard(const hb::Plan *p, int precision, int r, int n);
 int plan_set_outputs(hb::Plan *p, const hb_blocks *outs, std::string *err, cudaStream_t s);
 bool plan_outputs_equal(const hb::Plan *p, const hb_blocks *outs);
 int plan_precision(const hb::Plan *p);
+// FP64 build on the tensor cores: nonzero once if a wait in a finished build gave up
+int plan_host_error(hb::Plan *p);
 // Issue every stage on stream s.  timing: record the stage events (as graph
 // event nodes when capture is set).  *launches: kernels launched.
 int plan_run(hb::Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, std::string *err);

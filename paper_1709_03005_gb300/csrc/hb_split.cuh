@@ -8,16 +8,19 @@
 #include "hb_api_internal.cuh"
 #include "hb_tasks.cuh"
 
-// Panel slices and tensor map of a context (or of the context it borrows from).
-int mixed_prepare(hb_ctx *ctx, cudaStream_t s);
+// Panel slices and tensor maps of a context (or of the context it borrows from)
+// for one precision.
+int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s);
 // Identity of the panel a context reads (equal for contexts sharing integrals).
-const void *mixed_panel_key(const hb_ctx *ctx);
-int mixed_slices(const hb_ctx *ctx);
+const void *mixed_panel_key(const hb_ctx *ctx, int precision);
+int mixed_slices(const hb_ctx *ctx, int precision);
 // Diagonal panel rows (j, j) as float pairs [n_co][Kpad].
 const float2 *mixed_panel_diag(const hb_ctx *ctx);
 // Coefficient slices [S][Kpad/64][rows][64] bf16 and their tensor maps
 // tm[0..3]: 32-K stages at tile widths 32, 64, 128, and 64-K stages at 128.
-int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, CUtensorMap *tm, std::string *err);
+// exps (or null): the rows' exponents, kept apart from the slices.
+int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int16_t **exps, CUtensorMap *tm,
+                     std::string *err);
 int64_t blocks_split(int cn, int cnp, int N, int lg, int bn);
 int split_ntn(int N, int bn);
 // tile width (32, 64, 128) for a merged block of N columns over kblocks 64-wide
@@ -25,23 +28,25 @@ int split_ntn(int N, int bn);
 int split_cols_choice(int N, int kblocks, int force);
 // K stage (32, 64) of a launch of tile width bn over kblocks 64-wide K blocks
 int split_kstage_choice(int bn, int kblocks, int force);
+// tile width (32, 64) of the FP64 build
+int split_f64_cols_choice(int N, int force);
 int split_jpt(int cnp, int lg);
 int split_tile_heuristic(int cn, int cnp);
 // coefficient rows of Kin labels into slices of Kout columns, column k being
 // label perm[k] (null: label k)
 int g_slice(const hb::Grouped<hb::SliceTask> &g, int64_t R, int Kin, int Kout, const int32_t *perm, int S,
-            int skip_col, void *out, cudaStream_t s);
+            int skip_col, void *out, int16_t *exps, cudaStream_t s);
 // lg: tile arrangement (3..5, see SplitTask) and bn: tile width (32, 64,
 // 128); every task of g must use both.  tm_coef: the four coefficient maps.
 // kblocks: 64-wide K blocks of the panel rows; coef_planes: K blocks per
 // slice of the coefficient slices (the task's kc0 selects its label class)
 // shard_r, shard_n: the launch takes tiles shard_r, shard_r + shard_n, ... only
-int g_split(const hb_ctx *panel_ctx, int lg, int bn, const CUtensorMap *tm_coef, const hb::Grouped<hb::SplitTask> &g,
-            int kblocks, int coef_planes, const hb::ExpCol *cols, int *err, cudaStream_t s, int shard_r = 0,
-            int shard_n = 1);
+int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef,
+            const int16_t *coef_exps, const hb::Grouped<hb::SplitTask> &g, int kblocks, int coef_planes,
+            const hb::ExpCol *cols, int *err, cudaStream_t s, int shard_r = 0, int shard_n = 1);
 int64_t blocks_diag_rows(int j_lo, int j_hi, int n_nn);
 int diag_rows_ny(int n_nn);
-int g_diag_rows(const hb::Grouped<hb::DRTask> &g, cudaStream_t s);
+int g_diag_rows(const hb::Grouped<hb::DRTask> &g, int dfloat, cudaStream_t s);
 
 // Dense split-precision GEMM (Davidson block products).  An operand holds bf16
 // slices of R rows over Kpad columns, [S][Kpad/64][R][64], and its tensor map.

@@ -141,13 +141,13 @@ struct ATask {          // contracted coefficient rows A[(n,n')][k]
 // pair of one Hamiltonian.  The Eq. 7 GEMMs of all group pairs that read the
 // same continuum rectangle of the panel are merged into one, whose columns are
 // the state pairs of all of them; each column scatters to its own matrix.
-struct ExpCol {
+struct alignas(16) ExpCol {
+    double *lower, *upper;    // element (jj, jj') of the rectangle: lower[jj ld + jj'] and its mirror upper[jj' ld + jj]
+    int32_t ld;               // row length of its matrix
+    int32_t jmin;             // written where jj - jj' >= jmin (the lower triangle within one target group)
     const double *arow;       // contracted coefficient row A[(n,n')][0..Kpad)
-    double *H;                // continuum block of its Hamiltonian (ld x ld)
-    int64_t rbase, cbase;     // row_off + n cn, col_off + n' cn'
-    int64_t ld;
-    int32_t same, pad;        // same target group: write the lower triangle and mirror
 };
+static_assert(sizeof(ExpCol) == 32, "read as two 16-byte words");
 
 struct XTask {          // FP64 expansion of one merged block (Eq. 7)
     const double *P;
@@ -171,7 +171,7 @@ struct SplitTask {      // one merged block on the tensor cores
     int64_t col0;             // first column in the ExpCol table
 };
 
-struct DRTask {         // rows with j == j' of one group pair, in double-float
+struct DRTask {         // rows with j == j' of one group pair, in double-float or FP64
     const float2 *Pd;         // panel rows (j, j) as float pairs [n_co][Kpad]
     const float2 *A;          // coefficient rows as float pairs [n_nn][Ka]
     const int32_t *nn;
@@ -179,6 +179,7 @@ struct DRTask {         // rows with j == j' of one group pair, in double-float
     int n_nn, Kpad, Ka, n_co, j_lo, j_hi, cf, cn, cfp, cnp, same, ny;
     int64_t row_off, col_off, ld;
     double *H;
+    const double *P64, *A64;  // FP64 build: the panel and the coefficient rows
 };
 
 struct C4Task {         // class 4 of one target group against the L2 functions
@@ -295,8 +296,8 @@ int64_t blocks_gdiag_reduce(int n_to, int ns);
 size_t smem_gdiag(int ns);
 // shard_r, shard_n: only the blocks shard_r, shard_r + shard_n, ... of the grid do their tile
 int g_expand_fp64(const Grouped<XTask> &g, const ExpCol *cols, cudaStream_t s, int shard_r = 0, int shard_n = 1);
-// dfloat = 0: FP64 (128 threads, 32 states a pass); 1: double-float with
-// ns_tile states a pass (a multiple of 8 up to 64) and jt threads a block (32, 64 or 128)
+// dfloat = 0: FP64; 1: double-float; ns_tile states a pass (a multiple of 4 up
+// to 32, or in double-float of 8 up to 64) and jt threads a block (32, 64 or 128)
 int g_class4(const Grouped<C4Task> &g, int W, int dfloat, int ns_tile, int jt, cudaStream_t s);
 void class4_shape(int ns, int cn, int *ns_tile, int *jt);
 

@@ -102,6 +102,7 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
         cudaEventCreate(&e1);
         cudaEventRecord(e0, s);
     }
+    if (plan_host_error(b->plan)) return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel of an FP64 build gave up waiting");
     cudaError_t e = cudaGraphLaunch(b->exec, s);
     if (e != cudaSuccess) return bfail(HB_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(e));
     if (st) {

@@ -25,7 +25,6 @@ namespace hb {
 namespace {
 
 constexpr int kJ = 128;
-constexpr int kNS = 32;
 constexpr int kBatch = 32;
 
 __device__ __forceinline__ double x4(const Ints &I, int a, int b, int c, int j) {
@@ -72,13 +71,18 @@ __device__ double prototype_value(const Ints &I, const hb_pair &r, const uint64_
     return r.phase * (dir - exc);
 }
 
-template <int W>
+// Block = blockDim.x continuum orbitals of one L2 row; NS target states per
+// pass.  FP64 FMAs for states beyond the group's cost as much as the others on
+// this pipe: with one tile of 32 states and 128 threads, 20 states x 150
+// orbitals took 1.19 ms and 7 x 37 0.16 ms, now 0.53 and 0.05.
+template <int W, int NS>
 __global__ void __launch_bounds__(kJ)
 class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
-    __shared__ double cs[kBatch][kNS];
+    __shared__ double cs[kBatch][NS];
     __shared__ hb_pair rs[kBatch];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const C4Task &T = tasks[ti];
+    const int JT = blockDim.x;
     const Ints I = T.I;
     const hb_pair *__restrict__ pairs = T.pairs;
     const uint64_t *__restrict__ dets = T.dets;
@@ -86,22 +90,22 @@ class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk,
     const int ns = T.ns, cf = T.cf, cn = T.cn, cont_spin = T.cont_spin;
     const int lb = (int)(blockIdx.x - blk[ti]);
     const int l = lb / T.ny;
-    const int jl = (lb % T.ny) * kJ + threadIdx.x;
+    const int jl = (lb % T.ny) * JT + threadIdx.x;
     const bool jv = jl < cn;
     const int j = cf + (jv ? jl : 0);
     const int64_t b = T.row_ptr[l], e = T.row_ptr[l + 1];
-    for (int n0 = 0; n0 < ns; n0 += kNS) {
-        const int nc = min(kNS, ns - n0);
-        double acc[kNS];
+    for (int n0 = 0; n0 < ns; n0 += NS) {
+        const int nc = min(NS, ns - n0);
+        double acc[NS];
 #pragma unroll
-        for (int n = 0; n < kNS; ++n) acc[n] = 0.0;
+        for (int n = 0; n < NS; ++n) acc[n] = 0.0;
         for (int64_t p0 = b; p0 < e; p0 += kBatch) {
             const int cnt = (int)(e - p0 < kBatch ? e - p0 : kBatch);
             __syncthreads();
-            if (threadIdx.x < cnt) rs[threadIdx.x] = pairs[p0 + threadIdx.x];
+            for (int t = threadIdx.x; t < cnt; t += JT) rs[t] = pairs[p0 + t];
             __syncthreads();
-            for (int t = threadIdx.x; t < cnt * kNS; t += kJ) {
-                const int i = t / kNS, n = t % kNS;
+            for (int t = threadIdx.x; t < cnt * NS; t += JT) {
+                const int i = t / NS, n = t % NS;
                 cs[i][n] = n < nc ? C[(int64_t)rs[i].col * ns + n0 + n] : 0.0;
             }
             __syncthreads();
@@ -109,13 +113,13 @@ class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk,
                 const hb_pair r = rs[i];
                 const double y = prototype_value<W>(I, r, dets + (int64_t)r.col * 2 * W, j, cont_spin);
 #pragma unroll
-                for (int n = 0; n < kNS; ++n) acc[n] = fma(cs[i][n], y, acc[n]);
+                for (int n = 0; n < NS; ++n) acc[n] = fma(cs[i][n], y, acc[n]);
             }
         }
         if (jv) {
             double *out = T.Hlc + (int64_t)l * T.ld + T.col_off + jl;
 #pragma unroll
-            for (int n = 0; n < kNS; ++n)
+            for (int n = 0; n < NS; ++n)
                 if (n < nc) out[(int64_t)(n0 + n) * cn] = acc[n];
         }
     }
@@ -254,7 +258,7 @@ __global__ void split_df_kernel(const double *__restrict__ x, int64_t n, float2 
 int class4_ny(int cn, int jt) { return (cn + jt - 1) / jt; }
 int64_t blocks_class4(int n_l2, int cn, int jt) { return cn > 0 ? (int64_t)n_l2 * class4_ny(cn, jt) : 0; }
 
-// State tile and thread count of the mixed kernel for a group (host side):
+// State tile and thread count of either kernel for a group (host side):
 // the fewest passes over the states, then the smallest tile; the continuum
 // tile that leaves the fewest idle threads (ties to the larger block).
 void class4_shape(int ns, int cn, int *ns_tile, int *jt) {
@@ -281,13 +285,25 @@ void split_df(const double *x, int64_t n, float2 *out, cudaStream_t s) {
 int g_class4(const Grouped<C4Task> &g, int W, int dfloat, int ns_tile, int jt, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
     const unsigned grid = (unsigned)g.blocks;
+#define HB_C4(WW)                                                                          \
+    switch (ns_tile) {                                                                     \
+        case 4: class4_kernel<WW, 4><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;      \
+        case 8: class4_kernel<WW, 8><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;      \
+        case 12: class4_kernel<WW, 12><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+        case 16: class4_kernel<WW, 16><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+        case 20: class4_kernel<WW, 20><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+        case 24: class4_kernel<WW, 24><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+        case 28: class4_kernel<WW, 28><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+        default: class4_kernel<WW, 32><<<grid, jt, 0, s>>>(g.tasks, g.blk, g.n); break;    \
+    }
     if (!dfloat) {
         switch (W) {
-            case 1: class4_kernel<1><<<grid, kJ, 0, s>>>(g.tasks, g.blk, g.n); break;
-            case 2: class4_kernel<2><<<grid, kJ, 0, s>>>(g.tasks, g.blk, g.n); break;
-            case 3: class4_kernel<3><<<grid, kJ, 0, s>>>(g.tasks, g.blk, g.n); break;
-            default: class4_kernel<4><<<grid, kJ, 0, s>>>(g.tasks, g.blk, g.n); break;
+            case 1: HB_C4(1); break;
+            case 2: HB_C4(2); break;
+            case 3: HB_C4(3); break;
+            default: HB_C4(4); break;
         }
+#undef HB_C4
         return 1;
     }
 #define HB_C4DF(WW)                                                                                       \

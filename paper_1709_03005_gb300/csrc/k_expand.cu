@@ -144,11 +144,9 @@ expand_fp64_kernel(const XTask *__restrict__ tasks, const int64_t *__restrict__ 
             const int64_t m = m0 + ty * 4 + i;
             if (m >= M) continue;
             const int jj = (int)(m / cnp), jjp = (int)(m % cnp);
-            const int64_t r = c.rbase + jj;
-            const int64_t cc = c.cbase + jjp;
-            if (c.same && r < cc) continue;
-            c.H[r * c.ld + cc] = acc[i][j];
-            if (r != cc) c.H[cc * c.ld + r] = acc[i][j];
+            if (jj - jjp < c.jmin) continue;
+            c.lower[(int64_t)jj * c.ld + jjp] = acc[i][j];
+            c.upper[(int64_t)jjp * c.ld + jj] = acc[i][j];
         }
     }
 }

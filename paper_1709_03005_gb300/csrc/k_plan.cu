@@ -12,6 +12,7 @@
 // change).  A plan over many contexts is what a batch captures in a CUDA graph.
 #include <algorithm>
 #include <cstdio>
+#include <cstdint>
 #include <cstring>
 #include <map>
 #include <tuple>
@@ -83,7 +84,11 @@ struct Plan {
     std::vector<hb_ctx *> ctxs;
     std::vector<hb_blocks> outs;
     int precision = HB_FP64;
-    int W = 1, Kpad = 0, n_to = 0, S = 0, delta_col = 0;
+    int W = 1, Kpad = 0, n_to = 0, delta_col = 0;
+    // the expansion on the tensor cores (the mixed build always, the FP64 build
+    // where its slices fit the memory), its slices, and those of class 4
+    bool split_on = false;
+    int S = 0, c4_slices = 6;
     // panel columns per label class (Kc) and the coefficient slices' width
     // (Kw = every class); perm: the labels of the coefficient slice columns
     // (null without orbital symmetry)
@@ -134,9 +139,13 @@ struct Plan {
     bool upload_pending = false;
     // tensor-core operands
     void *coef = nullptr;
+    int16_t *coef_exps = nullptr;      // FP64 build: the coefficient rows' exponents
     CUtensorMap tm_coef[4];            // coefficient slices: 32-K stages at widths 32, 64, 128; 64-K at 128
     int64_t coef_rows = 0;
     int *err = nullptr;
+    // FP64 build on the tensor cores: its error word as of the last finished
+    // build (page-locked; such builds are not waited for)
+    int *host_err = nullptr;
     // classes 4, 2 and 8 run on a second stream beside the target side and
     // the expansion (they read only staged data and write their own blocks);
     // the target side and the expansion at higher priority, the second stream
@@ -337,12 +346,13 @@ void fill_tasks(Plan &p) {
                 blocks.back().ctx = ctx;
             }
             blocks[it->second].members.push_back(Member{ctx, &P, &out});
-            if (p.precision == HB_MIXED && p.shard_r == 0) {     // the j == j' rows: the first shard
+            if (p.split_on && p.shard_r == 0) {                  // the j == j' rows: the first shard
                 const int j_lo = std::max(A.cf, B.cf), j_hi = std::min(A.cf + A.cn, B.cf + B.cn);
                 // rows j == j' are of class 0 (irrep(j) ^ irrep(j) = 0)
                 p.drows.add(DRTask{mixed_panel_diag(ctx), P.A_df, P.nn, ctx->n_cls > 1 ? ctx->cls_labels : nullptr,
                                    P.n_nn, ctx->Kc, ctx->Kpad, ctx->n_co, j_lo, j_hi, A.cf, A.cn,
-                                   B.cf, B.cn, P.same, diag_rows_ny(P.n_nn), A.row_off, B.row_off, ctx->Dc, out.Hcc},
+                                   B.cf, B.cn, P.same, diag_rows_ny(P.n_nn), A.row_off, B.row_off, ctx->Dc, out.Hcc,
+                                   ctx->panel, P.A},
                             blocks_diag_rows(j_lo, j_hi, P.n_nn));
             }
         }
@@ -375,9 +385,9 @@ void fill_tasks(Plan &p) {
                 p.c4t.add(tt, items);
                 continue;
             }
-            int ns_tile = 32, jt = 128;
+            int ns_tile, jt;
+            class4_shape(G.ns, G.cn, &ns_tile, &jt);
             if (p.precision == HB_MIXED) {
-                class4_shape(G.ns, G.cn, &ns_tile, &jt);
                 auto cc = p.choice.c4.find({G.ns, G.cn});
                 if (cc != p.choice.c4.end()) { ns_tile = cc->second.first; jt = cc->second.second; }
                 if (ctx->force_c4_states) ns_tile = ctx->force_c4_states;
@@ -430,30 +440,31 @@ void fill_tasks(Plan &p) {
                     if (P.same && b > a) continue;
                     ExpCol c;
                     c.arow = P.A + (int64_t)t * m.ctx->Kpad;
-                    c.H = m.out->Hcc;
-                    c.rbase = A.row_off + (int64_t)a * A.cn;
-                    c.cbase = Bg.row_off + (int64_t)b * Bg.cn;
-                    c.ld = m.ctx->Dc;
-                    c.same = P.same;
-                    c.pad = 0;
+                    const int64_t ld = m.ctx->Dc, r = A.row_off + (int64_t)a * A.cn, cc = Bg.row_off + (int64_t)b * Bg.cn;
+                    c.ld = (int32_t)ld;
+                    c.lower = m.out->Hcc ? m.out->Hcc + r * ld + cc : nullptr;
+                    c.upper = m.out->Hcc ? m.out->Hcc + cc * ld + r : nullptr;
+                    // within one group a state pair n = n' has the whole rectangle; its upper half is the mirror's
+                    c.jmin = P.same && r == cc ? 0 : INT32_MIN;
                     p.cols.push_back(c);
                     ++t;
                 }
-            if (p.precision == HB_MIXED)
+            if (p.split_on)
                 p.slc.add(SliceTask{P.A, P.n_nn, coef_row + (mstart - col0)}, P.n_nn);   // a block per row
         }
         const int N = (int)((int64_t)p.cols.size() - col0);
         const BlockKey &k = B.key;
-        if (p.precision == HB_MIXED) {
+        if (p.split_on) {
             int lg = split_tile_heuristic(k.cn, k.cnp);
             auto tc = p.choice.tile.find({k.cn, k.cnp});
             if (tc != p.choice.tile.end()) lg = tc->second;
             if (B.ctx->force_tile) lg = B.ctx->force_tile;
-            const int bn = split_cols_choice(N, p.Kc / 64, B.ctx->force_cols);
-            const void *pkey = mixed_panel_key(B.ctx);
+            const int bn = p.precision == HB_MIXED ? split_cols_choice(N, p.Kc / 64, B.ctx->force_cols)
+                                                   : split_f64_cols_choice(N, B.ctx->force_cols);
+            const void *pkey = mixed_panel_key(B.ctx, p.precision);
             int gi = -1;
             for (size_t i = 0; i < p.split.size(); ++i)
-                if (mixed_panel_key(p.split[i].panel_ctx) == pkey && p.split[i].lg == lg && p.split[i].bn == bn)
+                if (mixed_panel_key(p.split[i].panel_ctx, p.precision) == pkey && p.split[i].lg == lg && p.split[i].bn == bn)
                     gi = (int)i;
             if (gi < 0) {
                 p.split.emplace_back();
@@ -609,24 +620,39 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     }
     bool any_pairs = false;
     for (int i = 0; i < n; ++i) any_pairs = any_pairs || !ctxs[i]->gps.empty();
-    if (precision == HB_MIXED && any_pairs) {
+    // the FP64 build's slices come out of a caller's workspace only where that
+    // was sized with them
+    bool room = precision == HB_MIXED;
+    if (!room) {
+        room = true;
+        for (int i = 0; i < n; ++i) {
+            const hb_ctx *owner = ctxs[i]->base ? ctxs[i]->base : ctxs[i];
+            for (const hb_ctx *c : {owner, (const hb_ctx *)ctxs[i]})
+                if (c->pool.base && (!c->pool.measured_f64 || (int64_t)c->pool.size + 512 < c->pool.measured))
+                    room = false;        // (its size is rounded to the allocator's 256 bytes)
+        }
+    }
+    if (any_pairs && room) {
         for (int i = 0; i < n && rc == HB_OK; ++i) {
             if (ctxs[i]->gps.empty()) continue;
-            rc = mixed_prepare(ctxs[i], s);
+            rc = mixed_prepare(ctxs[i], precision, s);
             if (rc != HB_OK) { *err = ctxs[i]->err; break; }
-            const int S = mixed_slices(ctxs[i]);
+            const int S = mixed_slices(ctxs[i], precision);
             if (p->S == 0) p->S = S;
             else if (S != p->S) { rc = HB_ERR_INVALID_ARG; *err = "contexts of one plan use different split_slices"; }
         }
+        p->split_on = rc == HB_OK && p->S > 0;
+        // an FP64 build without room for the slices adds its sums on the FP64 pipe
+        if (precision == HB_FP64 && rc == HB_ERR_OOM) rc = HB_OK;
         if (rc != HB_OK) { plan_destroy(p); return rc; }
         p->delta_col = ctxs[0]->delta_pos;   // the delta label's column (class 0 comes first)
     }
-    if (precision == HB_MIXED && p->S == 0) p->S = mixed_slices(ctxs[0]);
+    p->c4_slices = ctxs[0]->split_slices;
     // class 4 on the tensor cores: integral and CI slices, term-list sizes
     if (precision == HB_MIXED)
         for (int i = 0; i < n && rc == HB_OK; ++i) {
             if (ctxs[i]->n_l2 < 1 || ctxs[i]->c4_path == 1) continue;
-            rc = c4tc_prepare(ctxs[i], p->S, s);
+            rc = c4tc_prepare(ctxs[i], p->c4_slices, s);
             if (rc != HB_OK) *err = ctxs[i]->err;
         }
     if (precision == HB_MIXED)
@@ -654,9 +680,22 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         }
     }
     fill_tasks(*p);
-    if (precision == HB_MIXED && p->coef_rows > 0) {
-        rc = split_coef_alloc(ctxs[0], p->S, p->coef_rows, p->Kw, &p->coef, p->tm_coef, err);
+    if (p->split_on && p->coef_rows > 0) {
+        rc = split_coef_alloc(ctxs[0], p->S, p->coef_rows, p->Kw, &p->coef,
+                              precision == HB_FP64 ? &p->coef_exps : nullptr, p->tm_coef, err);
+        if (rc == HB_ERR_OOM && precision == HB_FP64) {
+            p->split_on = false;
+            p->split.clear();
+            fill_tasks(*p);
+            rc = HB_OK;
+        }
+        if (rc == HB_OK && p->split_on && precision == HB_FP64 &&
+            cudaMallocHost((void **)&p->host_err, sizeof(int)) != cudaSuccess) {
+            rc = HB_ERR_CUDA;
+            *err = "plan: page-locked error word";
+        }
         if (rc != HB_OK) { plan_destroy(p); return rc; }
+        if (p->host_err) *p->host_err = 0;
         ensure_split_events(*p);
     }
     pack_all(*p);
@@ -677,6 +716,11 @@ bool plan_outputs_equal(const Plan *p, const hb_blocks *outs) {
 }
 
 int plan_precision(const Plan *p) { return p->precision; }
+int plan_host_error(Plan *p) {
+    const int w = p->host_err ? *(volatile int *)p->host_err : 0;
+    if (w) *p->host_err = 0;
+    return w;
+}
 
 int plan_set_outputs(Plan *p, const hb_blocks *outs, std::string *err, cudaStream_t s) {
     p->outs.assign(outs, outs + p->outs.size());
@@ -741,7 +785,8 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
     // split expansion: tile arrangement per continuum rectangle (and panel)
     {
         std::map<std::tuple<const void *, int, int>, std::vector<const TuneSplit *>> cls;
-        for (auto &t : p->tune_split) cls[{mixed_panel_key(t.panel_ctx), t.t.cn, t.t.cnp}].push_back(&t);
+        for (auto &t : p->tune_split)
+            cls[{mixed_panel_key(t.panel_ctx, p->precision), t.t.cn, t.t.cnp}].push_back(&t);
         for (auto &kv : cls) {
             const int cn = std::get<1>(kv.first), cnp = std::get<2>(kv.first);
             const hb_ctx *pc = kv.second.front()->panel_ctx;
@@ -766,7 +811,8 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
                     }
                     if (ts.empty()) continue;
                     ms += time_tasks(p->ctxs[0], ts, nb, [&](const Grouped<SplitTask> &g) {
-                        g_split(pc, lg, bn, p->tm_coef, g, p->Kc / 64, p->Kw / 64, p->d_cols, p->err, s);
+                        g_split(pc, p->precision, lg, bn, p->tm_coef, p->coef_exps, g, p->Kc / 64, p->Kw / 64, p->d_cols,
+                                p->err, s);
                     }, s);
                 }
                 if (best_lg < 0) { best = def_ms = ms; best_lg = lg; }
@@ -920,7 +966,7 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         rec_on(p->ev[4], s2);
         cudaMemsetAsync(p->err + 1, 0, sizeof(int), s2);
         L += g_c4fill(p->c4f.g, s2);
-        L += g_c4tc(p->c4t.g, p->d_c4items, (int)p->c4items.size(), p->S, p->err + 1, s2);
+        L += g_c4tc(p->c4t.g, p->d_c4items, (int)p->c4items.size(), p->c4_slices, p->err + 1, s2);
         for (auto &v : p->c4v) L += g_class4(v.st.g, W, 1, v.ns_tile, v.jt, s2);
         rec_on(p->ev[3], s2);
         cudaEventRecord(p->c4_done, s2);
@@ -976,24 +1022,25 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     // expansion (Eq. 7): classes 1, 3, 5, 6, 7
     if (!ph2) {
         // phase 1 ends with the coefficient rows
-    } else if (p->precision == HB_MIXED) {
+    } else if (p->split_on || p->precision == HB_MIXED) {
         // with class 4 on the tensor cores, the expansion waits for it (see
         // the side stream above); the double-float class-4 kernel runs beside
         // the expansion, which was faster than running it first
         if (p->c4t.g.blocks > 0) cudaStreamWaitEvent(s, p->c4_done, 0);
         if (p->coef_rows > 0) {
             cudaMemsetAsync(p->err, 0, sizeof(int), s);
-            L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, s);
+            L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, p->coef_exps,
+                         s);
             for (size_t i = 0; i < p->split.size(); ++i) {
                 rec(p->ev_split[2 * i]);
-                LX += g_split(p->split[i].panel_ctx, p->split[i].lg, p->split[i].bn, p->tm_coef, p->split[i].st.g, p->Kc / 64, p->Kw / 64,
-                              p->d_cols, p->err, s,
-                              p->shard_r, p->shard_n);
+                LX += g_split(p->split[i].panel_ctx, p->precision, p->split[i].lg, p->split[i].bn, p->tm_coef, p->coef_exps,
+                              p->split[i].st.g, p->Kc / 64, p->Kw / 64, p->d_cols, p->err, s, p->shard_r, p->shard_n);
                 rec(p->ev_split[2 * i + 1]);
             }
-            // the rows with j == j' (double-float); beside the split kernel they
-            // slowed it by more than they saved
-            L += g_diag_rows(p->drows.g, s);
+            // the rows with j == j'; beside the split kernel they slowed it by
+            // more than they saved
+            L += g_diag_rows(p->drows.g, DF, s);
+            if (p->host_err) cudaMemcpyAsync(p->host_err, p->err, sizeof(int), cudaMemcpyDeviceToHost, s);
         }
     } else {
         LX += g_expand_fp64(p->x64.g, p->d_cols, s, p->shard_r, p->shard_n);
@@ -1039,7 +1086,7 @@ void plan_stats(Plan *p, hb_stats *st) {
         cudaEventElapsedTime(&st->ms_class4, p->ev[5], p->ev[3]);
         cudaEventElapsedTime(&st->ms_class4_kernel, p->ev[8], p->ev[3]);
     }
-    if (p->precision == HB_MIXED) {
+    if (p->split_on) {
         float total = 0.0f;
         for (size_t i = 0; i + 1 < p->ev_split.size(); i += 2) {
             float t = 0.0f;
@@ -1084,9 +1131,11 @@ void plan_destroy(Plan *p) {
     if (mem) {
         dfree(mem, p->dev);
         dfree(mem, p->coef);
+        dfree(mem, p->coef_exps);
         dfree(mem, p->err);
     }
     if (p->pinned) cudaFreeHost(p->pinned);
+    if (p->host_err) cudaFreeHost(p->host_err);
     delete p;
 }
 

@@ -4,37 +4,52 @@
 //
 // Both FP64 operands are split row by row into S bf16 slices (an error-free
 // splitting in the manner of Ozaki, Ogita, Oishi & Rump 2012): with 2^e the
-// smallest power of two above the row's largest magnitude,
-//   slice 0 = rint(x 2^{7-e}) 2^{e-7},  |integer| <= 128,
-//   slice i = rint(r_i 2^{7+7i-e}) 2^{e-7-7i}, |integer| <= 64  (i >= 1),
-// with r_i the remainder after slices 0..i-1, so S slices carry 7S bits.  The
-// row exponent is folded into the slice values, so every product of slice i of
-// a panel row with slice l of a coefficient row is an integer multiple of the
-// same unit 2^{e_row + e_col - 14 - 7(i+l)}.  The products with the same
-// s = i + l are summed by tcgen05.mma (kind::f16, bf16 inputs, FP32
-// accumulation in tensor memory) in K-chunks of 512: there every partial sum
-// stays below 2^24 units, so the FP32 accumulation is exact.  Separate TMEM
-// accumulators hold s = 0, 1, 2 and one holds s >= 3 (its rounding is below
-// 2^-45 of the result).  The epilogue drains the accumulators after each
-// chunk; the MMAs of the next chunk wait for that drain.  After each chunk the
-// epilogue warps fold the four accumulators into a double-float running sum
-// (TwoSum for s <= 2), and at the end write it as FP64.  Pairs with i + l >= S are dropped (below 2^-7S relative).
+// smallest power of two above the row's largest magnitude, x 2^(8+9(S-1)-e) is
+// rounded to an integer whose balanced base-512 digits d_0 .. d_{S-1} (|d_i| <=
+// 256, which bf16 holds exactly) are the slices, d_i 2^(-8-9i) apart from 2^e.
+// Products of slice i of a panel row with slice l of a coefficient row are
+// integer multiples of 2^(-16-9s), s = i + l; those with i + l < S are formed,
+// and summed per s by tcgen05.mma (kind::f16, FP32 accumulation in tensor
+// memory).  Up to 256 / (s + 1) terms every partial sum of such a sum stays
+// within 2^24 units, so the FP32 accumulation is exact; then the epilogue
+// takes the accumulator out and it starts again from zero.
 //
-// Kernel structure (one CTA per 128 x 128 output tile, 10 warps):
-//   warp 0  TMA producer: per 32-wide K stage and slice, one panel tile
-//           (128 x 32) and one coefficient tile (128 x 32), 64-byte swizzle,
-//           each slice in its own shared-memory slot with full/empty mbarriers
-//           so the MMAs start as slices land and slots refill as they free;
-//           two full sets of slots (six slices), so a stage loads while the
-//           one before it is multiplied
+// Mixed build: S = 5 (44 bits, 15 products).  s = 0, 1, 2 have accumulators of
+// their own, drained every 256, 128 and 64 terms into a double-float sum; s = 3
+// and 4 share the fourth, which need not be exact (its rounding is 2^-47 of
+// the row scales per product) and is added every 512 terms.  With base-128 digits the
+// same accuracy took 6 slices and 21 products, and all pairs s >= 3 shared an
+// accumulator seven bits further up: the sums here are 6 to 9 times closer to
+// 64 bits (4.5e-12 -> 7e-13 at 2422 labels, 1.7e-12 -> 1.8e-13 at 1367).  2422
+// labels x 1275 columns x 160000 rows: 14.2 -> 10.4 ms, 1367 x 210 x 22500: 358
+// -> 266 us.
+//
+// FP64 build: S = 7 (62 bits, 28 products), every s with an accumulator of its
+// own, and the row exponents kept apart from the digits.  The drained sums are
+// integers and are added as such (two 64-bit words per element, s <= 2 and
+// s >= 3), so the element is the correctly rounded sum of the 62-bit products,
+// whatever the order of the labels.  The FP64 pipe of this part runs at a
+// 1/1000 of the tensor rate: its sums took 14.0 ms where this takes 0.65 ms
+// (12.9 GFLOP), and rounded every one of the 1367 additions.
+//
+// Kernel structure (persistent CTAs on 128 x TBN output tiles, 10 warps):
+//   warp 0  TMA producer: per K stage (32 or 64 labels) and slice, one panel
+//           tile and one coefficient tile into a slot of a ring of as many
+//           slots as fit, with full/empty mbarriers
 //   warp 1  MMA issuer (one elected thread), TMEM allocation owner
-//   warps 2-9 epilogue: TMEM -> registers, double-float accumulation, FP64 out
-//           (two warps per TMEM lane quadrant, 64 columns each)
+//   warps 2-9 epilogue: TMEM -> registers, accumulation, FP64 out (two warps
+//           per TMEM lane quadrant)
+// A stage takes the pairs of the inexact accumulator first, those with slice 0
+// last, and then s = S-1 .. 0 of the exact ones.  So an accumulator due for draining is drained
+// behind the pairs that follow and those of the next stage that precede its
+// own (each accumulator has its own full/empty barriers), and slices S-1 .. 0
+// are released in that order, which is the order of the ring.
 // Every mbarrier wait is bounded; on a timeout the kernel records an error,
 // drains its own copies and MMAs, frees TMEM and returns.
 //
 // Rows with j == j' carry h_jj and the delta_jj' E term and so have a wide
-// dynamic range; the mixed kernel skips them and an FP64 kernel computes them.
+// dynamic range; the kernel skips them and diag_rows_kernel computes them (in
+// double-float or FP64).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -48,15 +63,19 @@
 
 namespace hb {
 
-struct MixedState {
-    int slices = 6;
-    int64_t panel_rows = 0;
-    __nv_bfloat16 *panel_slices = nullptr;   // [S][Kpad/64][n_co*n_co][64]
-    bool panel_ready = false;
-    bool borrowed_panel = false;
+// Panel slices of one precision, and their tensor maps.
+struct PanelSlices {
+    int slices = 0;
+    __nv_bfloat16 *buf = nullptr;            // [S][Kpad/64][n_co*n_co][64]
+    int16_t *exps = nullptr;                 // FP64: row exponents [n_co*n_co]
     // [stage width 32, 64][box of 8 x 16, 16 x 8, 32 x 4 continuum pairs (j' x j)]
-    CUtensorMap tm_panel[2][3];
-    float2 *pdiag = nullptr;                  // diagonal panel rows (j, j) as float pairs [n_co][Kpad]
+    CUtensorMap tm[2][3];
+    bool ready = false, borrowed = false;
+};
+
+struct MixedState {
+    PanelSlices panel[2];                    // HB_FP64, HB_MIXED
+    float2 *pdiag = nullptr;                 // mixed: diagonal panel rows (j, j) as float pairs [n_co][Kpad]
 };
 
 }  // namespace hb
@@ -79,28 +98,94 @@ constexpr int EPI_THREADS = 32 * EPI_WARPS;
 constexpr int EPI_COLS = BN / 2;             // columns per epilogue thread
 constexpr int NTHREADS = 64 + EPI_THREADS;
 
-// The expansion kernel's K pipeline: stages of KS = 32 K (64-byte operand
-// rows, 64-byte swizzle) or 64 K (128-byte rows and swizzle), and as many full
-// sets of S slots as fit 192 KB, so the copies of the next stages are in
-// flight while the stages before them are multiplied.  With one set (64-K
-// stages and 128 columns) odd stages use the slots in the order in which the
-// even ones free them (slot_of).  Its tile is 128 continuum pairs x TBN
-// columns (state pairs), TBN = 32, 64 or 128 chosen per merged block from its
-// column count; with TBN <= 64 the four accumulators are double-buffered in
-// tensor memory, so the MMAs of the next chunk run while the epilogue drains
-// the last one.  64-K stages serve 128-column tiles over long K (fewer waits
-// and copies per K), 32-K stages the rest (deeper prefetch).
-constexpr int XBUDGET = 192 * 1024;          // shared memory of the slots
+// The expansion kernel's K pipeline: stages of KS = 32 labels (64-byte operand
+// rows, 64-byte swizzle) or 64 (128-byte rows and swizzle), and a ring of as
+// many slice slots as fit, so the copies of the next stages are in flight
+// while the stages before them are multiplied.  Its tile is 128 continuum
+// pairs x TBN columns (state pairs), TBN = 32, 64 or 128 chosen per merged
+// block from its column count.  64-K stages serve 128-column tiles over long K
+// (fewer waits and copies per K), 32-K stages the rest (deeper prefetch).
+constexpr int XBUDGET = 7 * 32 * 1024;       // shared memory of the slots
 constexpr int XBARS = 24;                    // full and empty barriers: slots at most
+constexpr int XACC = 7;                      // accumulators at most
 constexpr int kK64Blocks = 32;               // 64-K stages from this many 64-wide K blocks up
+constexpr int kF64Slices = 7;                // slices of the FP64 build
 __host__ __device__ constexpr int xa_tile(int ks) { return BM * ks * 2; }
 // one slice of one stage: panel tile, then coefficient tile (multiples of 1 KB)
 __host__ __device__ constexpr int xslot(int tbn, int ks) { return (BM + tbn) * ks * 2; }
-__host__ __device__ constexpr int xsets(int S, int tbn, int ks) {
-    return XBUDGET / (S * xslot(tbn, ks)) < 4 ? XBUDGET / (S * xslot(tbn, ks)) : 4;
+__host__ __device__ constexpr int xslots(int tbn, int ks) {
+    return XBUDGET / xslot(tbn, ks) < XBARS ? XBUDGET / xslot(tbn, ks) : XBARS;
 }
-__host__ __device__ constexpr int xacc_bufs(int tbn) { return 8 * tbn <= 512 ? 2 : 1; }
-__host__ __device__ constexpr int xtmem_cols(int tbn) { return xacc_bufs(tbn) * 4 * tbn; }
+// accumulators: one per s below NEX, one for the rest
+__host__ __device__ constexpr int xaccs(int S, int nex) { return S <= nex ? S : nex + 1; }
+__host__ __device__ constexpr int xtmem_cols(int accs, int tbn) {
+    int c = 32;
+    while (c < accs * tbn) c *= 2;
+    return c;
+}
+// stages between drains of accumulator a: 256 / (a + 1) labels, rounded down to
+// a power of two, for an exact one, 512 for the inexact one
+__host__ __device__ constexpr int xperiod(int a, int nex, int ks) {
+    return (a >= nex ? 512 : a == 0 ? 256 : a == 1 ? 128 : a <= 3 ? 64 : 32) / ks;
+}
+// Whether accumulator a is drained after stage ks of nst.  a = 0 is drained
+// between the stages at which a = 1 is, so that at most two of the first three
+// come at once.
+template <int NEX, int KS>
+__device__ __forceinline__ bool acc_due(int a, int ks, int nst) {
+    const int per = xperiod(a, NEX, KS);
+    return ks == nst - 1 || (ks + 1 + (a == 0 ? per / 4 : 0)) % per == 0;
+}
+
+// The pairs (i, l) of a stage in order.
+struct PairOrder {
+    int n = 0;
+    int i[28] = {}, l[28] = {};
+};
+template <int S, int NEX>
+__host__ __device__ constexpr PairOrder pair_order() {
+    PairOrder o;
+    for (int m = S - 1; m >= 0; --m)              // inexact pairs, by their lower slice
+        for (int s = S - 1; s >= NEX; --s)
+            for (int i = 0; i <= s; ++i)
+                if ((i < s - i ? i : s - i) == m) {
+                    o.i[o.n] = i;
+                    o.l[o.n++] = s - i;
+                }
+    for (int s = (S < NEX ? S : NEX) - 1; s >= 0; --s)
+        for (int i = 0; i <= s; ++i) {
+            o.i[o.n] = i;
+            o.l[o.n++] = s - i;
+        }
+    return o;
+}
+// first and last pair that reads slice t; last pair of accumulator a
+__host__ __device__ constexpr int first_use(const PairOrder &o, int t) {
+    for (int p = 0; p < o.n; ++p)
+        if (o.i[p] == t || o.l[p] == t) return p;
+    return -1;
+}
+__host__ __device__ constexpr int last_use(const PairOrder &o, int t) {
+    int r = -1;
+    for (int p = 0; p < o.n; ++p)
+        if (o.i[p] == t || o.l[p] == t) r = p;
+    return r;
+}
+__host__ __device__ constexpr int last_of_acc(const PairOrder &o, int a, int nex) {
+    int r = -1;
+    for (int p = 0; p < o.n; ++p) {
+        const int s = o.i[p] + o.l[p];
+        if ((s < nex ? s : nex) == a) r = p;
+    }
+    return r;
+}
+__host__ __device__ constexpr int first_of_acc(const PairOrder &o, int a, int nex) {
+    for (int p = 0; p < o.n; ++p) {
+        const int s = o.i[p] + o.l[p];
+        if ((s < nex ? s : nex) == a) return p;
+    }
+    return -1;
+}
 
 __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tm, uint64_t *bar, int c0, int c1, int c2,
                                             int c3) {
@@ -184,50 +269,133 @@ __device__ __forceinline__ bool mma_block(uint64_t *full_bar, uint64_t *empty_ba
     return true;
 }
 
-// Slot of slice t in stage G: slot set G mod NSET, or with a single set the
-// release-ordered slots of odd stages.
-template <int S, int NSET>
-__device__ __forceinline__ int xslot_index(int G, int t) {
-    if (NSET >= 2) return (G % NSET) * S + t;
-    return (G & 1) ? slot_of<S>(1, t) : t;
+// What the MMA issuer carries through a launch.  due: the accumulators drained
+// after the current stage; fresh: those whose next MMA starts from zero; used:
+// those handed over before; epar: the parity of each one's next hand-back.
+struct MmaState {
+    uint64_t *full_bar, *empty_bar, *acc_full, *acc_empty;
+    uint32_t tmem, idesc;
+    uint64_t desc0;
+    int *err;
+    uint32_t due = 0, fresh = 0, used = 0, epar = 0;
+    uint32_t leader = 0;      // this lane issues
+};
+
+// Pair P of a stage and those after it; slice t of the stage is in slot sl[t],
+// whose use has parity sp[t].
+template <int S, int NEX, int TBN, int KS, int P>
+__device__ __forceinline__ bool mma_pairs(MmaState &m, const int (&sl)[S], const uint32_t (&sp)[S]) {
+    constexpr PairOrder O = pair_order<S, NEX>();
+    constexpr int XS = xslot(TBN, KS);
+    constexpr int i = O.i[P], l = O.l[P], a = i + l < NEX ? i + l : NEX;
+    constexpr bool wait_i = first_use(O, i) == P, wait_l = l != i && first_use(O, l) == P;
+    constexpr bool first_a = first_of_acc(O, a, NEX) == P, last_a = last_of_acc(O, a, NEX) == P;
+    if (wait_i && !mbar_wait_warp(&m.full_bar[sl[i]], sp[i], m.err, 4)) return false;
+    if (wait_l && !mbar_wait_warp(&m.full_bar[sl[l]], sp[l], m.err, 4)) return false;
+    if (first_a && (m.fresh >> a) & 1u) {
+        // the epilogue has taken this accumulator's last sums
+        if ((m.used >> a) & 1u) {
+            if (!mbar_wait_warp(&m.acc_empty[a], (m.epar >> a) & 1u, m.err, 3)) return false;
+            m.epar ^= 1u << a;
+        }
+        m.used |= 1u << a;
+    }
+    if (wait_i || wait_l || first_a) tc_fence_after();
+    const uint64_t da = m.desc0 + (uint32_t)((sl[i] * XS) >> 4), db = m.desc0 + (uint32_t)((sl[l] * XS + xa_tile(KS)) >> 4);
+#pragma unroll
+    for (int k = 0; k < KS / 16; ++k) {
+        const uint32_t acc = (first_a && k == 0) ? (~(m.fresh >> a) & 1u) : 1u;
+        mma_bf16_elect(m.tmem + a * TBN, da + 2 * k, db + 2 * k, m.idesc, acc, m.leader);
+    }
+    if (first_a) m.fresh &= ~(1u << a);
+    if (last_use(O, i) == P) mma_commit_elect(&m.empty_bar[sl[i]], m.leader);
+    if (l != i && last_use(O, l) == P) mma_commit_elect(&m.empty_bar[sl[l]], m.leader);
+    if (last_a && (m.due >> a) & 1u) {
+        mma_commit_elect(&m.acc_full[a], m.leader);
+        m.fresh |= 1u << a;
+    }
+    if constexpr (P + 1 < O.n) return mma_pairs<S, NEX, TBN, KS, P + 1>(m, sl, sp);
+    return true;
 }
 
-// One K stage of the expansion kernel (stage G, slots xslot_index), with
-// accumulators at TMEM column tacc: for each arriving slice t the pairs (i, l)
-// with max(i, l) = t and i + l < S, then the commits that free the slots read
-// for the last time.
-template <int S, int TBN, int KS, int NSET>
-__device__ __forceinline__ bool mma_stage(uint64_t *full_bar, uint64_t *empty_bar, int G, uint32_t tacc,
-                                          uint64_t desc0, uint32_t idesc, uint32_t &fresh, int *err) {
-    constexpr int XS = xslot(TBN, KS);
-    const uint32_t par = (uint32_t)((G / NSET) & 1);
+// One K stage of the expansion kernel.  Its slices lie in the ring from slot
+// `slot0` on, slice S-1 first, `par` being the parity of that slot's use
+// (flipped where the ring wraps).
+template <int S, int NEX, int TBN, int KS>
+__device__ __forceinline__ bool mma_stage(MmaState &m, int slot0, uint32_t par) {
+    constexpr int NS = xslots(TBN, KS);
+    int sl[S];
+    uint32_t sp[S];
 #pragma unroll
     for (int t = 0; t < S; ++t) {
-        if (!mbar_wait(&full_bar[xslot_index<S, NSET>(G, t)], par, err, 4)) return false;
-        tc_fence_after();
+        const int x = slot0 + (S - 1 - t);
+        sl[t] = x >= NS ? x - NS : x;
+        sp[t] = x >= NS ? par ^ 1u : par;
+    }
+    return mma_pairs<S, NEX, TBN, KS, 0>(m, sl, sp);
+}
+
+// One drained accumulator of the mixed kernel (NC columns of this thread's
+// TMEM lane): an exact one by TwoSum (2^-18 of the result for s = 2 still needs
+// it to keep the low word below an ulp of the high one), the inexact one
+// (2^-27) into the low word.
+template <bool EXACT, int NC>
+__device__ __forceinline__ void drain_df(uint32_t taddr, float (&hi)[NC], float (&lo)[NC]) {
+    static_assert(NC % 16 == 0, "columns are loaded 16 at a time");
 #pragma unroll
-        for (int i = 0; i <= t; ++i) {
+    for (int c0 = 0; c0 < NC; c0 += 32) {
+        uint32_t v[16], w[16];
+        tmem_ld16_async(taddr + c0, v);
+        if (c0 + 16 < NC) tmem_ld16_async(taddr + c0 + 16, w);
+        tmem_wait_ld();
+        tmem_regs_ready(v);
+        if (c0 + 16 < NC) tmem_regs_ready(w);
 #pragma unroll
-            for (int l = 0; l <= t; ++l) {
-                if ((i == t || l == t) && i + l < S) {
-                    const int s = i + l < 3 ? i + l : 3;
-                    const uint32_t offA = (uint32_t)(xslot_index<S, NSET>(G, i) * XS);
-                    const uint32_t offB = (uint32_t)(xslot_index<S, NSET>(G, l) * XS + xa_tile(KS));
-#pragma unroll
-                    for (int k = 0; k < KS / 16; ++k) {
-                        const uint32_t acc = (fresh >> s) & 1u ? 0u : 1u;
-                        mma_bf16(tacc + s * TBN, desc0 + ((offA + k * 32) >> 4), desc0 + ((offB + k * 32) >> 4),
-                                 idesc, acc);
-                        fresh &= ~(1u << s);
-                    }
-                }
+        for (int i = 0; i < 16; ++i) {
+            if (EXACT) df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
+            else lo[c0 + i] = __fadd_rn(lo[c0 + i], __uint_as_float(v[i]));
+            if (c0 + 16 < NC) {
+                constexpr int o = 16;
+                if (EXACT) df_add(hi[(c0 + o + i) % NC], lo[(c0 + o + i) % NC], __uint_as_float(w[i]));
+                else lo[(c0 + o + i) % NC] = __fadd_rn(lo[(c0 + o + i) % NC], __uint_as_float(w[i]));
             }
         }
-#pragma unroll
-        for (int i = 0; i < S; ++i)
-            if (release_step<S>(i) == t) mma_commit(&empty_bar[xslot_index<S, NSET>(G, i)]);
     }
-    return true;
+}
+
+// One drained accumulator of the FP64 kernel: its sums are integers of
+// 2^(-16-9s), added to word 0 (units of 2^-34, s <= 2) or 1 (2^-70).
+template <int SS, int NC>
+__device__ __forceinline__ void drain_int(uint32_t taddr, long long (&acc)[2][NC]) {
+    static_assert(NC % 16 == 0, "columns are loaded 16 at a time");
+    constexpr int w = SS <= 2 ? 0 : 1;
+    constexpr float to_int = (float)(1ull << (SS <= 2 ? 16 + 9 * SS : 0)) * 1.0f;
+    constexpr int lift = SS <= 2 ? 9 * (2 - SS) : 9 * (6 - SS);
+#pragma unroll
+    for (int c0 = 0; c0 < NC; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld16_async(taddr + c0, v);
+        tmem_wait_ld();
+        tmem_regs_ready(v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            float x = __uint_as_float(v[i]);
+            if (SS <= 2) x *= to_int;
+            else x = x * (float)(1ull << 40) * (float)(1ull << (16 + 9 * SS - 40));
+            acc[w][c0 + i] += (long long)__float2int_rn(x) * (1ll << lift);
+        }
+    }
+}
+
+// The FP64 element of the two words and the row and column exponents.
+constexpr int kExpNaN = 32767;               // exponent of a row with a value that is not finite
+__device__ __forceinline__ double int_words_to_double(long long a, long long b, int ea, int eb) {
+    if (ea == kExpNaN || eb == kExpNaN) return __longlong_as_double(0x7FF8000000000000ll);
+    const double v = fma((double)b, 0x1p-36, (double)a);
+    const int e = ea + eb - 34;
+    // |v| < 2^53: a power of two in the normal range leaves v in it, or takes it below
+    if (e > -960 && e < 960) return v * __hiloint2double((e + 1023) << 20, 0);
+    return scalbn(v, e);
 }
 
 // Fold one chunk's accumulators (NC columns of this thread's TMEM lane,
@@ -291,47 +459,46 @@ __device__ __forceinline__ TilePos tile_pos(const SplitTask *__restrict__ tasks,
 // Persistent: each CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // The slot ring, the accumulator hand-over and their barrier phases run on
 // across tiles, so the loads and MMAs of the next tile start while the
-// epilogue warps still write the last one out from registers.
-template <int S, int TBN, int KS>
+// epilogue warps still write the last one out from registers.  F64: the FP64
+// build's kernel (integer sums, exponents apart: pexp of the panel's rows,
+// n_co x n_co, cexp of the coefficient rows).
+template <int S, int TBN, int KS, bool F64>
 __global__ void __launch_bounds__(NTHREADS, 1)
 split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_constant__ CUtensorMap tm_coef,
                     const SplitTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int n_tiles,
-                    int kblocks, int coef_planes, const ExpCol *__restrict__ cols, int *err, int shard_r,
-                    int shard_n) {
+                    int kblocks, int coef_planes, const ExpCol *__restrict__ cols, const int16_t *__restrict__ pexp,
+                    const int16_t *__restrict__ cexp, int n_co, int *err, int shard_r, int shard_n) {
     // this launch's tiles: shard_r, shard_r + shard_n, ... (all of them unless
     // sharded), numbered t = 0, 1, ... so that every role walks the same list
     const int n_local = n_tiles > shard_r ? (n_tiles - shard_r + shard_n - 1) / shard_n : 0;
-    constexpr int XS = xslot(TBN, KS);
-    constexpr int NSET = xsets(S, TBN, KS);
-    constexpr int NACC = xacc_bufs(TBN);      // accumulator sets in tensor memory
-    constexpr int TCOLS = xtmem_cols(TBN);
+    constexpr int NEX = F64 ? S : 3;          // accumulators of one s each
+    constexpr int NACC = xaccs(S, NEX);
+    constexpr int XS = xslot(TBN, KS), NS = xslots(TBN, KS);
+    constexpr int TCOLS = xtmem_cols(NACC, TBN);
     constexpr int ECOLS = TBN / 2;            // columns per epilogue thread
-    constexpr int SPC = KCHUNK / KS;          // stages per exact chunk
     static_assert(KS == 32 || KS == 64, "stage width");
-    static_assert(NSET >= 1 && NSET * S <= XBARS, "slot sets");
+    static_assert(NS >= S && NS <= XBARS && NACC <= XACC && TCOLS <= 512, "slots and tensor memory");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *slots = base;                                         // [NSET][S][XS]
-    uint64_t *full_bar = (uint64_t *)(base + NSET * S * XS);      // [XBARS]
+    uint8_t *slots = base;                                         // [NS][XS]
+    uint64_t *full_bar = (uint64_t *)(base + NS * XS);             // [XBARS]
     uint64_t *empty_bar = full_bar + XBARS;                        // [XBARS]
-    uint64_t *acc_full = empty_bar + XBARS;                        // [2]
-    uint64_t *acc_empty = acc_full + 2;                            // [2]
-    uint64_t *final_bar = acc_empty + 2;                           // [1]
+    uint64_t *acc_full = empty_bar + XBARS;                        // [XACC]
+    uint64_t *acc_empty = acc_full + XACC;                         // [XACC]
+    uint64_t *final_bar = acc_empty + XACC;                        // [1]
     uint32_t *tmem_slot = (uint32_t *)(final_bar + 1);
-    // the epilogue's tile: arguments and column destinations, double-buffered
+    // the epilogue's tile, double-buffered
     __shared__ SplitTask ta[2];
     __shared__ TilePos tp[2];
-    __shared__ ExpCol colmeta[2][TBN];
     __shared__ int epi_fail;                 // an epilogue wait gave up (read only after a barrier)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nst = kblocks * (64 / KS);     // K stages per tile
-    const int nchunks = (nst + SPC - 1) / SPC;
 
     if (threadIdx.x == 0) {
         epi_fail = 0;
         for (int i = 0; i < XBARS; ++i) { mbar_init(&full_bar[i], 1); mbar_init(&empty_bar[i], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EPI_THREADS); }
+        for (int b = 0; b < XACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EPI_THREADS); }
         mbar_init(final_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -349,7 +516,8 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
     if (warp == 0) {
         // ------------------------------------------------------ TMA producer
         if (lane == 0) {
-            int G = 0;                            // K stages issued by this CTA over all its tiles
+            int sl = 0, loads = 0;               // next slot, copies issued so far
+            uint32_t par = 1;                    // parity of the release the slot waits for (none in the first round)
             bool ok = true;
             for (int t = blockIdx.x; t < n_local && ok; t += gridDim.x) {
                 const int tile = shard_r + shard_n * t;
@@ -357,55 +525,54 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                 const int cx = tasks[p.ti].cfp + p.jjp0, cy = tasks[p.ti].cf + p.jj0;
                 const int crow = (int)(tasks[p.ti].coef_row0 + p.n0);
                 const int kc0 = tasks[p.ti].kc0;      // the block's label class in the coefficient slices
-                for (int ks = 0; ks < nst && ok; ++ks, ++G) {
-                    // stage G uses its slots for the (G / NSET)-th time
-                    const int round = G / NSET;
+                for (int ks = 0; ks < nst && ok; ++ks) {
                     const int kx = KS == 64 ? 0 : (ks & 1) * 32;   // part of 64-wide K block kb
                     const int kb = KS == 64 ? ks : ks >> 1;
-                    for (int t = 0; t < S && ok; ++t) {
-                        const int sl = xslot_index<S, NSET>(G, t);
-                        // wait for the slot's release by the stage NSET before this one
-                        if (round > 0) ok = mbar_wait(&empty_bar[sl], (round - 1) & 1, err, 1);
+                    for (int i = S - 1; i >= 0 && ok; --i) {
+                        if (loads >= NS) ok = mbar_wait(&empty_bar[sl], par, err, 1);
                         if (!ok) break;
                         uint8_t *sA = slots + sl * XS;
                         mbar_expect_tx(&full_bar[sl], (uint32_t)XS);
-                        tma_load_4d(sA, &tm_panel, &full_bar[sl], kx, cx, cy, t * kblocks + kb);
+                        tma_load_4d(sA, &tm_panel, &full_bar[sl], kx, cx, cy, i * kblocks + kb);
                         tma_load_3d(sA + xa_tile(KS), &tm_coef, &full_bar[sl], kx, crow,
-                                    t * coef_planes + kc0 + kb);
+                                    i * coef_planes + kc0 + kb);
+                        if (loads < 2 * NS) ++loads;
+                        if (++sl == NS) { sl = 0; par ^= 1u; }
                     }
                 }
             }
-            // wait until this producer's copies of the last stage of every set have landed
-            for (int g = G > NSET ? G - NSET : 0; g < G; ++g)
-                for (int t = 0; t < S; ++t)
-                    mbar_wait(&full_bar[xslot_index<S, NSET>(g, t)], (g / NSET) & 1, err, 2);
+            // wait until this producer's last copy into every slot has landed
+            // (slots before `sl` were last filled in this round, the others in the one before)
+            for (int i = 0; i < NS && i < loads; ++i) {
+                const uint32_t fp = i < sl ? par ^ 1u : par;
+                mbar_wait(&full_bar[i], fp, err, 2);
+            }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc_bf16(BM, TBN);
-            // + (offset >> 4) per operand tile
-            const uint64_t desc0 = KS == 64 ? smem_desc_sw128(smem_u32(slots)) : smem_desc_sw64(smem_u32(slots));
-            bool ok = true;
-            int G = 0, C = 0;                     // K stages and chunks over all tiles
-            for (int t = blockIdx.x; t < n_local && ok; t += gridDim.x) {
-                for (int c = 0; c < nchunks && ok; ++c, ++C) {
-                    // chunk C fills accumulator set C mod NACC, drained after chunk C - NACC
-                    const int b = C % NACC;
-                    if (C >= NACC) ok = mbar_wait(&acc_empty[b], (C / NACC - 1) & 1, err, 3);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint32_t tacc = tmem + (uint32_t)(b * 4 * TBN);
-                    const int ks_end = min(nst, (c + 1) * SPC);
-                    uint32_t fresh = 0xFu;        // accumulators not yet written in this chunk
-                    for (int ks = c * SPC; ks < ks_end && ok; ++ks, ++G)
-                        ok = mma_stage<S, TBN, KS, NSET>(full_bar, empty_bar, G, tacc, desc0, idesc, fresh, err);
-                    if (ok) mma_commit(&acc_full[b]);     // accumulators of chunk C complete
-                }
+        MmaState m;
+        m.full_bar = full_bar; m.empty_bar = empty_bar; m.acc_full = acc_full; m.acc_empty = acc_empty;
+        m.tmem = __shfl_sync(0xffffffffu, tmem, 0);
+        m.idesc = instr_desc_bf16(BM, TBN);
+        // + (offset >> 4) per operand tile
+        m.desc0 = KS == 64 ? smem_desc_sw128(smem_u32(slots)) : smem_desc_sw64(smem_u32(slots));
+        m.err = err;
+        m.fresh = (1u << NACC) - 1u;
+        m.leader = elect_lane();
+        bool ok = true;
+        int sl = 0;
+        uint32_t par = 0;
+        for (int t = blockIdx.x; t < n_local && ok; t += gridDim.x)
+            for (int ks = 0; ks < nst && ok; ++ks) {
+                m.due = 0;
+#pragma unroll
+                for (int a = 0; a < NACC; ++a) m.due |= acc_due<NEX, KS>(a, ks, nst) ? 1u << a : 0u;
+                ok = mma_stage<S, NEX, TBN, KS>(m, sl, par);
+                sl += S;
+                if (sl >= NS) { sl -= NS; par ^= 1u; }
             }
-            mma_commit(final_bar);
-            mbar_wait(final_bar, 0, err, 5);
-        }
+        mma_commit_elect(final_bar, m.leader);
+        mbar_wait_warp(final_bar, 0, err, 5);
     } else {
         // ------------------------------------------------------ epilogue
         const int e = threadIdx.x - 64;          // 0 .. EPI_THREADS-1
@@ -413,7 +580,9 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
         const int q = warp & 3;                  // TMEM lane quadrant this warp may access
         const int col0 = (ew >> 2) * ECOLS;
         const int row = q * 32 + lane;           // tile row = TMEM lane
-        int C = 0, it = 0;
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)col0;
+        int it = 0;
+        uint32_t fpar = 0;                       // parity of each accumulator's next hand-over
         for (int t = blockIdx.x; t < n_local; t += gridDim.x, ++it) {
             const int tile = shard_r + shard_n * t;
             const int buf = it & 1;
@@ -426,48 +595,86 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
             // every epilogue thread reaches both barriers of a tile, so the
             // failure flag read after the first is the same for all of them
             named_bar_sync(1, EPI_THREADS);
-            if (epi_fail) break;
-            const SplitTask &a = ta[buf];
-            if (e < TBN) {
-                const int t = tp[buf].n0 + e;
-                ExpCol cm;
-                if (t < a.N) cm = cols[a.col0 + t];
-                else cm.H = nullptr;
-                colmeta[buf][e] = cm;
-            }
+            const bool failed = epi_fail != 0;
             named_bar_sync(1, EPI_THREADS);
-            float hi[ECOLS], lo[ECOLS];
+            if (failed) break;
+            const SplitTask &a = ta[buf];
+            // the column records are read when the tile is written out
+            if (e < TBN / 4 && tp[buf].n0 + 4 * e < a.N)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(cols + a.col0 + tp[buf].n0 + 4 * e));
+            float hi[F64 ? 1 : ECOLS], lo[F64 ? 1 : ECOLS];
+            long long wd[2][F64 ? ECOLS : 1];
+            if constexpr (F64) {
 #pragma unroll
-            for (int c = 0; c < ECOLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
+                for (int c = 0; c < ECOLS; ++c) { wd[0][c] = 0; wd[1][c] = 0; }
+            } else {
+#pragma unroll
+                for (int c = 0; c < ECOLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
+            }
             bool ok = true;
-            for (int c = 0; c < nchunks; ++c, ++C) {
-                const int b = C % NACC;
-                if (ok) ok = mbar_wait(&acc_full[b], (C / NACC) & 1, err, 6);
-                if (!ok) continue;
-                tc_fence_after();
-                drain_chunk<S>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 4 * TBN + col0), TBN, hi, lo);
-                tc_fence_before();
-                mbar_arrive(&acc_empty[b]);
+            for (int ks = 0; ks < nst; ++ks) {
+                // in the order in which the stage hands them over
+#pragma unroll
+                for (int b = NACC - 1; b >= 0; --b) {
+                    if (!acc_due<NEX, KS>(b, ks, nst)) continue;
+                    if (ok) ok = mbar_wait(&acc_full[b], (fpar >> b) & 1u, err, 6);
+                    fpar ^= 1u << b;
+                    if (!ok) continue;
+                    tc_fence_after();
+                    if constexpr (F64) {
+                        if (b == 0) drain_int<0>(tq, wd);
+                        else if (b == 1) drain_int<1>(tq + TBN, wd);
+                        else if (b == 2) drain_int<2>(tq + 2 * TBN, wd);
+                        else if (b == 3) drain_int<3>(tq + 3 * TBN, wd);
+                        else if (b == 4) drain_int<4>(tq + 4 * TBN, wd);
+                        else if (b == 5) drain_int<5>(tq + 5 * TBN, wd);
+                        else drain_int<6>(tq + 6 * TBN, wd);
+                    } else if (b < NEX) {
+                        drain_df<true>(tq + b * TBN, hi, lo);
+                    } else {
+                        drain_df<false>(tq + b * TBN, hi, lo);
+                    }
+                    tc_fence_before();
+                    mbar_arrive(&acc_empty[b]);
+                }
             }
             if (!ok) {
                 epi_fail = 1;
-                continue;                        // leaves at the next tile's first barrier
+                continue;                        // leaves at the next tile's first barriers
             }
             // the accumulators are free again: the MMAs of the next tile run
             // while this one is written out
             const int lg = a.bjp_log2;
             const int jj = tp[buf].jj0 + (row >> lg), jjp = tp[buf].jjp0 + (row & ((1 << lg) - 1));
             if (jj < a.cn && jjp < a.cnp && (a.cf + jj) != (a.cfp + jjp)) {
+                const int n0 = tp[buf].n0 + col0;
+                const int4 *__restrict__ cm = reinterpret_cast<const int4 *>(cols + a.col0 + n0);
+                int ea = 0;
+                if constexpr (F64) ea = __ldg(pexp + (int64_t)(a.cf + jj) * n_co + a.cfp + jjp);
+                // two columns' destinations are fetched together
 #pragma unroll
-                for (int c = 0; c < ECOLS; ++c) {
-                    const ExpCol &m = colmeta[buf][col0 + c];
-                    if (m.H) {
-                        const int64_t r = m.rbase + jj;
-                        const int64_t cc = m.cbase + jjp;
-                        if (!m.same || r >= cc) {
-                            const double v = df_to_double(hi[c], lo[c]);
-                            m.H[r * m.ld + cc] = v;
-                            if (r != cc) m.H[cc * m.ld + r] = v;
+                for (int c0 = 0; c0 < ECOLS; c0 += 2) {
+                    int4 d0[2], d1[2];
+                    int eb[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (n0 + c0 + u < a.N) {
+                            d0[u] = __ldg(cm + 2 * (c0 + u));
+                            d1[u] = __ldg(cm + 2 * (c0 + u) + 1);
+                            if constexpr (F64) eb[u] = __ldg(cexp + a.coef_row0 + n0 + c0 + u);
+                        }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int c = c0 + u;
+                        if (n0 + c < a.N && jj - jjp >= d1[u].y) {
+                            double v;
+                            if constexpr (F64) v = int_words_to_double(wd[0][c], wd[1][c], ea, eb[u]);
+                            else v = df_sum(hi[c], lo[c]);
+                            const int64_t ld = d1[u].x;
+                            double *lower = reinterpret_cast<double *>(((uint64_t)(uint32_t)d0[u].y << 32) | (uint32_t)d0[u].x);
+                            double *upper = reinterpret_cast<double *>(((uint64_t)(uint32_t)d0[u].w << 32) | (uint32_t)d0[u].z);
+                            lower[jj * ld + jjp] = v;
+                            upper[jjp * ld + jj] = v;
                         }
                     }
                 }
@@ -626,56 +833,70 @@ __global__ void dense_reduce_kernel(const float2 *__restrict__ part, int nsplit,
     Y[(int64_t)n * ldy + m] = df_to_double(h, l);
 }
 
-// One row into its S bf16 slices by a whole block (the digits of slice_row):
-// every thread reads its share of the row, the row exponent is reduced through
-// shared memory, then each thread writes the digits of its elements.  at(k)
-// gives element k (0 beyond the row's data).
+// Exponent e of an FP64 bit pattern, |x| in [2^(e-1), 2^e); zeros (and FP64
+// subnormals, taken as zero) give -2000, values that are not finite 1025.
+__device__ __forceinline__ int fp64_exponent(unsigned long long b) {
+    const int be = (int)((b >> 52) & 0x7FF);
+    return be == 0 ? -2000 : be - 1022;
+}
+
+// Balanced digits of x against a row exponent: first + step (S - 1) bits in
+// all, F = x 2^(bits - emax) rounded to nearest, the first digit of `first`
+// bits (|d| <= 2^first), the others of `step` (|d| <= 2^(step - 1)).  put(i, d)
+// takes digit i, the slice's value being d 2^(emax - first - step i).
+template <class Put>
+__device__ __forceinline__ void digits(double x, int emax, int S, int first, int step, Put put) {
+    long long F = 0;
+    if (emax > -2000) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+        const int be = (int)((b >> 52) & 0x7FF);
+        if (be != 0) {
+            const long long m = (long long)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52));   // x = m 2^(be-1075)
+            const int sh = (be - 1075) + first + step * (S - 1) - emax;
+            long long f;
+            if (sh >= 0) f = m << sh;                       // at most 62 bits
+            else if (sh > -63) f = (m + (1ll << (-sh - 1))) >> (-sh);
+            else f = 0;
+            F = (b >> 63) ? -f : f;
+        }
+    }
+    for (int i = 0; i < S; ++i) {
+        const int sh = step * (S - 1 - i);
+        const long long d = sh > 0 ? ((F + (1ll << (sh - 1))) >> sh) : F;   // nearest digit
+        F -= d << sh;
+        put(i, (float)d);
+    }
+}
+
+// Digit sizes of the expansion's slices, and of the Davidson products'.
+constexpr int kXFirst = 8, kXStep = 9, kDFirst = 7, kDStep = 7;
+
+// One row into its S bf16 slices by a whole block: every thread reads its
+// share of the row, the row exponent is reduced through shared memory, then
+// each thread writes the digits of its elements.  at(k) gives element k (0
+// beyond the row's data).  With `exps` the row exponent goes there and the
+// slices are those of x / 2^e.
 template <class At>
-__device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S,
-                                                __nv_bfloat16 *__restrict__ out) {
+__device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S, int first, int step,
+                                                __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps = nullptr) {
     __shared__ int red[32];
     int emax = -2000;
-    for (int k = threadIdx.x; k < Kpad; k += blockDim.x) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(at(k));
-        const int be = (int)((b >> 52) & 0x7FF);
-        if (be == 0) continue;                 // zero (FP64 subnormals ignored)
-        const int e = be - 1022;               // |x| in [2^(e-1), 2^e)
-        emax = e > emax ? e : emax;
-    }
+    for (int k = threadIdx.x; k < Kpad; k += blockDim.x)
+        emax = max(emax, fp64_exponent((unsigned long long)__double_as_longlong(at(k))));
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        const int o = __shfl_xor_sync(0xffffffffu, emax, off);
-        emax = o > emax ? o : emax;
-    }
+    for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
     const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     if ((threadIdx.x & 31) == 0) red[warp] = emax;
     __syncthreads();
     emax = -2000;
-    for (int w = 0; w < nw; ++w) emax = red[w] > emax ? red[w] : emax;
-    const int KB = Kpad / BKB;
+    for (int w = 0; w < nw; ++w) emax = max(emax, red[w]);
+    if (exps && threadIdx.x == 0) exps[dest] = (int16_t)(emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0));
+    const int KB = Kpad / BKB, e0 = exps ? 0 : emax;
     for (int k = threadIdx.x; k < Kpad; k += blockDim.x) {
-        long long F = 0;
-        if (emax > -2000) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(at(k));
-            const int be = (int)((b >> 52) & 0x7FF);
-            if (be != 0) {
-                const long long m = (long long)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52));   // x = m 2^(be-1075)
-                const int sh = (be - 1075) + 7 * S - emax;      // F = m 2^sh, rounded to nearest
-                long long f;
-                if (sh >= 0) f = m << sh;
-                else if (sh > -63) f = (m + (1ll << (-sh - 1))) >> (-sh);
-                else f = 0;
-                F = (b >> 63) ? -f : f;
-            }
-        }
         const int kb = k / BKB, kk = k % BKB;
-        for (int i = 0; i < S; ++i) {
-            const int sh = 7 * (S - 1 - i);
-            long long d = sh > 0 ? ((F + (1ll << (sh - 1))) >> sh) : F;   // nearest digit
-            F -= d << sh;
-            out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] =
-                __float2bfloat16_rn(ldexpf((float)d, emax - 7 - 7 * i));   // exact: |d| <= 128
-        }
+        digits(at(k), emax, S, first, step, [&](int i, float d) {
+            out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] = __float2bfloat16_rn(ldexpf(d, e0 - first - step * i));
+        });
     }
 }
 
@@ -688,58 +909,31 @@ slice_rows2_kernel(const double *__restrict__ X1, int64_t ld1, int K1, const dou
     const double *x1 = X1 + row * ld1;
     const double *x2 = X2 ? X2 + row * ld2 : nullptr;
     slice_row_block([&](int k) -> double { return k < K1 ? __ldg(x1 + k) : ((x2 && k < K1 + K2) ? __ldg(x2 + k - K1) : 0.0); },
-                    row, R, Kpad, S, out);
+                    row, R, Kpad, S, kDFirst, kDStep, out);
 }
 
 // ------------------------------------------------------------- slicing
-// One warp per row.  Row maximum |x|, e with max < 2^e; each element becomes
-// the 64-bit fixed-point integer F = round(x 2^{7S-e}) (|F| < 2^{7S}, built
-// from the FP64 bit pattern with integer operations), whose balanced base-128
-// digits d_0 .. d_{S-1} (d_0 in [-128, 128], the rest in [-64, 64]) are the
-// slices: slice i = d_i 2^{e-7-7i}.  Output layout [S][K/64][R][64] (R rows in
-// all), so a 64-wide K block of consecutive rows is contiguous.  Column
+// One warp per row (as slice_row_block).  Output layout [S][K/64][R][64] (R rows
+// in all), so a 64-wide K block of consecutive rows is contiguous.  Column
 // skip_col is zero.
 __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t dest, int64_t R, int Kpad, int S,
-                                          int skip_col, __nv_bfloat16 *__restrict__ out, int lane) {
+                                          int skip_col, __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps,
+                                          int lane) {
     const int KB = Kpad / BKB;
     // exponent of the row maximum from the bit patterns (no FP64 arithmetic)
     int emax = -2000;
-    for (int k = lane; k < Kpad; k += 32) {
-        if (k == skip_col) continue;
-        const unsigned long long b = (unsigned long long)__double_as_longlong(x[k]);
-        const int be = (int)((b >> 52) & 0x7FF);
-        if (be == 0) continue;                 // zero (FP64 subnormals ignored)
-        const int e = be - 1022;               // |x| in [2^(e-1), 2^e)
-        emax = e > emax ? e : emax;
-    }
+    for (int k = lane; k < Kpad; k += 32)
+        if (k != skip_col) emax = max(emax, fp64_exponent((unsigned long long)__double_as_longlong(x[k])));
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        const int o = __shfl_xor_sync(0xffffffffu, emax, off);
-        emax = o > emax ? o : emax;
-    }
+    for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
+    if (exps && lane == 0) exps[dest] = (int16_t)(emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0));
+    const int e0 = exps ? 0 : emax;
     for (int k = lane; k < Kpad; k += 32) {
-        long long F = 0;
-        if (k != skip_col && emax > -2000) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(x[k]);
-            const int be = (int)((b >> 52) & 0x7FF);
-            if (be != 0) {
-                const long long m = (long long)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52));   // x = m 2^(be-1075)
-                const int sh = (be - 1075) + 7 * S - emax;      // F = m 2^sh, rounded to nearest
-                long long f;
-                if (sh >= 0) f = m << sh;                       // sh <= 7S - 53 < 0 in practice
-                else if (sh > -63) f = (m + (1ll << (-sh - 1))) >> (-sh);
-                else f = 0;
-                F = (b >> 63) ? -f : f;
-            }
-        }
         const int kb = k / BKB, kk = k % BKB;
-        for (int i = 0; i < S; ++i) {
-            const int sh = 7 * (S - 1 - i);
-            long long d = sh > 0 ? ((F + (1ll << (sh - 1))) >> sh) : F;   // nearest digit (floor of F/2^sh + 1/2)
-            F -= d << sh;
-            const float v = ldexpf((float)d, emax - 7 - 7 * i);            // exact: |d| <= 128
-            out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] = __float2bfloat16_rn(v);
-        }
+        digits(k != skip_col ? x[k] : 0.0, emax, S, kXFirst, kXStep, [&](int i, float d) {
+            out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] =
+                __float2bfloat16_rn(ldexpf(d, e0 - kXFirst - kXStep * i));
+        });
     }
 }
 
@@ -747,11 +941,11 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
 // zeroed on the rows with j == j' (elsewhere that label is zero, or, with
 // orbital symmetry, the column holds another label).
 __global__ void slice_rows_kernel(const double *__restrict__ X, int64_t rows, int Kpad, int S, int skip_col,
-                                  int n_co, __nv_bfloat16 *__restrict__ out) {
+                                  int n_co, __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps) {
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     const bool diag = row / n_co == row % n_co;
-    slice_row(X + row * Kpad, row, rows, Kpad, S, diag ? skip_col : -1, out, threadIdx.x & 31);
+    slice_row(X + row * Kpad, row, rows, Kpad, S, diag ? skip_col : -1, out, exps, threadIdx.x & 31);
 }
 
 // Coefficient rows (Kin entries each) into slices of Kout columns: column k
@@ -761,7 +955,7 @@ __global__ void slice_rows_kernel(const double *__restrict__ X, int64_t rows, in
 __global__ void __launch_bounds__(256)
 slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int64_t R,
                    int Kin, int Kout, const int32_t *__restrict__ perm, int S, int skip_col,
-                   __nv_bfloat16 *__restrict__ out) {
+                   __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps) {
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const SliceTask &T = tasks[ti];
     const int64_t row = blockIdx.x - blk[ti];
@@ -770,7 +964,7 @@ slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restric
         if (k == skip_col) return 0.0;
         const int lab = perm ? __ldg(perm + k) : k;
         return (lab >= 0 && lab < Kin) ? __ldg(x + lab) : 0.0;
-    }, T.row0 + row, R, Kout, S, out);
+    }, T.row0 + row, R, Kout, S, kXFirst, kXStep, out, exps);
 }
 
 // Rows with j == j' (both ranges): H[(n,j),(n',j)] over all K, incl. delta,
@@ -847,6 +1041,57 @@ diag_rows_kernel(const DRTask *__restrict__ tasks, const int64_t *__restrict__ b
     if (r != c) T.H[c * T.ld + r] = v;
 }
 
+// The same in FP64, for the FP64 build: a thread adds one element's labels in
+// their order, so the sums do not depend on which labels a symmetry-blocked
+// panel leaves out (their terms are zero).  150 rows x 210 pairs x 1367 labels
+// hold the FP64 pipe for 68 us.
+constexpr int kD64k = 32;
+__global__ void __launch_bounds__(kDRthreads)
+diag_rows_f64_kernel(const DRTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+    __shared__ double sp[kDRj][kD64k + 1], sa[kDRt][kD64k + 1];
+    const int ti = task_of(blk, n_tasks, blockIdx.x);
+    const DRTask &T = tasks[ti];
+    const int lb = (int)(blockIdx.x - blk[ti]);
+    const int j0 = T.j_lo + (lb / T.ny) * kDRj, t0 = (lb % T.ny) * kDRt;
+    const int tl = threadIdx.x % kDRt, jl = threadIdx.x / kDRt;
+    const int j = j0 + jl, t = t0 + tl;
+    constexpr int per = kDRj * kD64k / kDRthreads;
+    double rp[per], ra[per];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < per; ++u) {
+            const int i = threadIdx.x + u * kDRthreads;
+            const int r = i / kD64k, k = k0 + i % kD64k;
+            const bool kin = k < T.Kpad;
+            const int lab = (kin && T.perm) ? __ldg(T.perm + k) : k;   // the label of panel column k
+            rp[u] = (kin && j0 + r < T.j_hi) ? __ldg(T.P64 + ((int64_t)(j0 + r) * T.n_co + j0 + r) * T.Kpad + k) : 0.0;
+            ra[u] = (kin && lab >= 0 && t0 + r < T.n_nn) ? __ldg(T.A64 + (int64_t)(t0 + r) * T.Ka + lab) : 0.0;
+        }
+    };
+    double v = 0.0;
+    fetch(0);
+    for (int k0 = 0; k0 < T.Kpad; k0 += kD64k) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < per; ++u) {
+            const int i = threadIdx.x + u * kDRthreads;
+            sp[i / kD64k][i % kD64k] = rp[u];
+            sa[i / kD64k][i % kD64k] = ra[u];
+        }
+        __syncthreads();
+        if (k0 + kD64k < T.Kpad) fetch(k0 + kD64k);
+#pragma unroll 8
+        for (int k = 0; k < kD64k; ++k) v = fma(sp[jl][k], sa[tl][k], v);
+    }
+    if (j >= T.j_hi || t >= T.n_nn) return;
+    const int na = T.nn[2 * t], nb = T.nn[2 * t + 1];
+    const int64_t r = T.row_off + (int64_t)na * T.cn + (j - T.cf);
+    const int64_t c = T.col_off + (int64_t)nb * T.cnp + (j - T.cfp);
+    if (T.same && r < c) return;
+    T.H[r * T.ld + c] = v;
+    if (r != c) T.H[c * T.ld + r] = v;
+}
+
 // Diagonal panel rows P[(j, j)][k] as float pairs.
 __global__ void panel_diag_df_kernel(const double *__restrict__ P, int n_co, int Kpad, float2 *__restrict__ out) {
     const int j = blockIdx.x;
@@ -880,7 +1125,9 @@ EncodeTiled encode_fn() {
 
 // dynamic shared memory of the expansion kernel: the operand slots, the
 // barriers and the 1 KB alignment
-static int split_smem_bytes(int S, int bn, int ks) { return xsets(S, bn, ks) * S * xslot(bn, ks) + 2048; }
+static int split_smem_bytes(int bn, int ks) {
+    return xslots(bn, ks) * xslot(bn, ks) + 1024 + (2 * XBARS + 2 * XACC + 2) * 8;
+}
 
 static int sm_count() {
     static int n = 0;
@@ -895,26 +1142,29 @@ static int sm_count() {
     return n;
 }
 
-template <int S>
+template <int S, bool F64>
 static cudaError_t set_smem_attr_s() {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(split_expand_kernel<S, 32, 32>, attr, split_smem_bytes(S, 32, 32));
+    cudaError_t e = cudaFuncSetAttribute(split_expand_kernel<S, 32, 32, F64>, attr, split_smem_bytes(32, 32));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(split_expand_kernel<S, 64, 32>, attr, split_smem_bytes(S, 64, 32));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 32>, attr, split_smem_bytes(S, 128, 32));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 64>, attr, split_smem_bytes(S, 128, 64));
+        e = cudaFuncSetAttribute(split_expand_kernel<S, 64, 32, F64>, attr, split_smem_bytes(64, 32));
+    if constexpr (!F64) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 32, F64>, attr, split_smem_bytes(128, 32));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 64, F64>, attr, split_smem_bytes(128, 64));
+    }
     return e;
 }
 
 static cudaError_t set_smem_attr(int S) {
     switch (S) {
-        case 2: return set_smem_attr_s<2>();
-        case 3: return set_smem_attr_s<3>();
-        case 4: return set_smem_attr_s<4>();
-        case 5: return set_smem_attr_s<5>();
-        default: return set_smem_attr_s<6>();
+        case 2: return set_smem_attr_s<2, false>();
+        case 3: return set_smem_attr_s<3, false>();
+        case 4: return set_smem_attr_s<4, false>();
+        case 5: return set_smem_attr_s<5, false>();
+        case 6: return set_smem_attr_s<6, false>();
+        default: return set_smem_attr_s<kF64Slices, true>();
     }
 }
 
@@ -923,47 +1173,56 @@ static int mixed_fail(hb_ctx *ctx, int code, const std::string &m) {
     return code;
 }
 
-// Panel slices and their tensor map, once per context (the integrals do not
-// change between builds); a context that borrows its integrals borrows these.
-int mixed_prepare(hb_ctx *ctx, cudaStream_t s) {
+// Panel slices and their tensor maps, once per context and precision (the
+// integrals do not change between builds); a context that borrows its
+// integrals borrows these.
+int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     if (!ctx->mixed) ctx->mixed = new MixedState();
     MixedState &M = *ctx->mixed;
-    if (M.panel_ready) return HB_OK;
+    PanelSlices &PS = M.panel[precision == HB_MIXED];
+    if (PS.ready) return HB_OK;
     if (ctx->base) {
-        int rc = mixed_prepare(ctx->base, s);
+        int rc = mixed_prepare(ctx->base, precision, s);
         if (rc != HB_OK) return mixed_fail(ctx, rc, ctx->base->err);
-        const MixedState &B = *ctx->base->mixed;
-        M.slices = B.slices;
-        M.panel_rows = B.panel_rows;
-        M.panel_slices = B.panel_slices;
-        for (int w = 0; w < 2; ++w)
-            for (int i = 0; i < 3; ++i) M.tm_panel[w][i] = B.tm_panel[w][i];
-        M.pdiag = B.pdiag;
-        M.borrowed_panel = true;
-        M.panel_ready = true;
+        PS = ctx->base->mixed->panel[precision == HB_MIXED];
+        PS.borrowed = true;
+        if (precision == HB_MIXED) M.pdiag = ctx->base->mixed->pdiag;
         return HB_OK;
     }
-    M.slices = ctx->split_slices;
-    if (M.slices < 2 || M.slices > MAXS) return mixed_fail(ctx, HB_ERR_INVALID_ARG, "split_slices must be 2..6");
+    PS.slices = precision == HB_MIXED ? ctx->expand_slices : kF64Slices;
+    if (precision == HB_MIXED && (PS.slices < 2 || PS.slices > MAXS))
+        return mixed_fail(ctx, HB_ERR_INVALID_ARG, "split_slices must be 2..6");
     if (!encode_fn()) return mixed_fail(ctx, HB_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
     const int64_t rows = (int64_t)ctx->n_co * ctx->n_co;
-    M.panel_rows = rows;
     // the panel's columns: every label, or with orbital symmetry the Kc labels
     // of each row's class
     const int Kc = ctx->Kc;
-    cudaError_t e = dmalloc(ctx, (void **)&M.panel_slices, sizeof(__nv_bfloat16) * (size_t)M.slices * rows * Kc);
-    if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_OOM, std::string("panel slices: ") + cudaGetErrorString(e));
-    ctx->dev_bytes += sizeof(__nv_bfloat16) * (size_t)M.slices * rows * Kc;
-    e = dmalloc_n(ctx, &M.pdiag, (size_t)ctx->n_co * Kc);
-    if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_OOM, std::string("panel rows: ") + cudaGetErrorString(e));
-    ctx->dev_bytes += sizeof(float2) * (size_t)ctx->n_co * Kc;
-    panel_diag_df_kernel<<<ctx->n_co, 256, 0, s>>>(ctx->panel, ctx->n_co, Kc, M.pdiag);
-    slice_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ctx->panel, rows, Kc, M.slices, ctx->delta_pos,
-                                                                 ctx->n_co, M.panel_slices);
+    const size_t bytes = sizeof(__nv_bfloat16) * (size_t)PS.slices * rows * Kc;
+    cudaError_t e = dmalloc(ctx, (void **)&PS.buf, bytes);
+    if (e == cudaSuccess && precision == HB_FP64) {
+        e = dmalloc_n(ctx, &PS.exps, (size_t)rows);
+        if (e != cudaSuccess) {
+            dfree(ctx, PS.buf);
+            PS.buf = nullptr;
+        }
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return mixed_fail(ctx, HB_ERR_OOM, std::string("panel slices: ") + cudaGetErrorString(e));
+    }
+    ctx->dev_bytes += bytes + (PS.exps ? sizeof(int16_t) * (size_t)rows : 0);
+    if (precision == HB_MIXED) {
+        e = dmalloc_n(ctx, &M.pdiag, (size_t)ctx->n_co * Kc);
+        if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_OOM, std::string("panel rows: ") + cudaGetErrorString(e));
+        ctx->dev_bytes += sizeof(float2) * (size_t)ctx->n_co * Kc;
+        panel_diag_df_kernel<<<ctx->n_co, 256, 0, s>>>(ctx->panel, ctx->n_co, Kc, M.pdiag);
+    }
+    slice_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ctx->panel, rows, Kc, PS.slices, ctx->delta_pos,
+                                                                 ctx->n_co, PS.buf, PS.exps);
     // 4D map over the panel slices [S*KB][j][j'][64]: coordinates (kk, j', j, plane)
     const int KB = Kc / BKB;
     cuuint64_t dims[4] = {(cuuint64_t)BKB, (cuuint64_t)ctx->n_co, (cuuint64_t)ctx->n_co,
-                          (cuuint64_t)M.slices * KB};
+                          (cuuint64_t)PS.slices * KB};
     cuuint64_t strides[3] = {(cuuint64_t)BKB * 2, (cuuint64_t)ctx->n_co * BKB * 2, (cuuint64_t)rows * BKB * 2};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = CUDA_SUCCESS;
@@ -973,32 +1232,46 @@ int mixed_prepare(hb_ctx *ctx, cudaStream_t s) {
             // a 32-K stage copies half a 64-wide K block (x = 0 or 32: 64-byte
             // aligned, 64-byte swizzle), a 64-K stage all of it (128-byte swizzle)
             cuuint32_t box[4] = {w ? 64u : 32u, (cuuint32_t)(1 << lg), (cuuint32_t)(BM >> lg), 1};
-            r = encode_fn()(&M.tm_panel[w][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, M.panel_slices, dims, strides,
+            r = encode_fn()(&PS.tm[w][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, PS.buf, dims, strides,
                             box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             w ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         }
     if (r != CUDA_SUCCESS) return mixed_fail(ctx, HB_ERR_CUDA, "panel tensor map: error " + std::to_string((int)r));
-    e = set_smem_attr(M.slices);
+    e = set_smem_attr(PS.slices);
     if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_CUDA, std::string("smem attribute: ") + cudaGetErrorString(e));
-    M.panel_ready = true;
+    PS.ready = true;
     return HB_OK;
 }
 
-const void *mixed_panel_key(const hb_ctx *ctx) { return ctx->mixed ? ctx->mixed->panel_slices : nullptr; }
+const void *mixed_panel_key(const hb_ctx *ctx, int precision) {
+    return ctx->mixed ? ctx->mixed->panel[precision == HB_MIXED].buf : nullptr;
+}
 const float2 *mixed_panel_diag(const hb_ctx *ctx) { return ctx->mixed ? ctx->mixed->pdiag : nullptr; }
-int mixed_slices(const hb_ctx *ctx) { return ctx->mixed ? ctx->mixed->slices : ctx->split_slices; }
+int mixed_slices(const hb_ctx *ctx, int precision) {
+    return precision == HB_MIXED ? (ctx->mixed ? ctx->mixed->panel[1].slices : ctx->expand_slices) : kF64Slices;
+}
 
 // Coefficient slices of `rows` rows in all: [S][Kpad/64][rows][64] bf16 and
 // four 3D maps: for 32-K stages one per tile width bn = 32, 64, 128 (box: bn
 // rows x half a K block of one slice plane, 64-byte swizzle), and for 64-K
 // stages one of 128 rows x a whole K block (128-byte swizzle).
-int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, CUtensorMap *tm, std::string *err) {
+// exps (FP64 build, or null): the rows' exponents.
+int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int16_t **exps, CUtensorMap *tm,
+                     std::string *err) {
     *buf = nullptr;
+    if (exps) *exps = nullptr;
     if (!encode_fn()) { *err = "cuTensorMapEncodeTiled is not available"; return HB_ERR_CUDA; }
     if (rows < 1) rows = 1;
     cudaError_t e = dmalloc(mem, buf, sizeof(__nv_bfloat16) * (size_t)S * rows * Kpad);
-    if (e != cudaSuccess) { *err = std::string("coefficient slices: ") + cudaGetErrorString(e); return HB_ERR_OOM; }
+    if (e == cudaSuccess && exps) e = dmalloc_n(mem, exps, (size_t)rows);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        dfree(mem, *buf);
+        *buf = nullptr;
+        *err = std::string("coefficient slices: ") + cudaGetErrorString(e);
+        return HB_ERR_OOM;
+    }
     const int KB = Kpad / BKB;
     cuuint64_t dims[3] = {(cuuint64_t)BKB, (cuuint64_t)rows, (cuuint64_t)S * KB};
     cuuint64_t strides[2] = {(cuuint64_t)BKB * 2, (cuuint64_t)rows * BKB * 2};
@@ -1013,6 +1286,7 @@ int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, CUt
     if (r != CUDA_SUCCESS) {
         dfree(mem, *buf);
         *buf = nullptr;
+        if (exps) { dfree(mem, *exps); *exps = nullptr; }
         *err = "coefficient tensor map: error " + std::to_string((int)r);
         return HB_ERR_CUDA;
     }
@@ -1036,13 +1310,18 @@ int split_cols_choice(int N, int kblocks, int force) {
     if (kblocks >= kK64Blocks) return 128;
     return N <= 32 ? 32 : (N <= 64 ? 64 : 128);
 }
+// The FP64 kernel's seven accumulators fit tensor memory up to 64 columns; its
+// sums are exact, so no shape changes a bit.
+int split_f64_cols_choice(int N, int force) { return force == 32 || (force == 0 && N <= 32) ? 32 : 64; }
 int split_jpt(int cnp, int lg) { return (cnp + (1 << lg) - 1) >> lg; }
 
-// Tile arrangement with the least padding of the cn x cnp rectangle (ties: 8 x 16).
+// Tile arrangement with the least padding of the cn x cnp rectangle; of equal
+// ones 16 x 8, whose warps (4 j x 8 j') write whole 32-byte sectors of both the
+// block and its mirror.
 int split_tile_heuristic(int cn, int cnp) {
-    int best = 4;
+    int best = 3;
     int64_t best_area = -1;
-    for (int lg : {4, 3, 5}) {
+    for (int lg : {3, 4, 5}) {
         const int bj = BM >> lg, bjp = 1 << lg;
         const int64_t area = (int64_t)((cn + bj - 1) / bj) * bj * ((cnp + bjp - 1) / bjp) * bjp;
         if (best_area < 0 || area < best_area) { best = lg; best_area = area; }
@@ -1051,10 +1330,10 @@ int split_tile_heuristic(int cn, int cnp) {
 }
 
 int g_slice(const Grouped<SliceTask> &g, int64_t R, int Kin, int Kout, const int32_t *perm, int S, int skip_col,
-            void *out, cudaStream_t s) {
+            void *out, int16_t *exps, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
     slice_rows_grouped<<<(unsigned)g.blocks, 256, 0, s>>>(g.tasks, g.blk, g.n, R, Kin, Kout, perm, S, skip_col,
-                                                          (__nv_bfloat16 *)out);
+                                                          (__nv_bfloat16 *)out, exps);
     return 1;
 }
 
@@ -1064,31 +1343,39 @@ int split_kstage_choice(int bn, int kblocks, int force) {
     return kblocks >= kK64Blocks ? 64 : 32;
 }
 
-int g_split(const hb_ctx *panel_ctx, int lg, int bn, const CUtensorMap *tm_coef, const Grouped<SplitTask> &g,
-            int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s, int shard_r, int shard_n) {
+int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef, const int16_t *coef_exps,
+            const Grouped<SplitTask> &g, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s,
+            int shard_r, int shard_n) {
     if (g.blocks <= 0) return 0;
-    if (bn != 32 && bn != 64 && bn != 128) return 0;
-    const MixedState &M = *panel_ctx->mixed;
-    const int ks = split_kstage_choice(bn, kblocks, panel_ctx->force_kstage);
-    const CUtensorMap &tm_panel = M.tm_panel[ks == 64 ? 1 : 0][lg - 3];
+    const bool f64 = precision != HB_MIXED;
+    if (bn != 32 && bn != 64 && (f64 || bn != 128)) return 0;
+    const PanelSlices &PS = panel_ctx->mixed->panel[!f64];
+    const int ks = f64 ? 32 : split_kstage_choice(bn, kblocks, panel_ctx->force_kstage);
+    const CUtensorMap &tm_panel = PS.tm[ks == 64 ? 1 : 0][lg - 3];
     const CUtensorMap &tm_c = tm_coef[ks == 64 ? 3 : (bn == 32 ? 0 : (bn == 64 ? 1 : 2))];
-    const size_t smem = split_smem_bytes(M.slices, bn, ks);
-    // persistent: one CTA per SM at most (each holds its SM's tensor memory or half of it)
+    const size_t smem = split_smem_bytes(bn, ks);
+    // persistent: one CTA per SM at most (each fills its SM's shared memory)
     const int n_tiles = (int)g.blocks;
     const int n_local = n_tiles > shard_r ? (n_tiles - shard_r + shard_n - 1) / shard_n : 0;
     if (n_local <= 0) return 0;
     const unsigned grid = (unsigned)std::min(n_local, sm_count());
-#define HB_SPLIT(SS, BB, KK)                                                                                    \
-    split_expand_kernel<SS, BB, KK><<<grid, NTHREADS, smem, s>>>(tm_panel, tm_c, g.tasks, g.blk, g.n, n_tiles, \
-                                                                kblocks, coef_planes, cols, err, shard_r, shard_n)
-#define HB_SPLIT_S(SS)                                 \
-    do {                                               \
-        if (bn == 32) HB_SPLIT(SS, 32, 32);            \
-        else if (bn == 64) HB_SPLIT(SS, 64, 32);       \
-        else if (ks == 32) HB_SPLIT(SS, 128, 32);      \
-        else HB_SPLIT(SS, 128, 64);                    \
+#define HB_SPLIT(SS, BB, KK, FF)                                                                                   \
+    split_expand_kernel<SS, BB, KK, FF><<<grid, NTHREADS, smem, s>>>(tm_panel, tm_c, g.tasks, g.blk, g.n, n_tiles, \
+                                                                     kblocks, coef_planes, cols, PS.exps, coef_exps,    \
+                                                                     panel_ctx->n_co, err, shard_r, shard_n)
+#define HB_SPLIT_S(SS)                                \
+    do {                                              \
+        if (bn == 32) HB_SPLIT(SS, 32, 32, false);        \
+        else if (bn == 64) HB_SPLIT(SS, 64, 32, false);   \
+        else if (ks == 32) HB_SPLIT(SS, 128, 32, false);  \
+        else HB_SPLIT(SS, 128, 64, false);                \
     } while (0)
-    switch (M.slices) {
+    if (f64) {
+        if (bn == 32) HB_SPLIT(kF64Slices, 32, 32, true);
+        else HB_SPLIT(kF64Slices, 64, 32, true);
+        return 1;
+    }
+    switch (PS.slices) {
         case 2: HB_SPLIT_S(2); break;
         case 3: HB_SPLIT_S(3); break;
         case 4: HB_SPLIT_S(4); break;
@@ -1106,9 +1393,10 @@ int64_t blocks_diag_rows(int j_lo, int j_hi, int n_nn) {
 }
 int diag_rows_ny(int n_nn) { return (n_nn + kDRt - 1) / kDRt; }
 
-int g_diag_rows(const Grouped<DRTask> &g, cudaStream_t s) {
+int g_diag_rows(const Grouped<DRTask> &g, int dfloat, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
-    diag_rows_kernel<<<(unsigned)g.blocks, kDRthreads, 0, s>>>(g.tasks, g.blk, g.n);
+    if (!dfloat) diag_rows_f64_kernel<<<(unsigned)g.blocks, kDRthreads, 0, s>>>(g.tasks, g.blk, g.n);
+    else diag_rows_kernel<<<(unsigned)g.blocks, kDRthreads, 0, s>>>(g.tasks, g.blk, g.n);
     return 1;
 }
 
@@ -1197,10 +1485,12 @@ int dense_split_gemm(int S, const DenseOperand &A, int64_t M, const DenseOperand
 
 void release_mixed(hb_ctx *ctx) {
     if (!ctx->mixed) return;
-    if (!ctx->mixed->borrowed_panel) {
-        dfree(ctx, ctx->mixed->panel_slices);
-        dfree(ctx, ctx->mixed->pdiag);
-    }
+    for (PanelSlices &P : ctx->mixed->panel)
+        if (!P.borrowed) {
+            dfree(ctx, P.buf);
+            dfree(ctx, P.exps);
+        }
+    if (!ctx->mixed->panel[1].borrowed) dfree(ctx, ctx->mixed->pdiag);
     delete ctx->mixed;
     ctx->mixed = nullptr;
 }
