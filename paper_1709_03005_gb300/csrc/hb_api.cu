@@ -633,7 +633,7 @@ int stage_problem(hb_ctx *ctx, const hb_problem *p, const hb_options *o, cudaStr
         DALLOC(P.W, (int64_t)A.ndet * B.ns);
         DALLOC(P.partial, (int64_t)tn_chunks(A.ndet) * nout);
         DALLOC(P.partial_s, P.same ? (int64_t)tn_chunks(A.ndet) * nout : 1);
-        DALLOC(P.gdiag, P.same ? (int64_t)tn_chunks(A.ndet) * 2 * p->n_to * nout : 1);
+        DALLOC(P.gdiag, P.same ? (int64_t)gdiag_chunks(A.ndet) * 2 * p->n_to * nout : 1);
         DALLOC(P.S, nout);
         DALLOC(P.E, nout);
         std::vector<int32_t> nn;
@@ -750,7 +750,7 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
     // the call that waits for it, or by the next one
     if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
     int launches = 0;
-    int rc = plan_run(plan, s, true, false, &launches, &err);
+    int rc = plan_launch(plan, s, &launches, &err);
     if (rc != HB_OK) return fail(ctx, rc, err);
     if (precision == HB_MIXED) {
         // the tensor-core kernel reports a bounded-wait timeout in a device word

@@ -29,6 +29,8 @@ int plan_host_error(hb::Plan *p);
 // Issue every stage on stream s.  timing: record the stage events (as graph
 // event nodes when capture is set).  *launches: kernels launched.
 int plan_run(hb::Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, std::string *err);
+// a whole build, replayed as a graph where the same one is repeated
+int plan_launch(hb::Plan *p, cudaStream_t s, int *launches, std::string *err);
 // After the stream has finished a timed run: per-stage times and counters.
 void plan_stats(hb::Plan *p, hb_stats *st);
 // Time the result-identical launch-shape candidates of every tunable stage

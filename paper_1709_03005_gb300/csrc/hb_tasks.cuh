@@ -79,6 +79,9 @@ struct IFTask {         // gamma items of the records of a group pair
     int W, n_to, n_elec;
     const int64_t *item_ptr;
     GammaItem *items;
+    int64_t item0;            // first item of the sort, whose chunks hold `chunk` items
+    int nc, chunk;
+    int64_t *off;             // the sort's counts per (key, chunk)
 };
 
 struct ZTask {          // zero n 8-byte words
@@ -112,6 +115,7 @@ struct GTask {          // gamma[key][n][n'] over the sorted items
     const double *Cp;
     const float2 *Cp_df;
     int nsp, ny;
+    int kpb;                  // keys a block (or warp) takes
     double *gamma;
 };
 
@@ -277,13 +281,15 @@ constexpr int kL2MirrorThreads = 256;
 // width: states per pass of the double-float kernel (16, 24 or 32; the
 // largest state count of the launch, rounded up, passes of 32 beyond)
 int g_sandwich(const Grouped<SWTask> &g, int dfloat, int width, cudaStream_t s);
-int g_sandwich_small(const Grouped<SWTask> &g, int dfloat, cudaStream_t s);    // nsp <= 32 (used for nsp <= 16)
+// nsp <= 32 (used for nsp <= 16); block_rows: a block per row, else 8 rows a block (the same sums)
+int g_sandwich_small(const Grouped<SWTask> &g, int dfloat, int block_rows, cudaStream_t s);
 int g_tn_partial(const Grouped<TNTask> &g, size_t smem, int dfloat, cudaStream_t s);
 int g_tn_reduce(const Grouped<TNTask> &g, int dfloat, cudaStream_t s);
-int g_item_fill(const Grouped<IFTask> &g, cudaStream_t s);
+// items and their counts per (key, chunk); block_rows: a block per row, else 8 rows a block
+int g_item_fill(const Grouped<IFTask> &g, int block_rows, cudaStream_t s);
 int g_zero(const Grouped<ZTask> &g, cudaStream_t s);
-int g_sort_hist(const Grouped<SortTask> &g, cudaStream_t s);
-int g_scan(const Grouped<ScanTask> &g, cudaStream_t s);
+// longest: entries of the longest table
+int g_scan(const Grouped<ScanTask> &g, int64_t longest, cudaStream_t s);
 int64_t blocks_scan(int64_t n);
 int g_sort_scatter(const Grouped<SortTask> &g, cudaStream_t s);
 int g_gamma(const Grouped<GTask> &g, size_t smem, int dfloat, cudaStream_t s);
@@ -310,8 +316,13 @@ int64_t blocks_tn_partial(int n_rows, int ns, int nsp);
 int64_t blocks_tn_reduce(int ns, int nsp);
 int64_t blocks_zero(int64_t n);
 int64_t blocks_sort(int64_t n_items, int n_keys);
-int64_t blocks_gamma(int n_keys, int ns, int nsp);
-int64_t blocks_gamma_warp(int n_keys);
+int sort_chunk_items(int64_t n_items, int n_keys);
+// keys a block (or warp) takes: one, or eight where most hold no items
+int gamma_keys_per(int64_t n_items, int n_keys);
+int64_t blocks_gamma(int n_keys, int kpb, int ns, int nsp);
+int64_t blocks_gamma_warp(int n_keys, int kpb);
+int64_t blocks_assemble(int n_nn, int Kpad);
+int gdiag_chunks(int ndet);
 int64_t blocks_expand_fp64(int cn, int cnp, int N);
 int64_t blocks_class4(int n_l2, int cn, int jt);
 int tn_ny(int ns, int nsp);

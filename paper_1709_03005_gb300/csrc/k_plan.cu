@@ -98,6 +98,8 @@ struct Plan {
     Stage<PVTask> pv;
     Stage<PVTask> pvd;                 // the diagonal records of same-group pairs
     Stage<SWTask> sw, sws;             // sandwich: lanes over records / over states
+    bool block_rows = true;            // a block per target row (else 8 rows a block)
+    int64_t scan_longest = 0;          // entries of the longest sort table
     int sw_width = 16;                 // states per pass of the record-lane sandwich
     Stage<TNTask> tn, tnr;
     Stage<IFTask> itf;
@@ -143,9 +145,13 @@ struct Plan {
     CUtensorMap tm_coef[4];            // coefficient slices: 32-K stages at widths 32, 64, 128; 64-K at 128
     int64_t coef_rows = 0;
     int *err = nullptr;
-    // FP64 build on the tensor cores: its error word as of the last finished
-    // build (page-locked; such builds are not waited for)
+    // the error words as of the last finished build (page-locked, behind the
+    // staged tables)
     int *host_err = nullptr;
+    // the plan as a graph, for builds repeated into the same blocks (plan_launch)
+    cudaGraphExec_t exec = nullptr;
+    int runs = 0;                      // builds into these blocks so far
+    bool no_graph = false;
     // classes 4, 2 and 8 run on a second stream beside the target side and
     // the expansion (they read only staged data and write their own blocks);
     // the target side and the expansion at higher priority, the second stream
@@ -155,7 +161,7 @@ struct Plan {
     // the target side's independent chains: the diagonal H^N values and the
     // gamma items (aux1), the diagonal gamma (aux2), beside the E, S chain
     cudaStream_t aux1 = nullptr, aux2 = nullptr;
-    cudaEvent_t k1_done = nullptr, items_done = nullptr, gd_done = nullptr, dv_done = nullptr;
+    cudaEvent_t k1_done = nullptr, items_done = nullptr, gd_done = nullptr, asm_done = nullptr, dr_done = nullptr;
     cudaEvent_t c4_done = nullptr;     // the tensor-core class-4 kernel has finished (side stream)
     // timers: start, target, expansion (main stream); class-4 end, L2 end, side
     // start (side stream); end after the join; L2 start, class-4 classification
@@ -223,6 +229,14 @@ void fill_tasks(Plan &p) {
     p.smem_tn = p.smem_gamma = p.smem_gd = 0;
     p.flops = 0.0;
     p.n_expand_tasks = 0;
+    p.scan_longest = 0;
+    // few target rows: a block per row, so that the longest does not set a
+    // stage's time; many: 8 rows a block (335400 blocks of one row, 42 records on
+    // average, took 448 us to start and end)
+    int64_t rows = 0;
+    for (const hb_ctx *c : p.ctxs)
+        for (auto &P : c->gps) rows += c->groups[P.g].ndet;
+    p.block_rows = rows <= 64 * 1024;
     int64_t coef_row = 0;
     // expansion blocks: the group pairs (of any context) that read the same
     // continuum rectangle of the same panel share one GEMM
@@ -274,7 +288,7 @@ void fill_tasks(Plan &p) {
             // groups per warp), lanes over the records otherwise
             {
                 const SWTask sw{P.pairs, P.rowptr + m0, P.val, nm, Cb, Cb_df, B.ns, P.W + (int64_t)m0 * B.ns};
-                if (B.ns <= 16) p.sws.add(sw, blocks_rows8(nm));
+                if (B.ns <= 16) p.sws.add(sw, p.block_rows ? nm : blocks_rows8(nm));
                 else p.sw.add(sw, nm);                        // a block per row
             }
             if (B.ns > 16) p.sw_width = std::max(p.sw_width, B.ns <= 24 ? 24 : 32);
@@ -299,15 +313,18 @@ void fill_tasks(Plan &p) {
                 i0 = ir.first;
                 n_it = ir.second - ir.first;
             }
-            p.itf.add(IFTask{P.pairs, P.rowptr + m0, nm, da, W, ctx->n_to, ctx->n_elec, P.item_ptr + m0, P.items},
-                      nm);                                    // a block per row
             const int nc = P.n_chunks;
+            p.itf.add(IFTask{P.pairs, P.rowptr + m0, nm, da, W, ctx->n_to, ctx->n_elec, P.item_ptr + m0, P.items, i0, nc,
+                             sort_chunk_items(n_it, n_keys), P.sort_off},
+                      p.block_rows ? nm : blocks_rows8(nm));
             const int64_t n_off = (int64_t)n_keys * nc;
             GammaItem *its = P.items + i0;
             p.zero.add(ZTask{P.sort_off, n_off + 1}, blocks_zero(n_off + 1));
             p.sort.add(SortTask{its, n_it, nc, n_keys, P.sort_off, P.sort_cur, P.order}, blocks_sort(n_it, n_keys));
             p.scan.add(ScanTask{P.sort_off, n_off, P.sort_cur, P.sort_part}, blocks_scan(n_off));
-            const GTask gt{its, P.order, P.sort_off, nc, n_keys, Ca, Ca_df, A.ns, Cb, Cb_df, B.ns, ny, P.gamma};
+            p.scan_longest = std::max(p.scan_longest, n_off);
+            const int kpb = gamma_keys_per(n_it, n_keys);
+            const GTask gt{its, P.order, P.sort_off, nc, n_keys, Ca, Ca_df, A.ns, Cb, Cb_df, B.ns, ny, kpb, P.gamma};
             const int nout = A.ns * B.ns;
             bool warp = nout <= 64;
             if (warp) {
@@ -316,9 +333,9 @@ void fill_tasks(Plan &p) {
                 p.tune_gamma.push_back(TuneGamma{gt});
             }
             if (warp) {
-                p.gamw.add(gt, blocks_gamma_warp(n_keys));
+                p.gamw.add(gt, blocks_gamma_warp(n_keys, kpb));
             } else {
-                p.gam.add(gt, blocks_gamma(n_keys, A.ns, B.ns));
+                p.gam.add(gt, blocks_gamma(n_keys, kpb, A.ns, B.ns));
                 p.smem_gamma = std::max(p.smem_gamma, smem_stage(A.ns, B.ns));
             }
             if (P.same) {
@@ -333,7 +350,7 @@ void fill_tasks(Plan &p) {
                              ctx->cont_spin, ctx->Kpad,
                              ctx->e_core, P.A, p.precision == HB_MIXED ? P.A_df : nullptr,
                              ctx->energy ? ctx->energy + A.e_off : nullptr, ctx->energy && p.shard_r != 0},
-                       P.n_nn);
+                       blocks_assemble(P.n_nn, ctx->Kpad));
             p.flops += 2.0 * (double)A.cn * B.cn * P.n_nn * class_label_count(ctx, A.cf, B.cf);
             ++p.n_expand_tasks;
             // the pair joins the expansion block of its continuum rectangle
@@ -548,10 +565,16 @@ int upload(Plan &p, std::string *err, cudaStream_t s) {
         if (p.pinned) cudaFreeHost(p.pinned);
         p.dev = nullptr;
         p.pinned = nullptr;
+        p.host_err = nullptr;
         p.dev_size = 0;
         e = dmalloc_n(p.ctxs[0], &p.dev, p.host.size());
-        if (e == cudaSuccess) e = cudaMallocHost((void **)&p.pinned, p.host.size());
-        if (e == cudaSuccess) p.dev_size = p.host.size();
+        const size_t tables = align256(p.host.size());
+        if (e == cudaSuccess) e = cudaMallocHost((void **)&p.pinned, tables + 256);
+        if (e == cudaSuccess) {
+            p.dev_size = p.host.size();
+            p.host_err = (int *)(p.pinned + tables);
+            p.host_err[0] = p.host_err[1] = 0;
+        }
     }
     if (e == cudaSuccess && !p.host.empty()) {
         memcpy(p.pinned, p.host.data(), p.host.size());
@@ -609,7 +632,7 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->side, cudaStreamNonBlocking, least);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->aux1, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->aux2, cudaStreamNonBlocking, greatest);
-    for (cudaEvent_t *ev : {&p->k1_done, &p->items_done, &p->gd_done, &p->dv_done})
+    for (cudaEvent_t *ev : {&p->k1_done, &p->items_done, &p->gd_done, &p->asm_done, &p->dr_done})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = dmalloc_n(ctxs[0], &p->err, 2);   // split kernel, class-4 kernel
     if (e == cudaSuccess) e = cudaMemsetAsync(p->err, 0, 2 * sizeof(int), s);
@@ -689,13 +712,7 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
             fill_tasks(*p);
             rc = HB_OK;
         }
-        if (rc == HB_OK && p->split_on && precision == HB_FP64 &&
-            cudaMallocHost((void **)&p->host_err, sizeof(int)) != cudaSuccess) {
-            rc = HB_ERR_CUDA;
-            *err = "plan: page-locked error word";
-        }
         if (rc != HB_OK) { plan_destroy(p); return rc; }
-        if (p->host_err) *p->host_err = 0;
         ensure_split_events(*p);
     }
     pack_all(*p);
@@ -722,7 +739,14 @@ int plan_host_error(Plan *p) {
     return w;
 }
 
+static void drop_graph(Plan *p) {
+    if (p->exec) cudaGraphExecDestroy(p->exec);
+    p->exec = nullptr;
+    p->runs = 0;
+}
+
 int plan_set_outputs(Plan *p, const hb_blocks *outs, std::string *err, cudaStream_t s) {
+    drop_graph(p);
     p->outs.assign(outs, outs + p->outs.size());
     fill_tasks(*p);
     ensure_split_events(*p);
@@ -865,8 +889,8 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
             size_t smem = 0;
             for (auto *t : kv.second) {
                 ts.push_back(t->t);
-                nbw.push_back(blocks_gamma_warp(t->t.n_keys));
-                nbb.push_back(blocks_gamma(t->t.n_keys, t->t.ns, t->t.nsp));
+                nbw.push_back(blocks_gamma_warp(t->t.n_keys, t->t.kpb));
+                nbb.push_back(blocks_gamma(t->t.n_keys, t->t.kpb, t->t.ns, t->t.nsp));
                 smem = std::max(smem, smem_stage(t->t.ns, t->t.nsp));
             }
             const int DF = p->precision == HB_MIXED ? 1 : 0;
@@ -877,6 +901,7 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { *err = std::string("autotune: ") + cudaGetErrorString(e); return HB_ERR_CUDA; }
+    drop_graph(p);
     p->choice = ch;
     p->tuned = true;
     fill_tasks(*p);
@@ -986,33 +1011,33 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     // target side (Eq. 8) in three chains that meet at the coefficient rows:
     // the diagonal gamma needs only the determinants and CI vectors
     cudaStreamWaitEvent(sb, p->fork, 0);
+    if (ph2 && p->coef_rows > 0) cudaMemsetAsync(p->err, 0, sizeof(int), sb);
     if (ph1) {
         L += g_gdiag(p->gdp.g, p->gdr.g, p->smem_gd, DF, sb);
-        cudaEventRecord(p->gd_done, sb);
         L += g_classify(p->cls_tt.g, W, 0, s);
         cudaEventRecord(p->k1_done, s);
         // the gamma items of the single-excitation records, sorted by key, and gamma
-        cudaStreamWaitEvent(sa, p->k1_done, 0);
-        // the diagonal H^N values (a sequential sum per row) beside the others
-        L += g_diag_values(p->pvd.g, W, DF, sa);
-        cudaEventRecord(p->dv_done, sa);
-        L += g_item_fill(p->itf.g, sa);
+        cudaStreamWaitEvent(sa, p->fork, 0);
         L += g_zero(p->zero.g, sa);
-        L += g_sort_hist(p->sort.g, sa);
-        L += g_scan(p->scan.g, sa);
+        cudaStreamWaitEvent(sa, p->k1_done, 0);
+        L += g_item_fill(p->itf.g, p->block_rows, sa);
+        L += g_scan(p->scan.g, p->scan_longest, sa);
         L += g_sort_scatter(p->sort.g, sa);
         L += g_gamma(p->gam.g, p->smem_gamma, DF, sa);
         L += g_gamma_warp(p->gamw.g, DF, sa);
         cudaEventRecord(p->items_done, sa);
+        // the diagonal H^N values beside the others
+        cudaStreamWaitEvent(sb, p->k1_done, 0);
+        L += g_diag_values(p->pvd.g, W, DF, sb);
+        cudaEventRecord(p->gd_done, sb);
         // H^N values, the sandwich and E, S
         L += g_pair_values(p->pv.g, W, DF, s);
-        cudaStreamWaitEvent(s, p->dv_done, 0);
+        cudaStreamWaitEvent(s, p->gd_done, 0);
         L += g_sandwich(p->sw.g, DF, p->sw_width, s);
-        L += g_sandwich_small(p->sws.g, DF, s);
+        L += g_sandwich_small(p->sws.g, DF, p->block_rows, s);
         L += g_tn_partial(p->tn.g, p->smem_tn, DF, s);
         L += g_tn_reduce(p->tnr.g, DF, s);
         cudaStreamWaitEvent(s, p->items_done, 0);
-        cudaStreamWaitEvent(s, p->gd_done, 0);
         L += g_assemble(p->asmb.g, DF, s);
     } else {
         cudaEventRecord(p->gd_done, sb);   // the auxiliary stream joins the capture
@@ -1028,7 +1053,18 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         // the expansion, which was faster than running it first
         if (p->c4t.g.blocks > 0) cudaStreamWaitEvent(s, p->c4_done, 0);
         if (p->coef_rows > 0) {
-            cudaMemsetAsync(p->err, 0, sizeof(int), s);
+            // the rows with j == j': beside a split kernel that fills the chip they
+            // slowed it by more than they saved; one that leaves most SMs idle has
+            // them beside it (10 us of the 160 of a build of dimension 110)
+            int64_t tiles = 0;
+            for (auto &g : p->split) tiles += g.st.g.blocks;
+            const bool beside = tiles <= 76;
+            if (beside) {
+                cudaEventRecord(p->asm_done, s);
+                cudaStreamWaitEvent(sb, p->asm_done, 0);
+                L += g_diag_rows(p->drows.g, DF, sb);
+                cudaEventRecord(p->dr_done, sb);
+            }
             L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, p->coef_exps,
                          s);
             for (size_t i = 0; i < p->split.size(); ++i) {
@@ -1037,10 +1073,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
                               p->split[i].st.g, p->Kc / 64, p->Kw / 64, p->d_cols, p->err, s, p->shard_r, p->shard_n);
                 rec(p->ev_split[2 * i + 1]);
             }
-            // the rows with j == j'; beside the split kernel they slowed it by
-            // more than they saved
-            L += g_diag_rows(p->drows.g, DF, s);
-            if (p->host_err) cudaMemcpyAsync(p->host_err, p->err, sizeof(int), cudaMemcpyDeviceToHost, s);
+            if (beside) cudaStreamWaitEvent(s, p->dr_done, 0);
+            else L += g_diag_rows(p->drows.g, DF, s);
         }
     } else {
         LX += g_expand_fp64(p->x64.g, p->d_cols, s, p->shard_r, p->shard_n);
@@ -1053,6 +1087,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     cudaStreamWaitEvent(s, p->join_main, 0);
     cudaStreamWaitEvent(s, p->join, 0);
     rec(p->ev[6]);
+    if (p->host_err && (p->split_on || p->precision == HB_MIXED))
+        cudaMemcpyAsync(p->host_err, p->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaGetLastError();
     p->launches = L;
     p->expand_launches = LX;
@@ -1102,14 +1138,58 @@ void plan_stats(Plan *p, hb_stats *st) {
 int plan_error_word(Plan *p, int *word) {
     *word = 0;
     if (!p->err) return HB_OK;
-    int w[2] = {0, 0};
-    if (cudaMemcpy(w, p->err, sizeof(w), cudaMemcpyDeviceToHost) != cudaSuccess) return HB_ERR_CUDA;
+    if (!p->host_err) return HB_OK;
+    const volatile int *w = p->host_err;      // copied behind the build, which the caller has waited for
     *word = w[0] ? w[0] : w[1];
+    return HB_OK;
+}
+
+// One build.  From the third into the same blocks on, the plan's launches (two
+// dozen kernels on four streams and the events between them, 60 us of host
+// time, longer than a small build runs) are replayed as one graph, captured
+// once.  Builds in a caller's capture, and those of a context that lives in a
+// caller's workspace (a graph may take device memory of its own), are
+// launched one by one.
+int plan_launch(Plan *p, cudaStream_t s, int *launches, std::string *err) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    if (!plain) cudaGetLastError();
+    bool owned = false;
+    for (const hb_ctx *c : p->ctxs) owned = owned || c->pool.base != nullptr;
+    if (!plain || owned || p->no_graph) return plan_run(p, s, true, false, launches, err);
+    if (!p->exec && ++p->runs >= 3) {
+        cudaStream_t cs = nullptr;
+        cudaGraph_t g = nullptr;
+        std::string e2;
+        bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            ok = plan_run(p, cs, true, true, nullptr, &e2) == HB_OK;
+            ok = cudaStreamEndCapture(cs, &g) == cudaSuccess && ok;
+        }
+        if (ok) ok = cudaGraphInstantiate(&p->exec, g, cudaGraphInstantiateFlagUseNodePriority) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+        if (cs) cudaStreamDestroy(cs);
+        if (!ok) {
+            cudaGetLastError();
+            p->exec = nullptr;
+            p->no_graph = true;
+        }
+    }
+    if (!p->exec) return plan_run(p, s, true, false, launches, err);
+    p->timed = true;
+    if (launches) *launches = p->launches;
+    const cudaError_t e = cudaGraphLaunch(p->exec, s);
+    if (e != cudaSuccess) {
+        *err = std::string("build graph: ") + cudaGetErrorString(e);
+        return HB_ERR_CUDA;
+    }
     return HB_OK;
 }
 
 void plan_destroy(Plan *p) {
     if (!p) return;
+    drop_graph(p);
     if (p->upload_pending) cudaEventSynchronize(p->uploaded);
     for (cudaEvent_t e : p->ev)
         if (e) cudaEventDestroy(e);
@@ -1120,7 +1200,7 @@ void plan_destroy(Plan *p) {
     if (p->join) cudaEventDestroy(p->join);
     if (p->join_main) cudaEventDestroy(p->join_main);
     if (p->c4_done) cudaEventDestroy(p->c4_done);
-    for (cudaEvent_t ev : {p->k1_done, p->items_done, p->gd_done, p->dv_done})
+    for (cudaEvent_t ev : {p->k1_done, p->items_done, p->gd_done, p->asm_done, p->dr_done})
         if (ev) cudaEventDestroy(ev);
     for (cudaStream_t st : {p->main, p->side, p->aux1, p->aux2})
         if (st) {
@@ -1135,7 +1215,6 @@ void plan_destroy(Plan *p) {
         dfree(mem, p->err);
     }
     if (p->pinned) cudaFreeHost(p->pinned);
-    if (p->host_err) cudaFreeHost(p->host_err);
     delete p;
 }
 

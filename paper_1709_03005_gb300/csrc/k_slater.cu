@@ -140,6 +140,51 @@ __device__ Acc element(const Ints &I, const uint64_t (&a)[2 * W], const uint64_t
     return v;
 }
 
+// <a|H|a> by a warp: lane j holds the j-th electron's orbital, electron i
+// meets the electrons before it; the lanes' sums are added in a fixed tree.
+__device__ __forceinline__ void warp_sum(AccD &v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v.v += __shfl_xor_sync(0xffffffffu, v.v, o);
+}
+__device__ __forceinline__ void warp_sum(AccF &v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, v.h, o), l = __shfl_xor_sync(0xffffffffu, v.l, o);
+        df_add2(v.h, v.l, h, l);
+    }
+}
+template <int W, class Acc>
+__device__ __forceinline__ Acc diag_element_warp(const Ints &I, const uint64_t (&a)[2 * W], uint16_t *occ) {
+    const int lane = threadIdx.x & 31;
+    const int n = I.n_to;
+    constexpr int sb = 64 * W;
+    int ne = 0;
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t bits = (uint32_t)(a[w] >> (32 * half));
+            if ((bits >> lane) & 1u)
+                occ[ne + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(64 * w + 32 * half + lane);
+            ne += __popc(bits);
+        }
+    __syncwarp();
+    Acc v;
+    for (int j = lane; j < ne; j += 32) {
+        const int q = occ[j], sq = q >= sb, oq = q - sq * sb;
+        v.add(I.h, I.h_df, (int64_t)oq * (I.n_orb + 1));
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) {
+            const int p = occ[i], sp = p >= sb, op = p - sp * sb;
+            v.add(I.jk, I.jk_df, (int64_t)op * n + oq);
+            if (sp == sq) v.sub(I.jk, I.jk_df, (int64_t)n * n + (int64_t)op * n + oq);
+        }
+    }
+    warp_sum(v);
+    __syncwarp();
+    return v;
+}
+
 __device__ __forceinline__ void store_value(const AccD &v, double *out, int64_t k) { out[k] = v.v; }
 __device__ __forceinline__ void store_value(const AccF &v, double *out, int64_t k) {
     reinterpret_cast<float2 *>(out)[k] = make_float2(v.h, v.l);
@@ -328,41 +373,6 @@ __device__ __forceinline__ double single_element(const Ints &I, const uint64_t (
     return odd ? -v : v;
 }
 
-// <a|H|a> by a warp: lane j holds the j-th electron's orbital, electron i
-// meets the electrons after it; the lanes' sums are added in a fixed tree.
-template <int W>
-__device__ __forceinline__ double diag_element_warp(const Ints &I, const uint64_t (&a)[2 * W], uint16_t *occ) {
-    const int lane = threadIdx.x & 31;
-    const int n = I.n_to;
-    constexpr int sb = 64 * W;
-    int ne = 0;
-#pragma unroll
-    for (int w = 0; w < 2 * W; ++w)
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const uint32_t bits = (uint32_t)(a[w] >> (32 * half));
-            if ((bits >> lane) & 1u)
-                occ[ne + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(64 * w + 32 * half + lane);
-            ne += __popc(bits);
-        }
-    __syncwarp();
-    double v = 0.0;
-    for (int j = lane; j < ne; j += 32) {
-        const int q = occ[j], sq = q >= sb, oq = q - sq * sb;
-        v += __ldg(I.h + (int64_t)oq * (I.n_orb + 1));
-#pragma unroll 4
-        for (int i = 0; i < j; ++i) {
-            const int p = occ[i], sp = p >= sb, op = p - sp * sb;
-            v += __ldg(I.jk + (int64_t)op * n + oq);
-            if (sp == sq) v -= __ldg(I.jk + (int64_t)n * n + (int64_t)op * n + oq);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncwarp();
-    return v;
-}
-
 template <int W>
 __global__ void __launch_bounds__(32 * kWarps)
 l2_values_kernel(const L2VTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
@@ -380,7 +390,7 @@ l2_values_kernel(const L2VTask *__restrict__ tasks, const int64_t *__restrict__ 
         if (row >= T.n || row < T.row_lo || row >= T.row_hi) return;
         uint64_t a[2 * W];
         load_det<W>(T.dets + (int64_t)row * 2 * W, a);
-        const double v = diag_element_warp<W>(I, a, occupied[warp]);
+        const double v = diag_element_warp<W, AccD>(I, a, occupied[warp]).value();
         if (lane == 0) {
             const int64_t at = __ldg(rp + row) + (__ldg(low + row + 1) - __ldg(low + row));
             T.col[at] = row;
@@ -586,12 +596,16 @@ __global__ void pair_values_kernel(const PVTask *__restrict__ tasks, const int64
 }
 
 // <D_m|H^N|D_m> of a same-group task: the record (m, m) of row m, found by
-// binary search over the row's ascending columns (a scan if that fails).
+// binary search over the row's ascending columns (a scan if that fails).  A
+// warp per row; the sum over all electron pairs by one thread took 11 us alone.
 template <int W, class Acc>
-__global__ void diag_values_kernel(const PVTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+__global__ void __launch_bounds__(32 * kWarps)
+diag_values_kernel(const PVTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+    __shared__ uint16_t occupied[kWarps][128 * W];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const PVTask &T = tasks[ti];
-    const int m = (int)((blockIdx.x - blk[ti]) * (int64_t)blockDim.x + threadIdx.x);
+    const int warp = threadIdx.x >> 5;
+    const int m = (int)((blockIdx.x - blk[ti]) * (int64_t)kWarps) + warp;
     if (m >= T.n_rows) return;
     int64_t lo = T.row_ptr[m], hi = T.row_ptr[m + 1] - 1, at = -1;
     while (lo <= hi) {
@@ -607,7 +621,8 @@ __global__ void diag_values_kernel(const PVTask *__restrict__ tasks, const int64
     if (at < 0 || T.pairs[at].degree != 0) return;
     uint64_t a[2 * W];
     load_det<W>(T.a + (int64_t)m * 2 * W, a);
-    store_value(diag_value<W, Acc>(T.I, a), T.val, at);
+    const Acc v = diag_element_warp<W, Acc>(T.I, a, occupied[warp]);
+    if ((threadIdx.x & 31) == 0) store_value(v, T.val, at);
 }
 
 __global__ void jk_kernel(Ints I, double *jk) {
@@ -627,7 +642,7 @@ void build_jk(const Ints &I, double *jk, cudaStream_t s) {
 }
 
 int64_t blocks_pair_values(int64_t n_pairs) { return (n_pairs + 255) / 256; }
-int64_t blocks_diag_values(int n_rows) { return (n_rows + 255) / 256; }
+int64_t blocks_diag_values(int n_rows) { return (n_rows + kWarps - 1) / kWarps; }
 
 int g_diag_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s) {
     if (g.blocks <= 0) return 0;

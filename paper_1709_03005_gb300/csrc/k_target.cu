@@ -11,6 +11,8 @@
 // stable counting sort so that every sum runs in a fixed order (no floating
 // point atomics anywhere).  Every stage is a grouped launch over the group
 // pairs of one or many Hamiltonians (one task per group pair).
+#include <algorithm>
+
 #include "hb_df.cuh"
 #include "hb_tasks.cuh"
 
@@ -74,31 +76,104 @@ sandwich_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__ bl
 }
 
 // The same for nsp <= 32: the lanes form G = 32 / P groups of P columns (P the
-// power of two >= nsp); group g takes records g, g+G, ... and the groups are
-// combined by a butterfly over the lanes that hold the same column.
+// power of two >= nsp).  A row's records are cut into four contiguous parts;
+// group g takes records g, g+G, ... of a part, the groups of a part are
+// combined by a butterfly over the lanes that hold the same column, the parts
+// in order.  A warp per row (four parts in flight), or a block per row with a
+// warp per part where the plan has few rows and the longest sets the time (300
+// rows, one of 300 records: 35 us, now 9): the same sums in the same order.
+template <bool DF>
+struct SmallSum {
+    float h = 0.0f, l = 0.0f;
+    double v = 0.0;
+    __device__ __forceinline__ void term(const SWTask &T, int64_t k, int nsp, int c) {
+        const int col = T.pairs[k].col;
+        if (DF) {
+            const float2 x = reinterpret_cast<const float2 *>(T.val)[k], y = __ldg(T.Cp_df + (int64_t)col * nsp + c);
+            df_fma(h, l, x.x, x.y, y.x, y.y);
+        } else {
+            v = fma(T.val[k], __ldg(T.Cp + (int64_t)col * nsp + c), v);
+        }
+    }
+    __device__ __forceinline__ void add(const SmallSum &o) {
+        if (DF) df_add2(h, l, o.h, o.l);
+        else v += o.v;
+    }
+    __device__ __forceinline__ void tree(int P) {
+        for (int off = 16; off >= P; off >>= 1) {
+            SmallSum o;
+            if (DF) {
+                o.h = __shfl_xor_sync(0xffffffffu, h, off);
+                o.l = __shfl_xor_sync(0xffffffffu, l, off);
+            } else {
+                o.v = __shfl_xor_sync(0xffffffffu, v, off);
+            }
+            add(o);
+        }
+    }
+    __device__ __forceinline__ void store(const SWTask &T, int64_t i) const {
+        if (DF) reinterpret_cast<float2 *>(T.Wout)[i] = make_float2(h, l);
+        else T.Wout[i] = v;
+    }
+};
+
+template <bool DF, bool BLOCK>
 __global__ void sandwich_small_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__ blk,
                                       int n_tasks) {
+    __shared__ SmallSum<DF> red[BLOCK ? 4 : 1][32];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const SWTask T = tasks[ti];
-    const int lane = threadIdx.x & 31;
-    const int row = (int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lb = (int)(blockIdx.x - blk[ti]);
+    const int row = BLOCK ? lb : lb * (blockDim.x >> 5) + w;
     if (row >= T.n_rows) return;
     const int nsp = T.nsp;
     int P = 1;
     while (P < nsp) P <<= 1;
     const int G = 32 / P, g = lane / P, c = lane % P;
     const int64_t b = T.row_ptr[row], e = T.row_ptr[row + 1];
-    double acc = 0.0;
-    if (c < nsp)
-        for (int64_t k = b + g; k < e; k += G) acc = fma(T.val[k], __ldg(T.Cp + (int64_t)T.pairs[k].col * nsp + c), acc);
-    for (int off = 16; off >= P; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (g == 0 && c < nsp) T.Wout[(int64_t)row * nsp + c] = acc;
+    const int64_t per = (e - b + 3) / 4;
+    SmallSum<DF> s[BLOCK ? 1 : 4];
+    if (BLOCK) {
+        const int64_t kb = min(e, b + w * per), ke = min(e, kb + per);
+        if (c < nsp)
+#pragma unroll 4
+            for (int64_t k = kb + g; k < ke; k += G) s[0].term(T, k, nsp, c);
+        s[0].tree(P);
+        red[w][lane] = s[0];
+        __syncthreads();
+        if (w == 0) {
+#pragma unroll
+            for (int u = 1; u < 4; ++u) s[0].add(red[u][lane]);
+        }
+    } else {
+        if (c < nsp)
+            for (int64_t i = g; i < per; i += G) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t k = b + u * per + i;
+                    if (k < e) s[u].term(T, k, nsp, c);
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < (BLOCK ? 1 : 4); ++u) s[u].tree(P);
+#pragma unroll
+        for (int u = 1; u < (BLOCK ? 1 : 4); ++u) s[0].add(s[u]);
+    }
+    if (g == 0 && c < nsp && (!BLOCK || w == 0)) s[0].store(T, (int64_t)row * nsp + c);
 }
 
 // partial[c][n][n'] = sum_{m in chunk c} C[m][n] * Wm[m][n']; rows staged in
 // batches, each thread keeps 4 outputs; the task's blocks are (chunk, y) with
 // y covering the outputs in steps of 1024.
 constexpr int kRowsPerChunk = 256;
+// rows per chunk of C^T W: short lists leave the chip idle in chunks of 256 (300
+// rows x 7 states: 16 us on 4 blocks, 5 us in chunks of 32)
+__host__ __device__ inline int tn_chunk_rows(int n_rows) { return n_rows < 4096 ? 32 : (n_rows < 16384 ? 64 : kRowsPerChunk); }
+__host__ __device__ inline int tn_chunk_count(int n_rows) {
+    const int k = tn_chunk_rows(n_rows);
+    return (n_rows + k - 1) / k;
+}
 // rows (or items) staged per batch so that the staging buffer stays <= 48 KB
 __host__ __device__ inline int stage_batch(int ns, int nsp) {
     const int b = 6144 / (ns + nsp);
@@ -114,8 +189,9 @@ __global__ void tn_partial_kernel(const TNTask *__restrict__ tasks, const int64_
     const int kRowBatch = stage_batch(ns, nsp);
     double *cs = sh;                      // [kRowBatch][ns]
     double *ws = sh + kRowBatch * ns;     // [kRowBatch][nsp]
-    const int m0 = c * kRowsPerChunk;
-    const int rows = min(kRowsPerChunk, T.n_rows - m0);
+    const int kChunk = tn_chunk_rows(T.n_rows);
+    const int m0 = c * kChunk;
+    const int rows = min(kChunk, T.n_rows - m0);
     const int nout = ns * nsp;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int r0 = 0; r0 < rows; r0 += kRowBatch) {
@@ -149,9 +225,10 @@ __global__ void reduce_partials_kernel(const TNTask *__restrict__ tasks, const i
     const int t = (int)(blockIdx.x - blk[ti]) * blockDim.x + threadIdx.x;
     const int n_out = T.ns * T.nsp;
     if (t >= n_out) return;
-    const int n_chunks = (T.n_rows + kRowsPerChunk - 1) / kRowsPerChunk;
+    const int n_chunks = tn_chunk_count(T.n_rows);
     double acc = 0.0;
-    for (int c = 0; c < n_chunks; ++c) acc += T.partial[(int64_t)c * n_out + t];
+#pragma unroll 8
+    for (int c = 0; c < n_chunks; ++c) acc += __ldg(T.partial + (int64_t)c * n_out + t);
     T.out[t] = acc;
 }
 
@@ -177,32 +254,39 @@ __global__ void item_count_kernel(const hb_pair *__restrict__ pairs, const int64
 // n_to^2 + r * n_to + q.  (A deg-0 record is a determinant with itself, m = m'
 // of one group; its diagonal contributions gamma(p, p) are the masked C^T C of
 // gdiag_partial_kernel below.)
-// One block per row: warp w of kIFWarps takes the w-th contiguous part of the
+// A block per row: warp w of kIFWarps takes the w-th contiguous part of the
 // row's records, counts its items, and writes them after those of the warps
-// before it, so the items keep the order of the records.
+// before it; or, where the plan has so many rows that they fill the chip, a
+// warp per row.  Either way the items keep the order of the records.  Each item
+// is counted under its key and sort chunk on the way (integer atomics: exact).
 constexpr int kIFWarps = 4;
 
-__global__ void __launch_bounds__(32 * kIFWarps)
+template <bool BLOCK>
+__global__ void __launch_bounds__(BLOCK ? 32 * kIFWarps : 256)
 item_fill_kernel(const IFTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     __shared__ int wcnt[kIFWarps];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const IFTask T = tasks[ti];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int row = (int)(blockIdx.x - blk[ti]);
+    const int lb = (int)(blockIdx.x - blk[ti]);
+    const int row = BLOCK ? lb : lb * 8 + w;
+    if (row >= T.n_rows) return;
     const int64_t b = T.row_ptr[row], e = T.row_ptr[row + 1];
-    const int64_t per = (e - b + kIFWarps - 1) / kIFWarps;
-    const int64_t kb = b + w * per, ke = min(e, kb + per);
-    int cnt = 0;
-    for (int64_t k = kb + lane; k - lane < ke; k += 32) {
-        const bool one = k < ke && T.pairs[k].degree == 1;
-        cnt += __popc(__ballot_sync(0xffffffffu, one));
-    }
-    if (lane == 0) wcnt[w] = cnt;
-    __syncthreads();
+    const int64_t per = BLOCK ? (e - b + kIFWarps - 1) / kIFWarps : e - b;
+    const int64_t kb = BLOCK ? b + w * per : b, ke = min(e, kb + per);
     int64_t pos = T.item_ptr[row];
-    for (int q = 0; q < w; ++q) pos += wcnt[q];
-    const int W = T.W, n_to = T.n_to;
-    const int sb = 64 * W;
+    if (BLOCK) {
+        int cnt = 0;
+        for (int64_t k = kb + lane; k - lane < ke; k += 32) {
+            const bool one = k < ke && T.pairs[k].degree == 1;
+            cnt += __popc(__ballot_sync(0xffffffffu, one));
+        }
+        if (lane == 0) wcnt[w] = cnt;
+        __syncthreads();
+        for (int q = 0; q < w; ++q) pos += wcnt[q];
+    }
+    const int n_to = T.n_to;
+    const int sb = 64 * T.W;
     for (int64_t k0 = kb; k0 < ke; k0 += 32) {
         const int64_t k = k0 + lane;
         int one = 0;
@@ -217,7 +301,10 @@ item_fill_kernel(const IFTask *__restrict__ tasks, const int64_t *__restrict__ b
             GammaItem it;
             it.key = s * n_to * n_to + p * n_to + q;
             it.m = r.row; it.mp = r.col; it.phase = r.phase;
-            T.items[pos + __popc(m & ((1u << lane) - 1u))] = it;
+            const int64_t at = pos + __popc(m & ((1u << lane) - 1u));
+            T.items[at] = it;
+            atomicAdd(reinterpret_cast<unsigned long long *>(T.off) + 1 + (int64_t)it.key * T.nc + (at - T.item0) / T.chunk,
+                      1ull);
         }
         pos += __popc(m);
     }
@@ -356,20 +443,6 @@ __global__ void zero_kernel(const ZTask *__restrict__ tasks, const int64_t *__re
     }
 }
 
-// histogram per (key, chunk) in off[1 + key * nc + chunk] (integer atomics: exact)
-__global__ void sort_hist_kernel(const SortTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
-    const int ti = task_of(blk, n_tasks, blockIdx.x);
-    const SortTask T = tasks[ti];
-    const int chunk = (int)(blockIdx.x - blk[ti]);
-    const int CS = sort_chunk_size(T.n_items, T.n_keys);
-    const int64_t base = (int64_t)chunk * CS;
-    unsigned long long *hist = (unsigned long long *)T.off;
-    for (int i = threadIdx.x; i < CS; i += blockDim.x) {
-        const int64_t k = base + i;
-        if (k < T.n_items) atomicAdd(hist + 1 + (int64_t)T.items[k].key * T.nc + chunk, 1ull);
-    }
-}
-
 // Three-phase scan per task over segments of kScanSeg entries:
 //   x[0] = 0, x[1..n] := inclusive scan of x[1..n], copy[0..n-1] := x[0..n-1].
 // Phase 1: each segment's sum into part[seg]; phase 2 (one block per task):
@@ -465,6 +538,33 @@ __global__ void __launch_bounds__(1024) scan_apply_kernel(const ScanTask *__rest
         }
 }
 
+// The whole table of a task by one block: where no table of the plan is longer
+// than kScanOne entries, one launch takes the place of three.
+constexpr int64_t kScanOne = 5 * kScanSeg;
+__global__ void __launch_bounds__(1024) scan_one_kernel(const ScanTask *__restrict__ tasks) {
+    __shared__ int64_t warp_sums[32];
+    const ScanTask T = tasks[blockIdx.x];
+    if (threadIdx.x == 0 && T.n > 0) {
+        T.x[0] = 0;
+        if (T.copy) T.copy[0] = 0;
+    }
+    int64_t carry = 0;
+    for (int64_t base = 0; base < T.n; base += kScanSeg) {
+        const int64_t i0 = base + threadIdx.x * 4;
+        int64_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = (i0 + k < T.n) ? T.x[1 + i0 + k] : 0;
+        const int64_t total = block_scan4(v, warp_sums);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k < T.n) {
+                T.x[1 + i0 + k] = v[k] + carry;
+                if (T.copy && i0 + k + 1 < T.n) T.copy[i0 + k + 1] = v[k] + carry;
+            }
+        carry += total;
+    }
+}
+
 // One warp per chunk walks its items in order, so equal keys keep their order.
 // cur: a copy of the exclusive offsets [key][chunk], advanced in place.
 __global__ void sort_scatter_kernel(const SortTask *__restrict__ tasks, const int64_t *__restrict__ blk,
@@ -498,15 +598,17 @@ __global__ void gamma_kernel(const GTask *__restrict__ tasks, const int64_t *__r
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const GTask T = tasks[ti];
     const int lb = (int)(blockIdx.x - blk[ti]);
-    const int key = lb / T.ny, by = lb % T.ny;
+    const int by = lb % T.ny;
     const int ns = T.ns, nsp = T.nsp;
     const int kItemBatch = stage_batch(ns, nsp);
     double *ca = sm;                          // [kItemBatch][ns]
     double *cb = sm + kItemBatch * ns;        // [kItemBatch][nsp]
+    // keys of this block: one, or several where most have no items
+    for (int key = lb / T.ny * T.kpb; key < min(T.n_keys, (lb / T.ny + 1) * T.kpb); ++key) {
     // with no items (nc == 0) both ends are off[0] = 0 and gamma is zero
     const int64_t b = T.off[(int64_t)key * T.nc];
     const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) return;      // empty key: never written, the coefficient rows read it as zero
+    if (b == e) continue;    // empty key: never written, the coefficient rows read it as zero
     const int nout = ns * nsp;
     // each thread keeps up to 4 outputs in registers
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -540,6 +642,7 @@ __global__ void gamma_kernel(const GTask *__restrict__ tasks, const int64_t *__r
         const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
         if (t < nout) T.gamma[(int64_t)key * nout + t] = acc[u];
     }
+    }
 }
 
 // The same for small outputs (ns * nsp <= 64): one warp per key, the lanes
@@ -548,12 +651,12 @@ __global__ void gamma_warp_kernel(const GTask *__restrict__ tasks, const int64_t
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const GTask T = tasks[ti];
     const int lane = threadIdx.x & 31;
-    const int key = (int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (key >= T.n_keys) return;
+    const int key0 = ((int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * T.kpb;
     const int ns = T.ns, nsp = T.nsp, nout = ns * nsp;
+    for (int key = key0; key < min(T.n_keys, key0 + T.kpb); ++key) {
     const int64_t b = T.off[(int64_t)key * T.nc];
     const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) return;
+    if (b == e) continue;
     double acc0 = 0.0, acc1 = 0.0;
     const int t0 = lane, t1 = lane + 32;
     const int a0 = t0 / nsp, c0 = t0 % nsp, a1 = t1 / nsp, c1 = t1 % nsp;
@@ -566,6 +669,7 @@ __global__ void gamma_warp_kernel(const GTask *__restrict__ tasks, const int64_t
     }
     if (t0 < nout) T.gamma[(int64_t)key * nout + t0] = acc0;
     if (t1 < nout) T.gamma[(int64_t)key * nout + t1] = acc1;
+    }
 }
 
 // ------------------------------------------------------ coefficient rows
@@ -581,53 +685,72 @@ __global__ void gamma_warp_kernel(const GTask *__restrict__ tasks, const int64_t
 // FP64 build: gamma and A in FP64.  Mixed build: gamma as (hi, lo) float
 // pairs, the sums in double-float, A written as float pairs (A_df, read by the
 // j == j' rows) and as FP64 (read by the slicing).
+// A block takes kAsmRows rows of a task and 256 labels: which keys a label adds
+// and whether they hold anything is worked out once for the rows, and the
+// gammas of neighbouring state pairs, which lie side by side, are read
+// together.  (A block per row over all labels took 312 us for the 11383 rows of
+// a twelve-Hamiltonian batch.)
+constexpr int kAsmRows = 8;
 template <bool DF>
-__global__ void assemble_kernel(const ATask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+__global__ void __launch_bounds__(256)
+assemble_kernel(const ATask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const ATask T = tasks[ti];
-    const int t = (int)(blockIdx.x - blk[ti]);
-    if (t >= T.n_nn) return;
-    const int n = T.nn[2 * t], np = T.nn[2 * t + 1];
+    const int lb = (int)(blockIdx.x - blk[ti]);
     const int ns = T.ns, nsp = T.nsp, n_to = T.n_to, Kpad = T.Kpad;
-    const int nout = ns * nsp, sidx = n * nsp + np;
+    const int nkb = (Kpad + 255) / 256;
+    const int t0 = lb / nkb * kAsmRows, k = lb % nkb * 256 + threadIdx.x;
+    const int nt = min(kAsmRows, T.n_nn - t0);
+    if (k >= Kpad) return;
+    const int nout = ns * nsp;
     const int Pt = n_to * (n_to + 1) / 2, nt2 = n_to * n_to;
-    auto present = [&](int key, bool diag) -> bool {
-        return (diag && T.same) || T.off[(int64_t)key * T.nc] != T.off[(int64_t)(key + 1) * T.nc];
+    // up to four keys, in the order of their sum
+    int key[4], n_key = 0;
+    auto add_key = [&](int q, bool diag) {
+        if ((diag && T.same) || T.off[(int64_t)q * T.nc] != T.off[(int64_t)(q + 1) * T.nc]) key[n_key++] = q;
     };
-    for (int k = threadIdx.x; k < Kpad; k += blockDim.x) {
+    bool neg = false;
+    if (k < Pt) {
+        // unpack k = r(r+1)/2 + s
+        int r = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
+        while ((r + 1) * (r + 2) / 2 <= k) ++r;
+        while (r * (r + 1) / 2 > k) --r;
+        const int s = k - r * (r + 1) / 2;
+#pragma unroll
+        for (int sp = 0; sp < 2; ++sp) {
+            add_key(sp * nt2 + r * n_to + s, r == s);
+            if (r != s) add_key(sp * nt2 + s * n_to + r, false);
+        }
+    } else if (k < Pt + nt2) {
+        const int pq = k - Pt;
+        add_key(T.cont_spin * nt2 + pq, pq / n_to == pq % n_to);
+        neg = true;
+    }
+#pragma unroll 4
+    for (int u = 0; u < nt; ++u) {
+        const int t = t0 + u;
+        const int n = T.nn[2 * t], np = T.nn[2 * t + 1], sidx = n * nsp + np;
         double v = 0.0;
         float vh = 0.0f, vl = 0.0f;
-        auto add_key = [&](int key, bool diag, bool neg) {
-            if (!present(key, diag)) return;
-            if (DF) {
-                const float2 g = reinterpret_cast<const float2 *>(T.gamma)[(int64_t)key * nout + sidx];
-                df_add2(vh, vl, neg ? -g.x : g.x, neg ? -g.y : g.y);
-            } else {
-                const double g = T.gamma[(int64_t)key * nout + sidx];
-                v += neg ? -g : g;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < n_key) {
+                if (DF) {
+                    const float2 g = reinterpret_cast<const float2 *>(T.gamma)[(int64_t)key[i] * nout + sidx];
+                    df_add2(vh, vl, neg ? -g.x : g.x, neg ? -g.y : g.y);
+                } else {
+                    const double g = T.gamma[(int64_t)key[i] * nout + sidx];
+                    v += neg ? -g : g;
+                }
             }
-        };
-        if (k < Pt) {
-            // unpack k = r(r+1)/2 + s
-            int r = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
-            while ((r + 1) * (r + 2) / 2 <= k) ++r;
-            while (r * (r + 1) / 2 > k) --r;
-            const int s = k - r * (r + 1) / 2;
-            for (int sp = 0; sp < 2; ++sp) {
-                add_key(sp * nt2 + r * n_to + s, r == s, false);
-                if (r != s) add_key(sp * nt2 + s * n_to + r, false, false);
-            }
-        } else if (k < Pt + nt2) {
-            const int pq = k - Pt;
-            add_key(T.cont_spin * nt2 + pq, pq / n_to == pq % n_to, true);
-        } else if (k == Pt + nt2) {
-            if (DF) { const float h = (float)T.S[sidx]; vh = h; vl = (float)(T.S[sidx] - (double)h); }
-            else v = T.S[sidx];
+        if (k == Pt + nt2) {
+            v = T.S[sidx];
         } else if (k == Pt + nt2 + 1) {
-            const double x = T.En ? ((T.same && n == np && !T.no_En) ? T.En[n] : 0.0)
-                                  : T.E[sidx] + T.e_core * T.S[sidx];
-            if (DF) { const float h = (float)x; vh = h; vl = (float)(x - (double)h); }
-            else v = x;
+            v = T.En ? ((T.same && n == np && !T.no_En) ? T.En[n] : 0.0) : T.E[sidx] + T.e_core * T.S[sidx];
+        }
+        if (DF && k >= Pt + nt2) {
+            vh = (float)v;
+            vl = (float)(v - (double)vh);
         }
         if (DF) {
             T.A_df[(int64_t)t * Kpad + k] = make_float2(vh, vl);
@@ -716,47 +839,6 @@ sandwich_df_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__
     }
 }
 
-__global__ void sandwich_small_df_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__ blk,
-                                         int n_tasks) {
-    const int ti = task_of(blk, n_tasks, blockIdx.x);
-    const SWTask T = tasks[ti];
-    const int lane = threadIdx.x & 31;
-    const int row = (int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (row >= T.n_rows) return;
-    const int nsp = T.nsp;
-    const float2 *val = reinterpret_cast<const float2 *>(T.val);
-    float2 *Wout = reinterpret_cast<float2 *>(T.Wout);
-    int P = 1;
-    while (P < nsp) P <<= 1;
-    const int G = 32 / P, g = lane / P, c = lane % P;
-    const int64_t b = T.row_ptr[row], e = T.row_ptr[row + 1];
-    // four independent partial sums (records i = 0, 1, 2, 3 mod 4 of this
-    // lane's stride), combined in a fixed order
-    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, l[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    if (c < nsp) {
-        int64_t k = b + g;
-        for (; k + 3 * G < e; k += 4 * G) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t kk = k + u * G;
-                const float2 v = val[kk];
-                const float2 x = __ldg(T.Cp_df + (int64_t)T.pairs[kk].col * nsp + c);
-                df_fma(h[u], l[u], v.x, v.y, x.x, x.y);
-            }
-        }
-        for (int u = 0; k < e; k += G, ++u) {
-            const float2 v = val[k];
-            const float2 x = __ldg(T.Cp_df + (int64_t)T.pairs[k].col * nsp + c);
-            df_fma(h[u], l[u], v.x, v.y, x.x, x.y);
-        }
-    }
-    df_add2(h[0], l[0], h[1], l[1]);
-    df_add2(h[2], l[2], h[3], l[3]);
-    df_add2(h[0], l[0], h[2], l[2]);
-    for (int off = 16; off >= P; off >>= 1) shfl_df_add(h[0], l[0], off);
-    if (g == 0 && c < nsp) Wout[(int64_t)row * nsp + c] = make_float2(h[0], l[0]);
-}
-
 __global__ void tn_partial_df_kernel(const TNTask *__restrict__ tasks, const int64_t *__restrict__ blk,
                                      int n_tasks) {
     extern __shared__ float2 shf[];
@@ -768,8 +850,9 @@ __global__ void tn_partial_df_kernel(const TNTask *__restrict__ tasks, const int
     const int kRowBatch = stage_batch(ns, nsp);
     float2 *cs = shf;                     // [kRowBatch][ns]
     float2 *ws = shf + kRowBatch * ns;    // [kRowBatch][nsp]
-    const int m0 = c * kRowsPerChunk;
-    const int rows = min(kRowsPerChunk, T.n_rows - m0);
+    const int kChunk = tn_chunk_rows(T.n_rows);
+    const int m0 = c * kChunk;
+    const int rows = min(kChunk, T.n_rows - m0);
     const int nout = ns * nsp;
     float ah[4] = {0.0f, 0.0f, 0.0f, 0.0f}, al[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int r0 = 0; r0 < rows; r0 += kRowBatch) {
@@ -805,11 +888,12 @@ __global__ void reduce_partials_df_kernel(const TNTask *__restrict__ tasks, cons
     const int t = (int)(blockIdx.x - blk[ti]) * blockDim.x + threadIdx.x;
     const int n_out = T.ns * T.nsp;
     if (t >= n_out) return;
-    const int n_chunks = (T.n_rows + kRowsPerChunk - 1) / kRowsPerChunk;
+    const int n_chunks = tn_chunk_count(T.n_rows);
     const float2 *partial = reinterpret_cast<const float2 *>(T.partial);
     float h = 0.0f, l = 0.0f;
+#pragma unroll 8
     for (int c = 0; c < n_chunks; ++c) {
-        const float2 x = partial[(int64_t)c * n_out + t];
+        const float2 x = __ldg(partial + (int64_t)c * n_out + t);
         df_add2(h, l, x.x, x.y);
     }
     T.out[t] = df_to_double(h, l);
@@ -820,14 +904,16 @@ __global__ void gamma_df_kernel(const GTask *__restrict__ tasks, const int64_t *
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const GTask T = tasks[ti];
     const int lb = (int)(blockIdx.x - blk[ti]);
-    const int key = lb / T.ny, by = lb % T.ny;
+    const int by = lb % T.ny;
     const int ns = T.ns, nsp = T.nsp;
     const int kItemBatch = stage_batch(ns, nsp);
     float2 *ca = smf;                         // [kItemBatch][ns]
     float2 *cb = smf + kItemBatch * ns;       // [kItemBatch][nsp]
+    // keys of this block: one, or several where most have no items
+    for (int key = lb / T.ny * T.kpb; key < min(T.n_keys, (lb / T.ny + 1) * T.kpb); ++key) {
     const int64_t b = T.off[(int64_t)key * T.nc];
     const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) return;
+    if (b == e) continue;
     const int nout = ns * nsp;
     float ah[4] = {0.0f, 0.0f, 0.0f, 0.0f}, al[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int64_t i0 = b; i0 < e; i0 += kItemBatch) {
@@ -866,6 +952,7 @@ __global__ void gamma_df_kernel(const GTask *__restrict__ tasks, const int64_t *
         const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
         if (t < nout) reinterpret_cast<float2 *>(T.gamma)[(int64_t)key * nout + t] = make_float2(ah[u], al[u]);
     }
+    }
 }
 
 __global__ void gamma_warp_df_kernel(const GTask *__restrict__ tasks, const int64_t *__restrict__ blk,
@@ -873,12 +960,12 @@ __global__ void gamma_warp_df_kernel(const GTask *__restrict__ tasks, const int6
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const GTask T = tasks[ti];
     const int lane = threadIdx.x & 31;
-    const int key = (int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (key >= T.n_keys) return;
+    const int key0 = ((int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * T.kpb;
     const int ns = T.ns, nsp = T.nsp, nout = ns * nsp;
+    for (int key = key0; key < min(T.n_keys, key0 + T.kpb); ++key) {
     const int64_t b = T.off[(int64_t)key * T.nc];
     const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) return;
+    if (b == e) continue;
     float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
     const int t0 = lane, t1 = lane + 32;
     const int a0 = t0 / nsp, c0 = t0 % nsp, a1 = t1 / nsp, c1 = t1 % nsp;
@@ -905,23 +992,32 @@ __global__ void gamma_warp_df_kernel(const GTask *__restrict__ tasks, const int6
     float2 *g = reinterpret_cast<float2 *>(T.gamma);
     if (t0 < nout) g[(int64_t)key * nout + t0] = make_float2(h0, l0);
     if (t1 < nout) g[(int64_t)key * nout + t1] = make_float2(h1, l1);
+    }
 }
 
 }  // namespace
 
 int64_t blocks_rows8(int64_t rows) { return (rows + 7) / 8; }
-int tn_chunks(int n_rows) { return (n_rows + kRowsPerChunk - 1) / kRowsPerChunk; }
+// chunks of any row count up to n_rows (a shard's rows may be cut finer than all of them)
+int tn_chunks(int n_rows) {
+    return std::max({tn_chunk_count(n_rows), tn_chunk_count(std::min(n_rows, 4095)), tn_chunk_count(std::min(n_rows, 16383))});
+}
 int tn_ny(int ns, int nsp) { return (ns * nsp + 1023) / 1024; }
-int64_t blocks_tn_partial(int n_rows, int ns, int nsp) { return (int64_t)tn_chunks(n_rows) * tn_ny(ns, nsp); }
+int64_t blocks_tn_partial(int n_rows, int ns, int nsp) { return (int64_t)tn_chunk_count(n_rows) * tn_ny(ns, nsp); }
 int64_t blocks_tn_reduce(int ns, int nsp) { return (ns * nsp + 255) / 256; }
 int64_t blocks_zero(int64_t n) { return (n + 1023) / 1024; }
 int sort_chunks(int64_t n_items, int n_keys) {
     const int c = sort_chunk_size(n_items, n_keys);
     return (int)((n_items + c - 1) / c);
 }
+int sort_chunk_items(int64_t n_items, int n_keys) { return sort_chunk_size(n_items, n_keys); }
 int64_t blocks_sort(int64_t n_items, int n_keys) { return sort_chunks(n_items, n_keys); }
-int64_t blocks_gamma(int n_keys, int ns, int nsp) { return (int64_t)n_keys * tn_ny(ns, nsp); }
-int64_t blocks_gamma_warp(int n_keys) { return (n_keys + 7) / 8; }
+int gamma_keys_per(int64_t n_items, int n_keys) { return n_items < 4 * (int64_t)n_keys ? 8 : 1; }
+int64_t blocks_gamma(int n_keys, int kpb, int ns, int nsp) { return (int64_t)((n_keys + kpb - 1) / kpb) * tn_ny(ns, nsp); }
+int64_t blocks_gamma_warp(int n_keys, int kpb) { return (n_keys + 8 * kpb - 1) / (8 * kpb); }
+int64_t blocks_assemble(int n_nn, int Kpad) {
+    return (int64_t)((n_nn + kAsmRows - 1) / kAsmRows) * ((Kpad + 255) / 256);
+}
 size_t smem_stage(int ns, int nsp) { return sizeof(double) * stage_batch(ns, nsp) * (ns + nsp); }
 
 void gamma_item_counts(const hb_pair *pairs, const int64_t *row_ptr, int n_rows, int n_elec,
@@ -945,9 +1041,11 @@ int g_sandwich(const Grouped<SWTask> &g, int dfloat, int width, cudaStream_t s) 
     }
     HB_GROUPED(sandwich_kernel, g, 32 * kSWWarps, 0, s);
 }
-int g_sandwich_small(const Grouped<SWTask> &g, int dfloat, cudaStream_t s) {
-    if (dfloat) HB_GROUPED(sandwich_small_df_kernel, g, 256, 0, s);
-    HB_GROUPED(sandwich_small_kernel, g, 256, 0, s);
+int g_sandwich_small(const Grouped<SWTask> &g, int dfloat, int block_rows, cudaStream_t s) {
+    if (dfloat && block_rows) HB_GROUPED((sandwich_small_kernel<true, true>), g, 128, 0, s);
+    if (dfloat) HB_GROUPED((sandwich_small_kernel<true, false>), g, 256, 0, s);
+    if (block_rows) HB_GROUPED((sandwich_small_kernel<false, true>), g, 128, 0, s);
+    HB_GROUPED((sandwich_small_kernel<false, false>), g, 256, 0, s);
 }
 int g_tn_partial(const Grouped<TNTask> &g, size_t smem, int dfloat, cudaStream_t s) {
     if (dfloat) HB_GROUPED(tn_partial_df_kernel, g, 256, smem, s);
@@ -957,9 +1055,11 @@ int g_tn_reduce(const Grouped<TNTask> &g, int dfloat, cudaStream_t s) {
     if (dfloat) HB_GROUPED(reduce_partials_df_kernel, g, 256, 0, s);
     HB_GROUPED(reduce_partials_kernel, g, 256, 0, s);
 }
-int g_item_fill(const Grouped<IFTask> &g, cudaStream_t s) { HB_GROUPED(item_fill_kernel, g, 32 * kIFWarps, 0, s); }
+int g_item_fill(const Grouped<IFTask> &g, int block_rows, cudaStream_t s) {
+    if (block_rows) HB_GROUPED(item_fill_kernel<true>, g, 32 * kIFWarps, 0, s);
+    HB_GROUPED(item_fill_kernel<false>, g, 256, 0, s);
+}
 int g_zero(const Grouped<ZTask> &g, cudaStream_t s) { HB_GROUPED(zero_kernel, g, 256, 0, s); }
-int g_sort_hist(const Grouped<SortTask> &g, cudaStream_t s) { HB_GROUPED(sort_hist_kernel, g, 256, 0, s); }
 int g_sort_scatter(const Grouped<SortTask> &g, cudaStream_t s) { HB_GROUPED(sort_scatter_kernel, g, 32, 0, s); }
 int g_gamma(const Grouped<GTask> &g, size_t smem, int dfloat, cudaStream_t s) {
     if (dfloat) HB_GROUPED(gamma_df_kernel, g, 256, smem, s);
@@ -989,18 +1089,25 @@ int g_gdiag(const Grouped<GDTask> &partial, const Grouped<GDTask> &reduce, size_
     return L;
 }
 
+int gdiag_chunks(int ndet) { return (ndet + kRowsPerChunk - 1) / kRowsPerChunk; }
 int64_t blocks_gdiag_partial(int ndet, int n_to, int ns) {
-    return (int64_t)tn_chunks(ndet) * 2 * n_to * tn_ny(ns, ns);
+    return (int64_t)gdiag_chunks(ndet) * 2 * n_to * tn_ny(ns, ns);
 }
 int64_t blocks_gdiag_reduce(int n_to, int ns) { return (int64_t)2 * n_to * ((ns * ns + 255) / 256); }
 size_t smem_gdiag(int ns) { return sizeof(double) * ns * gdiag_batch(ns); }
 
 int64_t blocks_scan(int64_t n) { return (n + kScanSeg - 1) / kScanSeg; }
 
-int g_scan(const Grouped<ScanTask> &g, cudaStream_t s) {
+int64_t scan_one_limit() { return kScanOne; }
+
+int g_scan(const Grouped<ScanTask> &g, int64_t longest, cudaStream_t s) {
     if (g.n <= 0) return 0;
     // empty tasks write nothing: their x[0] is zeroed before the histogram
     if (g.blocks <= 0) return 0;
+    if (longest <= kScanOne) {
+        scan_one_kernel<<<g.n, 1024, 0, s>>>(g.tasks);
+        return 1;
+    }
     scan_sums_kernel<<<(unsigned)g.blocks, 1024, 0, s>>>(g.tasks, g.blk, g.n);
     scan_part_kernel<<<g.n, 1024, 0, s>>>(g.tasks, g.n);
     scan_apply_kernel<<<(unsigned)g.blocks, 1024, 0, s>>>(g.tasks, g.blk, g.n);
