@@ -454,6 +454,62 @@ void hb::fill_diag(hb_ctx *ctx, const hb_blocks *H, DiagWork *w, cudaStream_t s)
 // w: ascending eigenvalues [n]; V: [n][nvec], column c is the c-th vector.
 namespace {
 
+// Dot products and updates of the small eigensolver, in pairs of doubles (the
+// host's 128-bit vectors) and eight independent sums: the compiler may not
+// reorder a sum, and a single one runs at the latency of an addition.  The
+// order is fixed by the length alone.
+typedef double vd2 __attribute__((vector_size(16), aligned(8), may_alias));
+inline vd2 ld2(const double *p) { return *reinterpret_cast<const vd2 *>(p); }
+inline void st2(double *p, vd2 v) { *reinterpret_cast<vd2 *>(p) = v; }
+
+inline double dot8(const double *a, const double *b, int n) {
+    vd2 s0 = {0.0, 0.0}, s1 = s0, s2 = s0, s3 = s0;
+    int i = 0;
+    for (; i + 8 <= n; i += 8) {
+        s0 += ld2(a + i) * ld2(b + i);
+        s1 += ld2(a + i + 2) * ld2(b + i + 2);
+        s2 += ld2(a + i + 4) * ld2(b + i + 4);
+        s3 += ld2(a + i + 6) * ld2(b + i + 6);
+    }
+    double r = 0.0;
+    for (; i < n; ++i) r += a[i] * b[i];
+    const vd2 t = (s0 + s1) + (s2 + s3);
+    return t[0] + t[1] + r;
+}
+inline void axpy(double *y, double c, const double *x, int n) {
+    const vd2 cc = {c, c};
+    int i = 0;
+    for (; i + 2 <= n; i += 2) st2(y + i, ld2(y + i) + cc * ld2(x + i));
+    for (; i < n; ++i) y[i] += c * x[i];
+}
+// row -= a x + b y over n entries; returns the new row times z
+inline double rank2_dot(double *row, double a, const double *x, double b, const double *y, const double *z, int n) {
+    const vd2 aa = {a, a}, bb = {b, b};
+    vd2 s0 = {0.0, 0.0}, s1 = s0, s2 = s0, s3 = s0;
+    int i = 0;
+    for (; i + 8 <= n; i += 8) {
+        const vd2 r0 = ld2(row + i) - (aa * ld2(x + i) + bb * ld2(y + i));
+        const vd2 r1 = ld2(row + i + 2) - (aa * ld2(x + i + 2) + bb * ld2(y + i + 2));
+        const vd2 r2 = ld2(row + i + 4) - (aa * ld2(x + i + 4) + bb * ld2(y + i + 4));
+        const vd2 r3 = ld2(row + i + 6) - (aa * ld2(x + i + 6) + bb * ld2(y + i + 6));
+        st2(row + i, r0);
+        st2(row + i + 2, r1);
+        st2(row + i + 4, r2);
+        st2(row + i + 6, r3);
+        s0 += r0 * ld2(z + i);
+        s1 += r1 * ld2(z + i + 2);
+        s2 += r2 * ld2(z + i + 4);
+        s3 += r3 * ld2(z + i + 6);
+    }
+    double r = 0.0;
+    for (; i < n; ++i) {
+        row[i] -= a * x[i] + b * y[i];
+        r += row[i] * z[i];
+    }
+    const vd2 t = (s0 + s1) + (s2 + s3);
+    return t[0] + t[1] + r;
+}
+
 struct Tridiag {
     std::vector<double> d, e;          // diagonal [n], off-diagonal [n-1]
     std::vector<double> vs, beta;      // reflector k: vs[k][k+1..n), beta[k]
@@ -471,17 +527,14 @@ Tridiag tridiagonalize(int n, std::vector<double> &A) {
     // reflector k from x = column k below the diagonal (x[i] for i > k):
     // v = x - alpha e_{k+1}, alpha = -sign(x_{k+1}) |x|, beta = 2 / v.v
     auto reflector = [&](int k, const double *x) {
-        double xn = 0.0;
-        for (int i = k + 1; i < n; ++i) xn += x[i] * x[i];
-        xn = std::sqrt(xn);
+        const double xn = std::sqrt(dot8(x + k + 1, x + k + 1, n - k - 1));
         ready[k] = 1;
         if (xn == 0.0) { t.e[k] = 0.0; skip[k] = 1; return; }
         const double alpha = x[k + 1] >= 0.0 ? -xn : xn;
         double *v = &t.vs[(size_t)k * n];
         for (int i = k + 1; i < n; ++i) v[i] = x[i];
         v[k + 1] -= alpha;
-        double vv = 0.0;
-        for (int i = k + 1; i < n; ++i) vv += v[i] * v[i];
+        const double vv = dot8(v + k + 1, v + k + 1, n - k - 1);
         t.e[k] = alpha;
         if (vv == 0.0) { skip[k] = 1; return; }
         t.beta[k] = 2.0 / vv;
@@ -512,15 +565,12 @@ Tridiag tridiagonalize(int n, std::vector<double> &A) {
 #pragma omp for schedule(static)
             for (int i = k + 1; i < n; ++i) {
                 const double *row = &A[(size_t)i * n];
-                double acc = 0.0;
-                for (int j = k + 1; j < n; ++j) acc += row[j] * v[j];
-                p[i] = bk * acc;
+                p[i] = bk * dot8(row + k + 1, v + k + 1, n - k - 1);
             }
         }
 #pragma omp single
         {
-            double pv = 0.0;
-            for (int i = k + 1; i < n; ++i) pv += p[i] * v[i];
+            const double pv = dot8(&p[k + 1], v + k + 1, n - k - 1);
             for (int i = k + 1; i < n; ++i) wv[i] = p[i] - 0.5 * bk * pv * v[i];
             // look-ahead: column k+1 after this step's update, and its reflector
             if (k + 3 < n) {
@@ -537,14 +587,9 @@ Tridiag tridiagonalize(int n, std::vector<double> &A) {
         for (int i = k + 1; i < n; ++i) {
             double *row = &A[(size_t)i * n];
             const double vi = v[i], wi = wv[i];
-            double acc = 0.0;
             if (next && i > nx) {
                 row[nx] -= vi * wv[nx] + wi * v[nx];
-                for (int j = nx + 1; j < n; ++j) {
-                    row[j] -= vi * wv[j] + wi * v[j];
-                    acc += row[j] * vn[j];
-                }
-                pn[i] = bn * acc;
+                pn[i] = bn * rank2_dot(row + nx + 1, vi, &wv[nx + 1], wi, v + nx + 1, vn + nx + 1, n - nx - 1);
             } else {
                 for (int j = k + 1; j < n; ++j) row[j] -= vi * wv[j] + wi * v[j];
             }
@@ -624,28 +669,41 @@ std::vector<double> tridiag_lowest(const Tridiag &t, int nvec) {
     std::vector<double> e2(n > 1 ? n - 1 : 0);
     for (int i = 0; i + 1 < n; ++i) e2[i] = t.e[i] * t.e[i];
     const double tiny = 1e-300 + 2.2e-16 * std::max(std::fabs(lo), std::fabs(hi)) * 1e-10;
-    auto below = [&](double x) {
-        int c = 0;
-        double q = t.d[0] - x;
-        if (q < 0.0) ++c;
-        for (int i = 1; i < n; ++i) {
-            if (q == 0.0) q = -tiny;
-            q = t.d[i] - x - e2[i - 1] / q;
-            if (q < 0.0) ++c;
-        }
-        return c;
-    };
+    // eight eigenvalues at a time: their counts run through the same pivots
+    // together, so the divisions of one do not wait for another's
     std::vector<double> w(nvec);
-#pragma omp parallel for schedule(dynamic, 4) if ((int64_t)nvec * n > 20000)
-    for (int j = 0; j < nvec; ++j) {
-        double a = lo, b = hi;
+    const int n8 = (nvec + 7) / 8;
+#pragma omp parallel for schedule(dynamic, 1) if ((int64_t)nvec * n > 4000)
+    for (int g = 0; g < n8; ++g) {
+        double a[8], b[8], mid[8], q[8];
+        int cnt[8];
+        for (int u = 0; u < 8; ++u) { a[u] = lo; b[u] = hi; }
         for (int it = 0; it < 2100; ++it) {
-            const double mid = 0.5 * (a + b);
-            if (mid <= a || mid >= b || b - a <= 2.0 * 2.2e-16 * std::max(std::fabs(a), std::fabs(b))) break;
-            if (below(mid) > j) b = mid;
-            else a = mid;
+            bool more = false;
+            for (int u = 0; u < 8; ++u) {
+                mid[u] = 0.5 * (a[u] + b[u]);
+                more = more || (mid[u] > a[u] && mid[u] < b[u] &&
+                                b[u] - a[u] > 2.0 * 2.2e-16 * std::max(std::fabs(a[u]), std::fabs(b[u])));
+            }
+            if (!more) break;
+            for (int u = 0; u < 8; ++u) {
+                q[u] = t.d[0] - mid[u];
+                cnt[u] = q[u] < 0.0;
+            }
+            for (int i = 1; i < n; ++i) {
+                const double di = t.d[i], ei = e2[i - 1];
+                for (int u = 0; u < 8; ++u) {
+                    const double p = q[u] == 0.0 ? -tiny : q[u];
+                    q[u] = di - mid[u] - ei / p;
+                    cnt[u] += q[u] < 0.0;
+                }
+            }
+            for (int u = 0; u < 8; ++u) {
+                if (cnt[u] > 8 * g + u) b[u] = mid[u];
+                else a[u] = mid[u];
+            }
         }
-        w[j] = 0.5 * (a + b);
+        for (int u = 0; u < 8 && 8 * g + u < nvec; ++u) w[8 * g + u] = 0.5 * (a[u] + b[u]);
     }
     return w;
 }
@@ -705,13 +763,9 @@ void tridiag_vector(const Tridiag &t, double lam, double tnorm, int seed, const 
     auto orth_normalise = [&]() {
         for (int pass = 0; pass < 2; ++pass)
             for (const double *q : cluster) {
-                double dot = 0.0;
-                for (int i = 0; i < n; ++i) dot += q[i] * y[i];
-                for (int i = 0; i < n; ++i) y[i] -= dot * q[i];
+                axpy(y, -dot8(q, y, n), q, n);
             }
-        double nrm = 0.0;
-        for (int i = 0; i < n; ++i) nrm += y[i] * y[i];
-        nrm = std::sqrt(nrm);
+        double nrm = std::sqrt(dot8(y, y, n));
         if (nrm == 0.0) { y[seed % n] = 1.0; nrm = 1.0; }
         for (int i = 0; i < n; ++i) y[i] /= nrm;
     };
@@ -747,9 +801,9 @@ void hb::small_eigh(int n, std::vector<double> A, std::vector<double> &w, std::v
         const double r = (i > 0 ? std::fabs(t.e[i - 1]) : 0.0) + (i + 1 < n ? std::fabs(t.e[i]) : 0.0);
         tnorm = std::max(tnorm, std::fabs(t.d[i]) + r);
     }
-    if (n >= 256 && 2 * nvec < n) {
-        // the wanted lowest by bisection (cheaper than all of them by QR on
-        // the large projected matrices); w then holds those nvec
+    if (n >= 48 && 2 * nvec < n) {
+        // the wanted lowest by bisection (cheaper than all of them by QR, whose
+        // rotations are a serial chain of square roots); w then holds those nvec
         const std::vector<double> low = tridiag_lowest(t, nvec);
         std::copy(low.begin(), low.end(), w.begin());
         w.resize(nvec);
@@ -781,10 +835,7 @@ void hb::small_eigh(int n, std::vector<double> A, std::vector<double> &w, std::v
         for (int k = n - 3; k >= 0; --k) {
             if (t.beta[k] == 0.0) continue;
             const double *v = &t.vs[(size_t)k * n];
-            double dot = 0.0;
-            for (int i = k + 1; i < n; ++i) dot += v[i] * y[i];
-            dot *= t.beta[k];
-            for (int i = k + 1; i < n; ++i) y[i] -= dot * v[i];
+            axpy(y + k + 1, -t.beta[k] * dot8(v + k + 1, y + k + 1, n - k - 1), v + k + 1, n - k - 1);
         }
         for (int i = 0; i < n; ++i) V[(size_t)i * nvec + c] = y[i];
     }
