@@ -24,8 +24,7 @@ struct GroupPair {
     int64_t n_pairs = 0, n_items = 0;
     int n_chunks = 0, n_nn = 0;
     int64_t *rowptr = nullptr;
-    int32_t *seg_off = nullptr;   // [ndet][segments] offsets of the column segments within each row
-    hb_pair *pairs = nullptr;
+    hb_pair *pairs = nullptr;   // (row, col) of every pair from hb_init on; the records are a build's
     double *val = nullptr;
     int64_t *item_ptr = nullptr;
     GammaItem *items = nullptr;
@@ -41,7 +40,6 @@ struct GroupPair {
 // Scratch of one target group against the L2 functions (class 4).
 struct GroupL2 {
     int64_t *rowptr = nullptr;
-    int32_t *seg_off = nullptr;
     hb_pair *pairs = nullptr;
     int64_t n_pairs = 0;
 };

@@ -31,13 +31,11 @@ struct Grouped {
 };
 
 // ----------------------------------------------------------------- tasks
-struct ClsTask {        // K1: classify rows of a against b into records
+struct ClsTask {        // K1: the records of a list of pairs (row of a, column of b)
     const uint64_t *a, *b;
-    int n_a, n_b, cont_spin, max_degree, lower;
-    const int64_t *row_ptr;
-    const int32_t *seg_off;   // [n_a][nseg] offsets of the column segments within each row
-    int nseg;
-    hb_pair *out;
+    int cont_spin;
+    int64_t n_pairs;
+    hb_pair *out;             // (row, col) given, the rest filled in
 };
 
 struct PVTask {         // <D_m|H^N|D'_m'> for the records of a group pair
@@ -311,6 +309,7 @@ void class4_shape(int ns, int cn, int *ns_tile, int *jt);
 // block counts of one task of each stage (host side)
 int64_t blocks_rows8(int64_t rows);                 // one warp per row, 8 warps a block
 int64_t blocks_seg_rows8(int64_t rows, int n_b);    // the same per column segment
+int64_t blocks_classify(int64_t n_pairs);
 int64_t blocks_pair_values(int64_t n_pairs);
 int64_t blocks_tn_partial(int n_rows, int ns, int nsp);
 int64_t blocks_tn_reduce(int ns, int nsp);

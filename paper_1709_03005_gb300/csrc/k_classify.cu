@@ -14,7 +14,7 @@ namespace hb {
 namespace {
 
 constexpr int kWarpsPerBlock = 8;
-constexpr int kSeg = kSegCols;   // columns per segment of the hot scans
+constexpr int kSeg = kSegCols;   // columns per segment of the L2 scan
 
 template <int W>
 __device__ __forceinline__ void load_det(const uint64_t *p, uint64_t (&x)[2 * W]) {
@@ -49,11 +49,26 @@ __device__ __forceinline__ int bits_of_diff(const uint64_t (&x)[2 * W], const ui
     return n;
 }
 
-// Sign exponent of <bra| a+_p1 a+_p2 a_h2 a_h1 |ket> for holes h1<h2 and
-// particles p1<p2 (keys in canonical order), ck(x) = # ket electrons below x.
-__device__ __forceinline__ int double_exponent(int ch1, int ch2, int cp1, int cp2, int kh1, int kh2,
-                                               int kp1, int kp2) {
-    return ch1 + ch2 - 1 + cp2 - (kh1 < kp2) - (kh2 < kp2) + cp1 - (kh1 < kp1) - (kh2 < kp1);
+// Parity of the number of electrons of x below each of up to four positions, added up.
+template <int W>
+__device__ __forceinline__ int parity_below(const uint64_t (&x)[2 * W], int p0, int p1, int p2, int p3) {
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) {
+        auto below = [&](int pos) -> uint64_t {
+            const int k = pos - 64 * w;
+            return k <= 0 ? 0ull : (k >= 64 ? ~0ull : (1ull << k) - 1ull);
+        };
+        n ^= __popcll(x[w] & (below(p0) ^ below(p1) ^ below(p2) ^ below(p3)));
+    }
+    return n & 1;
+}
+
+// Corrections to the sign of <bra| a+_p1 a+_p2 a_h2 a_h1 |ket> for holes h1<h2
+// and particles p1<p2 (keys in canonical order) beside the counts of ket
+// electrons below each.
+__device__ __forceinline__ int double_correction(int kh1, int kh2, int kp1, int kp2) {
+    return 1 + (kh1 < kp2) + (kh2 < kp2) + (kh1 < kp1) + (kh2 < kp1);
 }
 
 template <int W, int MODE>
@@ -71,13 +86,11 @@ __device__ __forceinline__ void make_record(const uint64_t (&a)[2 * W], const ui
         bits_of_diff<W>(b, a, h);
         bits_of_diff<W>(a, b, p);
         if (deg == 1) {
-            e = prefix_count(b, 2 * W, h[0]) + prefix_count(b, 2 * W, p[0]) - (h[0] < p[0]);
+            e = parity_below<W>(b, h[0], p[0], 0, 0) + (h[0] < p[0]);
             r.hole[0] = (int16_t)h[0];
             r.part[0] = (int16_t)p[0];
         } else if (deg == 2) {
-            e = double_exponent(prefix_count(b, 2 * W, h[0]), prefix_count(b, 2 * W, h[1]),
-                                prefix_count(b, 2 * W, p[0]), prefix_count(b, 2 * W, p[1]), h[0], h[1],
-                                p[0], p[1]);
+            e = parity_below<W>(b, h[0], h[1], p[0], p[1]) + double_correction(h[0], h[1], p[0], p[1]);
             r.hole[0] = (int16_t)h[0]; r.hole[1] = (int16_t)h[1];
             r.part[0] = (int16_t)p[0]; r.part[1] = (int16_t)p[1];
         }
@@ -86,22 +99,17 @@ __device__ __forceinline__ void make_record(const uint64_t (&a)[2 * W], const ui
         // Keys are doubled bit positions; v sits just above the last target
         // orbital of its spin.
         const int kv = cont_spin == 0 ? 2 * 64 * W - 1 : 2 * 128 * W - 1;
-        const int cv = cont_spin == 0 ? prefix_count(a, 2 * W, 64 * W) : prefix_count(a, 2 * W, 128 * W);
+        const int pv = cont_spin == 0 ? 64 * W : 128 * W;        // electrons below v: those of the spins up to its own
         int h[2], q[2];
         const int nh = bits_of_diff<W>(a, b, h);   // in chi only: d + 1
         const int nq = bits_of_diff<W>(b, a, q);   // in D only: d
         if (deg == 1 && nh >= 1) {
             const int kh = 2 * h[0];
-            e = prefix_count(a, 2 * W, h[0]) + cv - (kh < kv);
+            e = parity_below<W>(a, h[0], pv, 0, 0) + (kh < kv);
             r.hole[0] = (int16_t)h[0];
         } else if (deg == 2 && nh == 2 && nq == 1) {
-            const int kq = 2 * q[0];
-            int kp1, kp2, cp1, cp2;
-            const int cq = prefix_count(a, 2 * W, q[0]);
-            if (kq < kv) { kp1 = kq; cp1 = cq; kp2 = kv; cp2 = cv; }
-            else { kp1 = kv; cp1 = cv; kp2 = kq; cp2 = cq; }
-            e = double_exponent(prefix_count(a, 2 * W, h[0]), prefix_count(a, 2 * W, h[1]), cp1, cp2,
-                                2 * h[0], 2 * h[1], kp1, kp2);
+            const int kq = 2 * q[0], kp1 = min(kq, kv), kp2 = max(kq, kv);
+            e = parity_below<W>(a, h[0], h[1], q[0], pv) + double_correction(2 * h[0], 2 * h[1], kp1, kp2);
             r.hole[0] = (int16_t)h[0]; r.hole[1] = (int16_t)h[1];
             r.part[0] = (int16_t)q[0];
         }
@@ -215,105 +223,27 @@ k1_fill_kernel(const uint64_t *__restrict__ A, int n_a, const uint64_t *__restri
     fill_row<W, MODE>(A, B, n_b, cont_spin, max_degree, lower, row_ptr, out, row, threadIdx.x & 31);
 }
 
-// The same over many (a, b) tasks in one launch, with the column
-// determinants staged through shared memory: the 8 warps of a block (8 rows)
-// read each tile of columns from memory once, word-major so the lanes'
-// shared-memory reads are conflict free.
-template <int W>
-struct ColTile {
-    static constexpr int kCols = kSeg;       // a segment of column determinants
-};
-
-template <int W>
-__device__ __forceinline__ void stage_cols(uint64_t *tile, const uint64_t *__restrict__ B, int t0, int tn) {
-    constexpr int TC = ColTile<W>::kCols;
-    for (int i = threadIdx.x; i < tn * 2 * W; i += blockDim.x) {
-        const int c = i / (2 * W), w = i % (2 * W);
-        tile[w * TC + c] = __ldg(B + (int64_t)t0 * 2 * W + i);
-    }
-}
-
-template <int W>
-__device__ __forceinline__ void tile_det(const uint64_t *tile, int c, uint64_t (&b)[2 * W]) {
-#pragma unroll
-    for (int w = 0; w < 2 * W; ++w) b[w] = tile[w * ColTile<W>::kCols + c];
-}
-
-// Matches are queued per warp (in column order) and turned into records 32
-// at a time, one per lane, so the record work never runs with a lone lane.
+// A build's classification: hb_init has found the pairs within a double
+// excitation, in order, so a build works out degree, holes, particles and phase
+// of each listed pair (row, col), one per lane.  Searching all pairs again, in
+// tiles of 8 rows x 512 columns, took 0.80 + 0.34 ms for a batch of twelve
+// Hamiltonians (14e6 of 2e8 pairs couple) and 0.98 + 1.19 ms for 20000 target
+// determinants and 30000 L2 functions; now 0.27 + 0.02 and 0.20 + 0.03 ms, the
+// 24-byte records read and written.
 template <int W, int MODE>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock)
-k1_fill_grouped(const ClsTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
-    constexpr int TC = ColTile<W>::kCols;
-    __shared__ uint64_t tile[TC * 2 * W];
-    __shared__ int queue[kWarpsPerBlock][64];
+__global__ void __launch_bounds__(256)
+classify_kernel(const ClsTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const ClsTask &T = tasks[ti];
-    const int lb = (int)(blockIdx.x - blk[ti]);
-    // block = (8 rows, one segment of columns)
-    const int rb = lb / T.nseg, sg = lb % T.nseg;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int row = rb * kWarpsPerBlock + warp;
-    const bool active = row < T.n_a;
-    int *q = queue[warp];
-    uint64_t a[2 * W];
-    int limit = 0;
-    int64_t pos = 0, end = 0;
-    if (active) {
-        load_det<W>(T.a + (int64_t)row * 2 * W, a);
-        limit = T.lower ? min(T.n_b, row + 1) : T.n_b;
-        pos = T.row_ptr[row] + T.seg_off[(int64_t)row * T.nseg + sg];
-        end = T.row_ptr[row + 1];
-    }
-    const int last_row = min(T.n_a, (rb + 1) * kWarpsPerBlock) - 1;
-    const int blim = T.lower ? min(T.n_b, last_row + 1) : T.n_b;
-    const int t0 = sg * TC;
-    if (t0 >= blim) return;
-    const int tn = min(TC, blim - t0);
-    stage_cols<W>(tile, T.b, t0, tn);
-    __syncthreads();
-    // records for the first `cnt` queued columns
-    auto drain = [&](int cnt) {
-        if (lane < cnt) {
-            const int cl = q[lane];
-            uint64_t b[2 * W];
-            tile_det<W>(tile, cl, b);
-            const int deg = degree_of<W, MODE>(a, b);
-            const int64_t at = pos + lane;
-            if (at < end) {
-                hb_pair r;
-                make_record<W, MODE>(a, b, deg, T.cont_spin, row, t0 + cl, r);
-                T.out[at] = r;
-            }
-        }
-        pos += cnt;
-    };
-    const int cend = active ? min(tn, limit - t0) : 0;
-    int qn = 0;
-    for (int c0 = 0; c0 < cend; c0 += 32) {
-        const int cl = c0 + lane;
-        bool ok = false;
-        if (cl < cend) {
-            uint64_t b[2 * W];
-            tile_det<W>(tile, cl, b);
-            ok = degree_of<W, MODE>(a, b) <= T.max_degree;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        if (ok) q[qn + __popc(m & ((1u << lane) - 1u))] = cl;
-        qn += __popc(m);
-        __syncwarp();
-        if (qn >= 32) {
-            drain(32);
-            __syncwarp();
-            const int rest = qn - 32;
-            const int mv = lane < rest ? q[32 + lane] : 0;
-            __syncwarp();
-            if (lane < rest) q[lane] = mv;
-            qn = rest;
-            __syncwarp();
-        }
-    }
-    if (qn > 0) drain(qn);
+    const int64_t k = (blockIdx.x - blk[ti]) * (int64_t)256 + threadIdx.x;
+    if (k >= T.n_pairs) return;
+    const int2 rc = *reinterpret_cast<const int2 *>(T.out + k);
+    uint64_t a[2 * W], b[2 * W];
+    load_det<W>(T.a + (int64_t)rc.x * 2 * W, a);
+    load_det<W>(T.b + (int64_t)rc.y * 2 * W, b);
+    hb_pair r;
+    make_record<W, MODE>(a, b, degree_of<W, MODE>(a, b), T.cont_spin, rc.x, rc.y, r);
+    T.out[k] = r;
 }
 
 // Inclusive scan of x[1..n] in place (x[0] = 0 is set), single block.
@@ -417,6 +347,7 @@ void k1_seg_offsets(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int 
 }
 
 int64_t blocks_seg_rows8(int64_t rows, int n_b) { return ((rows + 7) / 8) * seg_count(n_b); }
+int64_t blocks_classify(int64_t n_pairs) { return (n_pairs + 255) / 256; }
 
 void exclusive_scan_inplace(int64_t *x, int n, cudaStream_t s) {
     scan_kernel<<<1, 1024, 0, s>>>(x, n);
@@ -424,9 +355,9 @@ void exclusive_scan_inplace(int64_t *x, int n, cudaStream_t s) {
 
 int g_classify(const Grouped<ClsTask> &g, int W, int mode, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
-    const dim3 grid((unsigned)g.blocks), block(32 * kWarpsPerBlock);
-#define HB_K1G(WW) (mode == 0 ? k1_fill_grouped<WW, 0><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n) \
-                              : k1_fill_grouped<WW, 1><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n))
+    const dim3 grid((unsigned)g.blocks), block(256);
+#define HB_K1G(WW) (mode == 0 ? classify_kernel<WW, 0><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n) \
+                              : classify_kernel<WW, 1><<<grid, block, 0, s>>>(g.tasks, g.blk, g.n))
     switch (W) {
         case 1: HB_K1G(1); break;
         case 2: HB_K1G(2); break;

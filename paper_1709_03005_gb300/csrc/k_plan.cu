@@ -275,9 +275,7 @@ void fill_tasks(Plan &p) {
             const double *Ca = ctx->ci + A.ci_off, *Cb = ctx->ci + B.ci_off;
             const float2 *Ca_df = ctx->ci_df ? ctx->ci_df + A.ci_off : nullptr;
             const float2 *Cb_df = ctx->ci_df ? ctx->ci_df + B.ci_off : nullptr;
-            p.cls_tt.add(ClsTask{da, db, A.ndet, B.ndet, ctx->cont_spin, 2, 0, P.rowptr, P.seg_off, seg_count(B.ndet),
-                                 P.pairs},
-                         blocks_seg_rows8(A.ndet, B.ndet));
+            p.cls_tt.add(ClsTask{da, db, ctx->cont_spin, P.n_pairs, P.pairs}, blocks_classify(P.n_pairs));
             const PVTask pvt{I, da, db, P.pairs, P.n_pairs, P.val, P.rowptr, A.ndet, P.same};
             p.pv.add(pvt, blocks_pair_values(P.n_pairs));
             if (P.same) p.pvd.add(pvt, blocks_diag_values(A.ndet));
@@ -380,9 +378,7 @@ void fill_tasks(Plan &p) {
             const GroupInfo &G = ctx->groups[g];
             GroupL2 &L = ctx->gl2[g];
             const uint64_t *dg = ctx->dets + G.det_off;
-            p.cls_tl2.add(ClsTask{ctx->l2, dg, ctx->n_l2, G.ndet, ctx->cont_spin, 2, 0, L.rowptr, L.seg_off,
-                                  seg_count(G.ndet), L.pairs},
-                          blocks_seg_rows8(ctx->n_l2, G.ndet));
+            p.cls_tl2.add(ClsTask{ctx->l2, dg, ctx->cont_spin, L.n_pairs, L.pairs}, blocks_classify(L.n_pairs));
             if (p.precision == HB_MIXED && c4tc_group_on(ctx, g)) {
                 C4FTask ft;
                 C4TTask tt;
