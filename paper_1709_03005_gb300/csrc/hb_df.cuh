@@ -79,6 +79,10 @@ __device__ __forceinline__ double df_sum(float hi, float lo) {
 // on the FP64 pipe; AccF sums the float pairs in double-float.
 struct AccD {
     double v = 0.0;
+    using Entry = double;
+    static __device__ __forceinline__ Entry entry(const double *t, const float2 *, int64_t i) { return __ldg(t + i); }
+    __device__ __forceinline__ void add_entry(Entry x) { v += x; }
+    __device__ __forceinline__ void sub_entry(Entry x) { v -= x; }
     __device__ __forceinline__ void add(const double *t, const float2 *, int64_t i) { v += __ldg(t + i); }
     __device__ __forceinline__ void sub(const double *t, const float2 *, int64_t i) { v -= __ldg(t + i); }
     __device__ __forceinline__ void neg() { v = -v; }
@@ -88,6 +92,10 @@ struct AccD {
 
 struct AccF {
     float h = 0.0f, l = 0.0f;
+    using Entry = float2;
+    static __device__ __forceinline__ Entry entry(const double *, const float2 *t, int64_t i) { return __ldg(t + i); }
+    __device__ __forceinline__ void add_entry(Entry x) { df_add2(h, l, x.x, x.y); }
+    __device__ __forceinline__ void sub_entry(Entry x) { df_add2(h, l, -x.x, -x.y); }
     __device__ __forceinline__ void add(const double *, const float2 *t, int64_t i) {
         const float2 x = __ldg(t + i);
         df_add2(h, l, x.x, x.y);

@@ -46,6 +46,7 @@ struct PVTask {         // <D_m|H^N|D'_m'> for the records of a group pair
     double *val;
     const int64_t *row_ptr;   // records of row m: [row_ptr[m], row_ptr[m + 1]), ascending columns
     int n_rows, same;         // same group: the diagonal records (m, m) go to g_diag_values
+    int steps;                // steps of 32 records a warp takes
 };
 
 // In the double-float launches of the stages below, val, Wout, Wm and partial
@@ -310,7 +311,7 @@ void class4_shape(int ns, int cn, int *ns_tile, int *jt);
 int64_t blocks_rows8(int64_t rows);                 // one warp per row, 8 warps a block
 int64_t blocks_seg_rows8(int64_t rows, int n_b);    // the same per column segment
 int64_t blocks_classify(int64_t n_pairs);
-int64_t blocks_pair_values(int64_t n_pairs);
+int64_t blocks_pair_values(int64_t n_pairs, int steps);
 int64_t blocks_tn_partial(int n_rows, int ns, int nsp);
 int64_t blocks_tn_reduce(int ns, int nsp);
 int64_t blocks_zero(int64_t n);

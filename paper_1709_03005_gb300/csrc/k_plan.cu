@@ -233,9 +233,12 @@ void fill_tasks(Plan &p) {
     // few target rows: a block per row, so that the longest does not set a
     // stage's time; many: 8 rows a block (335400 blocks of one row, 42 records on
     // average, took 448 us to start and end)
-    int64_t rows = 0;
-    for (const hb_ctx *c : p.ctxs)
+    int64_t rows = 0, tt_pairs = 0;
+    for (const hb_ctx *c : p.ctxs) {
         for (auto &P : c->gps) rows += c->groups[P.g].ndet;
+        tt_pairs += c->tt_pairs;
+    }
+    const int pv_steps = l2_value_steps(tt_pairs);   // one launch over all of them
     p.block_rows = rows <= 64 * 1024;
     int64_t coef_row = 0;
     // expansion blocks: the group pairs (of any context) that read the same
@@ -276,8 +279,9 @@ void fill_tasks(Plan &p) {
             const float2 *Ca_df = ctx->ci_df ? ctx->ci_df + A.ci_off : nullptr;
             const float2 *Cb_df = ctx->ci_df ? ctx->ci_df + B.ci_off : nullptr;
             p.cls_tt.add(ClsTask{da, db, ctx->cont_spin, P.n_pairs, P.pairs}, blocks_classify(P.n_pairs));
-            const PVTask pvt{I, da, db, P.pairs, P.n_pairs, P.val, P.rowptr, A.ndet, P.same};
-            p.pv.add(pvt, blocks_pair_values(P.n_pairs));
+            const PVTask pvt{I, da, db, P.pairs, P.n_pairs, P.val, P.rowptr, A.ndet, P.same,
+                             pv_steps};
+            p.pv.add(pvt, blocks_pair_values(P.n_pairs, pv_steps));
             if (P.same) p.pvd.add(pvt, blocks_diag_values(A.ndet));
             // the bra rows this rank contracts (all of them unless sharded)
             const auto mr = shard_range(A.ndet, p.shard_r, p.shard_n);

@@ -67,6 +67,8 @@ __device__ Acc diag_value(const Ints &I, const uint64_t (&d)[2 * W]) {
     return e;
 }
 
+// The integrals of up to eight electrons are in flight at a time; they are
+// added one by one in order.
 template <int W, class Acc>
 __device__ Acc single_value(const Ints &I, const uint64_t (&bra)[2 * W], const uint64_t (&ket)[2 * W], int hpos,
                             int ppos) {
@@ -81,10 +83,23 @@ __device__ Acc single_value(const Ints &I, const uint64_t (&bra)[2 * W], const u
         for (int w = 0; w < W; ++w) {
             uint64_t x = bra[s * W + w] & ket[s * W + w];
             while (x) {
-                const int k = 64 * w + __ffsll((long long)x) - 1;
-                x &= x - 1;
-                v.add(I.tttt, I.tttt_df, ph + pair_idx(k, k));
-                if (s == hs) v.sub(I.tttt, I.tttt_df, eri_idx(I, p, k, k, h));
+                typename Acc::Entry J[8], K[8];
+                int cnt = 0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (x) {
+                        const int k = 64 * w + __ffsll((long long)x) - 1;
+                        x &= x - 1;
+                        J[u] = Acc::entry(I.tttt, I.tttt_df, ph + pair_idx(k, k));
+                        if (s == hs) K[u] = Acc::entry(I.tttt, I.tttt_df, eri_idx(I, p, k, k, h));
+                        cnt = u + 1;
+                    }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u < cnt) {
+                        v.add_entry(J[u]);
+                        if (s == hs) v.sub_entry(K[u]);
+                    }
             }
         }
     }
@@ -333,43 +348,13 @@ __device__ __forceinline__ double double_element(const Ints &I, const uint64_t (
     return odd ? -v : v;
 }
 
-// sum of a single: the integrals of up to eight electrons in flight at a time,
-// added in the order of single_value
 template <int W>
 __device__ __forceinline__ double single_element(const Ints &I, const uint64_t (&a)[2 * W], const uint64_t (&b)[2 * W]) {
-    int hh[2], pp[2];
-    diff_bits<W>(b, a, hh);
-    diff_bits<W>(a, b, pp);
-    constexpr int sb = 64 * W;
-    const int odd = parity4<W>(b, hh[0], pp[0], 0, 0) ^ (hh[0] < pp[0]);
-    const int hs = hh[0] >= sb, h = hh[0] - hs * sb, p = pp[0] - (pp[0] >= sb) * sb;
-    double v = __ldg(I.h + (int64_t)p * I.n_orb + h);
-    const double *ph = I.tttt + pair_idx(p, h) * I.Pt;
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            uint64_t x = a[s * W + w] & b[s * W + w];
-            while (x) {
-                double J[8], K[8];
-                int cnt = 0;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (!x) { J[u] = K[u] = 0.0; continue; }
-                    const int k = 64 * w + __ffsll((long long)x) - 1;
-                    x &= x - 1;
-                    J[u] = __ldg(ph + pair_idx(k, k));
-                    K[u] = s == hs ? __ldg(I.tttt + eri_idx(I, p, k, k, h)) : 0.0;
-                    cnt = u + 1;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (u < cnt) {
-                        v += J[u];
-                        if (s == hs) v -= K[u];
-                    }
-            }
-        }
+    int h[2], p[2];
+    diff_bits<W>(b, a, h);
+    diff_bits<W>(a, b, p);
+    const int odd = parity4<W>(b, h[0], p[0], 0, 0) ^ (h[0] < p[0]);
+    const double v = single_value<W, AccD>(I, a, b, h[0], p[0]).value();
     return odd ? -v : v;
 }
 
@@ -572,27 +557,67 @@ __global__ void l2_mirror_fill_kernel(const int32_t *__restrict__ col, const int
 }
 
 // <A[row]|H|B[col]> for classified pairs (mode 0 records).  FP64: val as
-// doubles; double-float: val as (hi, lo) float pairs in the same 8 bytes.
+// doubles; double-float: val as (hi, lo) float pairs in the same 8 bytes.  As in
+// l2_values_kernel a warp takes 32 steps consecutive records, evaluates the
+// doubles as they come and queues the singles until 32 fill its lanes.
 template <int W, class Acc>
-__global__ void pair_values_kernel(const PVTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+__global__ void __launch_bounds__(32 * kWarps)
+pair_values_kernel(const PVTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
+    __shared__ int64_t queue[kWarps][64];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const PVTask &T = tasks[ti];
-    const int64_t k = (blockIdx.x - blk[ti]) * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= T.n_pairs) return;
     const Ints I = T.I;
-    const hb_pair r = T.pairs[k];
-    // within one group the diagonal records (O(N^2) sums, one per row) are
-    // left to diag_values_kernel, so that no warp here waits on one
-    if (r.degree == 0 && T.same) return;
-    uint64_t a[2 * W], b[2 * W];
-    load_det<W>(T.a + (int64_t)r.row * 2 * W, a);
-    load_det<W>(T.b + (int64_t)r.col * 2 * W, b);
-    Acc v;
-    if (r.degree == 0) v = diag_value<W, Acc>(I, a);
-    else if (r.degree == 1) v = single_value<W, Acc>(I, a, b, r.hole[0], r.part[0]);
-    else v = double_value<Acc>(I, W, r.hole[0], r.hole[1], r.part[0], r.part[1]);
-    if (r.degree > 0 && r.phase < 0) v.neg();
-    store_value(v, T.val, k);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t k0 = ((blockIdx.x - blk[ti]) * (int64_t)kWarps + warp) * 32 * T.steps;
+    int64_t *q = queue[warp];
+    int qn = 0;
+    auto drain = [&](int cnt) {
+        if (lane < cnt) {
+            const int64_t k = q[lane];
+            const hb_pair r = T.pairs[k];
+            uint64_t a[2 * W], b[2 * W];
+            load_det<W>(T.a + (int64_t)r.row * 2 * W, a);
+            load_det<W>(T.b + (int64_t)r.col * 2 * W, b);
+            Acc v = single_value<W, Acc>(I, a, b, r.hole[0], r.part[0]);
+            if (r.phase < 0) v.neg();
+            store_value(v, T.val, k);
+        }
+    };
+    for (int st = 0; st < T.steps; ++st) {
+        const int64_t k = k0 + 32 * st + lane;
+        bool single = false;
+        if (k < T.n_pairs) {
+            const hb_pair r = T.pairs[k];
+            if (r.degree == 1) {
+                single = true;
+            } else if (r.degree == 2) {
+                Acc v = double_value<Acc>(I, W, r.hole[0], r.hole[1], r.part[0], r.part[1]);
+                if (r.phase < 0) v.neg();
+                store_value(v, T.val, k);
+            } else if (!T.same) {
+                // within one group the diagonal records (O(N^2) sums, one per row)
+                // are left to diag_values_kernel
+                uint64_t a[2 * W];
+                load_det<W>(T.a + (int64_t)r.row * 2 * W, a);
+                store_value(diag_value<W, Acc>(I, a), T.val, k);
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, single);
+        if (single) q[qn + __popc(m & ((1u << lane) - 1u))] = k;
+        qn += __popc(m);
+        __syncwarp();
+        if (qn >= 32) {
+            drain(32);
+            __syncwarp();
+            const int rest = qn - 32;
+            const int64_t mv = lane < rest ? q[32 + lane] : 0;
+            __syncwarp();
+            if (lane < rest) q[lane] = mv;
+            qn = rest;
+            __syncwarp();
+        }
+    }
+    if (qn > 0) drain(qn);
 }
 
 // <D_m|H^N|D_m> of a same-group task: the record (m, m) of row m, found by
@@ -641,7 +666,10 @@ void build_jk(const Ints &I, double *jk, cudaStream_t s) {
     jk_kernel<<<(n + 255) / 256, 256, 0, s>>>(I, jk);
 }
 
-int64_t blocks_pair_values(int64_t n_pairs) { return (n_pairs + 255) / 256; }
+int64_t blocks_pair_values(int64_t n_pairs, int steps) {
+    const int64_t per = 32 * kWarps * (int64_t)steps;
+    return (n_pairs + per - 1) / per;
+}
 int64_t blocks_diag_values(int n_rows) { return (n_rows + kWarps - 1) / kWarps; }
 
 int g_diag_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s) {
