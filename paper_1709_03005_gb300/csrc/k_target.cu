@@ -77,9 +77,9 @@ sandwich_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__ bl
 
 // The same for nsp <= 32: the lanes form G = 32 / P groups of P columns (P the
 // power of two >= nsp).  A row's records are cut into four contiguous parts;
-// group g takes records g, g+G, ... of a part, the groups of a part are
-// combined by a butterfly over the lanes that hold the same column, the parts
-// in order.  A warp per row (four parts in flight), or a block per row with a
+// group g takes records g, g+G, ... of a part, a lane adds its parts in order,
+// and the groups are combined by a butterfly over the lanes that hold the same
+// column.  A warp per row (four parts in flight), or a block per row with a
 // warp per part where the plan has few rows and the longest sets the time (300
 // rows, one of 300 records: 35 us, now 9): the same sums in the same order.
 template <bool DF>
@@ -139,13 +139,11 @@ __global__ void sandwich_small_kernel(const SWTask *__restrict__ tasks, const in
         if (c < nsp)
 #pragma unroll 4
             for (int64_t k = kb + g; k < ke; k += G) s[0].term(T, k, nsp, c);
-        s[0].tree(P);
         red[w][lane] = s[0];
         __syncthreads();
-        if (w == 0) {
+        if (w != 0) return;
 #pragma unroll
-            for (int u = 1; u < 4; ++u) s[0].add(red[u][lane]);
-        }
+        for (int u = 1; u < 4; ++u) s[0].add(red[u][lane]);
     } else {
         if (c < nsp)
             for (int64_t i = g; i < per; i += G) {
@@ -156,11 +154,10 @@ __global__ void sandwich_small_kernel(const SWTask *__restrict__ tasks, const in
                 }
             }
 #pragma unroll
-        for (int u = 0; u < (BLOCK ? 1 : 4); ++u) s[u].tree(P);
-#pragma unroll
         for (int u = 1; u < (BLOCK ? 1 : 4); ++u) s[0].add(s[u]);
     }
-    if (g == 0 && c < nsp && (!BLOCK || w == 0)) s[0].store(T, (int64_t)row * nsp + c);
+    s[0].tree(P);
+    if (g == 0 && c < nsp) s[0].store(T, (int64_t)row * nsp + c);
 }
 
 // partial[c][n][n'] = sum_{m in chunk c} C[m][n] * Wm[m][n']; rows staged in
@@ -955,6 +952,9 @@ __global__ void gamma_df_kernel(const GTask *__restrict__ tasks, const int64_t *
     }
 }
 
+// The warp loads the (determinants, phase) of 32 items together and then walks
+// them in order, so that an item's CI rows do not wait for the two loads that
+// lead to them.
 __global__ void gamma_warp_df_kernel(const GTask *__restrict__ tasks, const int64_t *__restrict__ blk,
                                      int n_tasks) {
     const int ti = task_of(blk, n_tasks, blockIdx.x);
@@ -962,36 +962,49 @@ __global__ void gamma_warp_df_kernel(const GTask *__restrict__ tasks, const int6
     const int lane = threadIdx.x & 31;
     const int key0 = ((int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * T.kpb;
     const int ns = T.ns, nsp = T.nsp, nout = ns * nsp;
-    for (int key = key0; key < min(T.n_keys, key0 + T.kpb); ++key) {
-    const int64_t b = T.off[(int64_t)key * T.nc];
-    const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) continue;
-    float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
     const int t0 = lane, t1 = lane + 32;
-    const int a0 = t0 / nsp, c0 = t0 % nsp, a1 = t1 / nsp, c1 = t1 % nsp;
+    const int a0 = t0 < nout ? t0 / nsp : 0, c0 = t0 < nout ? t0 % nsp : 0;
+    const int a1 = t1 < nout ? t1 / nsp : 0, c1 = t1 < nout ? t1 % nsp : 0;
+    const bool two = nout > 32;
     // renormalise at the block kernel's batch ends, so both forms give the same bits
     const int kb = stage_batch(ns, nsp);
-    int since = 0;
-    for (int64_t i = b; i < e; ++i) {
-        const GammaItem it = T.items[T.order[i]];
-        const float sg = it.phase < 0 ? -1.0f : 1.0f;
-        if (t0 < nout) {
-            const float2 x = __ldg(T.C_df + (int64_t)it.m * ns + a0), y = __ldg(T.Cp_df + (int64_t)it.mp * nsp + c0);
-            df_fma(h0, l0, sg * x.x, sg * x.y, y.x, y.y);
+    for (int key = key0; key < min(T.n_keys, key0 + T.kpb); ++key) {
+        const int64_t b = T.off[(int64_t)key * T.nc];
+        const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
+        if (b == e) continue;
+        float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
+        int since = 0;
+        for (int64_t i0 = b; i0 < e; i0 += 32) {
+            const int cnt = (int)min((int64_t)32, e - i0);
+            int mm = 0, mp = 0;
+            float ph = 0.0f;
+            if (lane < cnt) {
+                const GammaItem it = T.items[T.order[i0 + lane]];
+                mm = it.m;
+                mp = it.mp;
+                ph = it.phase < 0 ? -1.0f : 1.0f;
+            }
+#pragma unroll 4
+            for (int i = 0; i < cnt; ++i) {
+                const int m = __shfl_sync(0xffffffffu, mm, i), q = __shfl_sync(0xffffffffu, mp, i);
+                const float sg = __shfl_sync(0xffffffffu, ph, i);
+                const float2 *cm = T.C_df + (int64_t)m * ns, *cq = T.Cp_df + (int64_t)q * nsp;
+                const float2 x = __ldg(cm + a0), y = __ldg(cq + c0);
+                df_fma(h0, l0, sg * x.x, sg * x.y, y.x, y.y);
+                if (two) {
+                    const float2 z = __ldg(cm + a1), u = __ldg(cq + c1);
+                    df_fma(h1, l1, sg * z.x, sg * z.y, u.x, u.y);
+                }
+                if (++since == kb || i0 + i + 1 == e) {
+                    since = 0;
+                    df_norm(h0, l0);
+                    df_norm(h1, l1);
+                }
+            }
         }
-        if (t1 < nout) {
-            const float2 x = __ldg(T.C_df + (int64_t)it.m * ns + a1), y = __ldg(T.Cp_df + (int64_t)it.mp * nsp + c1);
-            df_fma(h1, l1, sg * x.x, sg * x.y, y.x, y.y);
-        }
-        if (++since == kb || i + 1 == e) {
-            since = 0;
-            df_norm(h0, l0);
-            df_norm(h1, l1);
-        }
-    }
-    float2 *g = reinterpret_cast<float2 *>(T.gamma);
-    if (t0 < nout) g[(int64_t)key * nout + t0] = make_float2(h0, l0);
-    if (t1 < nout) g[(int64_t)key * nout + t1] = make_float2(h1, l1);
+        float2 *g = reinterpret_cast<float2 *>(T.gamma);
+        if (t0 < nout) g[(int64_t)key * nout + t0] = make_float2(h0, l0);
+        if (t1 < nout) g[(int64_t)key * nout + t1] = make_float2(h1, l1);
     }
 }
 
