@@ -860,29 +860,41 @@ __device__ __forceinline__ void digits(double x, int emax, int S, int first, int
             F = (b >> 63) ? -f : f;
         }
     }
-    for (int i = 0; i < S; ++i) {
+#pragma unroll
+    for (int i = 0; i < MAXS + 1; ++i) {
+        if (i >= S) break;
         const int sh = step * (S - 1 - i);
         const long long d = sh > 0 ? ((F + (1ll << (sh - 1))) >> sh) : F;   // nearest digit
         F -= d << sh;
-        put(i, (float)d);
+        put(i, __int_as_float(0x4B400000 + (int)d) - 12582912.0f);   // |d| < 2^22, exactly
     }
 }
 
 // Digit sizes of the expansion's slices, and of the Davidson products'.
 constexpr int kXFirst = 8, kXStep = 9, kDFirst = 7, kDStep = 7;
 
+// d 2^e for a digit d (at most 9 bits) and the exponent e of its slice; the
+// result, being exact in bf16, is its upper 16 bits.
+__device__ __forceinline__ uint32_t slice_bits(float d, int e) {
+    if (e >= -126 && e <= 100) return __float_as_uint(d * __int_as_float((e + 127) << 23)) >> 16;
+    return __bfloat16_as_ushort(__float2bfloat16_rn(ldexpf(d, e)));
+}
+
 // One row into its S bf16 slices by a whole block: every thread reads its
 // share of the row, the row exponent is reduced through shared memory, then
-// each thread writes the digits of its elements.  at(k) gives element k (0
-// beyond the row's data).  With `exps` the row exponent goes there and the
-// slices are those of x / 2^e.
+// each thread writes the digits of its elements, two neighbours to a store.
+// at(k) gives element k (0 beyond the row's data).  With `exps` the row exponent
+// goes there and the slices are those of x / 2^e.
 template <class At>
 __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S, int first, int step,
                                                 __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps = nullptr) {
     __shared__ int red[32];
     int emax = -2000;
-    for (int k = threadIdx.x; k < Kpad; k += blockDim.x)
-        emax = max(emax, fp64_exponent((unsigned long long)__double_as_longlong(at(k))));
+    for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
+        const double x0 = at(k), x1 = at(k + 1);
+        emax = max(emax, max(fp64_exponent((unsigned long long)__double_as_longlong(x0)),
+                             fp64_exponent((unsigned long long)__double_as_longlong(x1))));
+    }
 #pragma unroll
     for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
     const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -891,11 +903,14 @@ __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, 
     emax = -2000;
     for (int w = 0; w < nw; ++w) emax = max(emax, red[w]);
     if (exps && threadIdx.x == 0) exps[dest] = (int16_t)(emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0));
-    const int KB = Kpad / BKB, e0 = exps ? 0 : emax;
-    for (int k = threadIdx.x; k < Kpad; k += blockDim.x) {
-        const int kb = k / BKB, kk = k % BKB;
-        digits(at(k), emax, S, first, step, [&](int i, float d) {
-            out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] = __float2bfloat16_rn(ldexpf(d, e0 - first - step * i));
+    const int64_t plane = (int64_t)(Kpad / BKB) * R * BKB;
+    const int e0 = exps ? 0 : emax;
+    for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
+        uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(k / BKB) * R + dest) * BKB + k % BKB);
+        uint32_t lo[MAXS + 1];
+        digits(at(k), emax, S, first, step, [&](int i, float d) { lo[i] = slice_bits(d, e0 - first - step * i); });
+        digits(at(k + 1), emax, S, first, step, [&](int i, float d) {
+            o[i * (plane / 2)] = lo[i] | slice_bits(d, e0 - first - step * i) << 16;
         });
     }
 }
@@ -932,7 +947,7 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
         const int kb = k / BKB, kk = k % BKB;
         digits(k != skip_col ? x[k] : 0.0, emax, S, kXFirst, kXStep, [&](int i, float d) {
             out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] =
-                __float2bfloat16_rn(ldexpf(d, e0 - kXFirst - kXStep * i));
+                __ushort_as_bfloat16((unsigned short)slice_bits(d, e0 - kXFirst - kXStep * i));
         });
     }
 }
