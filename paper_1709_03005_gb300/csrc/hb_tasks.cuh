@@ -215,7 +215,7 @@ struct C4TTask {        // class 4 of one target group on the tensor cores
     int jpad;
     const int64_t *term_ptr;
     const int2 *terms;
-    int n_l2, n_jt, j0, cf, cn, ns;   // n_jt tiles of 128 orbitals from j0 (a multiple of 8)
+    int n_l2, n_jt, j0, tw, cf, cn, ns;   // n_jt tiles of tw orbitals from j0 (multiples of 8)
     const void *cs;                   // CI slices [S][c_rows][64] (bf16)
     int64_t c_rows;
     int64_t col_off, ld;
@@ -224,7 +224,7 @@ struct C4TTask {        // class 4 of one target group on the tensor cores
 
 struct C4Item {         // one work item of the tensor-core class-4 kernel
     int64_t t0;               // its first term
-    int ti, l, jt, nkb;       // task, L2 row, orbital tile, K blocks of 32 terms
+    int ti, l, jt, nkb;       // task, L2 row, orbital tile, K blocks of 16 terms
 };
 
 struct L2Task {         // classes 2 and 8 without the staged columns (no couplings, or an asymmetric list)

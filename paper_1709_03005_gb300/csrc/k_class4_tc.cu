@@ -20,15 +20,22 @@
 // sized once per plan and written every build from that build's pairs.
 //
 // Kernel (persistent, one CTA per SM, 13 warps):
-//   warp 0     MMA issuer (one thread) and TMEM owner (512 columns: two
-//              buffers of 4 accumulators x 64 states, so one work item's
-//              epilogue overlaps the next item's MMAs)
-//   warps 1-4  producers: cp.async gathers of 32 terms x (128 j + 64 n) per
-//              slice into 128-byte-swizzled MN-major tiles, 3 stages
+//   warp 0     MMA issuer and TMEM owner (512 columns: two buffers of 4
+//              accumulators x 64 states, taken by one chunk after the other, so
+//              a chunk's epilogue overlaps the next chunk's MMAs)
+//   warps 1-4  producers: cp.async gathers of 16 terms x (128 j + 64 n) per
+//              slice into 128-byte-swizzled MN-major tiles, 6 stages
 //   warps 5-12 epilogue: TMEM -> double-float (TwoSum for s <= 2) -> FP64
-// A work item is (L2 row, tile of 128 continuum orbitals); the tile starts on
-// a multiple of 8 orbitals so every 16-byte copy is aligned.  Every wait is
-// bounded; on a timeout the kernel records an error and leaves.
+// A work item is (L2 row, tile of at most 128 continuum orbitals); the tile
+// starts on a multiple of 8 orbitals so every 16-byte copy is aligned, and the
+// tiles of a row are of one width: 400 orbitals as 4 x 104 give every CTA the
+// same work, as 128 + 128 + 128 + 16 a quarter of the CTAs had little of it.
+// Every wait is bounded; on a timeout the kernel records an error and leaves.
+//
+// The slices of the 64 states lie side by side, so one MMA multiplies integral
+// slice i with the CI slices 0 .. 3 - i (N up to 256) into the neighbouring
+// accumulators s = i ..: 15 MMAs a K block for six slices instead of 21, and
+// the 128 orbitals of a slice are read from shared memory 15 times.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -52,7 +59,7 @@ struct C4TC {
         bool on = false;
         __nv_bfloat16 *cs = nullptr;            // [S][2 ndet + 1][64]
         int64_t c_rows = 0;
-        int64_t *term_ptr = nullptr;            // [n_l2 + 1], rows padded to multiples of 32 terms
+        int64_t *term_ptr = nullptr;            // [n_l2 + 1], rows padded to multiples of TKB terms
         std::vector<int64_t> term_ptr_host;
         int2 *terms = nullptr;                  // (x row, C row)
         int64_t n_terms = 0;
@@ -64,13 +71,13 @@ namespace {
 
 using namespace hb::tc;
 
-constexpr int TKB = 32;          // terms per K block
-constexpr int TBM = 128;         // continuum orbitals per tile (TMEM lanes)
+constexpr int TKB = 16;          // terms per K block (the K of one MMA)
+constexpr int TBM = 128;         // most continuum orbitals per tile (TMEM lanes)
 constexpr int TNP = 64;          // states per tile (N of the MMA)
-constexpr int TSTAGES = 3;
-constexpr int TCHUNK_KB = 8;     // K blocks per exact accumulation chunk (256 terms)
-constexpr int T_A_SLICE = 2 * (TKB / 8) * 1024;       // 8 KB: two 64-orbital atoms
-constexpr int T_B_SLICE = (TKB / 8) * 1024;           // 4 KB: one 64-state atom
+constexpr int TSTAGES = 6, TAHEAD = 3;   // stages; copies of TAHEAD + 1 of them in flight per producer thread
+constexpr int TCHUNK_KB = 16;    // K blocks per exact accumulation chunk (256 terms)
+constexpr int T_A_SLICE = 2 * (TKB / 8) * 1024;       // 4 KB: two 64-orbital atoms
+constexpr int T_B_SLICE = (TKB / 8) * 1024;           // 2 KB: one 64-state atom
 constexpr int T_PROD_WARPS = 4, T_EPI_WARPS = 8;
 constexpr int T_THREADS = 32 * (1 + T_PROD_WARPS + T_EPI_WARPS);
 constexpr int T_PROD_THREADS = 32 * T_PROD_WARPS, T_EPI_THREADS = 32 * T_EPI_WARPS;
@@ -291,13 +298,12 @@ __global__ void term_fill_kernel(const C4FTask *__restrict__ tasks, const int64_
 }
 
 // ------------------------------------------------------------- the kernel
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // 128-byte-swizzled MN-major descriptor: atoms of 64 MN elements x 8 K rows
@@ -385,69 +391,71 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
 
     if (warp == 0) {
         // ---------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc_bf16(TBM, TNP) | (1u << 15) | (1u << 16);   // both operands MN-major
-            const uint32_t sbase = smem_u32(base);
-            bool ok = true;
-            int G = 0, it = 0;
-            int cnt[2] = {0, 0};                // accumulator hand-overs per buffer
-            C4Item nx = load_item(items, n_items, blockIdx.x);
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
-                const C4Item cur = nx;
-                nx = load_item(items, n_items, item + gridDim.x);   // next record in flight
-                const int nkb = cur.nkb;
-                const int buf = it & 1;
-                for (int kb0 = 0; kb0 < nkb && ok; kb0 += TCHUNK_KB) {
-                    if (cnt[buf] > 0) ok = mbar_wait(&acc_empty[buf], (cnt[buf] - 1) & 1, err, 21);
+        const uint32_t idesc = instr_desc_bf16(TBM, 0) | (1u << 15) | (1u << 16);   // both operands MN-major; N added below
+        const uint32_t sbase = smem_u32(base), leader = elect_lane();
+        bool ok = true;
+        int q = 0, chunk = 0;
+        uint32_t par = 0;
+        C4Item nx = load_item(items, n_items, blockIdx.x);
+        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            const int nkb = nx.nkb;
+            nx = load_item(items, n_items, item + gridDim.x);   // next record in flight
+            for (int kb0 = 0; kb0 < nkb && ok; kb0 += TCHUNK_KB, ++chunk) {
+                const int buf = chunk & 1;
+                if (chunk > 1) ok = mbar_wait_warp(&acc_empty[buf], ((chunk >> 1) - 1) & 1, err, 21);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t acc0 = tmem + buf * 256;
+                const int kb1 = min(nkb, kb0 + TCHUNK_KB);
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    ok = mbar_wait_warp(&full_bar[q], par, err, 22);
                     if (!ok) break;
                     tc_fence_after();
-                    uint32_t fresh = 0xFu;
-                    const int kb1 = min(nkb, kb0 + TCHUNK_KB);
-                    for (int kb = kb0; kb < kb1 && ok; ++kb, ++G) {
-                        const int q = G % TSTAGES;
-                        ok = mbar_wait(&full_bar[q], (G / TSTAGES) & 1, err, 22);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t sa = sbase + q * STAGE, sbb = sa + S * T_A_SLICE;
+                    const uint32_t sa = sbase + q * STAGE, sbb = sa + S * T_A_SLICE;
+                    constexpr int n_acc = S < 4 ? S : 4;
 #pragma unroll
-                        for (int ks = 0; ks < TKB / 16; ++ks) {
+                    for (int i = 0; i < S; ++i) {
+                        const uint64_t ad = desc_mn(sa + i * T_A_SLICE, T_A_SLICE / 2, 1024);
+                        // CI slices 0 .. nm - 1 into accumulators i ..; the first integral slice starts all of them
+                        const int nm = i < n_acc ? n_acc - i : 0;
+                        if (nm > 0)
+                            mma_bf16_elect(acc0 + i * TNP, ad, desc_mn(sbb, T_B_SLICE, 1024),
+                                           idesc | ((uint32_t)(nm * TNP >> 3) << 17), i > 0 || kb > kb0 ? 1u : 0u, leader);
 #pragma unroll
-                            for (int i = 0; i < S; ++i) {
-#pragma unroll
-                                for (int l2 = 0; l2 < S; ++l2) {
-                                    if (i + l2 >= S) continue;
-                                    const int s = i + l2 < 3 ? i + l2 : 3;
-                                    const uint64_t ad = desc_mn(sa + i * T_A_SLICE + ks * 2048, T_A_SLICE / 2, 1024);
-                                    const uint64_t bd = desc_mn(sbb + l2 * T_B_SLICE + ks * 2048, T_A_SLICE / 2, 1024);
-                                    const uint32_t acc = (fresh >> s) & 1u ? 0u : 1u;
-                                    mma_bf16(tmem + buf * 256 + s * TNP, ad, bd, idesc, acc);
-                                    fresh &= ~(1u << s);
-                                }
-                            }
-                        }
-                        mma_commit(&empty_bar[q]);          // the stage is free once these MMAs complete
+                        for (int l2 = nm; l2 + i < S; ++l2)      // the rest into the last one
+                            mma_bf16_elect(acc0 + 3 * TNP, ad, desc_mn(sbb + l2 * T_B_SLICE, T_B_SLICE, 1024),
+                                           idesc | ((uint32_t)(TNP >> 3) << 17), 1u, leader);
                     }
-                    if (ok) mma_commit(&acc_full[buf]);
-                    ++cnt[buf];
+                    mma_commit_elect(&empty_bar[q], leader);          // the stage is free once these MMAs complete
+                    if (++q == TSTAGES) { q = 0; par ^= 1; }
                 }
+                if (ok) mma_commit_elect(&acc_full[buf], leader);
             }
-            mma_commit(final_bar);
-            mbar_wait(final_bar, 0, err, 23);
         }
+        mma_commit_elect(final_bar, leader);
+        mbar_wait_warp(final_bar, 0, err, 23);
     } else if (warp <= T_PROD_WARPS) {
         // ----------------------------------------------------------- producers
         // Thread pt copies, in every slice, the 16-byte chunks (tt, ch) with
-        // tt * 16 + ch = pt + 128 u (A, u < 4) and tt * 8 + ch = pt + 128 u
-        // (B, u < 2): six terms per stage, read one stage ahead.
+        // tt * 16 + ch = pt + 128 u (A, u < 2) and tt * 8 + ch = pt (B): three
+        // terms per stage, read one stage ahead, the item records two items.
         const int pt = threadIdx.x - 32;          // 0 .. T_PROD_THREADS-1
         constexpr int NA = TKB * 16 / T_PROD_THREADS, NB = TKB * 8 / T_PROD_THREADS;
         const uint32_t sbase = smem_u32(base);
         bool ok = true;
-        int G = 0;
+        int G = 0, q = 0, qf = 0;                 // stages issued; slots of the next one and of the next to publish
+        uint32_t par = 1;
         // the K blocks of this CTA in order: (item record, block) with the next one's terms in flight
         int item = blockIdx.x, kb = 0;
-        C4Item cur = load_item(items, n_items, item);
-        while (item < n_items && cur.nkb == 0) { item += gridDim.x; cur = load_item(items, n_items, item); }
+        C4Item cur = load_item(items, n_items, item), ahead = load_item(items, n_items, item + gridDim.x);
+        auto advance = [&](int &it, C4Item &r) {
+            do {
+                it += gridDim.x;
+                r = ahead;
+                ahead = load_item(items, n_items, it + gridDim.x);
+            } while (it < n_items && r.nkb == 0);
+        };
+        if (item < n_items && cur.nkb == 0) advance(item, cur);
         int2 ta[NA], tb[NB];
         auto load_terms = [&](const C4Item &it, int k, int2 (&xa)[NA], int2 (&xb)[NB]) {
             const int2 *terms = tasks[it.ti].terms + it.t0 + (int64_t)k * TKB;
@@ -456,6 +464,12 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
 #pragma unroll
             for (int u = 0; u < NB; ++u) xb[u] = __ldg(terms + (pt + T_PROD_THREADS * u) / 8);
         };
+        auto publish = [&] {
+            // the copies of this thread for that stage have landed: show them to the tensor cores
+            fence_async_smem();
+            mbar_arrive(&full_bar[qf]);
+            if (++qf == TSTAGES) qf = 0;
+        };
         if (item < n_items) load_terms(cur, 0, ta, tb);
         while (item < n_items && ok) {
             // the next K block of this CTA (possibly of a later item) and its terms
@@ -463,21 +477,17 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             C4Item nxt = cur;
             if (nkb >= cur.nkb) {
                 nkb = 0;
-                do {
-                    nitem += gridDim.x;
-                    nxt = load_item(items, n_items, nitem);
-                } while (nitem < n_items && nxt.nkb == 0);
+                advance(nitem, nxt);
             }
             int2 na[NA], nb[NB];
             if (nitem < n_items) load_terms(nxt, nkb, na, nb);
             const C4TTask &T = tasks[cur.ti];
-            const int j0 = T.j0 + cur.jt * TBM;
+            const int tw = T.tw, j0 = T.j0 + cur.jt * tw;
             const __nv_bfloat16 *cs = (const __nv_bfloat16 *)T.cs;
             const __nv_bfloat16 *xs = (const __nv_bfloat16 *)T.xs;
             const int64_t c_rows = T.c_rows, x_rows = T.x_rows;
             const int jpad = T.jpad;
-            const int q = G % TSTAGES;
-            if (G >= TSTAGES) ok = mbar_wait(&empty_bar[q], ((G / TSTAGES) - 1) & 1, err, 24);
+            if (G >= TSTAGES) ok = mbar_wait(&empty_bar[q], par, err, 24);
             if (!ok) break;
             const uint32_t sa = sbase + q * STAGE, sbb = sa + S * T_A_SLICE;
 #pragma unroll
@@ -489,27 +499,25 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
                     const int j = j0 + ch * 8;
                     const uint32_t off = (uint32_t)(i * T_A_SLICE + (ch >> 3) * (T_A_SLICE / 2) + (tt >> 3) * 1024 +
                                                     (tt & 7) * 128 + (((ch & 7) ^ (tt & 7)) << 4));
-                    const bool in = j + 8 <= jpad;
-                    const __nv_bfloat16 *src = xs + ((int64_t)i * x_rows + ta[u].x) * jpad + (in ? j : 0);
-                    cp_async16(sa + off, src, in ? 16u : 0u);
+                    // orbitals beyond the tile: rows of the product that nothing reads
+                    if (ch * 8 < tw && j + 8 <= jpad)
+                        cp_async16(sa + off, xs + ((int64_t)i * x_rows + ta[u].x) * jpad + j);
                 }
 #pragma unroll
                 for (int u = 0; u < NB; ++u) {
                     const int pidx = pt + T_PROD_THREADS * u;
                     const int tt = pidx / 8, ch = pidx % 8;
                     const uint32_t off = (uint32_t)(i * T_B_SLICE + (tt >> 3) * 1024 + (tt & 7) * 128 + ((ch ^ (tt & 7)) << 4));
-                    cp_async16(sbb + off, cs + ((int64_t)i * c_rows + tb[u].y) * TNP + ch * 8, 16u);
+                    cp_async16(sbb + off, cs + ((int64_t)i * c_rows + tb[u].y) * TNP + ch * 8);
                 }
             }
             cp_async_commit();
-            if (G > 1) {
-                // the copies of two stages back have landed: publish them to the
-                // tensor cores (three stages of copies in flight per thread)
-                cp_async_wait2();
-                fence_async_smem();
-                mbar_arrive(&full_bar[(G - 2) % TSTAGES]);
+            if (G >= TAHEAD) {
+                cp_async_wait<TAHEAD>();      // the stage TAHEAD back
+                publish();
             }
             ++G;
+            if (++q == TSTAGES) { q = 0; par ^= 1; }
             item = nitem;
             kb = nkb;
             cur = nxt;
@@ -518,17 +526,9 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
 #pragma unroll
             for (int u = 0; u < NB; ++u) tb[u] = nb[u];
         }
-        // the last two stages
-        if (ok && G > 1) {
-            cp_async_wait1();
-            fence_async_smem();
-            mbar_arrive(&full_bar[(G - 2) % TSTAGES]);
-        }
-        cp_async_wait0();
-        if (ok && G > 0) {
-            fence_async_smem();
-            mbar_arrive(&full_bar[(G - 1) % TSTAGES]);
-        }
+        cp_async_wait<0>();
+        if (ok)
+            for (int n = min(G, TAHEAD); n > 0; --n) publish();      // the last stages
     } else {
         // ------------------------------------------------------------ epilogue
         const int ew = warp - 1 - T_PROD_WARPS;   // 0 .. 7
@@ -536,35 +536,33 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
         const int col0 = (ew >> 2) * T_EPI_COLS;
         const int row = qd * 32 + lane;
         bool ok = true;
-        int it = 0;
-        int cnt[2] = {0, 0};
+        int chunk = 0;
         C4Item nx = load_item(items, n_items, blockIdx.x);
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
+        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
             const C4Item cur = nx;
             nx = load_item(items, n_items, item + gridDim.x);
             const C4TTask &T = tasks[cur.ti];
             const int nkb = cur.nkb;
-            const int buf = it & 1;
             float hi[T_EPI_COLS], lo[T_EPI_COLS];
 #pragma unroll
             for (int c = 0; c < T_EPI_COLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
-            for (int kb0 = 0; kb0 < nkb && ok; kb0 += TCHUNK_KB) {
-                ok = mbar_wait(&acc_full[buf], cnt[buf] & 1, err, 25);
+            for (int kb0 = 0; kb0 < nkb && ok; kb0 += TCHUNK_KB, ++chunk) {
+                const int buf = chunk & 1;
+                ok = mbar_wait(&acc_full[buf], (chunk >> 1) & 1, err, 25);
                 if (!ok) break;
                 tc_fence_after();
                 drain_c4<S>(tmem + ((uint32_t)(qd * 32) << 16) + buf * 256 + col0, hi, lo);
                 tc_fence_before();
                 mbar_arrive(&acc_empty[buf]);
-                ++cnt[buf];
             }
             if (!ok) break;
-            const int j = T.j0 + cur.jt * TBM + row;
-            if (j >= T.cf && j < T.cf + T.cn) {
+            const int j = T.j0 + cur.jt * T.tw + row;
+            if (row < T.tw && j >= T.cf && j < T.cf + T.cn) {
                 double *out = T.Hlc + (int64_t)cur.l * T.ld + T.col_off + (j - T.cf);
 #pragma unroll
                 for (int c = 0; c < T_EPI_COLS; ++c) {
                     const int n = col0 + c;
-                    if (n < T.ns) out[(int64_t)n * T.cn] = df_to_double(hi[c], lo[c]);
+                    if (n < T.ns) out[(int64_t)n * T.cn] = df_sum(hi[c], lo[c]);
                 }
             }
         }
@@ -687,8 +685,7 @@ int c4tc_prepare(hb_ctx *ctx, int S, cudaStream_t s) {
         fill_int_kernel<<<1, TNP, 0, s>>>(en, TNP, -2000);
         c_colexp_kernel<<<(Gi.ndet + 255) / 256, TNP, 0, s>>>(ctx->ci + Gi.ci_off, Gi.ndet, Gi.ns, en);
         c_slice_kernel<<<(unsigned)cg.c_rows, TNP, 0, s>>>(ctx->ci + Gi.ci_off, Gi.ndet, Gi.ns, S, en, cg.cs);
-        // the pairs of this build order, then the padded term counts per L2 row
-        k1_fill_pairs(ctx->l2, ctx->n_l2, dg, Gi.ndet, ctx->W, 1, ctx->cont_spin, 2, 0, L.rowptr, L.pairs, s);
+        // the padded term counts per L2 row (hb_init has made the records once)
         cudaMemsetAsync(cg.term_ptr, 0, sizeof(int64_t), s);
         term_count_kernel<<<(ctx->n_l2 + 7) / 8, 256, 0, s>>>(L.pairs, L.rowptr, ctx->n_l2, dg, ctx->W, ctx->n_to,
                                                                ctx->cont_spin, Gi.ndet, cg.term_ptr);
@@ -711,12 +708,20 @@ int c4tc_prepare(hb_ctx *ctx, int S, cudaStream_t s) {
     return HB_OK;
 }
 
+namespace {
+// Tiles of one width (a multiple of 8 orbitals) from a multiple of 8.
+struct C4Tiles { int j0, n, w; };
+C4Tiles c4_tiles(const GroupInfo &g) {
+    const int j0 = g.cf & ~7, span = g.cf + g.cn - j0, n = (span + TBM - 1) / TBM;
+    return {j0, n, ((span + n - 1) / n + 7) / 8 * 8};
+}
+}  // namespace
+
 void c4tc_items(const hb_ctx *ctx, int g, int ti, std::vector<C4Item> *items) {
     const C4TC &c = *(const C4TC *)ctx->c4tc;
     const C4TC::Group &cg = c.g[g];
     const GroupInfo &Gi = ctx->groups[g];
-    const int j0 = Gi.cf & ~7;
-    const int n_jt = (Gi.cf + Gi.cn - j0 + TBM - 1) / TBM;
+    const int n_jt = c4_tiles(Gi).n;
     for (int l = 0; l < ctx->n_l2; ++l) {
         const int64_t t0 = cg.term_ptr_host[l];
         const int nkb = (int)((cg.term_ptr_host[l + 1] - t0) / TKB);
@@ -733,11 +738,10 @@ void c4tc_tasks(const hb_ctx *ctx, int g, double *Hlc, C4FTask *fill, int64_t *f
     *fill = C4FTask{L.pairs, L.rowptr, ctx->n_l2, ctx->dets + Gi.det_off, ctx->W, ctx->n_to, ctx->cont_spin,
                     Gi.ndet, c.x_h0, c.x_zero, cg.term_ptr, cg.terms};
     *fill_blocks = (ctx->n_l2 + 7) / 8;
-    const int j0 = Gi.cf & ~7;
-    const int n_jt = (Gi.cf + Gi.cn - j0 + TBM - 1) / TBM;
-    *tc = C4TTask{c.xs, c.x_rows, c.jpad, cg.term_ptr, cg.terms, ctx->n_l2, n_jt, j0, Gi.cf, Gi.cn, Gi.ns, cg.cs,
+    const C4Tiles t = c4_tiles(Gi);
+    *tc = C4TTask{c.xs, c.x_rows, c.jpad, cg.term_ptr, cg.terms, ctx->n_l2, t.n, t.j0, t.w, Gi.cf, Gi.cn, Gi.ns, cg.cs,
                   cg.c_rows, Gi.row_off, ctx->Dc, Hlc};
-    *tc_items = (int64_t)ctx->n_l2 * n_jt;
+    *tc_items = (int64_t)ctx->n_l2 * t.n;
 }
 
 int g_c4fill(const Grouped<C4FTask> &g, cudaStream_t s) {
