@@ -19,18 +19,24 @@
 // the MMAs sum them exactly in FP32 over chunks of at most 256 terms.  The term lists (integral row, signed CI row) per L2 row are
 // sized once per plan and written every build from that build's pairs.
 //
-// Kernel (persistent, one CTA per SM, 13 warps):
+// Kernel (persistent, one CTA per SM, 12 warps):
 //   warp 0     MMA issuer and TMEM owner (512 columns: two buffers of 4
 //              accumulators x 64 states, taken by one chunk after the other, so
 //              a chunk's epilogue overlaps the next chunk's MMAs)
-//   warps 1-4  producers: cp.async gathers of 16 terms x (128 j + 64 n) per
-//              slice into 128-byte-swizzled MN-major tiles, 6 stages
-//   warps 5-12 epilogue: TMEM -> double-float (TwoSum for s <= 2) -> FP64
+//   warps 1-3  producers: cp.async gathers of 16 terms x (128 j + 64 n) per
+//              slice into 128-byte-swizzled MN-major tiles, 6 stages; each
+//              takes every third stage, so one looks up its terms while the
+//              others copy (four warps on every stage together: 5.7 for 5.1 ms)
+//   warps 4-11 epilogue: TMEM -> double-float (TwoSum for s <= 2) -> FP64
 // A work item is (L2 row, tile of at most 128 continuum orbitals); the tile
 // starts on a multiple of 8 orbitals so every 16-byte copy is aligned, and the
 // tiles of a row are of one width: 400 orbitals as 4 x 104 give every CTA the
 // same work, as 128 + 128 + 128 + 16 a quarter of the CTAs had little of it.
 // Every wait is bounded; on a timeout the kernel records an error and leaves.
+// 120000 items of 40 target and 400 continuum orbitals and 50 states (22 GB
+// gathered, 4.8 GB written) take 5.1 ms, 12.0 before the points above and below:
+// a warp's single lane issued an MMA in 98 cycles.  Now the epilogue's FP64
+// additions (4.7 ms without them) and the MMAs (990 cycles a K block) share it.
 //
 // The slices of the 64 states lie side by side, so one MMA multiplies integral
 // slice i with the CI slices 0 .. 3 - i (N up to 256) into the neighbouring
@@ -74,12 +80,12 @@ using namespace hb::tc;
 constexpr int TKB = 16;          // terms per K block (the K of one MMA)
 constexpr int TBM = 128;         // most continuum orbitals per tile (TMEM lanes)
 constexpr int TNP = 64;          // states per tile (N of the MMA)
-constexpr int TSTAGES = 6, TAHEAD = 3;   // stages; copies of TAHEAD + 1 of them in flight per producer thread
+constexpr int TSTAGES = 6, TAHEAD = 1;   // stages; copies of TAHEAD + 1 of them in flight per producer thread
 constexpr int TCHUNK_KB = 16;    // K blocks per exact accumulation chunk (256 terms)
 constexpr int T_A_SLICE = 2 * (TKB / 8) * 1024;       // 4 KB: two 64-orbital atoms
 constexpr int T_B_SLICE = (TKB / 8) * 1024;           // 2 KB: one 64-state atom
-constexpr int T_PROD_WARPS = 4, T_EPI_WARPS = 8;
-constexpr int T_THREADS = 32 * (1 + T_PROD_WARPS + T_EPI_WARPS);
+constexpr int T_PROD_GROUPS = 3, T_PROD_WARPS = 1, T_EPI_WARPS = 8;   // producer warps of a group
+constexpr int T_THREADS = 32 * (1 + T_PROD_GROUPS * T_PROD_WARPS + T_EPI_WARPS);
 constexpr int T_PROD_THREADS = 32 * T_PROD_WARPS, T_EPI_THREADS = 32 * T_EPI_WARPS;
 constexpr int T_EPI_COLS = TNP / 2;                   // columns per epilogue thread
 
@@ -298,8 +304,14 @@ __global__ void term_fill_kernel(const C4FTask *__restrict__ tasks, const int64_
 }
 
 // ------------------------------------------------------------- the kernel
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+// Predicated in the instruction itself: a branch around each copy kept the
+// copies of a stage from being issued together (7.1 for 5.6 ms).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool on) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %2, 0;\n\t"
+        "@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(dst), "l"(src), "r"((uint32_t)on)
+        : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -357,6 +369,8 @@ __device__ __forceinline__ void drain_c4(uint32_t tbase, float (&hi)[T_EPI_COLS]
         }
     }
 }
+
+static_assert(TSTAGES % T_PROD_GROUPS == 0, "a group's stages keep their slots");
 
 template <int S>
 __global__ void __launch_bounds__(T_THREADS, 1)
@@ -434,16 +448,16 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
         }
         mma_commit_elect(final_bar, leader);
         mbar_wait_warp(final_bar, 0, err, 23);
-    } else if (warp <= T_PROD_WARPS) {
+    } else if (warp <= T_PROD_GROUPS * T_PROD_WARPS) {
         // ----------------------------------------------------------- producers
         // Thread pt copies, in every slice, the 16-byte chunks (tt, ch) with
-        // tt * 16 + ch = pt + 128 u (A, u < 2) and tt * 8 + ch = pt (B): three
-        // terms per stage, read one stage ahead, the item records two items.
-        const int pt = threadIdx.x - 32;          // 0 .. T_PROD_THREADS-1
+        // tt * 16 + ch = pt + 32 u (A, u < 8) and tt * 8 + ch = pt + 32 u (B, u
+        // < 4), the terms read one stage ahead, the item records one item.
+        const int grp = (threadIdx.x - 32) / T_PROD_THREADS, pt = (threadIdx.x - 32) % T_PROD_THREADS;
         constexpr int NA = TKB * 16 / T_PROD_THREADS, NB = TKB * 8 / T_PROD_THREADS;
         const uint32_t sbase = smem_u32(base);
         bool ok = true;
-        int G = 0, q = 0, qf = 0;                 // stages issued; slots of the next one and of the next to publish
+        int G = 0, q = grp, qf = grp;             // own stages issued; slots of the next one and of the next to publish
         uint32_t par = 1;
         // the K blocks of this CTA in order: (item record, block) with the next one's terms in flight
         int item = blockIdx.x, kb = 0;
@@ -456,6 +470,13 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             } while (it < n_items && r.nkb == 0);
         };
         if (item < n_items && cur.nkb == 0) advance(item, cur);
+        auto next_block = [&](int &it, int &k, C4Item &r, int n) {
+            for (k += n; it < n_items && k >= r.nkb;) {
+                k -= r.nkb;
+                advance(it, r);
+            }
+        };
+        next_block(item, kb, cur, grp);
         int2 ta[NA], tb[NB];
         auto load_terms = [&](const C4Item &it, int k, int2 (&xa)[NA], int2 (&xb)[NB]) {
             const int2 *terms = tasks[it.ti].terms + it.t0 + (int64_t)k * TKB;
@@ -468,17 +489,15 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             // the copies of this thread for that stage have landed: show them to the tensor cores
             fence_async_smem();
             mbar_arrive(&full_bar[qf]);
-            if (++qf == TSTAGES) qf = 0;
+            qf += T_PROD_GROUPS;
+            if (qf >= TSTAGES) qf -= TSTAGES;
         };
-        if (item < n_items) load_terms(cur, 0, ta, tb);
+        if (item < n_items) load_terms(cur, kb, ta, tb);
         while (item < n_items && ok) {
-            // the next K block of this CTA (possibly of a later item) and its terms
-            int nitem = item, nkb = kb + 1;
+            // this group's next K block (possibly of a later item) and its terms
+            int nitem = item, nkb = kb;
             C4Item nxt = cur;
-            if (nkb >= cur.nkb) {
-                nkb = 0;
-                advance(nitem, nxt);
-            }
+            next_block(nitem, nkb, nxt, T_PROD_GROUPS);
             int2 na[NA], nb[NB];
             if (nitem < n_items) load_terms(nxt, nkb, na, nb);
             const C4TTask &T = tasks[cur.ti];
@@ -487,29 +506,32 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             const __nv_bfloat16 *xs = (const __nv_bfloat16 *)T.xs;
             const int64_t c_rows = T.c_rows, x_rows = T.x_rows;
             const int jpad = T.jpad;
-            if (G >= TSTAGES) ok = mbar_wait(&empty_bar[q], par, err, 24);
+            if (G >= TSTAGES / T_PROD_GROUPS) ok = mbar_wait(&empty_bar[q], par, err, 24);
             if (!ok) break;
             const uint32_t sa = sbase + q * STAGE, sbb = sa + S * T_A_SLICE;
+            // orbitals beyond the tile and states beyond the group's are rows and columns of the product that nothing reads
+            const int64_t xstep = x_rows * jpad, cstep = c_rows * TNP;
+            const int ns = T.ns;
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
+            for (int u = 0; u < NA; ++u) {
+                const int pidx = pt + T_PROD_THREADS * u;
+                const int tt = pidx / 16, ch = pidx % 16;
+                const int j = j0 + ch * 8;
+                const bool on = ch * 8 < tw && j + 8 <= jpad;
+                const uint32_t dst = sa + (uint32_t)((ch >> 3) * (T_A_SLICE / 2) + (tt >> 3) * 1024 + (tt & 7) * 128 +
+                                                     (((ch & 7) ^ (tt & 7)) << 4));
+                const __nv_bfloat16 *src = xs + (int64_t)ta[u].x * jpad + j;
 #pragma unroll
-                for (int u = 0; u < NA; ++u) {
-                    const int pidx = pt + T_PROD_THREADS * u;
-                    const int tt = pidx / 16, ch = pidx % 16;
-                    const int j = j0 + ch * 8;
-                    const uint32_t off = (uint32_t)(i * T_A_SLICE + (ch >> 3) * (T_A_SLICE / 2) + (tt >> 3) * 1024 +
-                                                    (tt & 7) * 128 + (((ch & 7) ^ (tt & 7)) << 4));
-                    // orbitals beyond the tile: rows of the product that nothing reads
-                    if (ch * 8 < tw && j + 8 <= jpad)
-                        cp_async16(sa + off, xs + ((int64_t)i * x_rows + ta[u].x) * jpad + j);
-                }
+                for (int i = 0; i < S; ++i) cp_async16(dst + i * T_A_SLICE, src + i * xstep, on);
+            }
 #pragma unroll
-                for (int u = 0; u < NB; ++u) {
-                    const int pidx = pt + T_PROD_THREADS * u;
-                    const int tt = pidx / 8, ch = pidx % 8;
-                    const uint32_t off = (uint32_t)(i * T_B_SLICE + (tt >> 3) * 1024 + (tt & 7) * 128 + ((ch ^ (tt & 7)) << 4));
-                    cp_async16(sbb + off, cs + ((int64_t)i * c_rows + tb[u].y) * TNP + ch * 8);
-                }
+            for (int u = 0; u < NB; ++u) {
+                const int pidx = pt + T_PROD_THREADS * u;
+                const int tt = pidx / 8, ch = pidx % 8;
+                const uint32_t dst = sbb + (uint32_t)((tt >> 3) * 1024 + (tt & 7) * 128 + ((ch ^ (tt & 7)) << 4));
+                const __nv_bfloat16 *src = cs + (int64_t)tb[u].y * TNP + ch * 8;
+#pragma unroll
+                for (int i = 0; i < S; ++i) cp_async16(dst + i * T_B_SLICE, src + i * cstep, ch * 8 < ns);
             }
             cp_async_commit();
             if (G >= TAHEAD) {
@@ -517,7 +539,8 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
                 publish();
             }
             ++G;
-            if (++q == TSTAGES) { q = 0; par ^= 1; }
+            q += T_PROD_GROUPS;
+            if (q >= TSTAGES) { q -= TSTAGES; par ^= 1; }
             item = nitem;
             kb = nkb;
             cur = nxt;
@@ -531,7 +554,7 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             for (int n = min(G, TAHEAD); n > 0; --n) publish();      // the last stages
     } else {
         // ------------------------------------------------------------ epilogue
-        const int ew = warp - 1 - T_PROD_WARPS;   // 0 .. 7
+        const int ew = warp - 1 - T_PROD_GROUPS * T_PROD_WARPS;   // 0 .. 7
         const int qd = warp & 3;                  // TMEM lane quadrant of this warp
         const int col0 = (ew >> 2) * T_EPI_COLS;
         const int row = qd * 32 + lane;
@@ -722,11 +745,16 @@ void c4tc_items(const hb_ctx *ctx, int g, int ti, std::vector<C4Item> *items) {
     const C4TC::Group &cg = c.g[g];
     const GroupInfo &Gi = ctx->groups[g];
     const int n_jt = c4_tiles(Gi).n;
-    for (int l = 0; l < ctx->n_l2; ++l) {
-        const int64_t t0 = cg.term_ptr_host[l];
-        const int nkb = (int)((cg.term_ptr_host[l + 1] - t0) / TKB);
-        for (int jt = 0; jt < n_jt; ++jt) items->push_back(C4Item{t0, ti, l, jt, nkb});
-    }
+    // tile by tile, so that what the CTAs gather at a time, a tile's columns of the
+    // integral slices, stays in the L2 cache (41 MB of 158 MB for 40 target and
+    // 400 continuum orbitals)
+    items->reserve(items->size() + (size_t)n_jt * ctx->n_l2);
+    for (int jt = 0; jt < n_jt; ++jt)
+        for (int l = 0; l < ctx->n_l2; ++l) {
+            const int64_t t0 = cg.term_ptr_host[l];
+            const int nkb = (int)((cg.term_ptr_host[l + 1] - t0) / TKB);
+            items->push_back(C4Item{t0, ti, l, jt, nkb});
+        }
 }
 
 void c4tc_tasks(const hb_ctx *ctx, int g, double *Hlc, C4FTask *fill, int64_t *fill_blocks, C4TTask *tc,
