@@ -6,6 +6,8 @@
 
 #include <stdint.h>
 
+#include "hb_df.cuh"
+
 namespace hb {
 namespace tc {
 
@@ -182,6 +184,18 @@ __device__ __forceinline__ void tmem_regs_ready(uint32_t (&r)[16]) {
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                    "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
                    "+r"(r[15]));
+}
+
+// 16 loaded columns into double-float sums, two columns at a time: EXACT by
+// TwoSum, otherwise into the low words.
+template <bool EXACT>
+__device__ __forceinline__ void fold16(const uint32_t (&v)[16], f2 *hi, f2 *lo) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const f2 x = f2_pack(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+        if (EXACT) df_add(hi[i], lo[i], x);
+        else lo[i] = f2_add(lo[i], x);
+    }
 }
 
 // Named barrier over the first n threads that reach it with this id.

@@ -181,11 +181,13 @@ __device__ __forceinline__ void prototype_df(const C4Task &T, const hb_pair &r, 
 }
 
 // Block = blockDim.x continuum orbitals (32, 64 or 128) of one L2 row; NS
-// target states per pass.
+// target states per pass, two to an f32x2 instruction.  The CI coefficients lie
+// in shared memory as high and low words, four states to a load.
 template <int W, int NS>
 __global__ void __launch_bounds__(kJ, NS <= 24 ? 6 : 1)
 class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
-    __shared__ float2 cs[kBatch][NS];
+    static_assert(NS % 4 == 0, "coefficients are read four states at a time");
+    __shared__ __align__(16) float ch[kBatch][NS], cl[kBatch][NS];
     __shared__ hb_pair rs[kBatch];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const C4Task &T = tasks[ti];
@@ -199,9 +201,9 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
     const int64_t b = T.row_ptr[l], e = T.row_ptr[l + 1];
     for (int n0 = 0; n0 < ns; n0 += NS) {
         const int nc = min(NS, ns - n0);
-        float ahi[NS], alo[NS];
+        f2 ahi[NS / 2], alo[NS / 2];
 #pragma unroll
-        for (int n = 0; n < NS; ++n) { ahi[n] = 0.0f; alo[n] = 0.0f; }
+        for (int n = 0; n < NS / 2; ++n) { ahi[n] = f2_pack(0.0f, 0.0f); alo[n] = f2_pack(0.0f, 0.0f); }
         for (int64_t p0 = b; p0 < e; p0 += kBatch) {
             const int cnt = (int)(e - p0 < kBatch ? e - p0 : kBatch);
             __syncthreads();
@@ -209,38 +211,38 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
             __syncthreads();
             for (int t = threadIdx.x; t < cnt * NS; t += JT) {
                 const int i = t / NS, n = t % NS;
-                cs[i][n] = n < nc ? __ldg(T.C_df + (int64_t)rs[i].col * ns + n0 + n) : make_float2(0.0f, 0.0f);
+                const float2 c = n < nc ? __ldg(T.C_df + (int64_t)rs[i].col * ns + n0 + n) : make_float2(0.0f, 0.0f);
+                ch[i][n] = c.x;
+                cl[i][n] = c.y;
             }
             __syncthreads();
             for (int i = 0; i < cnt; ++i) {
                 const hb_pair r = rs[i];
                 float yh, yl;
                 prototype_df<W>(T, r, T.dets + (int64_t)r.col * 2 * W, j, yh, yl);
+                const f2 y = f2_pack(yh, yh), ny = f2_pack(-yh, -yh), yl2 = f2_pack(yl, yl);
 #pragma unroll
-                for (int n = 0; n < NS; ++n) {
-                    const float2 c = cs[i][n];
-                    const float ph = c.x * yh;
-                    const float pe = fmaf(c.x, yh, -ph);              // exact error of ph
-                    const float pl = fmaf(c.x, yl, fmaf(c.y, yh, pe));
-                    float sum, err;
-                    df_two_sum(ahi[n], ph, sum, err);
-                    ahi[n] = sum;
-                    alo[n] = __fadd_rn(alo[n], __fadd_rn(err, pl));
+                for (int n = 0; n < NS; n += 4) {
+                    const ulonglong2 h4 = *reinterpret_cast<const ulonglong2 *>(&ch[i][n]);
+                    const ulonglong2 l4 = *reinterpret_cast<const ulonglong2 *>(&cl[i][n]);
+                    df_fma(ahi[n / 2], alo[n / 2], y, ny, yl2, f2{h4.x}, f2{l4.x});
+                    df_fma(ahi[n / 2 + 1], alo[n / 2 + 1], y, ny, yl2, f2{h4.y}, f2{l4.y});
                 }
             }
             // renormalise once per batch so the low words stay small
 #pragma unroll
-            for (int n = 0; n < NS; ++n) {
-                const float s = __fadd_rn(ahi[n], alo[n]);
-                alo[n] = __fsub_rn(alo[n], __fsub_rn(s, ahi[n]));
-                ahi[n] = s;
-            }
+            for (int n = 0; n < NS / 2; ++n) df_norm(ahi[n], alo[n]);
         }
         if (jv) {
             double *out = T.Hlc + (int64_t)l * T.ld + T.col_off + jl;
 #pragma unroll
-            for (int n = 0; n < NS; ++n)
-                if (n < nc) out[(int64_t)(n0 + n) * cn] = df_to_double(ahi[n], alo[n]);
+            for (int n = 0; n < NS; n += 2) {
+                float h0, h1, l0, l1;
+                f2_unpack(ahi[n / 2], h0, h1);
+                f2_unpack(alo[n / 2], l0, l1);
+                if (n < nc) out[(int64_t)(n0 + n) * cn] = df_to_double(h0, l0);
+                if (n + 1 < nc) out[(int64_t)(n0 + n + 1) * cn] = df_to_double(h1, l1);
+            }
         }
     }
 }

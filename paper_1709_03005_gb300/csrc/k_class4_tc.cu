@@ -92,15 +92,6 @@ constexpr int T_EPI_COLS = TNP / 2;                   // columns per epilogue th
 template <int S>
 constexpr int t_stage_bytes() { return S * (T_A_SLICE + T_B_SLICE); }
 
-// double-float accumulation: (hi, lo) += x, exact TwoSum on the high part
-__device__ __forceinline__ void df_add(float &hi, float &lo, float x) {
-    const float s = __fadd_rn(hi, x);
-    const float bp = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
-
 // ------------------------------------------------------------ digit helper
 // x = F 2^(e - 8S) with F = round(x 2^(8S - e)) from the FP64 bit pattern
 // (|x| < 2^e, so |F| < 2^(8S), at most 2^62 for S <= 6 ... 7); the balanced
@@ -340,7 +331,7 @@ __device__ __forceinline__ C4Item load_item(const C4Item *__restrict__ items, in
 // Fold one chunk of the four accumulators (T_EPI_COLS columns at this thread's
 // lane; accumulator s at column offset s * TNP) into the double-float sums.
 template <int S>
-__device__ __forceinline__ void drain_c4(uint32_t tbase, float (&hi)[T_EPI_COLS], float (&lo)[T_EPI_COLS]) {
+__device__ __forceinline__ void drain_c4(uint32_t tbase, f2 (&hi)[T_EPI_COLS / 2], f2 (&lo)[T_EPI_COLS / 2]) {
     constexpr int n_acc = S < 4 ? S : 4;
 #pragma unroll
     for (int c0 = 0; c0 < T_EPI_COLS; c0 += 16) {
@@ -349,22 +340,20 @@ __device__ __forceinline__ void drain_c4(uint32_t tbase, float (&hi)[T_EPI_COLS]
         if (n_acc > 1) tmem_ld16_async(tbase + TNP + c0, w);
         tmem_wait_ld();
         tmem_regs_ready(v);
-        if (n_acc > 1) tmem_regs_ready(w);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
-            if (n_acc > 1) df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(w[i]));
+        fold16<true>(v, &hi[c0 / 2], &lo[c0 / 2]);
+        if (n_acc > 1) {
+            tmem_regs_ready(w);
+            fold16<true>(w, &hi[c0 / 2], &lo[c0 / 2]);
         }
         if (n_acc > 2) {
             tmem_ld16_async(tbase + 2 * TNP + c0, v);
             if (n_acc > 3) tmem_ld16_async(tbase + 3 * TNP + c0, w);
             tmem_wait_ld();
             tmem_regs_ready(v);
-            if (n_acc > 3) tmem_regs_ready(w);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
-                if (n_acc > 3) lo[c0 + i] = __fadd_rn(lo[c0 + i], __uint_as_float(w[i]));
+            fold16<true>(v, &hi[c0 / 2], &lo[c0 / 2]);
+            if (n_acc > 3) {
+                tmem_regs_ready(w);
+                fold16<false>(w, &hi[c0 / 2], &lo[c0 / 2]);
             }
         }
     }
@@ -566,9 +555,9 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             nx = load_item(items, n_items, item + gridDim.x);
             const C4TTask &T = tasks[cur.ti];
             const int nkb = cur.nkb;
-            float hi[T_EPI_COLS], lo[T_EPI_COLS];
+            f2 hi[T_EPI_COLS / 2], lo[T_EPI_COLS / 2];
 #pragma unroll
-            for (int c = 0; c < T_EPI_COLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
+            for (int c = 0; c < T_EPI_COLS / 2; ++c) { hi[c] = f2_pack(0.0f, 0.0f); lo[c] = f2_pack(0.0f, 0.0f); }
             for (int kb0 = 0; kb0 < nkb && ok; kb0 += TCHUNK_KB, ++chunk) {
                 const int buf = chunk & 1;
                 ok = mbar_wait(&acc_full[buf], (chunk >> 1) & 1, err, 25);
@@ -583,9 +572,13 @@ class4_tc_kernel(const C4TTask *__restrict__ tasks, const C4Item *__restrict__ i
             if (row < T.tw && j >= T.cf && j < T.cf + T.cn) {
                 double *out = T.Hlc + (int64_t)cur.l * T.ld + T.col_off + (j - T.cf);
 #pragma unroll
-                for (int c = 0; c < T_EPI_COLS; ++c) {
+                for (int c = 0; c < T_EPI_COLS; c += 2) {
                     const int n = col0 + c;
-                    if (n < T.ns) out[(int64_t)n * T.cn] = df_sum(hi[c], lo[c]);
+                    float h0, h1, l0, l1;
+                    f2_unpack(hi[c / 2], h0, h1);
+                    f2_unpack(lo[c / 2], l0, l1);
+                    if (n < T.ns) out[(int64_t)n * T.cn] = df_sum(h0, l0);
+                    if (n + 1 < T.ns) out[(int64_t)(n + 1) * T.cn] = df_sum(h1, l1);
                 }
             }
         }

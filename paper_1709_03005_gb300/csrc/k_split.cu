@@ -225,15 +225,6 @@ __host__ __device__ constexpr int slot_of(int P, int t) {
     return 0;
 }
 
-// double-float accumulation: (hi, lo) += x, exact TwoSum on the high part
-__device__ __forceinline__ void df_add(float &hi, float &lo, float x) {
-    const float s = __fadd_rn(hi, x);
-    const float bp = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
-
 // One K block of MMAs, fully unrolled for slot parity P: for each arriving
 // slice t, the pairs (i, l) with max(i, l) = t and i + l < S, then the commits
 // that free the slots read for the last time.
@@ -339,8 +330,9 @@ __device__ __forceinline__ bool mma_stage(MmaState &m, int slot0, uint32_t par) 
 // TMEM lane): an exact one by TwoSum (2^-18 of the result for s = 2 still needs
 // it to keep the low word below an ulp of the high one), the inexact one
 // (2^-27) into the low word.
-template <bool EXACT, int NC>
-__device__ __forceinline__ void drain_df(uint32_t taddr, float (&hi)[NC], float (&lo)[NC]) {
+template <bool EXACT, int NP>
+__device__ __forceinline__ void drain_df(uint32_t taddr, f2 (&hi)[NP], f2 (&lo)[NP]) {
+    constexpr int NC = 2 * NP;
     static_assert(NC % 16 == 0, "columns are loaded 16 at a time");
 #pragma unroll
     for (int c0 = 0; c0 < NC; c0 += 32) {
@@ -350,16 +342,8 @@ __device__ __forceinline__ void drain_df(uint32_t taddr, float (&hi)[NC], float 
         tmem_wait_ld();
         tmem_regs_ready(v);
         if (c0 + 16 < NC) tmem_regs_ready(w);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (EXACT) df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
-            else lo[c0 + i] = __fadd_rn(lo[c0 + i], __uint_as_float(v[i]));
-            if (c0 + 16 < NC) {
-                constexpr int o = 16;
-                if (EXACT) df_add(hi[(c0 + o + i) % NC], lo[(c0 + o + i) % NC], __uint_as_float(w[i]));
-                else lo[(c0 + o + i) % NC] = __fadd_rn(lo[(c0 + o + i) % NC], __uint_as_float(w[i]));
-            }
-        }
+        fold16<EXACT>(v, &hi[c0 / 2], &lo[c0 / 2]);
+        if (c0 + 16 < NC) fold16<EXACT>(w, &hi[(c0 + 16) % NC / 2], &lo[(c0 + 16) % NC / 2]);
     }
 }
 
@@ -402,8 +386,9 @@ __device__ __forceinline__ double int_words_to_double(long long a, long long b, 
 // accumulator s at column offset s * stride) into the double-float sums:
 // s = 0, 1, 2 by TwoSum (2^-14 of the result for s = 2 still needs it to keep
 // the low word below an ulp of the high one), s >= 3 (2^-21) into the low word.
-template <int S, int NC>
-__device__ __forceinline__ void drain_chunk(uint32_t tbase, int stride, float (&hi)[NC], float (&lo)[NC]) {
+template <int S, int NP>
+__device__ __forceinline__ void drain_chunk(uint32_t tbase, int stride, f2 (&hi)[NP], f2 (&lo)[NP]) {
+    constexpr int NC = 2 * NP;
     constexpr int n_acc = S < 4 ? S : 4;       // accumulators written by the MMAs
     static_assert(NC % 16 == 0, "columns are loaded 16 at a time");
 #pragma unroll
@@ -414,22 +399,20 @@ __device__ __forceinline__ void drain_chunk(uint32_t tbase, int stride, float (&
         if (n_acc > 1) tmem_ld16_async(tbase + stride + c0, w);
         tmem_wait_ld();
         tmem_regs_ready(v);
-        if (n_acc > 1) tmem_regs_ready(w);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
-            if (n_acc > 1) df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(w[i]));
+        fold16<true>(v, &hi[c0 / 2], &lo[c0 / 2]);
+        if (n_acc > 1) {
+            tmem_regs_ready(w);
+            fold16<true>(w, &hi[c0 / 2], &lo[c0 / 2]);
         }
         if (n_acc > 2) {
             tmem_ld16_async(tbase + 2 * stride + c0, v);
             if (n_acc > 3) tmem_ld16_async(tbase + 3 * stride + c0, w);
             tmem_wait_ld();
             tmem_regs_ready(v);
-            if (n_acc > 3) tmem_regs_ready(w);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                df_add(hi[c0 + i], lo[c0 + i], __uint_as_float(v[i]));
-                if (n_acc > 3) lo[c0 + i] = __fadd_rn(lo[c0 + i], __uint_as_float(w[i]));
+            fold16<true>(v, &hi[c0 / 2], &lo[c0 / 2]);
+            if (n_acc > 3) {
+                tmem_regs_ready(w);
+                fold16<false>(w, &hi[c0 / 2], &lo[c0 / 2]);
             }
         }
     }
@@ -602,14 +585,14 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
             // the column records are read when the tile is written out
             if (e < TBN / 4 && tp[buf].n0 + 4 * e < a.N)
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(cols + a.col0 + tp[buf].n0 + 4 * e));
-            float hi[F64 ? 1 : ECOLS], lo[F64 ? 1 : ECOLS];
+            f2 hi[F64 ? 1 : ECOLS / 2], lo[F64 ? 1 : ECOLS / 2];
             long long wd[2][F64 ? ECOLS : 1];
             if constexpr (F64) {
 #pragma unroll
                 for (int c = 0; c < ECOLS; ++c) { wd[0][c] = 0; wd[1][c] = 0; }
             } else {
 #pragma unroll
-                for (int c = 0; c < ECOLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
+                for (int c = 0; c < ECOLS / 2; ++c) { hi[c] = f2_pack(0.0f, 0.0f); lo[c] = f2_pack(0.0f, 0.0f); }
             }
             bool ok = true;
             for (int ks = 0; ks < nst; ++ks) {
@@ -663,13 +646,18 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                             d1[u] = __ldg(cm + 2 * (c0 + u) + 1);
                             if constexpr (F64) eb[u] = __ldg(cexp + a.coef_row0 + n0 + c0 + u);
                         }
+                    float vh[2] = {}, vl[2] = {};
+                    if constexpr (!F64) {
+                        f2_unpack(hi[c0 / 2], vh[0], vh[1]);
+                        f2_unpack(lo[c0 / 2], vl[0], vl[1]);
+                    }
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         const int c = c0 + u;
                         if (n0 + c < a.N && jj - jjp >= d1[u].y) {
                             double v;
                             if constexpr (F64) v = int_words_to_double(wd[0][c], wd[1][c], ea, eb[u]);
-                            else v = df_sum(hi[c], lo[c]);
+                            else v = df_sum(vh[u], vl[u]);
                             const int64_t ld = d1[u].x;
                             double *lower = reinterpret_cast<double *>(((uint64_t)(uint32_t)d0[u].y << 32) | (uint32_t)d0[u].x);
                             double *upper = reinterpret_cast<double *>(((uint64_t)(uint32_t)d0[u].w << 32) | (uint32_t)d0[u].z);
@@ -789,9 +777,9 @@ dense_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
         const int q = warp & 3;
         const int col0 = (ew >> 2) * EPI_COLS;
         const int row = q * 32 + lane;
-        float hi[EPI_COLS], lo[EPI_COLS];
+        f2 hi[EPI_COLS / 2], lo[EPI_COLS / 2];
 #pragma unroll
-        for (int c = 0; c < EPI_COLS; ++c) { hi[c] = 0.0f; lo[c] = 0.0f; }
+        for (int c = 0; c < EPI_COLS / 2; ++c) { hi[c] = f2_pack(0.0f, 0.0f); lo[c] = f2_pack(0.0f, 0.0f); }
         bool ok = true;
         for (int c = 0; c < nchunks && ok; ++c) {
             ok = mbar_wait(acc_full, c & 1, err, 6);
@@ -805,9 +793,13 @@ dense_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_consta
         if (ok && m < a.M) {
             float2 *out = a.part + (int64_t)z * a.N * a.M + m;
 #pragma unroll
-            for (int c = 0; c < EPI_COLS; ++c) {
+            for (int c = 0; c < EPI_COLS; c += 2) {
                 const int n = n0 + col0 + c;
-                if (n < a.N) out[(int64_t)n * a.M] = make_float2(hi[c], lo[c]);
+                float h0, h1, l0, l1;
+                f2_unpack(hi[c / 2], h0, h1);
+                f2_unpack(lo[c / 2], l0, l1);
+                if (n < a.N) out[(int64_t)n * a.M] = make_float2(h0, l0);
+                if (n + 1 < a.N) out[(int64_t)(n + 1) * a.M] = make_float2(h1, l1);
             }
         }
     }

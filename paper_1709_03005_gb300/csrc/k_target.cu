@@ -787,30 +787,37 @@ sandwich_df_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__
     const int64_t kb = b + w * per, ke = min(e, kb + per);
     const bool vec = (nsp & 1) == 0 && (reinterpret_cast<uintptr_t>(T.Cp_df) & 15) == 0;
     for (int n0 = 0; n0 < nsp; n0 += W) {
-        float ah[W], al[W];
+        f2 sh2[W / 2], sl2[W / 2];
 #pragma unroll
-        for (int c = 0; c < W; ++c) { ah[c] = 0.0f; al[c] = 0.0f; }
+        for (int c = 0; c < W / 2; ++c) { sh2[c] = f2_pack(0.0f, 0.0f); sl2[c] = f2_pack(0.0f, 0.0f); }
         for (int64_t k = kb + lane; k < ke; k += 32) {
             const int col = T.pairs[k].col;
             const float2 v = val[k];
             const float2 *crow = T.Cp_df + (int64_t)col * nsp + n0;
+            const f2 vh = f2_pack(v.x, v.x), nvh = f2_pack(-v.x, -v.x), vl = f2_pack(v.y, v.y);
             if (vec) {
                 // n0 + c even and nsp even: the pair (c, c + 1) is in range together
 #pragma unroll
                 for (int c = 0; c < W; c += 2)
                     if (n0 + c < nsp) {
                         const float4 x = __ldg(reinterpret_cast<const float4 *>(crow + c));
-                        df_fma(ah[c], al[c], v.x, v.y, x.x, x.y);
-                        df_fma(ah[c + 1], al[c + 1], v.x, v.y, x.z, x.w);
+                        df_fma(sh2[c / 2], sl2[c / 2], vh, nvh, vl, f2_pack(x.x, x.z), f2_pack(x.y, x.w));
                     }
             } else {
 #pragma unroll
-                for (int c = 0; c < W; ++c)
+                for (int c = 0; c < W; c += 2)
                     if (n0 + c < nsp) {
                         const float2 x = __ldg(crow + c);
-                        df_fma(ah[c], al[c], v.x, v.y, x.x, x.y);
+                        const float2 z = n0 + c + 1 < nsp ? __ldg(crow + c + 1) : make_float2(0.0f, 0.0f);
+                        df_fma(sh2[c / 2], sl2[c / 2], vh, nvh, vl, f2_pack(x.x, z.x), f2_pack(x.y, z.y));
                     }
             }
+        }
+        float ah[W], al[W];
+#pragma unroll
+        for (int c = 0; c < W; c += 2) {
+            f2_unpack(sh2[c / 2], ah[c], ah[c + 1]);
+            f2_unpack(sl2[c / 2], al[c], al[c + 1]);
         }
 #pragma unroll
         for (int c = 0; c < W; ++c) {
