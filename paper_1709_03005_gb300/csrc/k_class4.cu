@@ -24,52 +24,93 @@ namespace hb {
 
 namespace {
 
-constexpr int kJ = 128;
+constexpr int kJ = 224;     // most threads of a block
 constexpr int kBatch = 32;
 
-__device__ __forceinline__ double x4(const Ints &I, int a, int b, int c, int j) {
-    // (a b | c j), target a, b, c and continuum index j
-    return __ldg(I.tttc + pair_idx(a, b) * ((int64_t)I.n_to * I.n_co) + (int64_t)c * I.n_co + j);
-}
+// A staged pair, worked out once for all orbitals and states: of degree 2 the
+// first elements of its direct and exchange rows of the (tt|tc) table, of degree
+// 1 (chi = D + t, the single excitation t -> j) the orbital t.
+struct PairRec {
+    int64_t dir, exc;      // -1: no such integral
+    int col, t;            // the determinant; t >= 0: degree 1
+    int neg, pad;
+};
 
 template <int W>
-__device__ double prototype_value(const Ints &I, const hb_pair &r, const uint64_t *__restrict__ D, int j,
-                                  int cont_spin) {
-    const int sb = 64 * W;
+__device__ __forceinline__ PairRec pair_rec(const C4Task &T, const hb_pair &r) {
+    const int sb = 64 * W, n_to = T.I.n_to, cont_spin = T.cont_spin;
+    PairRec p;
+    p.dir = p.exc = -1;
+    p.col = r.col;
+    p.t = -1;
+    p.neg = r.phase < 0;
+    p.pad = 0;
     if (r.degree == 1) {
-        // chi = D + t (spin cont_spin): single excitation t -> j
-        const int t = r.hole[0] % sb;
-        double v = __ldg(I.h + (int64_t)(I.n_to + j) * I.n_orb + t);
-#pragma unroll
-        for (int w = 0; w < 2 * W; ++w) {
-            uint64_t x = __ldg(D + w);
-            const int s = w / W;
-            while (x) {
-                const int k = 64 * (w % W) + __ffsll((long long)x) - 1;
-                x &= x - 1;
-                v += x4(I, k, k, t, j);                    // (jt|kk)
-                if (s == cont_spin) v -= x4(I, k, t, k, j); // (jk|kt)
-            }
-        }
-        return r.phase * v;
+        p.t = r.hole[0] % sb;
+        return p;
     }
     // degree 2: holes h1 < h2 in chi, particles {q, continuum} in D + j
     const int h1 = r.hole[0], h2 = r.hole[1], q = r.part[0];
     const int kq = 2 * q, kv = cont_spin == 0 ? 2 * 64 * W - 1 : 2 * 128 * W - 1;
     const int s1 = h1 / sb, s2 = h2 / sb, sq = q / sb;
     const int o1 = h1 % sb, o2 = h2 % sb, oq = q % sb;
-    double dir = 0.0, exc = 0.0;
+    // (q h1|j h2) and (q h2|j h1)
+    const int64_t x12 = (pair_idx(oq, o1) * n_to + o2) * T.I.n_co, x21 = (pair_idx(oq, o2) * n_to + o1) * T.I.n_co;
     if (kq < kv) {
-        // p1 = q, p2 = continuum
-        if (sq == s1 && cont_spin == s2) dir = x4(I, oq, o1, o2, j);   // (q h1|j h2)
-        if (sq == s2 && cont_spin == s1) exc = x4(I, oq, o2, o1, j);   // (q h2|j h1)
+        if (sq == s1 && cont_spin == s2) p.dir = x12;
+        if (sq == s2 && cont_spin == s1) p.exc = x21;
     } else {
-        // p1 = continuum, p2 = q
-        if (cont_spin == s1 && sq == s2) dir = x4(I, oq, o2, o1, j);   // (j h1|q h2)
-        if (cont_spin == s2 && sq == s1) exc = x4(I, oq, o1, o2, j);   // (j h2|q h1)
+        // the continuum orbital is the first particle
+        if (cont_spin == s1 && sq == s2) p.dir = x21;
+        if (cont_spin == s2 && sq == s1) p.exc = x12;
     }
-    return r.phase * (dir - exc);
+    return p;
 }
+
+// The integrals of a task, FP64 or as float pairs (Acc of hb_df.cuh), for
+// continuum orbital j.
+template <int W, class Acc>
+struct Prototype {
+    const double *x, *h;
+    const float2 *x_df, *h_df;
+    int64_t plane;
+    int n_co, cont_spin;
+    typename Acc::Entry dir, exc;
+    __device__ __forceinline__ Prototype(const C4Task &T, int j)
+        : x(T.I.tttc + j), h(T.I.h + (int64_t)(T.I.n_to + j) * T.I.n_orb), x_df(T.tttc_df + j),
+          h_df(T.h_df + (int64_t)(T.I.n_to + j) * T.I.n_orb), plane((int64_t)T.I.n_to * T.I.n_co), n_co(T.I.n_co),
+          cont_spin(T.cont_spin) {}
+    // starts the reads of a pair of degree 2
+    __device__ __forceinline__ void fetch(const PairRec &p) {
+        dir = exc = typename Acc::Entry{};
+        if (p.dir >= 0) dir = Acc::entry(x, x_df, p.dir);
+        if (p.exc >= 0) exc = Acc::entry(x, x_df, p.exc);
+    }
+    // <D_m + j|H|chi_l> without its sign; of degree 2 from what fetch read
+    __device__ __forceinline__ Acc value(const PairRec &p, const uint64_t *__restrict__ dets) const {
+        Acc v;
+        if (p.t < 0) {
+            v.add_entry(dir);
+            v.sub_entry(exc);
+            return v;
+        }
+        const uint64_t *D = dets + (int64_t)p.col * 2 * W;
+        const int t = p.t;
+        v.add(h, h_df, t);
+#pragma unroll
+        for (int w = 0; w < 2 * W; ++w) {
+            uint64_t y = __ldg(D + w);
+            const int s = w / W;
+            while (y) {
+                const int k = 64 * (w % W) + __ffsll((long long)y) - 1;
+                y &= y - 1;
+                v.add(x, x_df, pair_idx(k, k) * plane + (int64_t)t * n_co);                         // (jt|kk)
+                if (s == cont_spin) v.sub(x, x_df, pair_idx(k, t) * plane + (int64_t)k * n_co);     // (jk|kt)
+            }
+        }
+        return v;
+    }
+};
 
 // Block = blockDim.x continuum orbitals of one L2 row; NS target states per
 // pass.  FP64 FMAs for states beyond the group's cost as much as the others on
@@ -79,20 +120,19 @@ template <int W, int NS>
 __global__ void __launch_bounds__(kJ)
 class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     __shared__ double cs[kBatch][NS];
-    __shared__ hb_pair rs[kBatch];
+    __shared__ PairRec rs[kBatch];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const C4Task &T = tasks[ti];
     const int JT = blockDim.x;
-    const Ints I = T.I;
     const hb_pair *__restrict__ pairs = T.pairs;
     const uint64_t *__restrict__ dets = T.dets;
     const double *__restrict__ C = T.C;
-    const int ns = T.ns, cf = T.cf, cn = T.cn, cont_spin = T.cont_spin;
+    const int ns = T.ns, cf = T.cf, cn = T.cn;
     const int lb = (int)(blockIdx.x - blk[ti]);
     const int l = lb / T.ny;
     const int jl = (lb % T.ny) * JT + threadIdx.x;
-    const bool jv = jl < cn;
-    const int j = cf + (jv ? jl : 0);
+    const bool jv = jl < cn, wv = jl - (int)(threadIdx.x & 31) < cn;   // this lane's, this warp's orbitals exist
+    Prototype<W, AccD> proto(T, cf + (jv ? jl : 0));
     const int64_t b = T.row_ptr[l], e = T.row_ptr[l + 1];
     for (int n0 = 0; n0 < ns; n0 += NS) {
         const int nc = min(NS, ns - n0);
@@ -102,16 +142,19 @@ class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk,
         for (int64_t p0 = b; p0 < e; p0 += kBatch) {
             const int cnt = (int)(e - p0 < kBatch ? e - p0 : kBatch);
             __syncthreads();
-            for (int t = threadIdx.x; t < cnt; t += JT) rs[t] = pairs[p0 + t];
+            for (int t = threadIdx.x; t < cnt; t += JT) rs[t] = pair_rec<W>(T, pairs[p0 + t]);
             __syncthreads();
             for (int t = threadIdx.x; t < cnt * NS; t += JT) {
                 const int i = t / NS, n = t % NS;
                 cs[i][n] = n < nc ? C[(int64_t)rs[i].col * ns + n0 + n] : 0.0;
             }
             __syncthreads();
-            for (int i = 0; i < cnt; ++i) {
-                const hb_pair r = rs[i];
-                const double y = prototype_value<W>(I, r, dets + (int64_t)r.col * 2 * W, j, cont_spin);
+            proto.fetch(rs[0]);
+            for (int i = 0; i < (wv ? cnt : 0); ++i) {
+                AccD v = proto.value(rs[i], dets);
+                if (rs[i].neg) v.neg();
+                const double y = v.v;
+                if (i + 1 < cnt) proto.fetch(rs[i + 1]);     // in flight during the sums
 #pragma unroll
                 for (int n = 0; n < NS; ++n) acc[n] = fma(cs[i][n], y, acc[n]);
             }
@@ -126,69 +169,15 @@ class4_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk,
 }
 
 // ------------------------------------------------------- double-float path
-__device__ __forceinline__ float2 x4df(const C4Task &T, int a, int b, int c, int j) {
-    return __ldg(T.tttc_df + pair_idx(a, b) * ((int64_t)T.I.n_to * T.I.n_co) + (int64_t)c * T.I.n_co + j);
-}
-
-template <int W>
-__device__ __forceinline__ void prototype_df(const C4Task &T, const hb_pair &r, const uint64_t *__restrict__ D,
-                                             int j, float &vh, float &vl) {
-    const int sb = 64 * W;
-    const int cont_spin = T.cont_spin;
-    if (r.degree == 1) {
-        // chi = D + t (spin cont_spin): single excitation t -> j
-        const int t = r.hole[0] % sb;
-        const float2 h = __ldg(T.h_df + (int64_t)(T.I.n_to + j) * T.I.n_orb + t);
-        vh = h.x;
-        vl = h.y;
-#pragma unroll
-        for (int w = 0; w < 2 * W; ++w) {
-            uint64_t x = __ldg(D + w);
-            const int s = w / W;
-            while (x) {
-                const int k = 64 * (w % W) + __ffsll((long long)x) - 1;
-                x &= x - 1;
-                const float2 a = x4df(T, k, k, t, j);                 // (jt|kk)
-                df_add2(vh, vl, a.x, a.y);
-                if (s == cont_spin) {
-                    const float2 b = x4df(T, k, t, k, j);             // (jk|kt)
-                    df_add2(vh, vl, -b.x, -b.y);
-                }
-            }
-        }
-    } else {
-        // degree 2: holes h1 < h2 in chi, particles {q, continuum} in D + j
-        const int h1 = r.hole[0], h2 = r.hole[1], q = r.part[0];
-        const int kq = 2 * q, kv = cont_spin == 0 ? 2 * 64 * W - 1 : 2 * 128 * W - 1;
-        const int s1 = h1 / sb, s2 = h2 / sb, sq = q / sb;
-        const int o1 = h1 % sb, o2 = h2 % sb, oq = q % sb;
-        float2 dir = make_float2(0.0f, 0.0f), exc = make_float2(0.0f, 0.0f);
-        if (kq < kv) {
-            if (sq == s1 && cont_spin == s2) dir = x4df(T, oq, o1, o2, j);   // (q h1|j h2)
-            if (sq == s2 && cont_spin == s1) exc = x4df(T, oq, o2, o1, j);   // (q h2|j h1)
-        } else {
-            if (cont_spin == s1 && sq == s2) dir = x4df(T, oq, o2, o1, j);   // (j h1|q h2)
-            if (cont_spin == s2 && sq == s1) exc = x4df(T, oq, o1, o2, j);   // (j h2|q h1)
-        }
-        vh = dir.x;
-        vl = dir.y;
-        df_add2(vh, vl, -exc.x, -exc.y);
-    }
-    if (r.phase < 0) {
-        vh = -vh;
-        vl = -vl;
-    }
-}
-
 // Block = blockDim.x continuum orbitals (32, 64 or 128) of one L2 row; NS
 // target states per pass, two to an f32x2 instruction.  The CI coefficients lie
 // in shared memory as high and low words, four states to a load.
 template <int W, int NS>
-__global__ void __launch_bounds__(kJ, NS <= 24 ? 6 : 1)
+__global__ void __launch_bounds__(kJ, NS <= 24 ? 3 : 1)
 class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
     static_assert(NS % 4 == 0, "coefficients are read four states at a time");
     __shared__ __align__(16) float ch[kBatch][NS], cl[kBatch][NS];
-    __shared__ hb_pair rs[kBatch];
+    __shared__ PairRec rs[kBatch];
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const C4Task &T = tasks[ti];
     const int JT = blockDim.x;
@@ -196,8 +185,9 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
     const int lb = (int)(blockIdx.x - blk[ti]);
     const int l = lb / T.ny;
     const int jl = (lb % T.ny) * JT + threadIdx.x;
-    const bool jv = jl < cn;
-    const int j = T.cf + (jv ? jl : 0);
+    const bool jv = jl < cn, wv = jl - (int)(threadIdx.x & 31) < cn;   // this lane's, this warp's orbitals exist
+    Prototype<W, AccF> proto(T, T.cf + (jv ? jl : 0));
+    const uint64_t *__restrict__ dets = T.dets;
     const int64_t b = T.row_ptr[l], e = T.row_ptr[l + 1];
     for (int n0 = 0; n0 < ns; n0 += NS) {
         const int nc = min(NS, ns - n0);
@@ -207,7 +197,7 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
         for (int64_t p0 = b; p0 < e; p0 += kBatch) {
             const int cnt = (int)(e - p0 < kBatch ? e - p0 : kBatch);
             __syncthreads();
-            for (int t = threadIdx.x; t < cnt; t += JT) rs[t] = T.pairs[p0 + t];
+            for (int t = threadIdx.x; t < cnt; t += JT) rs[t] = pair_rec<W>(T, T.pairs[p0 + t]);
             __syncthreads();
             for (int t = threadIdx.x; t < cnt * NS; t += JT) {
                 const int i = t / NS, n = t % NS;
@@ -216,11 +206,12 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
                 cl[i][n] = c.y;
             }
             __syncthreads();
-            for (int i = 0; i < cnt; ++i) {
-                const hb_pair r = rs[i];
-                float yh, yl;
-                prototype_df<W>(T, r, T.dets + (int64_t)r.col * 2 * W, j, yh, yl);
-                const f2 y = f2_pack(yh, yh), ny = f2_pack(-yh, -yh), yl2 = f2_pack(yl, yl);
+            proto.fetch(rs[0]);
+            for (int i = 0; i < (wv ? cnt : 0); ++i) {
+                AccF v = proto.value(rs[i], dets);
+                if (rs[i].neg) v.neg();
+                const f2 y = f2_pack(v.h, v.h), ny = f2_pack(-v.h, -v.h), yl2 = f2_pack(v.l, v.l);
+                if (i + 1 < cnt) proto.fetch(rs[i + 1]);     // in flight during the sums
 #pragma unroll
                 for (int n = 0; n < NS; n += 4) {
                     const ulonglong2 h4 = *reinterpret_cast<const ulonglong2 *>(&ch[i][n]);
@@ -240,8 +231,8 @@ class4_df_kernel(const C4Task *__restrict__ tasks, const int64_t *__restrict__ b
                 float h0, h1, l0, l1;
                 f2_unpack(ahi[n / 2], h0, h1);
                 f2_unpack(alo[n / 2], l0, l1);
-                if (n < nc) out[(int64_t)(n0 + n) * cn] = df_to_double(h0, l0);
-                if (n + 1 < nc) out[(int64_t)(n0 + n + 1) * cn] = df_to_double(h1, l1);
+                if (n < nc) out[(int64_t)(n0 + n) * cn] = df_sum(h0, l0);
+                if (n + 1 < nc) out[(int64_t)(n0 + n + 1) * cn] = df_sum(h1, l1);
             }
         }
     }
@@ -270,13 +261,10 @@ void class4_shape(int ns, int cn, int *ns_tile, int *jt) {
     const int passes = (ns + 31) / 32;
     const int need = (ns + passes - 1) / passes;
     *ns_tile = need <= 4 ? 4 : (need + 3) / 4 * 4;
-    int best = 128;
-    int64_t best_idle = (int64_t)((cn + 127) / 128) * 128 - cn;
-    for (int t : {64, 32}) {
-        const int64_t idle = (int64_t)((cn + t - 1) / t) * t - cn;
-        if (idle < best_idle) { best = t; best_idle = idle; }
-    }
-    *jt = best;
+    // one block for the whole row where the orbitals allow it (the pairs and CI
+    // rows are staged once), else blocks of one size
+    const int tiles = (cn + kJ - 1) / kJ, per = tiles > 0 ? (cn + tiles - 1) / tiles : 1;
+    *jt = (per + 31) / 32 * 32;
 }
 
 void split_df(const double *x, int64_t n, float2 *out, cudaStream_t s) {
