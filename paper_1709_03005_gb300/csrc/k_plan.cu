@@ -166,7 +166,7 @@ struct Plan {
     // timers: start, target, expansion (main stream); class-4 end, L2 end, side
     // start (side stream); end after the join; L2 start, class-4 classification
     // end (side stream); split kernels
-    cudaEvent_t ev[9] = {};
+    cudaEvent_t ev[8] = {};
     std::vector<cudaEvent_t> ev_split;
     int launches = 0, expand_launches = 0;
     bool timed = false;
@@ -974,35 +974,27 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     // reduced coefficient rows in place, classes 4, 2, 8 and the expansion (2)
     const bool ph1 = p->phase != 2, ph2 = p->phase != 1;
     if (ph2) L += g_classify(p->cls_tl2.g, W, 1, s2);
-    rec_on(p->ev[8], s2);
     if (!ph2) {
         rec_on(p->ev[7], s2);
         rec_on(p->ev[4], s2);
         rec_on(p->ev[3], s2);
-    } else if (p->c4t.g.blocks > 0) {
-        // the tensor-core class-4 kernel and the expansion kernel each hold
-        // whole SMs until their work is done, and the L2 rows' blocks do not
-        // fit beside either: the L2 rows run beside the target side, then
-        // class 4, and the expansion starts once both are done
+    } else {
+        // the L2 rows first, which fit beside the target side.  The tensor-core
+        // class-4 kernel and the expansion kernel each hold whole SMs until
+        // their work is done: with it, the expansion starts once it is done
         rec_on(p->ev[7], s2);
         L += g_l2_csr(p->l2.g, W, s2);
         L += g_l2_values(p->l2v.g, W, s2);
         L += g_l2_mirror(p->l2m.g, s2);
         rec_on(p->ev[4], s2);
-        cudaMemsetAsync(p->err + 1, 0, sizeof(int), s2);
-        L += g_c4fill(p->c4f.g, s2);
-        L += g_c4tc(p->c4t.g, p->d_c4items, (int)p->c4items.size(), p->c4_slices, p->err + 1, s2);
-        for (auto &v : p->c4v) L += g_class4(v.st.g, W, 1, v.ns_tile, v.jt, s2);
-        rec_on(p->ev[3], s2);
-        cudaEventRecord(p->c4_done, s2);
-    } else {
+        if (p->c4t.g.blocks > 0) {
+            cudaMemsetAsync(p->err + 1, 0, sizeof(int), s2);
+            L += g_c4fill(p->c4f.g, s2);
+            L += g_c4tc(p->c4t.g, p->d_c4items, (int)p->c4items.size(), p->c4_slices, p->err + 1, s2);
+        }
         for (auto &v : p->c4v) L += g_class4(v.st.g, W, p->precision == HB_MIXED ? 1 : 0, v.ns_tile, v.jt, s2);
         rec_on(p->ev[3], s2);
-        rec_on(p->ev[7], s2);
-        L += g_l2_csr(p->l2.g, W, s2);
-        L += g_l2_values(p->l2v.g, W, s2);
-        L += g_l2_mirror(p->l2m.g, s2);
-        rec_on(p->ev[4], s2);
+        cudaEventRecord(p->c4_done, s2);
     }
     cudaEventRecord(p->join, s2);
     s = p->main;
@@ -1050,14 +1042,18 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     } else if (p->split_on || p->precision == HB_MIXED) {
         // with class 4 on the tensor cores, the expansion waits for it (see
         // the side stream above); the double-float class-4 kernel runs beside
-        // the expansion, which was faster than running it first
-        if (p->c4t.g.blocks > 0) cudaStreamWaitEvent(s, p->c4_done, 0);
+        // the expansion, which was faster than running it first (615 against 719
+        // us at dimension 8000).  The FP64 one holds an SM too long for that: an
+        // expansion whose CTAs share out their tiles waits (1.63 against 1.80
+        // ms), one with fewer tiles than SMs does not (138 against 158 us at
+        // dimension 959).
+        int64_t tiles = 0;
+        for (auto &g : p->split) tiles += g.st.g.blocks;
+        if (p->c4t.g.blocks > 0 || (p->precision != HB_MIXED && tiles > 152)) cudaStreamWaitEvent(s, p->c4_done, 0);
         if (p->coef_rows > 0) {
             // the rows with j == j': beside a split kernel that fills the chip they
             // slowed it by more than they saved; one that leaves most SMs idle has
             // them beside it (10 us of the 160 of a build of dimension 110)
-            int64_t tiles = 0;
-            for (auto &g : p->split) tiles += g.st.g.blocks;
             const bool beside = tiles <= 76;
             if (beside) {
                 cudaEventRecord(p->asm_done, s);
@@ -1111,17 +1107,10 @@ void plan_stats(Plan *p, hb_stats *st) {
     cudaEventElapsedTime(&st->ms_target, p->ev[0], p->ev[1]);
     cudaEventElapsedTime(&st->ms_expand, p->ev[1], p->ev[2]);
     cudaEventElapsedTime(&st->ms_l2, p->ev[7], p->ev[4]);
-    if (p->c4t.g.blocks > 0) {
-        // class-4 classification, then (after the L2 rows) the tensor-core part
-        float a = 0.0f, b = 0.0f;
-        cudaEventElapsedTime(&a, p->ev[5], p->ev[7]);
-        cudaEventElapsedTime(&b, p->ev[4], p->ev[3]);
-        st->ms_class4 = a + b;
-        st->ms_class4_kernel = b;
-    } else {
-        cudaEventElapsedTime(&st->ms_class4, p->ev[5], p->ev[3]);
-        cudaEventElapsedTime(&st->ms_class4_kernel, p->ev[8], p->ev[3]);
-    }
+    // class-4 classification, then (after the L2 rows) the rest
+    cudaEventElapsedTime(&st->ms_class4, p->ev[5], p->ev[7]);
+    cudaEventElapsedTime(&st->ms_class4_kernel, p->ev[4], p->ev[3]);
+    st->ms_class4 += st->ms_class4_kernel;
     if (p->split_on) {
         float total = 0.0f;
         for (size_t i = 0; i + 1 < p->ev_split.size(); i += 2) {
