@@ -34,14 +34,15 @@
 // same work, as 128 + 128 + 128 + 16 a quarter of the CTAs had little of it.
 // Every wait is bounded; on a timeout the kernel records an error and leaves.
 // 120000 items of 40 target and 400 continuum orbitals and 50 states (22 GB
-// gathered, 4.8 GB written) take 5.1 ms, 12.0 before the points above and below:
-// a warp's single lane issued an MMA in 98 cycles.  Now the epilogue's FP64
-// additions (4.7 ms without them) and the MMAs (990 cycles a K block) share it.
+// gathered, 4.8 GB written) take 4.7 ms, 12.0 before the points above and
+// below: a warp's single lane issued an MMA in 98 cycles.  The MMAs now take
+// 990 cycles a K block, and the epilogue's FP64 additions almost as long.
 //
 // The slices of the 64 states lie side by side, so one MMA multiplies integral
 // slice i with the CI slices 0 .. 3 - i (N up to 256) into the neighbouring
 // accumulators s = i ..: 15 MMAs a K block for six slices instead of 21, and
 // the 128 orbitals of a slice are read from shared memory 15 times.
+
 #include <cuda_bf16.h>
 
 #include <algorithm>

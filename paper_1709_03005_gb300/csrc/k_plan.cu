@@ -620,7 +620,8 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     }
     int rc = HB_OK;
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 9 && e == cudaSuccess; ++i) e = cudaEventCreate(&p->ev[i]);
+    for (cudaEvent_t &ev : p->ev)
+        if (e == cudaSuccess) e = cudaEventCreate(&ev);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->uploaded, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);

@@ -560,6 +560,9 @@ __global__ void l2_mirror_fill_kernel(const int32_t *__restrict__ col, const int
 // doubles; double-float: val as (hi, lo) float pairs in the same 8 bytes.  As in
 // l2_values_kernel a warp takes 32 steps consecutive records, evaluates the
 // doubles as they come and queues the singles until 32 fill its lanes.
+// 12.6e6 records of 20000 determinants: 0.43 -> 0.21 ms; 14e6 of a batch of
+// twelve: 0.42 -> 0.26 ms (with one step a warp, whose queue holds a few singles
+// at most, 0.64).
 template <int W, class Acc>
 __global__ void __launch_bounds__(32 * kWarps)
 pair_values_kernel(const PVTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {

@@ -770,7 +770,9 @@ __device__ __forceinline__ void shfl_df_add(float &h, float &l, int off) {
 // Passes of W states, one block per row as in sandwich_kernel: a lane of warp
 // w sums every 32nd record of the warp's part of the row for all W states of
 // the pass, the warp reduces by a fixed xor tree and warp 0 adds the warps in
-// order.  The coefficient pairs are read 16 bytes at a time where aligned.
+// order.  The coefficient pairs are read 16 bytes at a time where aligned; two
+// states to an f32x2 instruction (20000 rows of 630 records, 50 states: 1.63 ms
+// in single instructions, 1.16 so).
 template <int W>
 __global__ void __launch_bounds__(32 * kSWWarps)
 sandwich_df_kernel(const SWTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks) {
