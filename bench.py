@@ -29,6 +29,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import subprocess
 import sys
@@ -426,22 +427,24 @@ def run_ours(args, rank, world, local_rank):
     del host
 
     peaks = measured_peaks()
-    if precision == hb.HB_MIXED:
+    if st.expand_tensor_flops > 0:
         kern_ms = gemm_ms
         tflops = st.expand_tensor_flops
+        products = round(tflops / st.expand_flops)       # S (S + 1) / 2 of S slices per operand
+        slices = round((math.sqrt(8 * products + 1) - 1) / 2)
         pk = peaks.get("bf16_tflops")
         fp64eq = st.expand_flops / (kern_ms / 1e3) / 1e12 if kern_ms else None
         pipe = tflops / (kern_ms / 1e3) / 1e12 if kern_ms else None
         roof = {"bound": "tensor", "unit": "TFLOP/s", "peak": pk,
                 "peak_source": "measured bf16 burst (of measured)",
-                "kernel": "split_expand_kernel: Eq. 7 contraction on bf16 tensor cores, 6 slices per operand",
+                "kernel": f"split_expand_kernel: Eq. 7 contraction on bf16 tensor cores, {slices} slices per operand",
                 "achieved": fp64eq, "flops_per_launch": st.expand_flops,
                 "flops_definition": "algorithmic FP64-equivalent flops 2 K (elements) of Eq. 7 per launch",
                 "kernel_ms": kern_ms,
                 "pipe_achieved": pipe, "pipe_frac": pipe / pk if pipe and pk else None,
                 "pipe_flops_per_launch": tflops,
-                "pipe_definition": "bf16 tensor flops issued: the 21 slice-pair products of every FP64-equivalent "
-                                   "product",
+                "pipe_definition": f"bf16 tensor flops issued: the {products} slice-pair products of every "
+                                   "FP64-equivalent product",
                 "traffic": profiled_traffic("split_expand_kernel", "paper_1709_03005_gb300/csrc/k_split.cu",
                                             None if args.set else args.config)}
     else:
