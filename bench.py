@@ -606,7 +606,7 @@ def run_ours(args, rank, world, local_rank):
         out = {"metric": "H elements/sec", "value": value, "unit": "H elements/s", "n_gpus": world,
                "steps": args.steps, "warmup": args.warmup, "ms_per_step": total_ms / args.steps,
                "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-               "dtype": "bf16x6-split/f32->f64" if precision == hb.HB_MIXED else "f64", "data": "synthetic",
+               "dtype": "bf16x5-split/f32->f64" if precision == hb.HB_MIXED else "f64", "data": "synthetic",
                "config": {"workload": workload_text(args), "dim": dim,
                           "positions": positions(dim), "l2_flush": "256 MB write between timed steps",
                           "parallelism": f"replicas x{world}", "precision": args.precision},
