@@ -49,6 +49,8 @@
  * Streams: `stream` is a cudaStream_t passed as void*; NULL means the legacy
  * default stream.  Work is enqueued on it; calls that must read a device
  * result (counts, convergence) synchronise that stream before returning.
+ * Builds of one context (its own, sharded ones, those of a batch) share its
+ * scratch: a build enqueued on another stream waits for the one before.
  */
 #ifndef HB_H
 #define HB_H

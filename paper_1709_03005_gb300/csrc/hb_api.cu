@@ -730,6 +730,7 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
     // other output blocks)
     hb::Plan *plan = (hb::Plan *)ctx->plan;
     std::string err;
+    plan_wait_last(&ctx, 1, s);
     if (plan && plan_precision(plan) != precision) {
         cudaStreamSynchronize(s);
         plan_destroy(plan);
@@ -754,6 +755,7 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
     if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
     int launches = 0;
     int rc = plan_launch(plan, s, &launches, &err);
+    plan_mark_built(plan, s);
     if (rc != HB_OK) return fail(ctx, rc, err);
     if (precision == HB_MIXED) {
         // the tensor-core kernel reports a bounded-wait timeout in a device word
@@ -886,6 +888,7 @@ extern "C" int hb_build_contract(hb_ctx *ctx, int32_t precision, int32_t rank, i
     CK(cudaSetDevice(ctx->device));
     // the contraction writes no output block: a cached plan of this share is
     // used as it is, a new one is made without outputs
+    plan_wait_last(&ctx, 1, s);
     hb::Plan *p = (hb::Plan *)ctx->shard_plan;
     if (!p || !plan_is_shard(p, precision, rank, nranks)) {
         hb_blocks none{};
@@ -906,6 +909,7 @@ extern "C" int hb_build_contract(hb_ctx *ctx, int32_t precision, int32_t rank, i
         CK(cudaMemcpyAsync(partial + off, P.A, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
         off += (int64_t)n;
     }
+    plan_mark_built(p, s);
     if (st) {
         memset(st, 0, sizeof(*st));
         st->kernel_launches = launches;
@@ -928,6 +932,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     hb::Plan *p = nullptr;
+    plan_wait_last(&ctx, 1, s);
     rc = shard_plan(ctx, precision, rank, nranks, out, &p, s);
     if (rc != HB_OK) return rc;
     // the summed coefficient rows of all ranks in place of this rank's
@@ -944,6 +949,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
     int launches = 0;
     rc = plan_run(p, s, false, false, &launches, &err);
     plan_set_phase(p, 0);
+    plan_mark_built(p, s);
     if (rc != HB_OK) return fail(ctx, rc, err);
     if (precision == HB_MIXED) {
         int word = 0;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <map>
+#include <memory>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -45,6 +46,13 @@ struct GroupL2 {
 };
 
 struct MixedState;   // split-precision operands (k_split.cu)
+
+// The end of a build on its caller's stream; shared by the plan that records it
+// and the contexts whose last build it was.
+struct BuildEvent {
+    cudaEvent_t e = nullptr;
+    ~BuildEvent() { if (e) cudaEventDestroy(e); }
+};
 
 // Device memory a context takes after hb_init (build plans, tensor-core
 // slices and tables, double-float copies, solver scratch): cudaMalloc, or,
@@ -161,6 +169,9 @@ struct hb_ctx {
     hb::DevPool pool;        // device memory beyond the staged problem
     hb_ctx *base = nullptr;  // context whose staged integrals this one borrows (or null)
     void *plan = nullptr;    // cached grouped-launch plan of this context's own builds (k_plan.cu)
+    // the end of this context's last build: its scratch (records, sort tables,
+    // coefficient rows) serves every build, so the next one waits for it
+    std::shared_ptr<hb::BuildEvent> last_build;
     void *shard_plan = nullptr;   // cached plan of this context's share of a sharded build
     void *diag = nullptr;   // Davidson workspace (k_davidson.cu)
     void *mlp = nullptr;    // learned preconditioner weights (k_mlp.cu)

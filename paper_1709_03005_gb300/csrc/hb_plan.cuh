@@ -29,6 +29,11 @@ int plan_host_error(hb::Plan *p);
 // Issue every stage on stream s.  timing: record the stage events (as graph
 // event nodes when capture is set).  *launches: kernels launched.
 int plan_run(hb::Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, std::string *err);
+// Order stream s behind the last build of each context (whatever stream, plan or
+// batch it ran by); and record the end of a build of p on s as that of its
+// contexts.  Neither does anything on a stream that is being captured.
+void plan_wait_last(hb_ctx *const *ctxs, int n, cudaStream_t s);
+void plan_mark_built(hb::Plan *p, cudaStream_t s);
 // a whole build, replayed as a graph where the same one is repeated
 int plan_launch(hb::Plan *p, cudaStream_t s, int *launches, std::string *err);
 // After the stream has finished a timed run: per-stage times and counters.

@@ -56,6 +56,7 @@ extern "C" int hb_batch_create(hb_batch **out, hb_ctx *const *ctxs, int32_t n, i
     b->outs.assign(outs, outs + n);
     cudaStream_t s = (cudaStream_t)stream;
     std::string err;
+    plan_wait_last(ctxs, n, s);
     // the plan prepares the tensor-core operands and uploads its task tables
     int rc = plan_create(ctxs, n, outs, precision, &b->plan, &err, s);
     if (rc != HB_OK) { delete b; return bfail(rc, err); }
@@ -97,6 +98,7 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
     if (!b || !b->exec) return bfail(HB_ERR_INVALID_ARG, "batch is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    plan_wait_last(b->ctxs.data(), (int)b->ctxs.size(), s);
     if (st) {
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -105,6 +107,7 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
     if (plan_host_error(b->plan)) return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel of an FP64 build gave up waiting");
     cudaError_t e = cudaGraphLaunch(b->exec, s);
     if (e != cudaSuccess) return bfail(HB_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(e));
+    plan_mark_built(b->plan, s);
     if (st) {
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);

@@ -163,6 +163,7 @@ struct Plan {
     cudaStream_t aux1 = nullptr, aux2 = nullptr;
     cudaEvent_t k1_done = nullptr, items_done = nullptr, gd_done = nullptr, asm_done = nullptr, dr_done = nullptr;
     cudaEvent_t c4_done = nullptr;     // the tensor-core class-4 kernel has finished (side stream)
+    std::shared_ptr<BuildEvent> built; // the end of this plan's last build on its caller's stream
     // timers: start, target, expansion (main stream); class-4 end, L2 end, side
     // start (side stream); end after the join; L2 start, class-4 classification
     // end (side stream); split kernels
@@ -635,6 +636,8 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->aux2, cudaStreamNonBlocking, greatest);
     for (cudaEvent_t *ev : {&p->k1_done, &p->items_done, &p->gd_done, &p->asm_done, &p->dr_done})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    p->built = std::make_shared<BuildEvent>();
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->built->e, cudaEventDisableTiming);
     if (e == cudaSuccess) e = dmalloc_n(ctxs[0], &p->err, 2);   // split kernel, class-4 kernel
     if (e == cudaSuccess) e = cudaMemsetAsync(p->err, 0, 2 * sizeof(int), s);
     if (e != cudaSuccess) {
@@ -1134,6 +1137,30 @@ int plan_error_word(Plan *p, int *word) {
     return HB_OK;
 }
 
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();      // the legacy stream while another stream is captured
+    return true;
+}
+
+void plan_wait_last(hb_ctx *const *ctxs, int n, cudaStream_t s) {
+    if (capturing(s)) return;
+    const BuildEvent *before = nullptr;
+    for (int i = 0; i < n; ++i) {
+        const BuildEvent *b = ctxs[i]->last_build.get();
+        if (b && b != before) cudaStreamWaitEvent(s, b->e, 0);
+        before = b;
+    }
+}
+
+void plan_mark_built(Plan *p, cudaStream_t s) {
+    if (capturing(s)) return;
+    cudaEventRecord(p->built->e, s);
+    for (hb_ctx *c : p->ctxs)
+        if (c->last_build != p->built) c->last_build = p->built;
+}
+
 // One build.  From the third into the same blocks on, the plan's launches (two
 // dozen kernels on four streams and the events between them, 60 us of host
 // time, longer than a small build runs) are replayed as one graph, captured
@@ -1141,9 +1168,7 @@ int plan_error_word(Plan *p, int *word) {
 // caller's workspace (a graph may take device memory of its own), are
 // launched one by one.
 int plan_launch(Plan *p, cudaStream_t s, int *launches, std::string *err) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool plain = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-    if (!plain) cudaGetLastError();
+    const bool plain = !capturing(s);
     bool owned = false;
     for (const hb_ctx *c : p->ctxs) owned = owned || c->pool.base != nullptr;
     if (!plain || owned || p->no_graph) return plan_run(p, s, true, false, launches, err);
