@@ -10,9 +10,11 @@
 namespace hb {
 
 // Make the integral slices (or borrow the base context's), the CI slices of
-// every group with 1..64 states and the term-list row pointers (this runs the
-// class-4 classification once).  S: slices per operand.
-int c4tc_prepare(hb_ctx *ctx, int S, cudaStream_t s);
+// every group with 1..64 states and the term-list row pointers.  Both operands
+// take c4tc_slices(ctx) slices.
+int c4tc_prepare(hb_ctx *ctx, cudaStream_t s);
+// Slices per operand: those of the context that owns the integral tables.
+int c4tc_slices(const hb_ctx *ctx);
 // Whether group g of ctx has tensor-core class-4 operands.
 bool c4tc_group_on(const hb_ctx *ctx, int g);
 // The term-fill and kernel tasks of group g writing into Hlc, with their

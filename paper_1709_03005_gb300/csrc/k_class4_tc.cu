@@ -632,8 +632,11 @@ bool c4tc_group_on(const hb_ctx *ctx, int g) {
 
 int c4tc_min_states(const hb_ctx *ctx) { return ctx->c4_path == 2 ? 1 : 32; }
 
-int c4tc_prepare(hb_ctx *ctx, int S, cudaStream_t s) {
+int c4tc_slices(const hb_ctx *ctx) { return (ctx->base ? ctx->base : ctx)->split_slices; }
+
+int c4tc_prepare(hb_ctx *ctx, cudaStream_t s) {
     if (ctx->c4tc) return HB_OK;
+    const int S = c4tc_slices(ctx);
     if (S < 2 || S > 6) return c4_fail(ctx, HB_ERR_INVALID_ARG, "slices must be 2..6");
     bool any = false;      // nothing to make unless some group takes the tensor-core path
     for (int g = 0; g < ctx->n_groups; ++g) {
@@ -652,7 +655,7 @@ int c4tc_prepare(hb_ctx *ctx, int S, cudaStream_t s) {
     if (c->x_rows >= (1ll << 31)) return c4_fail(ctx, HB_ERR_INVALID_ARG, "integral table too large");
     cudaError_t e = cudaSuccess;
     if (ctx->base) {
-        int rc = c4tc_prepare(ctx->base, S, s);
+        int rc = c4tc_prepare(ctx->base, s);
         if (rc != HB_OK) return c4_fail(ctx, rc, ctx->base->err);
         const C4TC *b = (const C4TC *)ctx->base->c4tc;
         c->xs = b->xs;

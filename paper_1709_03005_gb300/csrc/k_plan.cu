@@ -88,7 +88,7 @@ struct Plan {
     // the expansion on the tensor cores (the mixed build always, the FP64 build
     // where its slices fit the memory), its slices, and those of class 4
     bool split_on = false;
-    int S = 0, c4_slices = 6;
+    int S = 0, c4_slices = 0;
     // panel columns per label class (Kc) and the coefficient slices' width
     // (Kw = every class); perm: the labels of the coefficient slice columns
     // (null without orbital symmetry)
@@ -664,9 +664,14 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
             if (ctxs[i]->gps.empty()) continue;
             rc = mixed_prepare(ctxs[i], precision, s);
             if (rc != HB_OK) { *err = ctxs[i]->err; break; }
-            const int S = mixed_slices(ctxs[i], precision);
-            if (p->S == 0) p->S = S;
-            else if (S != p->S) { rc = HB_ERR_INVALID_ARG; *err = "contexts of one plan use different split_slices"; }
+            // a panel of fewer slices than the plan's reads the leading ones of the coefficient rows
+            p->S = std::max(p->S, mixed_slices(ctxs[i], precision));
+            const int s4 = c4tc_slices(ctxs[i]);
+            if (p->c4_slices == 0) p->c4_slices = s4;
+            else if (precision == HB_MIXED && s4 != p->c4_slices) {
+                rc = HB_ERR_INVALID_ARG;
+                *err = "contexts of one plan use different split_slices";
+            }
         }
         p->split_on = rc == HB_OK && p->S > 0;
         // an FP64 build without room for the slices adds its sums on the FP64 pipe
@@ -674,12 +679,11 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         if (rc != HB_OK) { plan_destroy(p); return rc; }
         p->delta_col = ctxs[0]->delta_pos;   // the delta label's column (class 0 comes first)
     }
-    p->c4_slices = ctxs[0]->split_slices;
     // class 4 on the tensor cores: integral and CI slices, term-list sizes
     if (precision == HB_MIXED)
         for (int i = 0; i < n && rc == HB_OK; ++i) {
             if (ctxs[i]->n_l2 < 1 || ctxs[i]->c4_path == 1) continue;
-            rc = c4tc_prepare(ctxs[i], p->c4_slices, s);
+            rc = c4tc_prepare(ctxs[i], s);
             if (rc != HB_OK) *err = ctxs[i]->err;
         }
     if (precision == HB_MIXED)
