@@ -61,7 +61,7 @@ struct C4TC {
     int64_t x_rows = 0, x_h0 = 0, x_zero = 0;   // rows: (tt|tc) rows, then h^T rows, then a zero row
     int jpad = 0;
     __nv_bfloat16 *xs = nullptr;
-    bool borrowed = false;
+    bool borrowed = false, groups_done = false;
     struct Group {
         bool on = false;
         __nv_bfloat16 *cs = nullptr;            // [S][2 ndet + 1][64]
@@ -634,16 +634,11 @@ int c4tc_min_states(const hb_ctx *ctx) { return ctx->c4_path == 2 ? 1 : 32; }
 
 int c4tc_slices(const hb_ctx *ctx) { return (ctx->base ? ctx->base : ctx)->split_slices; }
 
-int c4tc_prepare(hb_ctx *ctx, cudaStream_t s) {
+// The integral slices of a context, or those it borrows.
+static int c4tc_tables(hb_ctx *ctx, cudaStream_t s) {
     if (ctx->c4tc) return HB_OK;
     const int S = c4tc_slices(ctx);
     if (S < 2 || S > 6) return c4_fail(ctx, HB_ERR_INVALID_ARG, "slices must be 2..6");
-    bool any = false;      // nothing to make unless some group takes the tensor-core path
-    for (int g = 0; g < ctx->n_groups; ++g) {
-        const GroupInfo &Gi = ctx->groups[g];
-        any = any || (Gi.ns >= c4tc_min_states(ctx) && Gi.ns <= TNP && Gi.cn > 0 && Gi.ndet > 0 && ctx->n_l2 > 0);
-    }
-    if (!any) return HB_OK;
     C4TC *c = new C4TC();
     ctx->c4tc = c;
     c->S = S;
@@ -653,33 +648,50 @@ int c4tc_prepare(hb_ctx *ctx, cudaStream_t s) {
     c->x_rows = c->x_zero + 1;
     c->jpad = (ctx->n_co + 7) / 8 * 8;
     if (c->x_rows >= (1ll << 31)) return c4_fail(ctx, HB_ERR_INVALID_ARG, "integral table too large");
-    cudaError_t e = cudaSuccess;
     if (ctx->base) {
-        int rc = c4tc_prepare(ctx->base, s);
+        // whether or not a group of the base context takes the tensor cores itself
+        int rc = c4tc_tables(ctx->base, s);
         if (rc != HB_OK) return c4_fail(ctx, rc, ctx->base->err);
-        const C4TC *b = (const C4TC *)ctx->base->c4tc;
-        c->xs = b->xs;
+        c->xs = ((const C4TC *)ctx->base->c4tc)->xs;
         c->borrowed = true;
-    } else {
-        int *ex = nullptr;
-        e = dmalloc_n(ctx, &ex, (size_t)(ctx->n_co > 0 ? ctx->n_co : 1));
-        if (e == cudaSuccess) e = c4_alloc(ctx, &c->xs, (size_t)S * c->x_rows * c->jpad);
-        if (e != cudaSuccess) {
-            dfree(ctx, ex);
-            return c4_fail(ctx, HB_ERR_OOM, cudaGetErrorString(e));
-        }
-        if (ctx->n_co > 0) {
-            fill_int_kernel<<<(ctx->n_co + 255) / 256, 256, 0, s>>>(ex, ctx->n_co, -2000);
-            x_colexp_kernel<<<(unsigned)((c->x_rows + 63) / 64), 128, 0, s>>>(ctx->tttc, ctx->h, n_tc_rows, ctx->n_to,
-                                                                           ctx->n_co, ctx->n_orb, c->x_rows, ex);
-        }
-        x_slice_kernel<<<(unsigned)((c->x_rows * c->jpad + 255) / 256), 256, 0, s>>>(ctx->tttc, ctx->h, n_tc_rows, ctx->n_to, ctx->n_co, ctx->n_orb, c->x_rows,
-                                            c->jpad, S, ex, c->xs);
-        e = cudaStreamSynchronize(s);
-        dfree(ctx, ex);
-        if (e != cudaSuccess) return c4_fail(ctx, HB_ERR_CUDA, cudaGetErrorString(e));
+        if (!c->xs) return c4_fail(ctx, HB_ERR_OOM, "the base context has none");
+        return HB_OK;
     }
-    e = set_attr<2>();
+    int *ex = nullptr;
+    cudaError_t e = dmalloc_n(ctx, &ex, (size_t)(ctx->n_co > 0 ? ctx->n_co : 1));
+    if (e == cudaSuccess) e = c4_alloc(ctx, &c->xs, (size_t)S * c->x_rows * c->jpad);
+    if (e != cudaSuccess) {
+        dfree(ctx, ex);
+        return c4_fail(ctx, HB_ERR_OOM, cudaGetErrorString(e));
+    }
+    if (ctx->n_co > 0) {
+        fill_int_kernel<<<(ctx->n_co + 255) / 256, 256, 0, s>>>(ex, ctx->n_co, -2000);
+        x_colexp_kernel<<<(unsigned)((c->x_rows + 63) / 64), 128, 0, s>>>(ctx->tttc, ctx->h, n_tc_rows, ctx->n_to,
+                                                                       ctx->n_co, ctx->n_orb, c->x_rows, ex);
+    }
+    x_slice_kernel<<<(unsigned)((c->x_rows * c->jpad + 255) / 256), 256, 0, s>>>(ctx->tttc, ctx->h, n_tc_rows, ctx->n_to, ctx->n_co, ctx->n_orb, c->x_rows,
+                                        c->jpad, S, ex, c->xs);
+    e = cudaStreamSynchronize(s);
+    dfree(ctx, ex);
+    if (e != cudaSuccess) return c4_fail(ctx, HB_ERR_CUDA, cudaGetErrorString(e));
+    return HB_OK;
+}
+
+int c4tc_prepare(hb_ctx *ctx, cudaStream_t s) {
+    if (ctx->c4tc && ((C4TC *)ctx->c4tc)->groups_done) return HB_OK;
+    bool any = false;      // nothing to make unless some group takes the tensor-core path
+    for (int g = 0; g < ctx->n_groups; ++g) {
+        const GroupInfo &Gi = ctx->groups[g];
+        any = any || (Gi.ns >= c4tc_min_states(ctx) && Gi.ns <= TNP && Gi.cn > 0 && Gi.ndet > 0 && ctx->n_l2 > 0);
+    }
+    if (!any) return HB_OK;
+    const int rc = c4tc_tables(ctx, s);
+    C4TC *c = (C4TC *)ctx->c4tc;
+    if (c) c->groups_done = true;
+    // without tables (found no room before, which was reported then) the double-float kernel takes every group
+    if (rc != HB_OK || !c->xs) return rc;
+    const int S = c->S;
+    cudaError_t e = set_attr<2>();
     if (e == cudaSuccess) e = set_attr<3>();
     if (e == cudaSuccess) e = set_attr<4>();
     if (e == cudaSuccess) e = set_attr<5>();

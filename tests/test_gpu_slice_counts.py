@@ -88,3 +88,25 @@ def test_batches(a, b, accepted):
     lib.hb_batch_destroy(handle)
     for h in hams:
         h.close()
+
+
+def test_base_without_a_wide_group():
+    """A base context none of whose groups takes class 4 on the tensor cores lends the tables all the same."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    P = _problem()
+    narrow = synth.make_config("mid", n_co=20, n_state=3, n_l2=60, seed=77)
+    for name in ("h", "eri_tttt", "eri_tttc", "eri_ttcc", "eri_tctc"):
+        setattr(narrow, name, getattr(P, name))
+    want = hb.Hamiltonian(P)
+    ref = _build(want)
+    base = hb.Hamiltonian(narrow)
+    _build(base)
+    H = hb.Hamiltonian(P, base=base)
+    b = _build(H)
+    assert "class4 tensor cores" in H.tuning_report()
+    for k in ("Hcc", "Hlc", "val"):
+        assert torch.equal(b[k], ref[k]), k
+    _build(base)
+    for h in (H, base, want):
+        h.close()
