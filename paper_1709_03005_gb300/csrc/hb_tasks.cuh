@@ -91,8 +91,8 @@ struct ZTask {          // zero n 8-byte words
 struct SortTask {       // stable counting sort of the gamma items by key
     const GammaItem *items;
     int64_t n_items;
-    int nc, n_keys;
-    int64_t *off, *cur;
+    int nc, chunk;            // chunks of the offset table; items of one
+    int64_t *cur;
     int32_t *order;
 };
 
@@ -315,7 +315,9 @@ int64_t blocks_pair_values(int64_t n_pairs, int steps);
 int64_t blocks_tn_partial(int n_rows, int ns, int nsp);
 int64_t blocks_tn_reduce(int ns, int nsp);
 int64_t blocks_zero(int64_t n);
-int64_t blocks_sort(int64_t n_items, int n_keys);
+int64_t blocks_sort(int64_t n_items, int chunk);
+// items per sort chunk: those of the whole list, whose table of chunks a part of
+// it (a shard's rows) then fits
 int sort_chunk_items(int64_t n_items, int n_keys);
 // keys a block (or warp) takes: one, or eight where most hold no items
 int gamma_keys_per(int64_t n_items, int n_keys);

@@ -316,14 +316,14 @@ void fill_tasks(Plan &p) {
                 i0 = ir.first;
                 n_it = ir.second - ir.first;
             }
-            const int nc = P.n_chunks;
+            const int nc = P.n_chunks, chunk = sort_chunk_items(P.n_items, n_keys);
             p.itf.add(IFTask{P.pairs, P.rowptr + m0, nm, da, W, ctx->n_to, ctx->n_elec, P.item_ptr + m0, P.items, i0, nc,
-                             sort_chunk_items(n_it, n_keys), P.sort_off},
+                             chunk, P.sort_off},
                       p.block_rows ? nm : blocks_rows8(nm));
             const int64_t n_off = (int64_t)n_keys * nc;
             GammaItem *its = P.items + i0;
             p.zero.add(ZTask{P.sort_off, n_off + 1}, blocks_zero(n_off + 1));
-            p.sort.add(SortTask{its, n_it, nc, n_keys, P.sort_off, P.sort_cur, P.order}, blocks_sort(n_it, n_keys));
+            p.sort.add(SortTask{its, n_it, nc, chunk, P.sort_cur, P.order}, blocks_sort(n_it, chunk));
             p.scan.add(ScanTask{P.sort_off, n_off, P.sort_cur, P.sort_part}, blocks_scan(n_off));
             p.scan_longest = std::max(p.scan_longest, n_off);
             const int kpb = gamma_keys_per(n_it, n_keys);

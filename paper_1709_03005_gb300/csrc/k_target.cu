@@ -570,7 +570,7 @@ __global__ void sort_scatter_kernel(const SortTask *__restrict__ tasks, const in
     const SortTask T = tasks[ti];
     const int chunk = (int)(blockIdx.x - blk[ti]);
     const int lane = threadIdx.x;
-    const int CS = sort_chunk_size(T.n_items, T.n_keys);
+    const int CS = T.chunk;
     const int64_t base = (int64_t)chunk * CS;
     for (int i0 = 0; i0 < CS; i0 += 32) {
         const int64_t k = base + i0 + lane;
@@ -1033,7 +1033,7 @@ int sort_chunks(int64_t n_items, int n_keys) {
     return (int)((n_items + c - 1) / c);
 }
 int sort_chunk_items(int64_t n_items, int n_keys) { return sort_chunk_size(n_items, n_keys); }
-int64_t blocks_sort(int64_t n_items, int n_keys) { return sort_chunks(n_items, n_keys); }
+int64_t blocks_sort(int64_t n_items, int chunk) { return (n_items + chunk - 1) / chunk; }
 int gamma_keys_per(int64_t n_items, int n_keys) { return n_items < 4 * (int64_t)n_keys ? 8 : 1; }
 int64_t blocks_gamma(int n_keys, int kpb, int ns, int nsp) { return (int64_t)((n_keys + kpb - 1) / kpb) * tn_ny(ns, nsp); }
 int64_t blocks_gamma_warp(int n_keys, int kpb) { return (n_keys + 8 * kpb - 1) / (8 * kpb); }
