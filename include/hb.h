@@ -361,7 +361,7 @@ int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int32_t nranks
    molecule): the integrals, the expansion panel and its tensor-core slices are
    borrowed from `base`, which must outlive this context.  The caller
    guarantees that p's integral arrays equal base's (only their shapes are
-   checked). */
+   checked).  HB_ERR_INVALID_ARG for target groups on a base that has none. */
 int hb_init_shared(hb_ctx **ctx, const hb_problem *p, const hb_options *o, hb_ctx *base, void *stream);
 
 /* Batched build of n staged contexts into outs[0..n) (Section 2.2 classes for

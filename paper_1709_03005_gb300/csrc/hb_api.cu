@@ -484,6 +484,8 @@ int stage_problem(hb_ctx *ctx, const hb_problem *p, const hb_options *o, cudaStr
     const bool shared = ctx->base != nullptr;
     if (shared) {
         // integrals, their tables and the expansion panel belong to the base context
+        if (p->n_groups > 0 && (!ctx->base->panel || !ctx->base->tttc))
+            return fail(ctx, HB_ERR_INVALID_ARG, "the base context has no target groups, and so no continuum integrals to lend");
         ctx->h = ctx->base->h; ctx->tttt = ctx->base->tttt; ctx->tttc = ctx->base->tttc;
         ctx->jk = ctx->base->jk; ctx->panel = ctx->base->panel;
     } else {
