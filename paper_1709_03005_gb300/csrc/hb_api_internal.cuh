@@ -172,6 +172,9 @@ struct hb_ctx {
     // the end of this context's last build: its scratch (records, sort tables,
     // coefficient rows) serves every build, so the next one waits for it
     std::shared_ptr<hb::BuildEvent> last_build;
+    // the tables made on first use (panel slices, double-float copies): a build on
+    // another stream, of this context or of one that borrows them, waits for it
+    std::shared_ptr<hb::BuildEvent> tables_made;
     void *shard_plan = nullptr;   // cached plan of this context's share of a sharded build
     void *diag = nullptr;   // Davidson workspace (k_davidson.cu)
     void *mlp = nullptr;    // learned preconditioner weights (k_mlp.cu)

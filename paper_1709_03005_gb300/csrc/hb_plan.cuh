@@ -34,6 +34,10 @@ int plan_run(hb::Plan *p, cudaStream_t s, bool timing, bool capture, int *launch
 // contexts.  Neither does anything on a stream that is being captured.
 void plan_wait_last(hb_ctx *const *ctxs, int n, cudaStream_t s);
 void plan_mark_built(hb::Plan *p, cudaStream_t s);
+// Around what makes tables of a context and its base on s: behind what was made
+// of them before, and recorded for what reads them next.
+void plan_wait_tables(hb_ctx *ctx, cudaStream_t s);
+void plan_mark_tables(hb_ctx *ctx, cudaStream_t s);
 // a whole build, replayed as a graph where the same one is repeated
 int plan_launch(hb::Plan *p, cudaStream_t s, int *launches, std::string *err);
 // After the stream has finished a timed run: per-stage times and counters.

@@ -645,6 +645,18 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         plan_destroy(p);
         return HB_ERR_CUDA;
     }
+    // the tables below may have been made on another stream, by a build that is still running
+    struct TableOrder {
+        hb_ctx *const *ctxs;
+        int n;
+        cudaStream_t s;
+        TableOrder(hb_ctx *const *c, int n_, cudaStream_t s_) : ctxs(c), n(n_), s(s_) {
+            for (int i = 0; i < n; ++i) plan_wait_tables(ctxs[i], s);
+        }
+        ~TableOrder() {
+            for (int i = 0; i < n; ++i) plan_mark_tables(ctxs[i], s);
+        }
+    } order(ctxs, n, s);
     bool any_pairs = false;
     for (int i = 0; i < n; ++i) any_pairs = any_pairs || !ctxs[i]->gps.empty();
     // the FP64 build's slices come out of a caller's workspace only where that
@@ -1155,6 +1167,24 @@ void plan_wait_last(hb_ctx *const *ctxs, int n, cudaStream_t s) {
         const BuildEvent *b = ctxs[i]->last_build.get();
         if (b && b != before) cudaStreamWaitEvent(s, b->e, 0);
         before = b;
+    }
+}
+
+void plan_wait_tables(hb_ctx *ctx, cudaStream_t s) {
+    if (capturing(s)) return;
+    for (const hb_ctx *c : {ctx, ctx->base})
+        if (c && c->tables_made) cudaStreamWaitEvent(s, c->tables_made->e, 0);
+}
+
+void plan_mark_tables(hb_ctx *ctx, cudaStream_t s) {
+    if (capturing(s)) return;
+    for (hb_ctx *c : {ctx, ctx->base}) {
+        if (!c) continue;
+        if (!c->tables_made) {
+            c->tables_made = std::make_shared<BuildEvent>();
+            cudaEventCreateWithFlags(&c->tables_made->e, cudaEventDisableTiming);
+        }
+        cudaEventRecord(c->tables_made->e, s);
     }
 }
 

@@ -52,3 +52,32 @@ def test_base_without_groups():
         assert torch.equal(b[k], ref[k]), k
     H.close()
     B.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tables_made_on_another_stream(precision):
+    """The first build of a borrowing context, on another stream, beside the base's
+    first build (or contraction) that makes the tables and is held up ahead of them."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    base, P = _base_and_problem()
+    ref = _reference(P, precision)
+    B = hb.Hamiltonian(base)
+    H = hb.Hamiltonian(P, base=B)
+    out = H.allocate()
+    x, part = B.allocate(), torch.empty(B.shard_coef_len(), dtype=torch.float64, device="cuda")
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(400_000_000)          # 0.2 s
+        if precision == 0:
+            B.build(0, x, stream=a, stats=False)
+        else:
+            B.build_contract(1, 0, 1, part, stream=a)
+    H.build(precision, out, stream=b, stats=False)
+    b.synchronize()
+    for k in KEYS:
+        assert torch.equal(out[k], ref[k]), k
+    torch.cuda.synchronize()
+    H.close()
+    B.close()
