@@ -269,8 +269,9 @@ int hb_query(const hb_ctx *ctx, hb_layout *out);
    hb_set_workspace gives the context a device buffer of `bytes` bytes that the
    caller owns and keeps alive until hb_destroy (or until the context is no
    longer used).  Whatever a previous build or solve had set up is released
-   first.  A build or solve whose set-up does not fit returns HB_ERR_OOM.  A
-   workspace can be set once per context.  Errors: HB_ERR_INVALID_ARG (NULL,
+   first, but for tables that a batch of the context reads.  A build or solve
+   whose set-up does not fit returns HB_ERR_OOM.  A workspace can be set once
+   per context.  Errors: HB_ERR_INVALID_ARG (NULL,
    a workspace already set), HB_ERR_CUDA. */
 int hb_workspace_size(hb_ctx *ctx, int32_t precision, int32_t diag_k, int32_t precond, int64_t *bytes,
                       void *stream);

@@ -355,6 +355,7 @@ extern "C" int hb_init_shared(hb_ctx **out, const hb_problem *p, const hb_option
         return fail(nullptr, HB_ERR_INVALID_ARG, "problem orbitals differ from the base context");
     hb_ctx *ctx = new hb_ctx();
     ctx->base = base;
+    ctx->base_gen = base->tables_gen;
     int rc = init_context(ctx, p, o, (cudaStream_t)stream);
     if (rc != HB_OK) { g_last_error = ctx->err; hb_destroy(ctx); return rc; }
     *out = ctx;
@@ -727,6 +728,7 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
         return fail(ctx, HB_ERR_INVALID_ARG, "L2 CSR arrays are NULL");
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
+    refresh_borrowed(ctx);
     // the build as a plan of grouped launches over this context's group pairs,
     // kept between builds (made again for another precision, re-pointed for
     // other output blocks)
@@ -890,6 +892,7 @@ extern "C" int hb_build_contract(hb_ctx *ctx, int32_t precision, int32_t rank, i
     CK(cudaSetDevice(ctx->device));
     // the contraction writes no output block: a cached plan of this share is
     // used as it is, a new one is made without outputs
+    refresh_borrowed(ctx);
     plan_wait_last(&ctx, 1, s);
     hb::Plan *p = (hb::Plan *)ctx->shard_plan;
     if (!p || !plan_is_shard(p, precision, rank, nranks)) {
@@ -934,6 +937,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     hb::Plan *p = nullptr;
+    refresh_borrowed(ctx);
     plan_wait_last(&ctx, 1, s);
     rc = shard_plan(ctx, precision, rank, nranks, out, &p, s);
     if (rc != HB_OK) return rc;
@@ -1082,8 +1086,14 @@ extern "C" const char *hb_last_error(const hb_ctx *ctx) {
     return ctx ? ctx->err.c_str() : g_last_error.c_str();
 }
 
+// A context that borrows tables its base has released since lets go of what it
+// made from them; its next build makes both again.
+void hb::refresh_borrowed(hb_ctx *ctx) {
+    if (ctx->base && ctx->base_gen != ctx->base->tables_gen) release_lazy(ctx);
+}
+
 void hb::release_lazy(hb_ctx *ctx) {
-    if (ctx->plan || ctx->shard_plan) cudaDeviceSynchronize();
+    cudaDeviceSynchronize();      // builds of this context, of borrowing ones and of batches
     if (ctx->plan) {
         plan_destroy((hb::Plan *)ctx->plan);
         ctx->plan = nullptr;
@@ -1092,9 +1102,12 @@ void hb::release_lazy(hb_ctx *ctx) {
         plan_destroy((hb::Plan *)ctx->shard_plan);
         ctx->shard_plan = nullptr;
     }
+    hb::release_diag(ctx);
+    if (*ctx->batches > 0) return;
+    ++ctx->tables_gen;
+    if (ctx->base) ctx->base_gen = ctx->base->tables_gen;
     release_mixed(ctx);
     hb::release_c4tc(ctx);
-    hb::release_diag(ctx);
     // the double-float copies (ensure_df) are the allocations after hb_init's
     const size_t n0 = ctx->pool.init_allocs;
     if (ctx->allocs.size() > n0) {

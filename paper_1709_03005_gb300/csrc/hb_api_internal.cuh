@@ -82,6 +82,7 @@ cudaError_t dmalloc_n(hb_ctx *ctx, T **p, size_t n) {
 // Drop the build plan, tensor-core operands, double-float copies and solver
 // scratch of a context (they are made again on next use).
 void release_lazy(hb_ctx *ctx);
+void refresh_borrowed(hb_ctx *ctx);
 
 // Target groups as the build sees them when some groups are given over CSFs
 // or share their determinants (k_csf.cu): merged groups with zeroed host CI
@@ -175,6 +176,12 @@ struct hb_ctx {
     // the tables made on first use (panel slices, double-float copies): a build on
     // another stream, of this context or of one that borrows them, waits for it
     std::shared_ptr<hb::BuildEvent> tables_made;
+    // Batches whose launch graph reads those tables of this context: while there
+    // are any, release_lazy keeps them.  tables_gen counts the releases; a context
+    // that borrows them (base_gen: the count it borrowed at) lets go of what it
+    // made from released ones before its next build (refresh_borrowed).
+    std::shared_ptr<int> batches = std::make_shared<int>(0);
+    int64_t tables_gen = 0, base_gen = 0;
     void *shard_plan = nullptr;   // cached plan of this context's share of a sharded build
     void *diag = nullptr;   // Davidson workspace (k_davidson.cu)
     void *mlp = nullptr;    // learned preconditioner weights (k_mlp.cu)

@@ -20,6 +20,7 @@ struct hb_batch {
     hb::Plan *plan = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    std::vector<std::shared_ptr<int>> members;   // the member contexts' and their bases' counts of batches
     size_t nodes = 0;
     int launches = 0;
 };
@@ -39,6 +40,7 @@ void batch_free(hb_batch *b) {
         cudaDeviceSynchronize();
         plan_destroy(b->plan);
     }
+    for (auto &m : b->members) --*m;
     delete b;
 }
 }  // namespace
@@ -56,10 +58,17 @@ extern "C" int hb_batch_create(hb_batch **out, hb_ctx *const *ctxs, int32_t n, i
     b->outs.assign(outs, outs + n);
     cudaStream_t s = (cudaStream_t)stream;
     std::string err;
+    for (int i = 0; i < n; ++i) hb::refresh_borrowed(ctxs[i]);
+    for (int i = 0; i < n; ++i)
+        for (hb_ctx *c : {ctxs[i], ctxs[i]->base})
+            if (c) {
+                ++*c->batches;
+                b->members.push_back(c->batches);
+            }
     plan_wait_last(ctxs, n, s);
     // the plan prepares the tensor-core operands and uploads its task tables
     int rc = plan_create(ctxs, n, outs, precision, &b->plan, &err, s);
-    if (rc != HB_OK) { delete b; return bfail(rc, err); }
+    if (rc != HB_OK) { batch_free(b); return bfail(rc, err); }
     // pick the launch shapes by timing them on this batch's own tasks
     rc = plan_autotune(b->plan, s, &err);
     if (rc != HB_OK) { batch_free(b); return bfail(rc, err); }

@@ -81,3 +81,74 @@ def test_tables_made_on_another_stream(precision):
     torch.cuda.synchronize()
     H.close()
     B.close()
+
+
+def _overwrite_freed():
+    """Fill what the device has just been given back with NaN patterns."""
+    import torch
+    x = [torch.full((1 << 20,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(64)]
+    torch.cuda.synchronize()
+    del x
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tables_released_by_the_base(precision):
+    """The base measures and takes a workspace, which releases the tables it had
+    lent: the borrowing context's builds, replayed ones too, do not read them any more."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    base, P = _base_and_problem()
+    ref, ref_base = _reference(P, precision), _reference(base, precision)
+    B = hb.Hamiltonian(base)
+    H = hb.Hamiltonian(P, base=B)
+    out = H.allocate()
+    for _ in range(4):
+        H.build(precision, out)
+    need = B.workspace_size(precision)
+    _overwrite_freed()
+    out["Hcc"].fill_(0.0)
+    H.build(precision, out)
+    torch.cuda.synchronize()
+    for k in KEYS:
+        assert torch.equal(out[k], ref[k]), k
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    B.set_workspace(ws)
+    _overwrite_freed()
+    x, _ = B.build(precision)
+    out["Hcc"].fill_(0.0)
+    H.build(precision, out)
+    torch.cuda.synchronize()
+    for k in KEYS:
+        assert torch.equal(out[k], ref[k]) and torch.equal(x[k], ref_base[k]), k
+    H.close()
+    B.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tables_of_a_batch_stay(precision):
+    """Members of a batch measure and take a workspace: the batch's graph still reads their tables."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    base, P = _base_and_problem()
+    B = hb.Batch([base, P], precision)
+    B.launch()
+    torch.cuda.synchronize()
+    ref = [{k: v.clone() for k, v in b.items()} for b in B.blocks]
+    ws = []
+    for h in B.hams:
+        ws.append(torch.empty(h.workspace_size(precision), dtype=torch.uint8, device="cuda"))
+        h.set_workspace(ws[-1])
+    _overwrite_freed()
+    for b in B.blocks:
+        b["Hcc"].fill_(0.0)
+    B.launch()
+    torch.cuda.synchronize()
+    for b, r in zip(B.blocks, ref):
+        for k in KEYS:
+            assert torch.equal(b[k], r[k]), k
+    for h, r in zip(B.hams, ref):
+        b, _ = h.build(precision)
+        torch.cuda.synchronize()
+        for k in KEYS:
+            assert torch.equal(b[k], r[k]), k
+    B.close()
