@@ -715,7 +715,12 @@ extern "C" int64_t hb_group_offset(const hb_ctx *ctx, int32_t g) {
     return g == ctx->n_groups ? ctx->Dc : ctx->groups[g].row_off;
 }
 
-static const char *const kF64Timeout = "a tensor-core kernel of an FP64 build gave up waiting";
+// An FP64 build is left running; a wait that gave up in it is reported by the
+// call that waits for it, or by the next one.
+static std::string gave_up(const char *which, int word) {
+    return std::string("a tensor-core kernel of ") + which + " gave up waiting (split expansion: codes 1-6, class 4: codes 21-26; code " +
+           std::to_string(word) + ")";
+}
 
 extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *out, hb_stats *st,
                                void *stream) {
@@ -735,6 +740,7 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
     hb::Plan *plan = (hb::Plan *)ctx->plan;
     std::string err;
     plan_wait_last(&ctx, 1, s);
+    if (const int w = plan_last_error(ctx)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build before this one", w));
     if (plan && plan_precision(plan) != precision) {
         cudaStreamSynchronize(s);
         plan_destroy(plan);
@@ -754,24 +760,18 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
         int rc = plan_set_outputs(plan, out, &err, s);
         if (rc != HB_OK) return fail(ctx, rc, err);
     }
-    // an FP64 build is left running; a wait that gave up in it is reported by
-    // the call that waits for it, or by the next one
-    if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
+    plan_clear_error(plan, s);
     int launches = 0;
     int rc = plan_launch(plan, s, &launches, &err);
     plan_mark_built(plan, s);
     if (rc != HB_OK) return fail(ctx, rc, err);
     if (precision == HB_MIXED) {
-        // the tensor-core kernel reports a bounded-wait timeout in a device word
-        int word = 0;
         CK(cudaStreamSynchronize(s));
-        if (plan_error_word(plan, &word) != HB_OK) return fail(ctx, HB_ERR_CUDA, "reading the mixed error word");
-        if (word != 0)
-            return fail(ctx, HB_ERR_TIMEOUT, "a tensor-core kernel (split expansion, codes 1-6, or class 4, codes 21-26) gave up waiting (code " + std::to_string(word) + ")");
+        if (const int w = plan_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build", w));
     }
     if (st) {
         plan_stats(plan, st);                    // waits for the build
-        if (plan_host_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
+        if (const int w = plan_error(plan)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build", w));
     }
     return HB_OK;
 }
@@ -894,12 +894,14 @@ extern "C" int hb_build_contract(hb_ctx *ctx, int32_t precision, int32_t rank, i
     // used as it is, a new one is made without outputs
     refresh_borrowed(ctx);
     plan_wait_last(&ctx, 1, s);
+    if (const int w = plan_last_error(ctx)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build before this one", w));
     hb::Plan *p = (hb::Plan *)ctx->shard_plan;
     if (!p || !plan_is_shard(p, precision, rank, nranks)) {
         hb_blocks none{};
         rc = shard_plan(ctx, precision, rank, nranks, &none, &p, s);
         if (rc != HB_OK) return rc;
     }
+    plan_clear_error(p, s);
     // the stage timers belong to whole builds: this phase runs untimed
     plan_set_phase(p, 1);
     std::string err;
@@ -939,6 +941,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
     hb::Plan *p = nullptr;
     refresh_borrowed(ctx);
     plan_wait_last(&ctx, 1, s);
+    if (const int w = plan_last_error(ctx)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build before this one", w));
     rc = shard_plan(ctx, precision, rank, nranks, out, &p, s);
     if (rc != HB_OK) return rc;
     // the summed coefficient rows of all ranks in place of this rank's
@@ -949,7 +952,7 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
         if (precision == HB_MIXED && P.A_df) split_df(P.A, (int64_t)n, P.A_df, s);
         off += (int64_t)n;
     }
-    if (plan_host_error(p)) return fail(ctx, HB_ERR_TIMEOUT, kF64Timeout);
+    plan_clear_error(p, s);
     plan_set_phase(p, 2);
     std::string err;
     int launches = 0;
@@ -958,10 +961,8 @@ extern "C" int hb_build_expand(hb_ctx *ctx, int32_t precision, int32_t rank, int
     plan_mark_built(p, s);
     if (rc != HB_OK) return fail(ctx, rc, err);
     if (precision == HB_MIXED) {
-        int word = 0;
         CK(cudaStreamSynchronize(s));
-        if (plan_error_word(p, &word) != HB_OK) return fail(ctx, HB_ERR_CUDA, "reading the mixed error word");
-        if (word != 0) return fail(ctx, HB_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (code " + std::to_string(word) + ")");
+        if (const int w = plan_error(p)) return fail(ctx, HB_ERR_TIMEOUT, gave_up("the build", w));
     }
     if (st) {
         memset(st, 0, sizeof(*st));

@@ -51,6 +51,12 @@ struct MixedState;   // split-precision operands (k_split.cu)
 // and the contexts whose last build it was.
 struct BuildEvent {
     cudaEvent_t e = nullptr;
+    // the build's error words (split expansion, class 4; nonzero: a wait gave up),
+    // copied behind it into the plan's page-locked memory, kept here once that is gone
+    int kept[2] = {0, 0};
+    volatile int *err = kept;
+    int injected = 0, inject_next = 0;     // test hook: the error of this build, of the next one
+    int word() const { return err[0] ? err[0] : (err[1] ? err[1] : injected); }
     ~BuildEvent() { if (e) cudaEventDestroy(e); }
 };
 
@@ -173,6 +179,7 @@ struct hb_ctx {
     // the end of this context's last build: its scratch (records, sort tables,
     // coefficient rows) serves every build, so the next one waits for it
     std::shared_ptr<hb::BuildEvent> last_build;
+    bool error_told = false;     // the caller knows of that build's error
     // the tables made on first use (panel slices, double-float copies): a build on
     // another stream, of this context or of one that borrows them, waits for it
     std::shared_ptr<hb::BuildEvent> tables_made;

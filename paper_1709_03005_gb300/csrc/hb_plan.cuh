@@ -24,8 +24,13 @@ bool plan_is_shard(const hb::Plan *p, int precision, int r, int n);
 int plan_set_outputs(hb::Plan *p, const hb_blocks *outs, std::string *err, cudaStream_t s);
 bool plan_outputs_equal(const hb::Plan *p, const hb_blocks *outs);
 int plan_precision(const hb::Plan *p);
-// FP64 build on the tensor cores: nonzero once if a wait in a finished build gave up
-int plan_host_error(hb::Plan *p);
+// Error word of the context's last build, once: 0 after the call that returned it
+// (whichever call of the interface that was), or while the build runs.
+int plan_last_error(hb_ctx *ctx);
+// The same of the build of p that the caller has just waited for.
+int plan_error(hb::Plan *p);
+// Before a launch of p on s: zero the words of an error that has been returned.
+void plan_clear_error(hb::Plan *p, cudaStream_t s);
 // Issue every stage on stream s.  timing: record the stage events (as graph
 // event nodes when capture is set).  *launches: kernels launched.
 int plan_run(hb::Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, std::string *err);
@@ -49,6 +54,4 @@ int plan_autotune(hb::Plan *p, cudaStream_t s, std::string *err);
 bool plan_tuned(const hb::Plan *p);
 // The launch shapes in use, as text.
 std::string plan_report(const hb::Plan *p);
-// Bounded-wait status word of the tensor-core kernel (0: fine).
-int plan_error_word(hb::Plan *p, int *word);
 void plan_destroy(hb::Plan *p);

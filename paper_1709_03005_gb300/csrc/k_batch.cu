@@ -23,6 +23,7 @@ struct hb_batch {
     std::vector<std::shared_ptr<int>> members;   // the member contexts' and their bases' counts of batches
     size_t nodes = 0;
     int launches = 0;
+    bool launched = false, error_told = false;   // the caller knows of the last launch's error
 };
 
 namespace {
@@ -107,16 +108,23 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
     if (!b || !b->exec) return bfail(HB_ERR_INVALID_ARG, "batch is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (b->launched && !b->error_told)
+        if (const int w = plan_error(b->plan)) {
+            b->error_told = true;
+            return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel of the launch before this one gave up waiting (code " + std::to_string(w) + ")");
+        }
     plan_wait_last(b->ctxs.data(), (int)b->ctxs.size(), s);
     if (st) {
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         cudaEventRecord(e0, s);
     }
-    if (plan_host_error(b->plan)) return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel of an FP64 build gave up waiting");
+    plan_clear_error(b->plan, s);
     cudaError_t e = cudaGraphLaunch(b->exec, s);
     if (e != cudaSuccess) return bfail(HB_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(e));
     plan_mark_built(b->plan, s);
+    b->launched = true;
+    b->error_told = false;
     if (st) {
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
@@ -131,9 +139,10 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
     if (b->precision == HB_MIXED) {
         e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bfail(HB_ERR_CUDA, cudaGetErrorString(e));
-        int word = 0;
-        if (plan_error_word(b->plan, &word) != HB_OK) return bfail(HB_ERR_CUDA, "reading the mixed error word");
-        if (word) return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (code " + std::to_string(word) + ")");
+        if (const int w = plan_error(b->plan)) {
+            b->error_told = true;
+            return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (code " + std::to_string(w) + ")");
+        }
     }
     return HB_OK;
 }

@@ -146,7 +146,8 @@ struct Plan {
     int64_t coef_rows = 0;
     int *err = nullptr;
     // the error words as of the last finished build (page-locked, behind the
-    // staged tables)
+    // staged tables; built->err).  On the device they stay set until the error has
+    // been returned, so that no build that follows hides it
     int *host_err = nullptr;
     // the plan as a graph, for builds repeated into the same blocks (plan_launch)
     cudaGraphExec_t exec = nullptr;
@@ -555,6 +556,15 @@ void bind_all(Plan &p) {
     p.d_c4items = (const C4Item *)(p.dev + p.off_c4items);
 }
 
+// The error words out of the page-locked memory, which is about to go.
+void release_words(Plan &p) {
+    if (!p.host_err) return;
+    cudaEventSynchronize(p.built->e);
+    for (int i = 0; i < 2; ++i) p.built->kept[i] = p.built->err[i];
+    p.built->err = p.built->kept;
+    p.host_err = nullptr;
+}
+
 // Copy the packed tables through the pinned staging buffer (which is reused
 // only after the previous copy from it has finished).
 int upload(Plan &p, std::string *err, cudaStream_t s) {
@@ -562,6 +572,7 @@ int upload(Plan &p, std::string *err, cudaStream_t s) {
     if (p.upload_pending) e = cudaEventSynchronize(p.uploaded);
     p.upload_pending = false;
     if (e == cudaSuccess && p.host.size() > p.dev_size) {
+        release_words(p);
         if (p.dev) dfree(p.ctxs[0], p.dev);
         if (p.pinned) cudaFreeHost(p.pinned);
         p.dev = nullptr;
@@ -574,7 +585,9 @@ int upload(Plan &p, std::string *err, cudaStream_t s) {
         if (e == cudaSuccess) {
             p.dev_size = p.host.size();
             p.host_err = (int *)(p.pinned + tables);
-            p.host_err[0] = p.host_err[1] = 0;
+            p.host_err[0] = p.built->kept[0];
+            p.host_err[1] = p.built->kept[1];
+            p.built->err = p.host_err;
         }
     }
     if (e == cudaSuccess && !p.host.empty()) {
@@ -753,10 +766,28 @@ bool plan_outputs_equal(const Plan *p, const hb_blocks *outs) {
 }
 
 int plan_precision(const Plan *p) { return p->precision; }
-int plan_host_error(Plan *p) {
-    const int w = p->host_err ? *(volatile int *)p->host_err : 0;
-    if (w) *p->host_err = 0;
+
+int plan_last_error(hb_ctx *ctx) {
+    if (!ctx->last_build || ctx->error_told) return 0;
+    const int w = ctx->last_build->word();
+    ctx->error_told = w != 0;
     return w;
+}
+
+int plan_error(Plan *p) {
+    const int w = p->built->word();
+    if (w)
+        for (hb_ctx *c : p->ctxs)
+            if (c->last_build == p->built) c->error_told = true;
+    return w;
+}
+
+void plan_clear_error(Plan *p, cudaStream_t s) {
+    BuildEvent &b = *p->built;
+    if (b.word() == 0) return;
+    cudaEventSynchronize(b.e);             // builds enqueued before the error was known have copied it too
+    b.err[0] = b.err[1] = b.injected = 0;
+    cudaMemsetAsync(p->err, 0, 2 * sizeof(int), s);
 }
 
 static void drop_graph(Plan *p) {
@@ -919,6 +950,7 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
             ch.gamma_warp[kv.first] = mb < kGain * mw ? 0 : 1;     // the warp form unless clearly slower
         }
     }
+    cudaMemsetAsync(p->err, 0, 2 * sizeof(int), s);     // a candidate's errors are not a build's
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { *err = std::string("autotune: ") + cudaGetErrorString(e); return HB_ERR_CUDA; }
     drop_graph(p);
@@ -1008,7 +1040,6 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         L += g_l2_mirror(p->l2m.g, s2);
         rec_on(p->ev[4], s2);
         if (p->c4t.g.blocks > 0) {
-            cudaMemsetAsync(p->err + 1, 0, sizeof(int), s2);
             L += g_c4fill(p->c4f.g, s2);
             L += g_c4tc(p->c4t.g, p->d_c4items, (int)p->c4items.size(), p->c4_slices, p->err + 1, s2);
         }
@@ -1023,7 +1054,6 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     // target side (Eq. 8) in three chains that meet at the coefficient rows:
     // the diagonal gamma needs only the determinants and CI vectors
     cudaStreamWaitEvent(sb, p->fork, 0);
-    if (ph2 && p->coef_rows > 0) cudaMemsetAsync(p->err, 0, sizeof(int), sb);
     if (ph1) {
         L += g_gdiag(p->gdp.g, p->gdr.g, p->smem_gd, DF, sb);
         L += g_classify(p->cls_tt.g, W, 0, s);
@@ -1103,7 +1133,7 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
     cudaStreamWaitEvent(s, p->join_main, 0);
     cudaStreamWaitEvent(s, p->join, 0);
     rec(p->ev[6]);
-    if (p->host_err && (p->split_on || p->precision == HB_MIXED))
+    if (p->host_err && ph2 && (p->split_on || p->precision == HB_MIXED))
         cudaMemcpyAsync(p->host_err, p->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaGetLastError();
     p->launches = L;
@@ -1144,15 +1174,6 @@ void plan_stats(Plan *p, hb_stats *st) {
     }
 }
 
-int plan_error_word(Plan *p, int *word) {
-    *word = 0;
-    if (!p->err) return HB_OK;
-    if (!p->host_err) return HB_OK;
-    const volatile int *w = p->host_err;      // copied behind the build, which the caller has waited for
-    *word = w[0] ? w[0] : w[1];
-    return HB_OK;
-}
-
 static bool capturing(cudaStream_t s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
@@ -1191,8 +1212,12 @@ void plan_mark_tables(hb_ctx *ctx, cudaStream_t s) {
 void plan_mark_built(Plan *p, cudaStream_t s) {
     if (capturing(s)) return;
     cudaEventRecord(p->built->e, s);
-    for (hb_ctx *c : p->ctxs)
+    p->built->injected = p->built->inject_next;
+    p->built->inject_next = 0;
+    for (hb_ctx *c : p->ctxs) {
         if (c->last_build != p->built) c->last_build = p->built;
+        c->error_told = false;
+    }
 }
 
 // One build.  From the third into the same blocks on, the plan's launches (two
@@ -1240,6 +1265,7 @@ void plan_destroy(Plan *p) {
     if (!p) return;
     drop_graph(p);
     if (p->upload_pending) cudaEventSynchronize(p->uploaded);
+    release_words(*p);
     for (cudaEvent_t e : p->ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : p->ev_split)
@@ -1265,6 +1291,14 @@ void plan_destroy(Plan *p) {
     }
     if (p->pinned) cudaFreeHost(p->pinned);
     delete p;
+}
+
+// Test hook (host only, not part of the interface): the error word of the
+// context's last build, or of its plan's next one, as if a wait had given up.
+extern "C" int hb_test_build_error(hb_ctx *ctx, int word, int next) {
+    if (!ctx || !ctx->last_build) return HB_ERR_INVALID_ARG;
+    (next ? ctx->last_build->inject_next : ctx->last_build->injected) = word;
+    return HB_OK;
 }
 
 // Test hook (host only, not part of the interface): the tile width and K stage
