@@ -290,7 +290,11 @@ int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
    and the other class-4 groups in double-float on the FP32 pipes; classes 2
    and 8 in FP64.  The results are written as FP64.  `st` may be NULL.
    Errors: HB_ERR_INVALID_ARG, HB_ERR_OOM, HB_ERR_CUDA, HB_ERR_TIMEOUT (a
-   bounded wait of a tensor-core kernel gave up). */
+   bounded wait of a tensor-core kernel gave up: blocks are incomplete).  An
+   FP64 build with st == NULL, a sharded one and a batch launched so are left
+   running when the call returns; their HB_ERR_TIMEOUT comes, once, from the
+   next call for the context (or the batch) that builds, which then builds
+   nothing, or from hb_diag. */
 int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *out, hb_stats *st,
                     void *stream);
 
@@ -304,7 +308,8 @@ int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *out, hb_sta
    largest wanted residual has not halved over 10 iterations (counted in
    st->mlp_fallbacks).  Returns
    HB_ERR_NOT_CONVERGED after max_iter iterations (evals then hold the current
-   Ritz values). */
+   Ritz values), HB_ERR_TIMEOUT if a wait gave up in a product, or in the
+   context's last build and no call has returned that yet. */
 int hb_diag(hb_ctx *ctx, const hb_blocks *H, int32_t k, double tol, int32_t max_iter,
             int32_t precond, const double *v0, double *evals, double *evecs, hb_stats *st,
             void *stream);

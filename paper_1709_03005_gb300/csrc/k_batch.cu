@@ -139,6 +139,8 @@ extern "C" int hb_batch_launch(hb_batch *b, hb_stats *st, void *stream) {
     if (b->precision == HB_MIXED) {
         e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bfail(HB_ERR_CUDA, cudaGetErrorString(e));
+    }
+    if (b->precision == HB_MIXED || st) {        // the launch has been waited for
         if (const int w = plan_error(b->plan)) {
             b->error_told = true;
             return bfail(HB_ERR_TIMEOUT, "a tensor-core kernel gave up waiting (code " + std::to_string(w) + ")");

@@ -22,6 +22,7 @@
 
 #include "hb_api_internal.cuh"
 #include "hb_davidson.cuh"
+#include "hb_plan.cuh"
 
 using namespace hb;
 
@@ -1185,6 +1186,13 @@ extern "C" int hb_diag(hb_ctx *ctx, const hb_blocks *H, int32_t k, double tol, i
     std::vector<double> dh(n);
     cudaMemcpyAsync(dh.data(), w->d, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
+    // an FP64 build may have been left running: its error is known now
+    if (const int word = plan_last_error(ctx)) {
+        if (tensor) release_tensor_products(ctx, w);
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return diag_fail(ctx, HB_ERR_TIMEOUT, "a tensor-core kernel of the build gave up waiting (code " + std::to_string(word) + ")");
+    }
     const int64_t ld = n;
     // --- initial block
     int m = 0;

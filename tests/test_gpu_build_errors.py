@@ -100,3 +100,42 @@ def test_shard_is_told_once(precision):
     H.build_expand(precision, 0, 1, red, x)
     _same(x, ref)
     H.close()
+
+
+def test_solve_after_a_failed_fp64_build():
+    from paper_1709_03005_gb300 import hb
+    H = hb.Hamiltonian(synth.make_config("c1"))
+    x, _ = H.build(0)
+    ref, _, _ = H.diag(x, 2)
+    for flags in (hb.HB_PRECOND_DIAG, hb.HB_PRECOND_DIAG | hb.HB_DIAG_TENSOR):
+        _inject(H, 5, 1)
+        H.build(0, x, stats=False)
+        _times_out(lambda: H.diag(x, 2, precond=flags))
+        ev, _, _ = H.diag(x, 2)
+        assert (ev == ref).all()
+    H.close()
+
+
+def test_change_of_precision_after_a_failed_fp64_build():
+    from paper_1709_03005_gb300 import hb
+    H = hb.Hamiltonian(synth.make_config("c1"))
+    ref, _ = H.build(1)
+    x, _ = H.build(0)
+    _inject(H, 5, 1)
+    H.build(0, x, stats=False)
+    _times_out(lambda: H.build(1, x))
+    H.build(1, x)
+    _same(x, ref)
+    H.close()
+
+
+def test_fp64_batch_that_waits():
+    from paper_1709_03005_gb300 import hb
+    B = hb.Batch([synth.make_config("c1")], 0)
+    B.launch()
+    ref = {k: v.clone() for k, v in B.blocks[0].items()}
+    _inject(B.hams[0], 5, 1)
+    _times_out(B.launch)
+    B.launch()
+    _same(B.blocks[0], ref)
+    B.close()
