@@ -1205,27 +1205,25 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     // of each row's class
     const int Kc = ctx->Kc;
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)PS.slices * rows * Kc;
-    cudaError_t e = dmalloc(ctx, (void **)&PS.buf, bytes);
-    if (e == cudaSuccess && precision == HB_FP64) {
-        e = dmalloc_n(ctx, &PS.exps, (size_t)rows);
-        if (e != cudaSuccess) {
-            dfree(ctx, PS.buf);
-            PS.buf = nullptr;
+    const size_t extra = precision == HB_MIXED ? sizeof(float2) * (size_t)ctx->n_co * Kc : sizeof(int16_t) * (size_t)rows;
+    // everything that can fail comes before the kernels; a failure leaves nothing behind
+    auto undo = [&](int code, const std::string &m) {
+        dfree(ctx, PS.buf);
+        dfree(ctx, PS.exps);
+        PS.buf = nullptr;
+        PS.exps = nullptr;
+        if (precision == HB_MIXED) {
+            dfree(ctx, M.pdiag);
+            M.pdiag = nullptr;
         }
-    }
+        return mixed_fail(ctx, code, m);
+    };
+    cudaError_t e = dmalloc(ctx, (void **)&PS.buf, bytes);
+    if (e == cudaSuccess) e = precision == HB_MIXED ? dmalloc(ctx, (void **)&M.pdiag, extra) : dmalloc(ctx, (void **)&PS.exps, extra);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return mixed_fail(ctx, HB_ERR_OOM, std::string("panel slices: ") + cudaGetErrorString(e));
+        return undo(HB_ERR_OOM, std::string("panel slices: ") + cudaGetErrorString(e));
     }
-    ctx->dev_bytes += bytes + (PS.exps ? sizeof(int16_t) * (size_t)rows : 0);
-    if (precision == HB_MIXED) {
-        e = dmalloc_n(ctx, &M.pdiag, (size_t)ctx->n_co * Kc);
-        if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_OOM, std::string("panel rows: ") + cudaGetErrorString(e));
-        ctx->dev_bytes += sizeof(float2) * (size_t)ctx->n_co * Kc;
-        panel_diag_df_kernel<<<ctx->n_co, 256, 0, s>>>(ctx->panel, ctx->n_co, Kc, M.pdiag);
-    }
-    slice_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ctx->panel, rows, Kc, PS.slices, ctx->delta_pos,
-                                                                 ctx->n_co, PS.buf, PS.exps);
     // 4D map over the panel slices [S*KB][j][j'][64]: coordinates (kk, j', j, plane)
     const int KB = Kc / BKB;
     cuuint64_t dims[4] = {(cuuint64_t)BKB, (cuuint64_t)ctx->n_co, (cuuint64_t)ctx->n_co,
@@ -1244,9 +1242,13 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
                             w ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         }
-    if (r != CUDA_SUCCESS) return mixed_fail(ctx, HB_ERR_CUDA, "panel tensor map: error " + std::to_string((int)r));
+    if (r != CUDA_SUCCESS) return undo(HB_ERR_CUDA, "panel tensor map: error " + std::to_string((int)r));
     e = set_smem_attr(PS.slices);
-    if (e != cudaSuccess) return mixed_fail(ctx, HB_ERR_CUDA, std::string("smem attribute: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) return undo(HB_ERR_CUDA, std::string("smem attribute: ") + cudaGetErrorString(e));
+    ctx->dev_bytes += bytes + extra;
+    if (precision == HB_MIXED) panel_diag_df_kernel<<<ctx->n_co, 256, 0, s>>>(ctx->panel, ctx->n_co, Kc, M.pdiag);
+    slice_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ctx->panel, rows, Kc, PS.slices, ctx->delta_pos,
+                                                                 ctx->n_co, PS.buf, PS.exps);
     PS.ready = true;
     return HB_OK;
 }

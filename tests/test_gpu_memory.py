@@ -1,0 +1,39 @@
+"""Device memory of the tables made on first use: what a failed set-up leaves, and
+what an FP64 build takes."""
+import ctypes as C
+
+import pytest
+
+from paper_1709_03005_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_1709_03005_gb300 import build_ext
+    build_ext.build()
+
+
+def test_failed_setup_holds_nothing():
+    """A workspace that takes the panel slices of a mixed build and no more: every
+    attempt fails alike, and none of them keeps the slices."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    P = synth.make_config("mid")
+    H = hb.Hamiltonian(P)
+    L = H.layout
+    Kc = (L.n_labels + 63) // 64 * 64
+    slices = 5 * 2 * P.n_co ** 2 * Kc
+    H.set_workspace(torch.empty(slices + 4096, dtype=torch.uint8, device="cuda"))
+    held = L.device_bytes
+    seen = set()
+    for _ in range(3):
+        with pytest.raises(hb.HBError) as e:
+            H.build(hb.HB_MIXED)
+        assert e.value.code == hb.HB_ERR_OOM
+        seen.add(str(e.value))
+        hb._check(H.lib.hb_query(H.ctx, C.byref(L)), H.ctx)
+        assert L.device_bytes == held
+    assert len(seen) == 1
+    H.close()
