@@ -1093,8 +1093,14 @@ int64_t hb::diag_workspace_bytes(const hb_ctx *ctx, int k, int precond) {
     return t;
 }
 
+// On failure nothing is kept: buffers of an earlier call, of another size, must
+// not pass for this one's.
 int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t s) {
     DiagWork *w = (DiagWork *)ctx->diag;
+    auto no_room = [&](const std::string &m) {
+        release_diag(ctx);
+        return diag_fail(ctx, HB_ERR_OOM, m);
+    };
     const int64_t n = ctx->dim;
     if (!w) {
         w = new DiagWork();
@@ -1107,6 +1113,7 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
         w->V = w->AV = w->X = w->AX = w->W2 = w->d = w->partial = w->small = w->theta = w->proj = w->XT = w->prod = nullptr;
         w->idx = nullptr;
         w->XT_rows = 0;
+        w->mmax = 0;
         const size_t vec = (size_t)mmax * n;
         cudaError_t e = dmalloc_n(ctx, &w->V, vec);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->AV, vec);
@@ -1121,7 +1128,7 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->theta, (size_t)mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->idx, (size_t)mmax);
         if (e == cudaSuccess && ctx->Dc > 0) e = dmalloc_n(ctx, &w->prod, (size_t)product_doubles(n, mmax));
-        if (e != cudaSuccess) return diag_fail(ctx, HB_ERR_OOM, std::string("Davidson workspace: ") + cudaGetErrorString(e));
+        if (e != cudaSuccess) return no_room(std::string("Davidson workspace: ") + cudaGetErrorString(e));
         w->mmax = mmax;
         w->n = n;
     }
@@ -1130,13 +1137,13 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
         w->XT = nullptr;
         w->XT_rows = 0;
         cudaError_t e = dmalloc_n(ctx, &w->XT, (size_t)ctx->n_l2 * w->mmax);
-        if (e != cudaSuccess) return diag_fail(ctx, HB_ERR_OOM, "Davidson interleaved-vector buffer");
+        if (e != cudaSuccess) return no_room("Davidson interleaved-vector buffer");
         w->XT_rows = (int64_t)ctx->n_l2 * w->mmax;
     }
     if (ctx->Dc > 0 && ctx->n_l2 > 0 && (!w->HlcT || w->HlcT_src != H->Hlc)) {
         if (!w->HlcT) {
             cudaError_t e = dmalloc_n(ctx, &w->HlcT, (size_t)ctx->Dc * ctx->n_l2);
-            if (e != cudaSuccess) return diag_fail(ctx, HB_ERR_OOM, "Davidson transpose buffer");
+            if (e != cudaSuccess) return no_room("Davidson transpose buffer");
         }
         w->HlcT_src = H->Hlc;
     }

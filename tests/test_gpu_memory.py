@@ -37,3 +37,22 @@ def test_failed_setup_holds_nothing():
         assert L.device_bytes == held
     assert len(seen) == 1
     H.close()
+
+
+def test_solve_after_one_without_room():
+    """A workspace for a solve of 2 pairs: one of 24 finds no room, the next of 2 runs as before."""
+    import numpy as np
+    import torch
+    from paper_1709_03005_gb300 import hb
+    H = hb.Hamiltonian(synth.make_config("mid"))
+    x, _ = H.build(0)
+    need = H.workspace_size(-1, 2) - (14 << 20)      # most of its allowance for the autotuner
+    H.set_workspace(torch.empty(need, dtype=torch.uint8, device="cuda"))
+    ref, _, _ = H.diag(x, 2)
+    for _ in range(2):
+        with pytest.raises(hb.HBError) as e:
+            H.diag(x, 24)
+        assert e.value.code == hb.HB_ERR_OOM
+        ev, _, _ = H.diag(x, 2)
+        assert np.array_equal(ev, ref)
+    H.close()
