@@ -28,6 +28,7 @@ int fail(hb_ctx *ctx, int code, const std::string &msg) {
 }
 
 int cuda_fail(hb_ctx *ctx, cudaError_t e, const char *what) {
+    cudaGetLastError();      // reported here, and not by the next call's check
     return fail(ctx, e == cudaErrorMemoryAllocation ? HB_ERR_OOM : HB_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -76,7 +77,10 @@ cudaError_t dmalloc(hb_ctx *ctx, void **p, size_t bytes) {
         *p = P.base + off;
     } else {
         cudaError_t e = cudaMalloc(p, bytes);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) {
+            cudaGetLastError();      // returned here, and not by the next check of a launch
+            return e;
+        }
     }
     P.live[*p] = bytes;
     P.live_bytes += bytes;

@@ -597,6 +597,7 @@ int upload(Plan &p, std::string *err, cudaStream_t s) {
         if (e == cudaSuccess) p.upload_pending = true;
     }
     if (e != cudaSuccess) {
+        cudaGetLastError();
         *err = std::string("plan upload: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? HB_ERR_OOM : HB_ERR_CUDA;
     }

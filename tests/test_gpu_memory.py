@@ -56,3 +56,36 @@ def test_solve_after_one_without_room():
         ev, _, _ = H.diag(x, 2)
         assert np.array_equal(ev, ref)
     H.close()
+
+
+def _fill_device_but(left):
+    """Take all device memory but about `left` bytes."""
+    import torch
+    torch.cuda.empty_cache()
+    return torch.empty(max(torch.cuda.mem_get_info()[0] - left, 0), dtype=torch.uint8, device="cuda")
+
+
+def test_error_of_an_allocation_is_returned_once():
+    """A solve that finds no memory; what follows it with room again succeeds."""
+    import numpy as np
+    import torch
+    from paper_1709_03005_gb300 import hb
+    P = synth.make_config("c2")
+    H = hb.Hamiltonian(P)
+    x, _ = H.build(1)
+    rest = _fill_device_but(64 << 20)
+    with pytest.raises(hb.HBError) as e:
+        H.diag(x, 20, 1e-6)
+    assert e.value.code == hb.HB_ERR_OOM
+    with pytest.raises(hb.HBError) as e:
+        hb.Hamiltonian(P)
+    assert e.value.code == hb.HB_ERR_OOM
+    del rest
+    torch.cuda.empty_cache()
+    ev, _, _ = H.diag(x, 20, 1e-6)
+    G = hb.Hamiltonian(P)
+    y, _ = G.build(1)
+    assert torch.equal(x["Hcc"], y["Hcc"])
+    assert np.isfinite(ev).all()
+    G.close()
+    H.close()
