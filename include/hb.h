@@ -282,8 +282,10 @@ int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
 
 /* Build every class (1-8) into the caller's device buffers.  precision:
    HB_FP64 (double arithmetic; the sums of Eq. 7 exact sums of 62-bit products
-   of the operands, rounded once, on the tensor cores where the operand slices
-   fit the memory) or HB_MIXED: the continuum-continuum
+   of the operands, rounded once, on the tensor cores where the operand slices,
+   14 bytes for every 8 of the expansion panel, are at most an eighth of the
+   free device memory, or within a workspace measured with them; they are given
+   back where a mixed build or a solve of the context finds no room) or HB_MIXED: the continuum-continuum
    contraction (Eq. 7), and class 4 (Eq. 5) of groups of 32..64 states (see
    hb_options.class4_path), on bf16 tensor cores with split operands, exact
    FP32 accumulation and double-float recovery; the target-side contraction

@@ -754,6 +754,8 @@ extern "C" int hb_build_blocks(hb_ctx *ctx, int32_t precision, const hb_blocks *
     if (!plan) {
         hb_ctx *one[1] = {ctx};
         int rc = plan_create(one, 1, out, precision, &plan, &err, s);
+        if (rc == HB_ERR_OOM && precision == HB_MIXED && release_f64_slices(ctx))
+            rc = plan_create(one, 1, out, precision, &plan, &err, s);
         if (rc != HB_OK) return fail(ctx, rc, err);
         ctx->plan = plan;
         if (ctx->autotune) {
@@ -867,6 +869,8 @@ static int shard_plan(hb_ctx *ctx, int precision, int rank, int nranks, const hb
     if (!p) {
         hb_ctx *one[1] = {ctx};
         int rc = plan_create(one, 1, out, precision, &p, &err, s, rank, nranks);
+        if (rc == HB_ERR_OOM && precision == HB_MIXED && release_f64_slices(ctx))
+            rc = plan_create(one, 1, out, precision, &p, &err, s, rank, nranks);
         if (rc != HB_OK) return fail(ctx, rc, err);
         ctx->shard_plan = p;
     } else if (!plan_outputs_equal(p, out)) {
@@ -989,6 +993,7 @@ extern "C" int hb_workspace_size(hb_ctx *ctx, int32_t precision, int32_t diag_k,
     release_lazy(ctx);
     const size_t live0 = ctx->pool.live_bytes;
     ctx->pool.peak_bytes = live0;
+    bool f64_split = false;
     if (precision != -1) {
         hb_blocks none{};
         hb_ctx *one[1] = {ctx};
@@ -997,6 +1002,7 @@ extern "C" int hb_workspace_size(hb_ctx *ctx, int32_t precision, int32_t diag_k,
         int rc = plan_create(one, 1, &none, precision, &plan, &err, s);
         if (rc != HB_OK) { release_lazy(ctx); return fail(ctx, rc, err); }
         cudaStreamSynchronize(s);
+        f64_split = precision == HB_FP64 && plan_split_on(plan);
         plan_destroy(plan);
     }
     // the build's set-up stays while a solve runs, so the two add up
@@ -1006,7 +1012,7 @@ extern "C" int hb_workspace_size(hb_ctx *ctx, int32_t precision, int32_t diag_k,
     // the autotuner's timing buffers and the allocator's alignment
     need += (16 << 20) + need / 64;
     ctx->pool.measured = need;
-    ctx->pool.measured_f64 = precision == HB_FP64;
+    ctx->pool.measured_f64 = f64_split;
     *bytes = need;
     return HB_OK;
 }

@@ -74,7 +74,7 @@ struct DevPool {
     size_t live_bytes = 0, peak_bytes = 0;
     size_t init_allocs = 0;                      // hb_ctx::allocs made by hb_init
     int64_t measured = 0;                        // the last hb_workspace_size result
-    bool measured_f64 = false;                   // and whether it was for an FP64 build
+    bool measured_f64 = false;                   // and whether it was for an FP64 build with its slices
 };
 cudaError_t dmalloc(hb_ctx *ctx, void **p, size_t bytes);
 void dfree(hb_ctx *ctx, void *p);

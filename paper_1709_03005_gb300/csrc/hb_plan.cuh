@@ -24,6 +24,7 @@ bool plan_is_shard(const hb::Plan *p, int precision, int r, int n);
 int plan_set_outputs(hb::Plan *p, const hb_blocks *outs, std::string *err, cudaStream_t s);
 bool plan_outputs_equal(const hb::Plan *p, const hb_blocks *outs);
 int plan_precision(const hb::Plan *p);
+bool plan_split_on(const hb::Plan *p);      // the expansion on the tensor cores
 // Error word of the context's last build, once: 0 after the call that returned it
 // (whichever call of the interface that was), or while the build runs.
 int plan_last_error(hb_ctx *ctx);

@@ -11,6 +11,11 @@
 // Panel slices and tensor maps of a context (or of the context it borrows from)
 // for one precision.
 int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s);
+// Whether an FP64 build may take `bytes` of the context's memory for its slices.
+bool f64_slices_fit(const hb_ctx *ctx, size_t bytes);
+// Give back the panel slices of FP64 builds (and the plans that read them), which
+// such a build can do without; false where there are none or a batch reads them.
+bool release_f64_slices(hb_ctx *ctx);
 // Identity of the panel a context reads (equal for contexts sharing integrals).
 const void *mixed_panel_key(const hb_ctx *ctx, int precision);
 int mixed_slices(const hb_ctx *ctx, int precision);

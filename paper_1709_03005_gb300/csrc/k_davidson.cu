@@ -23,6 +23,7 @@
 #include "hb_api_internal.cuh"
 #include "hb_davidson.cuh"
 #include "hb_plan.cuh"
+#include "hb_split.cuh"
 
 using namespace hb;
 
@@ -1168,6 +1169,7 @@ extern "C" int hb_diag(hb_ctx *ctx, const hb_blocks *H, int32_t k, double tol, i
     const int b = (int)std::min<int64_t>(n, k + std::max(4, std::min(16, k / 2)));
     const int mmax = (int)std::min<int64_t>(n, (int64_t)ctx->diag_basis * b);
     int rc = ensure_diag_work(ctx, H, mmax, s);
+    if (rc == HB_ERR_OOM && release_f64_slices(ctx)) rc = ensure_diag_work(ctx, H, mmax, s);
     if (rc != HB_OK) return rc;
     DiagWork *w = (DiagWork *)ctx->diag;
     Ops ops{ctx, H, s, n, ctx->Dc, ctx->n_l2, w};
@@ -1184,6 +1186,7 @@ extern "C" int hb_diag(hb_ctx *ctx, const hb_blocks *H, int32_t k, double tol, i
     if (tensor) {
         // slices of the fixed operands, once per call
         rc = setup_tensor_products(ctx, H, w, mmax, s);
+        if (rc == HB_ERR_OOM && release_f64_slices(ctx)) rc = setup_tensor_products(ctx, H, w, mmax, s);
         if (rc != HB_OK) return rc;
         ops.launches += 2;
     }

@@ -685,6 +685,19 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
                     room = false;        // (its size is rounded to the allocator's 256 bytes)
         }
     }
+    // the coefficient slices of an FP64 build come first: without room for them
+    // the panel's are not made
+    int64_t rows = 0;
+    for (int i = 0; i < n; ++i)
+        for (auto &P : ctxs[i]->gps) rows += P.n_nn;
+    if (any_pairs && room && precision == HB_FP64) {
+        const int S = mixed_slices(ctxs[0], precision);
+        rc = f64_slices_fit(ctxs[0], 2 * (size_t)S * rows * p->Kw)
+                 ? split_coef_alloc(ctxs[0], S, rows, p->Kw, &p->coef, &p->coef_exps, p->tm_coef, err) : HB_ERR_OOM;
+        room = rc == HB_OK;
+        if (rc == HB_ERR_OOM) rc = HB_OK;
+        if (rc != HB_OK) { plan_destroy(p); return rc; }
+    }
     if (any_pairs && room) {
         for (int i = 0; i < n && rc == HB_OK; ++i) {
             if (ctxs[i]->gps.empty()) continue;
@@ -701,7 +714,13 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         }
         p->split_on = rc == HB_OK && p->S > 0;
         // an FP64 build without room for the slices adds its sums on the FP64 pipe
-        if (precision == HB_FP64 && rc == HB_ERR_OOM) rc = HB_OK;
+        if (precision == HB_FP64 && rc == HB_ERR_OOM) {
+            rc = HB_OK;
+            dfree(ctxs[0], p->coef);
+            dfree(ctxs[0], p->coef_exps);
+            p->coef = nullptr;
+            p->coef_exps = nullptr;
+        }
         if (rc != HB_OK) { plan_destroy(p); return rc; }
         p->delta_col = ctxs[0]->delta_pos;   // the delta label's column (class 0 comes first)
     }
@@ -738,14 +757,7 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     }
     fill_tasks(*p);
     if (p->split_on && p->coef_rows > 0) {
-        rc = split_coef_alloc(ctxs[0], p->S, p->coef_rows, p->Kw, &p->coef,
-                              precision == HB_FP64 ? &p->coef_exps : nullptr, p->tm_coef, err);
-        if (rc == HB_ERR_OOM && precision == HB_FP64) {
-            p->split_on = false;
-            p->split.clear();
-            fill_tasks(*p);
-            rc = HB_OK;
-        }
+        if (!p->coef) rc = split_coef_alloc(ctxs[0], p->S, p->coef_rows, p->Kw, &p->coef, nullptr, p->tm_coef, err);
         if (rc != HB_OK) { plan_destroy(p); return rc; }
         ensure_split_events(*p);
     }
@@ -767,6 +779,7 @@ bool plan_outputs_equal(const Plan *p, const hb_blocks *outs) {
 }
 
 int plan_precision(const Plan *p) { return p->precision; }
+bool plan_split_on(const Plan *p) { return p->split_on; }
 
 int plan_last_error(hb_ctx *ctx) {
     if (!ctx->last_build || ctx->error_told) return 0;

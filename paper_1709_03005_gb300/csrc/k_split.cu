@@ -57,6 +57,7 @@
 #include <mutex>
 
 #include "hb_api_internal.cuh"
+#include "hb_plan.cuh"
 #include "hb_split.cuh"
 #include "hb_df.cuh"
 #include "hb_tc.cuh"
@@ -1180,6 +1181,20 @@ static int mixed_fail(hb_ctx *ctx, int code, const std::string &m) {
     return code;
 }
 
+// The slices of an FP64 build are 14 bytes for every 8 of the panel, and it can do
+// without them: outside a caller's workspace (sized with them or not) they take
+// no more than an eighth of the memory that is free, so that the caller, other
+// contexts and the solve find about what they found before.
+bool f64_slices_fit(const hb_ctx *ctx, size_t bytes) {
+    if (ctx->pool.base) return true;
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return bytes <= free / 8;
+}
+
 // Panel slices and their tensor maps, once per context and precision (the
 // integrals do not change between builds); a context that borrows its
 // integrals borrows these.
@@ -1205,6 +1220,8 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     // of each row's class
     const int Kc = ctx->Kc;
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)PS.slices * rows * Kc;
+    if (precision == HB_FP64 && !f64_slices_fit(ctx, bytes))
+        return mixed_fail(ctx, HB_ERR_OOM, "panel slices: more than an FP64 build may take");
     const size_t extra = precision == HB_MIXED ? sizeof(float2) * (size_t)ctx->n_co * Kc : sizeof(int16_t) * (size_t)rows;
     // everything that can fail comes before the kernels; a failure leaves nothing behind
     auto undo = [&](int code, const std::string &m) {
@@ -1490,6 +1507,25 @@ int dense_split_gemm(int S, const DenseOperand &A, int64_t M, const DenseOperand
     const int64_t tot = M * N;
     dense_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, nsplit, (int)M, (int)N, Y, ldy);
     return 2;
+}
+
+bool release_f64_slices(hb_ctx *ctx) {
+    hb_ctx *owner = ctx->base ? ctx->base : ctx;
+    if (!owner->mixed || !owner->mixed->panel[0].ready || *owner->batches > 0) return false;
+    cudaDeviceSynchronize();
+    for (hb_ctx *c : {ctx, owner})
+        for (void **p : {&c->plan, &c->shard_plan})
+            if (*p && plan_precision((Plan *)*p) == HB_FP64) {
+                plan_destroy((Plan *)*p);
+                *p = nullptr;
+            }
+    PanelSlices &PS = owner->mixed->panel[0];
+    dfree(owner, PS.buf);
+    dfree(owner, PS.exps);
+    PS = PanelSlices();
+    if (ctx != owner && ctx->mixed) ctx->mixed->panel[0] = PanelSlices();
+    ++owner->tables_gen;          // other borrowing contexts let go of them before their next build
+    return true;
 }
 
 void release_mixed(hb_ctx *ctx) {

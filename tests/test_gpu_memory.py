@@ -89,3 +89,69 @@ def test_error_of_an_allocation_is_returned_once():
     assert np.isfinite(ev).all()
     G.close()
     H.close()
+
+
+def _build64(H, x=None):
+    import torch
+    b, st = H.build(0, x)
+    torch.cuda.synchronize()
+    return b, st
+
+
+def test_fp64_slices_take_an_eighth_of_the_free_memory():
+    """0.44 GB of slices beside 2 GB of free memory: the build adds its sums on the FP64 pipe, and holds no more than it did."""
+    import torch
+    from paper_1709_03005_gb300 import hb
+    P = synth.make_config("c2")
+    H = hb.Hamiltonian(P)
+    x = H.allocate()
+    rest = _fill_device_but(2 << 30)
+    before = torch.cuda.mem_get_info()[0]
+    _, st = _build64(H, x)
+    assert st.expand_tensor_flops == 0.0
+    assert before - torch.cuda.mem_get_info()[0] < 64 << 20
+    want = {k: v.clone() for k, v in x.items()}
+    del rest
+    torch.cuda.empty_cache()
+    H.close()
+    H = hb.Hamiltonian(P)
+    _, st = _build64(H, x)
+    assert st.expand_tensor_flops > 0.0
+    scale = want["Hcc"].abs().max()
+    assert (x["Hcc"] - want["Hcc"]).abs().max() <= 1e-13 * scale
+    assert torch.equal(x["Hlc"], want["Hlc"]) and torch.equal(x["val"], want["val"])
+    H.close()
+
+
+@pytest.mark.parametrize("what", ["solve", "mixed"])
+def test_fp64_slices_are_given_back(what):
+    """What finds no room beside the slices of an earlier FP64 build takes theirs."""
+    import numpy as np
+    import torch
+    from paper_1709_03005_gb300 import hb
+    P = synth.make_config("c2")
+    H = hb.Hamiltonian(P)
+    if what == "solve":
+        x, _ = _build64(H)
+        ref, _, _ = H.diag(x, 20, 1e-6)
+    else:
+        x, _ = H.build(1)
+        ref = {k: v.clone() for k, v in x.items()}
+    H.close()
+    H = hb.Hamiltonian(P)
+    _, st = _build64(H, x)
+    assert st.expand_tensor_flops > 0.0
+    y = torch.zeros_like(x["Hcc"])
+    rest = _fill_device_but(128 << 20)
+    if what == "solve":
+        ev, _, _ = H.diag(x, 20, 1e-6)
+        assert np.array_equal(ev, ref)
+    else:
+        H.build(1, x)
+        torch.cuda.synchronize()
+        for k in ref:
+            assert torch.equal(x[k], ref[k]), k
+    _build64(H, x)
+    del rest, y
+    torch.cuda.empty_cache()
+    H.close()
