@@ -208,12 +208,21 @@ spmm_csr_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
 // fixed order, so the sums are deterministic.  Chunks of 512 entries left a
 // 1980-row solve on 12 blocks that all computed 32 columns of its 12: 146 us a
 // projection, now 9 us.
-constexpr int kGramTile = 32, kGramSub = 32;
-int gram_chunk(int64_t n) {
-    if (n >= 32768) return 512;
+// More than kGramTiles tiles fill the chip in chunks of 512, whose partial sums
+// take less memory (the 1296 vectors of 200 roots: 0.8 GB at dimension 30000, 2 GB
+// in 147 chunks).
+constexpr int kGramTile = 32, kGramSub = 32, kGramTiles = 16;
+int64_t gram_tiles(int p, int q) { return (int64_t)((p + kGramTile - 1) / kGramTile) * ((q + kGramTile - 1) / kGramTile); }
+int gram_chunk(int64_t n, int p, int q) {
+    if (n >= 32768 || gram_tiles(p, q) > kGramTiles) return 512;
     return (int)std::max<int64_t>(kGramSub, (n / 152 + kGramSub - 1) / kGramSub * kGramSub);
 }
-int gram_chunks(int64_t n) { return (int)((n + gram_chunk(n) - 1) / gram_chunk(n)); }
+int gram_chunks(int64_t n, int p, int q) { return (int)((n + gram_chunk(n, p, q) - 1) / gram_chunk(n, p, q)); }
+// doubles of the partial sums of up to mmax vectors against as many
+int64_t gram_doubles(int64_t n, int mmax) {
+    const int64_t few = std::min<int64_t>((int64_t)mmax * mmax, kGramTiles * kGramTile * kGramTile);
+    return std::max(gram_chunks(n, 1, 1) * few, (n + 511) / 512 * mmax * mmax);
+}
 __global__ void __launch_bounds__(256)
 gram_partial_kernel(const double *__restrict__ X, int64_t ldx, int p, const double *__restrict__ Y, int64_t ldy, int q,
                     int64_t n, int chunk, double *__restrict__ partial) {
@@ -935,9 +944,9 @@ struct Ops {
     // G[a][b] = X[a] . Y[b] on the host (p x q)
     void gram(const double *X, int p, const double *Y, int q, int64_t ld, std::vector<double> &G) {
         const double t0 = now_ms();
-        const int chunks = gram_chunks(n);
-        dim3 g(chunks, ((p + kGramTile - 1) / kGramTile) * ((q + kGramTile - 1) / kGramTile));
-        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n), w->partial);
+        const int chunks = gram_chunks(n, p, q);
+        dim3 g(chunks, (unsigned)gram_tiles(p, q));
+        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n, p, q), w->partial);
         reduce_kernel<<<(p * q + 31) / 32, 256, 0, s>>>(w->partial, chunks, p * q, w->small);
         launches += 2;
         proj_flops += 2.0 * p * q * (double)n;
@@ -950,8 +959,8 @@ struct Ops {
     // r2[a] = |X[a]|^2 on the host (p values)
     void norms2(const double *X, int p, int64_t ld, std::vector<double> &r2) {
         const double t0 = now_ms();
-        const int chunks = gram_chunks(n);
-        norms_partial_kernel<<<dim3(chunks, p), 256, 0, s>>>(X, ld, p, n, gram_chunk(n), w->partial);
+        const int chunks = gram_chunks(n, p, 1);
+        norms_partial_kernel<<<dim3(chunks, p), 256, 0, s>>>(X, ld, p, n, gram_chunk(n, p, 1), w->partial);
         reduce_kernel<<<(p + 31) / 32, 256, 0, s>>>(w->partial, chunks, p, w->small);
         launches += 2;
         proj_flops += 2.0 * p * (double)n;
@@ -984,9 +993,9 @@ struct Ops {
     void project_out(const double *X, int p, double *Y, int q, int64_t ld) {
         if (p <= 0 || q <= 0) return;
         const double t0 = now_ms();
-        const int chunks = gram_chunks(n);
-        dim3 g(chunks, ((p + kGramTile - 1) / kGramTile) * ((q + kGramTile - 1) / kGramTile));
-        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n), w->partial);
+        const int chunks = gram_chunks(n, p, q);
+        dim3 g(chunks, (unsigned)gram_tiles(p, q));
+        gram_partial_kernel<<<g, 256, 0, s>>>(X, ld, p, Y, ld, q, n, gram_chunk(n, p, q), w->partial);
         reduce_kernel<<<(p * q + 31) / 32, 256, 0, s>>>(w->partial, chunks, p * q, w->proj);
         dim3 g2((unsigned)((n + 15) / 16), (q + 15) / 16);
         combine_kernel<<<g2, 64, 0, s>>>(X, ld, p, w->proj, q, n, Y, ld, 1.0, -1.0);
@@ -1072,8 +1081,7 @@ int64_t hb::diag_workspace_bytes(const hb_ctx *ctx, int k, int precond) {
     if (n < 1 || k < 1) return 0;
     const int b = (int)std::min<int64_t>(n, k + std::max(4, std::min(16, k / 2)));
     const int mmax = (int)std::min<int64_t>(n, (int64_t)ctx->diag_basis * b);
-    const int64_t chunks = gram_chunks(n);
-    int64_t t = 5 * r(8.0 * mmax * n) + r(8.0 * n) + r(8.0 * chunks * mmax * mmax) + 2 * r(8.0 * mmax * mmax) +
+    int64_t t = 5 * r(8.0 * mmax * n) + r(8.0 * n) + r(8.0 * gram_doubles(n, mmax)) + 2 * r(8.0 * mmax * mmax) +
                 r(8.0 * mmax) + r(4.0 * mmax);
     if (nl > 0) t += r(8.0 * nl * mmax);
     if (Dc > 0) t += r(8.0 * product_doubles(n, mmax));
@@ -1122,8 +1130,7 @@ int hb::ensure_diag_work(hb_ctx *ctx, const hb_blocks *H, int mmax, cudaStream_t
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->AX, vec);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->W2, vec);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->d, (size_t)n);
-        const int chunks = gram_chunks(n);
-        if (e == cudaSuccess) e = dmalloc_n(ctx, &w->partial, (size_t)chunks * mmax * mmax);
+        if (e == cudaSuccess) e = dmalloc_n(ctx, &w->partial, (size_t)gram_doubles(n, mmax));
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->small, (size_t)mmax * mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->proj, (size_t)mmax * mmax);
         if (e == cudaSuccess) e = dmalloc_n(ctx, &w->theta, (size_t)mmax);

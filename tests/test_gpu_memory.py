@@ -155,3 +155,23 @@ def test_fp64_slices_are_given_back(what):
     del rest, y
     torch.cuda.empty_cache()
     H.close()
+
+
+def test_scratch_of_many_roots():
+    """200 roots of dimension 959 (up to 959 vectors): the partial sums of the
+    projections take no more than the vectors do, and the solve is right."""
+    import numpy as np
+    import torch
+    from oracle import coracle
+    from paper_1709_03005_gb300 import hb
+    P = synth.make_config("mid")
+    H = hb.Hamiltonian(P)
+    need = H.workspace_size(-1, 200)
+    vectors = 5 * 8 * H.dim * H.dim
+    assert need <= 3 * vectors
+    x, _ = _build64(H)
+    H.set_workspace(torch.empty(need, dtype=torch.uint8, device="cuda"))
+    ev, _, _ = H.diag(x, 200, 1e-8, 200)
+    ref = np.linalg.eigvalsh(coracle.Oracle(P).dense())[:200]
+    np.testing.assert_allclose(ev, ref, atol=1e-8, rtol=0)
+    H.close()
