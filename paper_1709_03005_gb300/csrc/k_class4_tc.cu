@@ -14,10 +14,12 @@
 //     exponent per continuum orbital j;
 //   C slices [S][2 ndet + 1][64] per group: +c, -c and a zero row, one exponent
 //     per state n;
-// split into balanced base-256 digits, so every slice-pair product of a term
-// has the unit 2^(e_j + e_n - 16 - 8 s), at most 2^16 units for s <= 2, and
-// the MMAs sum them exactly in FP32 over chunks of at most 256 terms.  The term lists (integral row, signed CI row) per L2 row are
-// sized once per plan and written every build from that build's pairs.
+// split into balanced base-256 digits (|d_0| <= 256, the others 128), so that the
+// products of a term with i + l = s are multiples of 2^(e_j + e_n - 16 - 8 s):
+// 65536 of them at most for s = 0 and 1, 81920 for s = 2, and the MMAs sum them
+// exactly in FP32 over chunks of 192 terms (2^24 / 81920 = 204).  The term lists
+// (integral row, signed CI row) per L2 row are sized once per plan and written
+// every build from that build's pairs.
 //
 // Kernel (persistent, one CTA per SM, 12 warps):
 //   warp 0     MMA issuer and TMEM owner (512 columns: two buffers of 4
@@ -82,7 +84,7 @@ constexpr int TKB = 16;          // terms per K block (the K of one MMA)
 constexpr int TBM = 128;         // most continuum orbitals per tile (TMEM lanes)
 constexpr int TNP = 64;          // states per tile (N of the MMA)
 constexpr int TSTAGES = 6, TAHEAD = 1;   // stages; copies of TAHEAD + 1 of them in flight per producer thread
-constexpr int TCHUNK_KB = 16;    // K blocks per exact accumulation chunk (256 terms)
+constexpr int TCHUNK_KB = 12;    // K blocks per exact accumulation chunk (192 terms)
 constexpr int T_A_SLICE = 2 * (TKB / 8) * 1024;       // 4 KB: two 64-orbital atoms
 constexpr int T_B_SLICE = (TKB / 8) * 1024;           // 2 KB: one 64-state atom
 constexpr int T_PROD_GROUPS = 3, T_PROD_WARPS = 1, T_EPI_WARPS = 8;   // producer warps of a group
