@@ -113,11 +113,13 @@ __device__ __forceinline__ void stage_params(const float *params, float *P) {
 // products of a sample (forward, input gradient, weight gradient) are register
 // tiles (8 samples x 4 units, or 4 x 4 weights), so the kernel runs on the FP32
 // pipe: 8.7 kFMA a sample, 23 us for 65536 samples at the full rate.  The
-// gradient sums stay in registers over all tiles of a block; each block then
-// writes one row of partial sums, and a second kernel adds the rows in order.
+// gradient sums stay in registers over all tiles of a block, in two levels: those
+// of kFold tiles (1024 samples), then the sum of these, so that the chain of FP32
+// additions does not grow with the window; each block then writes one row of
+// partial sums, and a second kernel adds the rows in order.
 // Measured at 65536 samples: 76 us + 6 us, against 172 + 2375 us when the
 // activations went through memory and each parameter walked the samples alone.
-constexpr int kTile = 128, kLd = kTile + 4, kTrainThreads = 256;
+constexpr int kTile = 128, kLd = kTile + 4, kTrainThreads = 256, kFold = 8;
 constexpr int kTrainSmem = (3 * MLP_W * kLd + MLP_IN * kLd + 2 * MLP_W * MLP_W + MLP_W * MLP_IN + 3 * MLP_W + 2 * kTile) *
                            (int)sizeof(float);
 
@@ -179,7 +181,30 @@ mlp_train_kernel(const float *__restrict__ params, const float *__restrict__ fea
     // b1, b2, w3 of unit wa over samples 32 (t % 4) ..; b3 and the loss on thread t < kTile
     const int ga = t / 16, gc = t % 16, wa = t / 4, wq = t % 4;
     float g2[4][4] = {}, g1[2] = {0.0f, 0.0f}, gb1 = 0.0f, gb2 = 0.0f, gw3 = 0.0f, gb3 = 0.0f, gl = 0.0f;
+    // and those of the tiles folded so far (b3 and the loss take one sample a tile and thread)
+    float s2[4][4] = {}, s1[2] = {0.0f, 0.0f}, sb1 = 0.0f, sb2 = 0.0f, sw3 = 0.0f;
+    auto fold = [&](float &s, float &g) {
+        s += g;
+        g = 0.0f;
+    };
+    auto fold_all = [&] {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) fold(s2[i][j], g2[i][j]);
+        fold(s1[0], g1[0]);
+        fold(s1[1], g1[1]);
+        fold(sb1, gb1);
+        fold(sb2, gb2);
+        fold(sw3, gw3);
+    };
+    int held = 0;                              // tiles in the first level
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        if (held == kFold) {
+            fold_all();
+            held = 0;
+        }
+        ++held;
         const int64_t i0 = tile * kTile;
         const int valid = (int)min((int64_t)kTile, n - i0);
         __syncthreads();
@@ -301,23 +326,24 @@ mlp_train_kernel(const float *__restrict__ params, const float *__restrict__ fea
             if (((s >> 2) & 3) == wq) gb1 += (d.x + d.y) + (d.z + d.w);
         }
     }
+    fold_all();
     float *out = partial + (int64_t)blockIdx.x * (MLP_NPARAM + 1);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) out[OFF_W2 + (ga + 16 * i) * MLP_W + gc + 16 * j] = g2[i][j];
-    out[OFF_W1 + wa * MLP_IN + 2 * wq] = g1[0];
-    out[OFF_W1 + wa * MLP_IN + 2 * wq + 1] = g1[1];
+        for (int j = 0; j < 4; ++j) out[OFF_W2 + (ga + 16 * i) * MLP_W + gc + 16 * j] = s2[i][j];
+    out[OFF_W1 + wa * MLP_IN + 2 * wq] = s1[0];
+    out[OFF_W1 + wa * MLP_IN + 2 * wq + 1] = s1[1];
 #pragma unroll
     for (int h = 1; h < 4; h <<= 1) {
-        gb1 += __shfl_xor_sync(0xffffffffu, gb1, h);
-        gb2 += __shfl_xor_sync(0xffffffffu, gb2, h);
-        gw3 += __shfl_xor_sync(0xffffffffu, gw3, h);
+        sb1 += __shfl_xor_sync(0xffffffffu, sb1, h);
+        sb2 += __shfl_xor_sync(0xffffffffu, sb2, h);
+        sw3 += __shfl_xor_sync(0xffffffffu, sw3, h);
     }
     if (wq == 0) {
-        out[OFF_B1 + wa] = gb1;
-        out[OFF_B2 + wa] = gb2;
-        out[OFF_W3 + wa] = gw3;
+        out[OFF_B1 + wa] = sb1;
+        out[OFF_B2 + wa] = sb2;
+        out[OFF_W3 + wa] = sw3;
     }
     __syncthreads();
     if (t < kTile) {
