@@ -281,9 +281,11 @@ int hb_set_workspace(hb_ctx *ctx, void *dev_ptr, size_t bytes);
 int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
 
 /* Build every class (1-8) into the caller's device buffers.  precision:
-   HB_FP64 (double arithmetic; the sums of Eq. 7 exact sums of 62-bit products
-   of the operands, rounded once, on the tensor cores where the operand slices,
-   14 bytes for every 8 of the expansion panel, are at most an eighth of the
+   HB_FP64 (double arithmetic; the sums of Eq. 7 exact sums of the products of
+   the operands' 62 leading bits, counted from the largest entry of a row of
+   labels, rounded once, or sums in double where the magnitudes of the terms
+   are so small beside those largest entries that these are closer; on the
+   tensor cores where the operand slices, 16 bytes for every 8 of the expansion panel, are at most an eighth of the
    free device memory, or within a workspace measured with them; they are given
    back where a mixed build or a solve of the context finds no room) or HB_MIXED: the continuum-continuum
    contraction (Eq. 7), and class 4 (Eq. 5) of groups of 32..64 states (see

@@ -23,7 +23,8 @@ int mixed_slices(const hb_ctx *ctx, int precision);
 const float2 *mixed_panel_diag(const hb_ctx *ctx);
 // Coefficient slices [S][Kpad/64][rows][64] bf16 and their tensor maps
 // tm[0..3]: 32-K stages at tile widths 32, 64, 128, and 64-K stages at 128.
-// exps (or null): the rows' exponents, kept apart from the slices.
+// exps (or null): the rows' exponents, kept apart from the slices (S then counts
+// the magnitudes too).
 int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int16_t **exps, CUtensorMap *tm,
                      std::string *err);
 int64_t blocks_split(int cn, int cnp, int N, int lg, int bn);
@@ -49,6 +50,16 @@ int g_slice(const hb::Grouped<hb::SliceTask> &g, int64_t R, int Kin, int Kout, c
 int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef,
             const int16_t *coef_exps, const hb::Grouped<hb::SplitTask> &g, int kblocks, int coef_planes,
             const hb::ExpCol *cols, int *err, cudaStream_t s, int shard_r = 0, int shard_n = 1);
+// FP64 build: a bit an element (SplitTask::weak0), set where the digits are not good
+// enough, from the magnitudes; g: the blocks of `digits` (g_split's) in tiles of
+// kWeakCols columns.  g_weak_sums, after both, sums those elements in FP64; g: the
+// same tasks with blocks_weak_sums blocks each.
+constexpr int kWeakCols = 128;
+int64_t blocks_weak_sums(int cn, int cnp, int N);
+int g_weak_sums(const hb_ctx *panel_ctx, const hb::Grouped<hb::SplitTask> &g, const hb::Grouped<hb::SplitTask> &digits,
+                const uint32_t *weak, int kblocks, const hb::ExpCol *cols, cudaStream_t s, int shard_r, int shard_n);
+int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const hb::Grouped<hb::SplitTask> &g,
+                uint32_t *weak, int kblocks, int coef_planes, const hb::ExpCol *cols, int *err, cudaStream_t s);
 int64_t blocks_diag_rows(int j_lo, int j_hi, int n_nn);
 int diag_rows_ny(int n_nn);
 int g_diag_rows(const hb::Grouped<hb::DRTask> &g, int dfloat, cudaStream_t s);

@@ -170,6 +170,8 @@ struct SplitTask {      // one merged block on the tensor cores
     int bjp_log2;             // tile of (128 >> bjp_log2) j x (1 << bjp_log2) j' continuum pairs (3..5)
     int bn;                   // columns per tile (32, 64, 128): the launch's tile width
     int kc0;                  // first 64-wide K block of the block's label class in the coefficient slices
+    int weak_words;           // FP64: the block's bits, a bit an element, in words of 32 columns, [word][row]
+    int64_t weak0;            // and the first of them
     int64_t coef_row0;        // first row of the block in the coefficient slices
     int64_t col0;             // first column in the ExpCol table
 };

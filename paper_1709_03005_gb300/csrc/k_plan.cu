@@ -57,6 +57,7 @@ struct SplitGroup {
     int lg = 4;                        // tile arrangement of every task of the launch
     int bn = 128;                      // tile width (columns) of every task of the launch
     Stage<SplitTask> st;
+    Stage<SplitTask> weak, fix;        // FP64: the same blocks for the magnitudes and for the sums in FP64
 };
 
 // Tunable launch shapes.  Every candidate of a choice computes bit-identical
@@ -144,6 +145,8 @@ struct Plan {
     int16_t *coef_exps = nullptr;      // FP64 build: the coefficient rows' exponents
     CUtensorMap tm_coef[4];            // coefficient slices: 32-K stages at widths 32, 64, 128; 64-K at 128
     int64_t coef_rows = 0;
+    uint32_t *weak = nullptr;          // FP64: the bits of the elements summed in FP64
+    int64_t weak_words = 0;
     int *err = nullptr;
     // the error words as of the last finished build (page-locked, behind the
     // staged tables; built->err).  On the device they stay set until the error has
@@ -163,6 +166,7 @@ struct Plan {
     // gamma items (aux1), the diagonal gamma (aux2), beside the E, S chain
     cudaStream_t aux1 = nullptr, aux2 = nullptr;
     cudaEvent_t k1_done = nullptr, items_done = nullptr, gd_done = nullptr, asm_done = nullptr, dr_done = nullptr;
+    cudaEvent_t slices_done = nullptr, bits_done = nullptr;
     cudaEvent_t c4_done = nullptr;     // the tensor-core class-4 kernel has finished (side stream)
     std::shared_ptr<BuildEvent> built; // the end of this plan's last build on its caller's stream
     // timers: start, target, expansion (main stream); class-4 end, L2 end, side
@@ -224,7 +228,12 @@ void fill_tasks(Plan &p) {
     p.x64.clear(); p.slc.clear(); p.drows.clear(); p.l2.clear(); p.l2v.clear(); p.l2m.clear();
     for (auto &v : p.c4v) v.st.clear();
     p.c4f.clear(); p.c4t.clear();
-    for (auto &sg : p.split) sg.st.clear();
+    for (auto &sg : p.split) {
+        sg.st.clear();
+        sg.weak.clear();
+        sg.fix.clear();
+    }
+    p.weak_words = 0;
     p.cols.clear();
     p.c4items.clear();
     p.tune_split.clear(); p.tune_c4.clear(); p.tune_gamma.clear();
@@ -502,7 +511,17 @@ void fill_tasks(Plan &p) {
             t.coef_row0 = coef_row;
             t.col0 = col0;
             t.kc0 = B.ctx->class_of(k.cf, k.cfp) * (p.Kc / 64);
+            t.weak_words = (N + 31) / 32;
+            t.weak0 = p.weak_words;
             p.split[gi].st.add(t, blocks_split(k.cn, k.cnp, N, lg, bn));
+            if (p.precision == HB_FP64) {
+                p.weak_words += (int64_t)k.cn * k.cnp * t.weak_words;
+                p.split[gi].fix.add(t, blocks_weak_sums(k.cn, k.cnp, N));
+                SplitTask m = t;
+                m.bn = kWeakCols;
+                m.ntn = split_ntn(N, kWeakCols);
+                p.split[gi].weak.add(m, blocks_split(k.cn, k.cnp, N, lg, kWeakCols));
+            }
             p.tune_split.push_back(TuneSplit{B.ctx, t});
             coef_row += N;
         } else {
@@ -529,7 +548,11 @@ void pack_all(Plan &p) {
     stage_pack(p.gdp, p.host); stage_pack(p.gdr, p.host); stage_pack(p.tn, p.host); stage_pack(p.tnr, p.host); stage_pack(p.itf, p.host);
     stage_pack(p.zero, p.host); stage_pack(p.sort, p.host); stage_pack(p.scan, p.host); stage_pack(p.gam, p.host);
     stage_pack(p.asmb, p.host); stage_pack(p.x64, p.host); stage_pack(p.slc, p.host);
-    for (auto &sg : p.split) stage_pack(sg.st, p.host);
+    for (auto &sg : p.split) {
+        stage_pack(sg.st, p.host);
+        stage_pack(sg.weak, p.host);
+        stage_pack(sg.fix, p.host);
+    }
     stage_pack(p.drows, p.host); stage_pack(p.l2, p.host); stage_pack(p.l2v, p.host); stage_pack(p.l2m, p.host);
     for (auto &v : p.c4v) stage_pack(v.st, p.host);
     stage_pack(p.c4f, p.host); stage_pack(p.c4t, p.host);
@@ -548,7 +571,11 @@ void bind_all(Plan &p) {
     stage_bind(p.gdp, p.dev); stage_bind(p.gdr, p.dev); stage_bind(p.tn, p.dev); stage_bind(p.tnr, p.dev); stage_bind(p.itf, p.dev);
     stage_bind(p.zero, p.dev); stage_bind(p.sort, p.dev); stage_bind(p.scan, p.dev); stage_bind(p.gam, p.dev);
     stage_bind(p.asmb, p.dev); stage_bind(p.x64, p.dev); stage_bind(p.slc, p.dev);
-    for (auto &sg : p.split) stage_bind(sg.st, p.dev);
+    for (auto &sg : p.split) {
+        stage_bind(sg.st, p.dev);
+        stage_bind(sg.weak, p.dev);
+        stage_bind(sg.fix, p.dev);
+    }
     stage_bind(p.drows, p.dev); stage_bind(p.l2, p.dev); stage_bind(p.l2v, p.dev); stage_bind(p.l2m, p.dev);
     for (auto &v : p.c4v) stage_bind(v.st, p.dev);
     stage_bind(p.c4f, p.dev); stage_bind(p.c4t, p.dev);
@@ -648,7 +675,7 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->side, cudaStreamNonBlocking, least);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->aux1, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->aux2, cudaStreamNonBlocking, greatest);
-    for (cudaEvent_t *ev : {&p->k1_done, &p->items_done, &p->gd_done, &p->asm_done, &p->dr_done})
+    for (cudaEvent_t *ev : {&p->k1_done, &p->items_done, &p->gd_done, &p->asm_done, &p->dr_done, &p->slices_done, &p->bits_done})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     p->built = std::make_shared<BuildEvent>();
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->built->e, cudaEventDisableTiming);
@@ -692,8 +719,8 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         for (auto &P : ctxs[i]->gps) rows += P.n_nn;
     if (any_pairs && room && precision == HB_FP64) {
         const int S = mixed_slices(ctxs[0], precision);
-        rc = f64_slices_fit(ctxs[0], 2 * (size_t)S * rows * p->Kw)
-                 ? split_coef_alloc(ctxs[0], S, rows, p->Kw, &p->coef, &p->coef_exps, p->tm_coef, err) : HB_ERR_OOM;
+        rc = f64_slices_fit(ctxs[0], 2 * (size_t)(S + 1) * rows * p->Kw)
+                 ? split_coef_alloc(ctxs[0], S + 1, rows, p->Kw, &p->coef, &p->coef_exps, p->tm_coef, err) : HB_ERR_OOM;
         room = rc == HB_OK;
         if (rc == HB_ERR_OOM) rc = HB_OK;
         if (rc != HB_OK) { plan_destroy(p); return rc; }
@@ -756,6 +783,11 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         }
     }
     fill_tasks(*p);
+    if (p->split_on && precision == HB_FP64 && dmalloc_n(ctxs[0], &p->weak, (size_t)p->weak_words) != cudaSuccess) {
+        p->split_on = false;         // no room after all: the sums on the FP64 pipe
+        p->split.clear();
+        fill_tasks(*p);
+    }
     if (p->split_on && p->coef_rows > 0) {
         if (!p->coef) rc = split_coef_alloc(ctxs[0], p->S, p->coef_rows, p->Kw, &p->coef, nullptr, p->tm_coef, err);
         if (rc != HB_OK) { plan_destroy(p); return rc; }
@@ -900,8 +932,8 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
                     }
                     if (ts.empty()) continue;
                     ms += time_tasks(p->ctxs[0], ts, nb, [&](const Grouped<SplitTask> &g) {
-                        g_split(pc, p->precision, lg, bn, p->tm_coef, p->coef_exps, g, p->Kc / 64, p->Kw / 64, p->d_cols,
-                                p->err, s);
+                        g_split(pc, p->precision, lg, bn, p->tm_coef, p->coef_exps, g, p->Kc / 64,
+                                p->Kw / 64, p->d_cols, p->err, s);
                     }, s);
                 }
                 if (best_lg < 0) { best = def_ms = ms; best_lg = lg; }
@@ -1113,7 +1145,8 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
         // dimension 959).
         int64_t tiles = 0;
         for (auto &g : p->split) tiles += g.st.g.blocks;
-        if (p->c4t.g.blocks > 0 || (p->precision != HB_MIXED && tiles > 152)) cudaStreamWaitEvent(s, p->c4_done, 0);
+        const bool after_c4 = p->c4t.g.blocks > 0 || (p->precision != HB_MIXED && tiles > 152);
+        if (after_c4 && DF) cudaStreamWaitEvent(s, p->c4_done, 0);
         if (p->coef_rows > 0) {
             // the rows with j == j': beside a split kernel that fills the chip they
             // slowed it by more than they saved; one that leaves most SMs idle has
@@ -1127,11 +1160,29 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
             }
             L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, p->coef_exps,
                          s);
+            // FP64: the bits of the elements that the digits are not good enough for,
+            // in CTAs that fit beside class 4's
+            if (!DF) {
+                cudaEventRecord(p->slices_done, s);
+                cudaStreamWaitEvent(sa, p->slices_done, 0);
+                for (auto &g : p->split)
+                    L += g_weak_bits(g.panel_ctx, g.lg, p->tm_coef, g.weak.g, p->weak, p->Kc / 64, p->Kw / 64, p->d_cols,
+                                     p->err, sa);
+                cudaEventRecord(p->bits_done, sa);
+            }
+            if (after_c4 && !DF) cudaStreamWaitEvent(s, p->c4_done, 0);
             for (size_t i = 0; i < p->split.size(); ++i) {
                 rec(p->ev_split[2 * i]);
                 LX += g_split(p->split[i].panel_ctx, p->precision, p->split[i].lg, p->split[i].bn, p->tm_coef, p->coef_exps,
-                              p->split[i].st.g, p->Kc / 64, p->Kw / 64, p->d_cols, p->err, s, p->shard_r, p->shard_n);
+                              p->split[i].st.g, p->Kc / 64, p->Kw / 64,
+                              p->d_cols, p->err, s, p->shard_r, p->shard_n);
                 rec(p->ev_split[2 * i + 1]);
+            }
+            if (!DF) {
+                cudaStreamWaitEvent(s, p->bits_done, 0);
+                for (auto &g : p->split)
+                    L += g_weak_sums(g.panel_ctx, g.fix.g, g.st.g, p->weak, p->Kc / 64, p->d_cols, s, p->shard_r,
+                                     p->shard_n);
             }
             if (beside) cudaStreamWaitEvent(s, p->dr_done, 0);
             else L += g_diag_rows(p->drows.g, DF, s);
@@ -1289,7 +1340,7 @@ void plan_destroy(Plan *p) {
     if (p->join) cudaEventDestroy(p->join);
     if (p->join_main) cudaEventDestroy(p->join_main);
     if (p->c4_done) cudaEventDestroy(p->c4_done);
-    for (cudaEvent_t ev : {p->k1_done, p->items_done, p->gd_done, p->asm_done, p->dr_done})
+    for (cudaEvent_t ev : {p->k1_done, p->items_done, p->gd_done, p->asm_done, p->dr_done, p->slices_done, p->bits_done})
         if (ev) cudaEventDestroy(ev);
     for (cudaStream_t st : {p->main, p->side, p->aux1, p->aux2})
         if (st) {
@@ -1301,6 +1352,7 @@ void plan_destroy(Plan *p) {
         dfree(mem, p->dev);
         dfree(mem, p->coef);
         dfree(mem, p->coef_exps);
+        dfree(mem, p->weak);
         dfree(mem, p->err);
     }
     if (p->pinned) cudaFreeHost(p->pinned);

@@ -27,10 +27,26 @@
 // FP64 build: S = 7 (62 bits, 28 products), every s with an accumulator of its
 // own, and the row exponents kept apart from the digits.  The drained sums are
 // integers and are added as such (two 64-bit words per element, s <= 2 and
-// s >= 3), so the element is the correctly rounded sum of the 62-bit products,
-// whatever the order of the labels.  The FP64 pipe of this part runs at a
-// 1/1000 of the tensor rate: its sums took 14.0 ms where this takes 0.65 ms
-// (12.9 GFLOP), and rounded every one of the 1367 additions.
+// s >= 3), so the element is the correctly rounded sum of the products of the
+// operands' 62 leading bits, whatever the order of the labels.  The FP64 pipe of
+// this part runs at a 1/1000 of the tensor rate: its sums took 14.0 ms where this
+// takes 0.65 ms (12.9 GFLOP), and rounded every one of the 1367 additions.
+//   What the digits leave out is relative to the largest entries of the two rows:
+// K labels err by less than K 2^-60 of their product, typically by 2^-63 sqrt(K),
+// and sums in FP64 by about 2^-54 M, M = sum |p_k a_k|.  Where the large entries of
+// the one row meet zeros or tiny entries of the other (h_jj' of 50 and S = 0
+// between groups, beside integrals of 1e-6) M can be so small that FP64 is closer.
+// So the FP64 build carries an eighth slice, the magnitudes to 8 bits rounded down,
+// whose product is a lower bound of M: an element with 0 < M < sqrt(K) 2^-9 of the
+// scales (there the typical errors are alike; at least 2^-7, where the bounds are)
+// is summed in FP64 (fp64_elements_kernel).  Magnitudes below 2^-9 count as 2^-40,
+// so M = 0 means that no two entries meet, and the sum is exactly zero; a row with a
+// value that is not finite is all 2^-40.  Molecular integrals and target densities stay far above the line
+// (the lowest 1e-3 of M lies at 0.05 to 0.6 of the scales, the line at 0.03 to 0.08).
+// The magnitudes are multiplied by a launch of their own (this kernel with one
+// slice and 128-wide tiles), which leaves a bit an element, beside what comes before
+// the digits: an eighth pair of tiles in every stage of those made them 22 % slower
+// (0.65 -> 0.79 ms).
 //
 // Kernel structure (persistent CTAs on 128 x TBN output tiles, 10 warps):
 //   warp 0  TMA producer: per K stage (32 or 64 labels) and slice, one panel
@@ -54,6 +70,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "hb_api_internal.cuh"
@@ -67,7 +84,7 @@ namespace hb {
 // Panel slices of one precision, and their tensor maps.
 struct PanelSlices {
     int slices = 0;
-    __nv_bfloat16 *buf = nullptr;            // [S][Kpad/64][n_co*n_co][64]
+    __nv_bfloat16 *buf = nullptr;            // [S][Kpad/64][n_co*n_co][64] (FP64: S + 1, the last the magnitudes)
     int16_t *exps = nullptr;                 // FP64: row exponents [n_co*n_co]
     // [stage width 32, 64][box of 8 x 16, 16 x 8, 32 x 4 continuum pairs (j' x j)]
     CUtensorMap tm[2][3];
@@ -110,7 +127,12 @@ constexpr int XBUDGET = 7 * 32 * 1024;       // shared memory of the slots
 constexpr int XBARS = 24;                    // full and empty barriers: slots at most
 constexpr int XACC = 7;                      // accumulators at most
 constexpr int kK64Blocks = 32;               // 64-K stages from this many 64-wide K blocks up
-constexpr int kF64Slices = 7;                // slices of the FP64 build
+constexpr int kF64Slices = 7;                // digit slices of the FP64 build
+constexpr int kF64Planes = kF64Slices + 1;   // and its magnitudes
+constexpr int kWeakSlots = 3;                // ring of the magnitudes' launch, whose CTAs fit beside class 4's
+// what the kernel computes: the mixed and the FP64 build's sums, and the bits of
+// the elements whose magnitudes are too small for the digits
+enum : int { kMixedSums, kF64Sums, kWeakBits };
 __host__ __device__ constexpr int xa_tile(int ks) { return BM * ks * 2; }
 // one slice of one stage: panel tile, then coefficient tile (multiples of 1 KB)
 __host__ __device__ constexpr int xslot(int tbn, int ks) { return (BM + tbn) * ks * 2; }
@@ -131,9 +153,10 @@ __host__ __device__ constexpr int xperiod(int a, int nex, int ks) {
 }
 // Whether accumulator a is drained after stage ks of nst.  a = 0 is drained
 // between the stages at which a = 1 is, so that at most two of the first three
-// come at once.
+// come at once.  Without exact accumulators (magnitudes) the end alone counts.
 template <int NEX, int KS>
 __device__ __forceinline__ bool acc_due(int a, int ks, int nst) {
+    if (NEX == 0) return ks == nst - 1;
     const int per = xperiod(a, NEX, KS);
     return ks == nst - 1 || (ks + 1 + (a == 0 ? per / 4 : 0)) % per == 0;
 }
@@ -313,9 +336,8 @@ __device__ __forceinline__ bool mma_pairs(MmaState &m, const int (&sl)[S], const
 // One K stage of the expansion kernel.  Its slices lie in the ring from slot
 // `slot0` on, slice S-1 first, `par` being the parity of that slot's use
 // (flipped where the ring wraps).
-template <int S, int NEX, int TBN, int KS>
+template <int S, int NEX, int TBN, int KS, int NS>
 __device__ __forceinline__ bool mma_stage(MmaState &m, int slot0, uint32_t par) {
-    constexpr int NS = xslots(TBN, KS);
     int sl[S];
     uint32_t sp[S];
 #pragma unroll
@@ -370,6 +392,25 @@ __device__ __forceinline__ void drain_int(uint32_t taddr, long long (&acc)[2][NC
             acc[w][c0 + i] += (long long)__float2int_rn(x) * (1ll << lift);
         }
     }
+}
+
+// The magnitude sums of 32 columns: bit c set where the digits of column c are
+// not good enough (see the head of this file).
+__device__ __forceinline__ uint32_t drain_weak(uint32_t taddr, float line) {
+    uint32_t weak = 0;
+#pragma unroll
+    for (int c0 = 0; c0 < 32; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld16_async(taddr + c0, v);
+        tmem_wait_ld();
+        tmem_regs_ready(v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float x = __uint_as_float(v[i]);
+            if (x > 0.0f && x < line) weak |= 1u << (c0 + i);
+        }
+    }
+    return weak;
 }
 
 // The FP64 element of the two words and the row and column exponents.
@@ -443,21 +484,24 @@ __device__ __forceinline__ TilePos tile_pos(const SplitTask *__restrict__ tasks,
 // Persistent: each CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // The slot ring, the accumulator hand-over and their barrier phases run on
 // across tiles, so the loads and MMAs of the next tile start while the
-// epilogue warps still write the last one out from registers.  F64: the FP64
+// epilogue warps still write the last one out from registers.  kF64Sums: the FP64
 // build's kernel (integer sums, exponents apart: pexp of the panel's rows,
-// n_co x n_co, cexp of the coefficient rows).
-template <int S, int TBN, int KS, bool F64>
+// n_co x n_co, cexp of the coefficient rows).  kWeakBits: a bit an element in `weak`,
+// set where the sum of the magnitudes (plane `plane0` of the slices) is below `line`.
+template <int S, int TBN, int KS, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_constant__ CUtensorMap tm_coef,
                     const SplitTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int n_tiles,
                     int kblocks, int coef_planes, const ExpCol *__restrict__ cols, const int16_t *__restrict__ pexp,
-                    const int16_t *__restrict__ cexp, int n_co, int *err, int shard_r, int shard_n) {
+                    const int16_t *__restrict__ cexp, uint32_t *__restrict__ weak, int plane0, float line, int n_co,
+                    int *err, int shard_r, int shard_n) {
     // this launch's tiles: shard_r, shard_r + shard_n, ... (all of them unless
     // sharded), numbered t = 0, 1, ... so that every role walks the same list
     const int n_local = n_tiles > shard_r ? (n_tiles - shard_r + shard_n - 1) / shard_n : 0;
-    constexpr int NEX = F64 ? S : 3;          // accumulators of one s each
+    constexpr bool F64 = MODE == kF64Sums, WEAK = MODE == kWeakBits;
+    constexpr int NEX = WEAK ? 0 : F64 ? S : 3;   // accumulators of one s each
     constexpr int NACC = xaccs(S, NEX);
-    constexpr int XS = xslot(TBN, KS), NS = xslots(TBN, KS);
+    constexpr int XS = xslot(TBN, KS), NS = WEAK ? kWeakSlots : xslots(TBN, KS);
     constexpr int TCOLS = xtmem_cols(NACC, TBN);
     constexpr int ECOLS = TBN / 2;            // columns per epilogue thread
     static_assert(KS == 32 || KS == 64, "stage width");
@@ -513,13 +557,14 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                     const int kx = KS == 64 ? 0 : (ks & 1) * 32;   // part of 64-wide K block kb
                     const int kb = KS == 64 ? ks : ks >> 1;
                     for (int i = S - 1; i >= 0 && ok; --i) {
+                        const int plane = i + (WEAK ? plane0 : 0);
                         if (loads >= NS) ok = mbar_wait(&empty_bar[sl], par, err, 1);
                         if (!ok) break;
                         uint8_t *sA = slots + sl * XS;
                         mbar_expect_tx(&full_bar[sl], (uint32_t)XS);
-                        tma_load_4d(sA, &tm_panel, &full_bar[sl], kx, cx, cy, i * kblocks + kb);
+                        tma_load_4d(sA, &tm_panel, &full_bar[sl], kx, cx, cy, plane * kblocks + kb);
                         tma_load_3d(sA + xa_tile(KS), &tm_coef, &full_bar[sl], kx, crow,
-                                    i * coef_planes + kc0 + kb);
+                                    plane * coef_planes + kc0 + kb);
                         if (loads < 2 * NS) ++loads;
                         if (++sl == NS) { sl = 0; par ^= 1u; }
                     }
@@ -551,7 +596,7 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                 m.due = 0;
 #pragma unroll
                 for (int a = 0; a < NACC; ++a) m.due |= acc_due<NEX, KS>(a, ks, nst) ? 1u << a : 0u;
-                ok = mma_stage<S, NEX, TBN, KS>(m, sl, par);
+                ok = mma_stage<S, NEX, TBN, KS, NS>(m, sl, par);
                 sl += S;
                 if (sl >= NS) { sl -= NS; par ^= 1u; }
             }
@@ -586,9 +631,11 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
             // the column records are read when the tile is written out
             if (e < TBN / 4 && tp[buf].n0 + 4 * e < a.N)
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(cols + a.col0 + tp[buf].n0 + 4 * e));
-            f2 hi[F64 ? 1 : ECOLS / 2], lo[F64 ? 1 : ECOLS / 2];
+            f2 hi[MODE ? 1 : ECOLS / 2], lo[MODE ? 1 : ECOLS / 2];
             long long wd[2][F64 ? ECOLS : 1];
-            if constexpr (F64) {
+            uint32_t bits[2] = {0, 0};               // weak columns
+            if constexpr (WEAK) {
+            } else if constexpr (F64) {
 #pragma unroll
                 for (int c = 0; c < ECOLS; ++c) { wd[0][c] = 0; wd[1][c] = 0; }
             } else {
@@ -605,7 +652,9 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                     fpar ^= 1u << b;
                     if (!ok) continue;
                     tc_fence_after();
-                    if constexpr (F64) {
+                    if constexpr (WEAK) {
+                        for (int w = 0; w < 2; ++w) bits[w] = drain_weak(tq + 32 * w, line);
+                    } else if constexpr (F64) {
                         if (b == 0) drain_int<0>(tq, wd);
                         else if (b == 1) drain_int<1>(tq + TBN, wd);
                         else if (b == 2) drain_int<2>(tq + 2 * TBN, wd);
@@ -630,7 +679,14 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
             // while this one is written out
             const int lg = a.bjp_log2;
             const int jj = tp[buf].jj0 + (row >> lg), jjp = tp[buf].jjp0 + (row & ((1 << lg) - 1));
-            if (jj < a.cn && jjp < a.cnp && (a.cf + jj) != (a.cfp + jjp)) {
+            const bool in = jj < a.cn && jjp < a.cnp && (a.cf + jj) != (a.cfp + jjp);
+            if constexpr (WEAK) {
+                const int w0 = (tp[buf].n0 + col0) >> 5;
+#pragma unroll
+                for (int w = 0; w < 2; ++w)
+                    if (in && 32 * (w0 + w) < a.N)
+                        weak[a.weak0 + (int64_t)(w0 + w) * a.cn * a.cnp + (int64_t)jj * a.cnp + jjp] = bits[w];
+            } else if (in) {
                 const int n0 = tp[buf].n0 + col0;
                 const int4 *__restrict__ cm = reinterpret_cast<const int4 *>(cols + a.col0 + n0);
                 int ea = 0;
@@ -675,6 +731,83 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+    }
+}
+
+// The weak elements of an FP64 build summed in FP64 after the digits: a warp takes
+// 32 rows (orbital pairs, one a lane) x 32 columns, and of those up to four elements
+// of a column at a time, a lane every 32nd label in their order, so that the sums do
+// not depend on which labels a symmetry-blocked panel leaves out.  digit_blk: the
+// first tile of every task in the digits' launch, of whose tiles this shard takes
+// every shard_n-th.  It reads a bit an element; were all elements weak, 22500 pairs x
+// 210 columns over 1367 labels, it would take 15.5 ms, bound by the FP64 pipe, which
+// takes 14.0 for all sums.
+__global__ void __launch_bounds__(256)
+fp64_elements_kernel(const SplitTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks,
+                     const int64_t *__restrict__ digit_blk, const uint32_t *__restrict__ weak,
+                     const double *__restrict__ panel, int n_co, int Kc, int K, const int32_t *__restrict__ labels,
+                     const ExpCol *__restrict__ all_cols, int shard_r, int shard_n) {
+    constexpr unsigned full = 0xffffffffu;
+    const int ti = task_of(blk, n_tasks, blockIdx.x), lane = threadIdx.x & 31;
+    const SplitTask &T = tasks[ti];
+    const int64_t rows = (int64_t)T.cn * T.cnp, padded = (rows + 31) / 32 * 32;
+    const int64_t i = (blockIdx.x - blk[ti]) * (int64_t)256 + threadIdx.x;
+    const int w = (int)(i / padded);               // the same in a warp
+    const int64_t row = i % padded;
+    if (w >= T.weak_words) return;
+    const int jj = (int)(row / T.cnp), jjp = (int)(row % T.cnp);
+    uint32_t todo = row < rows && T.cf + jj != T.cfp + jjp ? weak[T.weak0 + w * rows + row] : 0;
+    const int nc = T.N - 32 * w;
+    todo &= nc >= 32 ? ~0u : (1u << nc) - 1u;
+    uint32_t any = __reduce_or_sync(full, todo);
+    if (any == 0) return;
+    const int tile_m = (jj / (BM >> T.bjp_log2)) * T.jpt_tiles + (jjp >> T.bjp_log2);
+    const unsigned long long mine = (unsigned long long)(panel + ((int64_t)(T.cf + jj) * n_co + T.cfp + jjp) * Kc);
+    const int32_t *__restrict__ lab = labels ? labels + T.kc0 * 64 : nullptr;
+    while (any) {
+        const int c = 32 * w + __ffs(any) - 1;
+        unsigned left = __ballot_sync(full, ((todo >> (__ffs(any) - 1)) & 1u) &&
+                                                (digit_blk[ti] + (int64_t)tile_m * T.ntn + c / T.bn) % shard_n == shard_r);
+        any &= any - 1;
+        const ExpCol e = all_cols[T.col0 + c];
+        while (left) {
+            int src[4], n = 0;
+            const double *p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                src[u] = left ? __ffs(left) - 1 : src[0];
+                n += left != 0;
+                left &= left - 1;
+                p[u] = (const double *)__shfl_sync(full, mine, src[u]);
+            }
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int l = lane; l < K; l += 32) {
+                int k = l;                        // the label's panel column
+                if (lab) {
+                    int b = 0, t = Kc;            // (padding columns, label -1, come last)
+                    while (b < t) {
+                        const int m = (b + t) / 2, x = __ldg(lab + m);
+                        if (x >= 0 && x < l) b = m + 1;
+                        else t = m;
+                    }
+                    if (b == Kc || __ldg(lab + b) != l) continue;
+                    k = b;
+                }
+                const double a = __ldg(e.arow + l);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (u < n) v[u] = fma(__ldg(p[u] + k), a, v[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                for (int o = 16; o; o >>= 1) v[u] += __shfl_xor_sync(full, v[u], o);
+                if (u < n && lane == src[u] && jj - jjp >= e.jmin) {
+                    e.lower[(int64_t)jj * e.ld + jjp] = v[u];
+                    e.upper[(int64_t)jjp * e.ld + jj] = v[u];
+                }
+            }
+        }
     }
 }
 
@@ -873,11 +1006,23 @@ __device__ __forceinline__ uint32_t slice_bits(float d, int e) {
     return __bfloat16_as_ushort(__float2bfloat16_rn(ldexpf(d, e)));
 }
 
+// Magnitude of x against a row exponent as a bf16: the leading 8 bits of |x| / 2^emax,
+// rounded down, in units of 2^-8; 2^-40 where they are zero and x is not, or where a
+// value of the row is not finite.
+__device__ __forceinline__ uint32_t magnitude_bits(double x, int emax) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if ((b << 1) == 0) return 0;
+    const int be = (int)((b >> 52) & 0x7FF), sh = 1075 - 8 - be + emax;      // 45 or more
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const uint32_t top = be != 0 && emax > -2000 && emax <= 1024 && sh < 64 ? (uint32_t)(m >> sh) : 0;
+    return top ? slice_bits((float)top, -8) : (127 - 40) << 7;
+}
+
 // One row into its S bf16 slices by a whole block: every thread reads its
 // share of the row, the row exponent is reduced through shared memory, then
 // each thread writes the digits of its elements, two neighbours to a store.
 // at(k) gives element k (0 beyond the row's data).  With `exps` the row exponent
-// goes there and the slices are those of x / 2^e.
+// goes there, the slices are those of x / 2^e, and slice S holds the magnitudes.
 template <class At>
 __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S, int first, int step,
                                                 __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps = nullptr) {
@@ -905,6 +1050,7 @@ __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, 
         digits(at(k + 1), emax, S, first, step, [&](int i, float d) {
             o[i * (plane / 2)] = lo[i] | slice_bits(d, e0 - first - step * i) << 16;
         });
+        if (exps) o[S * (plane / 2)] = magnitude_bits(at(k), emax) | magnitude_bits(at(k + 1), emax) << 16;
     }
 }
 
@@ -942,6 +1088,9 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
             out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] =
                 __ushort_as_bfloat16((unsigned short)slice_bits(d, e0 - kXFirst - kXStep * i));
         });
+        if (exps)
+            out[(((int64_t)S * KB + kb) * R + dest) * BKB + kk] =
+                __ushort_as_bfloat16((unsigned short)(k != skip_col ? magnitude_bits(x[k], emax) : 0));
     }
 }
 
@@ -1133,8 +1282,8 @@ EncodeTiled encode_fn() {
 
 // dynamic shared memory of the expansion kernel: the operand slots, the
 // barriers and the 1 KB alignment
-static int split_smem_bytes(int bn, int ks) {
-    return xslots(bn, ks) * xslot(bn, ks) + 1024 + (2 * XBARS + 2 * XACC + 2) * 8;
+static int split_smem_bytes(int bn, int ks, int slots = 0) {
+    return (slots ? slots : xslots(bn, ks)) * xslot(bn, ks) + 1024 + (2 * XBARS + 2 * XACC + 2) * 8;
 }
 
 static int sm_count() {
@@ -1150,29 +1299,32 @@ static int sm_count() {
     return n;
 }
 
-template <int S, bool F64>
+template <int S, int MODE>
 static cudaError_t set_smem_attr_s() {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(split_expand_kernel<S, 32, 32, F64>, attr, split_smem_bytes(32, 32));
+    cudaError_t e = cudaFuncSetAttribute(split_expand_kernel<S, 32, 32, MODE>, attr, split_smem_bytes(32, 32));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(split_expand_kernel<S, 64, 32, F64>, attr, split_smem_bytes(64, 32));
-    if constexpr (!F64) {
+        e = cudaFuncSetAttribute(split_expand_kernel<S, 64, 32, MODE>, attr, split_smem_bytes(64, 32));
+    if constexpr (MODE == kMixedSums) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 32, F64>, attr, split_smem_bytes(128, 32));
+            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 32, MODE>, attr, split_smem_bytes(128, 32));
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 64, F64>, attr, split_smem_bytes(128, 64));
+            e = cudaFuncSetAttribute(split_expand_kernel<S, 128, 64, MODE>, attr, split_smem_bytes(128, 64));
+    } else if (e == cudaSuccess) {
+        e = cudaFuncSetAttribute(split_expand_kernel<1, kWeakCols, 64, kWeakBits>, attr,
+                                 split_smem_bytes(kWeakCols, 64, kWeakSlots));
     }
     return e;
 }
 
 static cudaError_t set_smem_attr(int S) {
     switch (S) {
-        case 2: return set_smem_attr_s<2, false>();
-        case 3: return set_smem_attr_s<3, false>();
-        case 4: return set_smem_attr_s<4, false>();
-        case 5: return set_smem_attr_s<5, false>();
-        case 6: return set_smem_attr_s<6, false>();
-        default: return set_smem_attr_s<kF64Slices, true>();
+        case 2: return set_smem_attr_s<2, kMixedSums>();
+        case 3: return set_smem_attr_s<3, kMixedSums>();
+        case 4: return set_smem_attr_s<4, kMixedSums>();
+        case 5: return set_smem_attr_s<5, kMixedSums>();
+        case 6: return set_smem_attr_s<6, kMixedSums>();
+        default: return set_smem_attr_s<kF64Slices, kF64Sums>();
     }
 }
 
@@ -1181,7 +1333,7 @@ static int mixed_fail(hb_ctx *ctx, int code, const std::string &m) {
     return code;
 }
 
-// The slices of an FP64 build are 14 bytes for every 8 of the panel, and it can do
+// The slices of an FP64 build are 16 bytes for every 8 of the panel, and it can do
 // without them: outside a caller's workspace (sized with them or not) they take
 // no more than an eighth of the memory that is free, so that the caller, other
 // contexts and the solve find about what they found before.
@@ -1219,7 +1371,8 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     // the panel's columns: every label, or with orbital symmetry the Kc labels
     // of each row's class
     const int Kc = ctx->Kc;
-    const size_t bytes = sizeof(__nv_bfloat16) * (size_t)PS.slices * rows * Kc;
+    const int planes = precision == HB_FP64 ? kF64Planes : PS.slices;
+    const size_t bytes = sizeof(__nv_bfloat16) * (size_t)planes * rows * Kc;
     if (precision == HB_FP64 && !f64_slices_fit(ctx, bytes))
         return mixed_fail(ctx, HB_ERR_OOM, "panel slices: more than an FP64 build may take");
     const size_t extra = precision == HB_MIXED ? sizeof(float2) * (size_t)ctx->n_co * Kc : sizeof(int16_t) * (size_t)rows;
@@ -1244,7 +1397,7 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     // 4D map over the panel slices [S*KB][j][j'][64]: coordinates (kk, j', j, plane)
     const int KB = Kc / BKB;
     cuuint64_t dims[4] = {(cuuint64_t)BKB, (cuuint64_t)ctx->n_co, (cuuint64_t)ctx->n_co,
-                          (cuuint64_t)PS.slices * KB};
+                          (cuuint64_t)planes * KB};
     cuuint64_t strides[3] = {(cuuint64_t)BKB * 2, (cuuint64_t)ctx->n_co * BKB * 2, (cuuint64_t)rows * BKB * 2};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = CUDA_SUCCESS;
@@ -1369,6 +1522,37 @@ int split_kstage_choice(int bn, int kblocks, int force) {
     return kblocks >= kK64Blocks ? 64 : 32;
 }
 
+// The line of a panel's weak elements (see the head of this file): half-way between
+// two sums of magnitudes, which are multiples of 2^-16 but for the 2^-40 ones, so
+// that the order in which they are added does not matter.
+static float weak_line(int K) {
+    const double at = std::max(std::sqrt((double)K) / 512.0, 1.0 / 128.0);
+    return (float)((std::floor(at * 65536.0) + 0.5) / 65536.0);
+}
+
+int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const Grouped<SplitTask> &g,
+                uint32_t *weak, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s) {
+    if (g.blocks <= 0) return 0;
+    const PanelSlices &PS = panel_ctx->mixed->panel[0];
+    const unsigned grid = (unsigned)std::min((int)g.blocks, sm_count());
+    split_expand_kernel<1, kWeakCols, 64, kWeakBits><<<grid, NTHREADS, split_smem_bytes(kWeakCols, 64, kWeakSlots), s>>>(
+        PS.tm[1][lg - 3], tm_coef[3], g.tasks, g.blk, g.n, (int)g.blocks, kblocks, coef_planes, cols, nullptr, nullptr,
+        weak, kF64Slices, weak_line(panel_ctx->K), panel_ctx->n_co, err, 0, 1);
+    return 1;
+}
+
+int64_t blocks_weak_sums(int cn, int cnp, int N) {
+    return (((int64_t)cn * cnp + 31) / 32 * 32 * ((N + 31) / 32) + 255) / 256;
+}
+int g_weak_sums(const hb_ctx *panel_ctx, const Grouped<SplitTask> &g, const Grouped<SplitTask> &digits,
+                const uint32_t *weak, int kblocks, const ExpCol *cols, cudaStream_t s, int shard_r, int shard_n) {
+    if (g.blocks <= 0) return 0;
+    fp64_elements_kernel<<<(unsigned)g.blocks, 256, 0, s>>>(
+        g.tasks, g.blk, g.n, digits.blk, weak, panel_ctx->panel, panel_ctx->n_co, kblocks * 64, panel_ctx->K,
+        panel_ctx->n_cls > 1 ? panel_ctx->cls_labels : nullptr, cols, shard_r, shard_n);
+    return 1;
+}
+
 int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef, const int16_t *coef_exps,
             const Grouped<SplitTask> &g, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s,
             int shard_r, int shard_n) {
@@ -1385,20 +1569,21 @@ int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtens
     const int n_local = n_tiles > shard_r ? (n_tiles - shard_r + shard_n - 1) / shard_n : 0;
     if (n_local <= 0) return 0;
     const unsigned grid = (unsigned)std::min(n_local, sm_count());
-#define HB_SPLIT(SS, BB, KK, FF)                                                                                   \
-    split_expand_kernel<SS, BB, KK, FF><<<grid, NTHREADS, smem, s>>>(tm_panel, tm_c, g.tasks, g.blk, g.n, n_tiles, \
-                                                                     kblocks, coef_planes, cols, PS.exps, coef_exps,    \
-                                                                     panel_ctx->n_co, err, shard_r, shard_n)
-#define HB_SPLIT_S(SS)                                \
-    do {                                              \
-        if (bn == 32) HB_SPLIT(SS, 32, 32, false);        \
-        else if (bn == 64) HB_SPLIT(SS, 64, 32, false);   \
-        else if (ks == 32) HB_SPLIT(SS, 128, 32, false);  \
-        else HB_SPLIT(SS, 128, 64, false);                \
+#define HB_SPLIT(SS, BB, KK, MM)                                                                                   \
+    split_expand_kernel<SS, BB, KK, MM><<<grid, NTHREADS, smem, s>>>(tm_panel, tm_c, g.tasks, g.blk, g.n, n_tiles, \
+                                                                     kblocks, coef_planes, cols, PS.exps, coef_exps, \
+                                                                     nullptr, 0, 0.0f, panel_ctx->n_co, err, shard_r, \
+                                                                     shard_n)
+#define HB_SPLIT_S(SS)                                       \
+    do {                                                     \
+        if (bn == 32) HB_SPLIT(SS, 32, 32, kMixedSums);      \
+        else if (bn == 64) HB_SPLIT(SS, 64, 32, kMixedSums); \
+        else if (ks == 32) HB_SPLIT(SS, 128, 32, kMixedSums);\
+        else HB_SPLIT(SS, 128, 64, kMixedSums);              \
     } while (0)
     if (f64) {
-        if (bn == 32) HB_SPLIT(kF64Slices, 32, 32, true);
-        else HB_SPLIT(kF64Slices, 64, 32, true);
+        if (bn == 32) HB_SPLIT(kF64Slices, 32, 32, kF64Sums);
+        else HB_SPLIT(kF64Slices, 64, 32, kF64Sums);
         return 1;
     }
     switch (PS.slices) {
