@@ -151,7 +151,8 @@ typedef struct {
     int32_t split_tile;       /* 0 = chosen; 3, 4, 5: tensor-core tiles of (128 >> v) j x (1 << v) j' */
     int32_t class4_states;    /* 0 = chosen; 4, 8, ..., 32, 40, 48, 56, 64: target states per pass of the
                                  double-float class-4 kernel */
-    int32_t class4_threads;   /* 0 = chosen; 32, 64, 128: continuum orbitals per class-4 block */
+    int32_t class4_threads;   /* 0 = chosen (up to 224); 32, 64, 128: continuum orbitals per block of the
+                                 double-float class-4 kernel */
     int32_t class4_path;      /* mixed build, class 4: 0 = tensor cores for groups of 32..64 states and
                                  the double-float kernel for the rest; 1 = the double-float kernel
                                  only; 2 = tensor cores for every group of 1..64 states */
@@ -215,7 +216,7 @@ typedef struct {
     double max_residual;
     float ms_matvec;
     float ms_rr;              /* hb_diag: host time of the small eigenproblems */
-    double expand_tensor_flops;  /* mixed: bf16 tensor flops of the split products */
+    double expand_tensor_flops;  /* bf16 tensor flops of the split products (0: sums on the FP64 pipe) */
     float ms_gram;            /* hb_diag: projections (device sums and their copy to the host) */
     float ms_combine;         /* hb_diag: basis combinations (coefficients to the device, kernel) */
     float ms_class4_kernel;   /* the class-4 kernels after their classification (part of ms_class4) */
@@ -281,13 +282,15 @@ int hb_set_workspace(hb_ctx *ctx, void *dev_ptr, size_t bytes);
 int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
 
 /* Build every class (1-8) into the caller's device buffers.  precision:
-   HB_FP64 (double arithmetic; the sums of Eq. 7 exact sums of the products of
-   the operands' 62 leading bits, counted from the largest entry of a row of
-   labels, rounded once, or sums in double where the magnitudes of the terms
-   are so small beside those largest entries that these are closer; on the
-   tensor cores where the operand slices, 16 bytes for every 8 of the expansion panel, are at most an eighth of the
-   free device memory, or within a workspace measured with them; they are given
-   back where a mixed build or a solve of the context finds no room) or HB_MIXED: the continuum-continuum
+   HB_FP64 (double arithmetic; the sums of Eq. 7 on the tensor cores as exact
+   sums of the products of the operands' 62 leading bits, counted from the
+   largest entry of a row of labels, rounded once; elements whose terms are
+   small beside those largest entries are summed in double.  The operand
+   slices, 16 bytes for every 8 of the expansion panel, are made where they are
+   at most an eighth of the free device memory or within a workspace measured
+   with them, and given back where a mixed build or a solve of the context
+   finds no room; without them all sums are in double) or HB_MIXED: the
+   continuum-continuum
    contraction (Eq. 7), and class 4 (Eq. 5) of groups of 32..64 states (see
    hb_options.class4_path), on bf16 tensor cores with split operands, exact
    FP32 accumulation and double-float recovery; the target-side contraction

@@ -611,7 +611,7 @@ int stage_problem(hb_ctx *ctx, const hb_problem *p, const hb_options *o, cudaStr
     if (!ctx->l2_low_ptr) {
         // no listed columns: builds search the L2 pairs by segments
         DALLOC(ctx->l2_seg_off, (int64_t)std::max(p->n_l2, 1) * seg_count(p->n_l2));
-        k1_seg_offsets(ctx->l2, p->n_l2, ctx->l2, p->n_l2, W, 0, 2, 0, ctx->l2_seg_off, s);
+        k1_seg_offsets(ctx->l2, p->n_l2, W, ctx->l2_seg_off, s);
     }
     // --- per group pair scratch; the gamma item count needs the records
     const int n_keys = 2 * p->n_to * p->n_to;
@@ -1076,8 +1076,8 @@ extern "C" int hb_dump(const hb_ctx *ctx, const char *path) {
     fprintf(f, "orbitals: %d target + %d continuum, n_words %d, electrons %d + 1 (continuum spin %s)\n", ctx->n_to,
             ctx->n_co, ctx->W, ctx->n_elec, ctx->cont_spin == HB_SPIN_ALPHA ? "alpha" : "beta");
     fprintf(f, "dimension %lld = contracted %lld + L2 %d\n", (long long)ctx->dim, (long long)ctx->Dc, ctx->n_l2);
-    fprintf(f, "labels K %d (padded %d), e_core %.17g, split slices %d\n", ctx->K, ctx->Kpad, ctx->e_core,
-            ctx->split_slices);
+    fprintf(f, "labels K %d (padded %d), e_core %.17g, split slices %d (expansion %d)\n", ctx->K, ctx->Kpad,
+            ctx->e_core, ctx->split_slices, ctx->expand_slices);
     fprintf(f, "expansion panel: %d label class%s of %d columns%s\n", ctx->n_cls, ctx->n_cls > 1 ? "es" : "",
             ctx->Kc, ctx->n_cls > 1 ? " (orbital symmetry)" : "");
     for (int g = 0; g < ctx->n_groups; ++g) {

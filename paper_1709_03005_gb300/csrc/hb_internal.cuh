@@ -58,9 +58,9 @@ struct GammaItem {
 // segments of kSegCols, each with its own output offset within the row.
 constexpr int kSegCols = 512;
 int seg_count(int n_b);
-// seg_off[row][seg]: matches of the row in the segments before seg.
-void k1_seg_offsets(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int W, int mode, int max_degree,
-                    int lower, int32_t *seg_off, cudaStream_t s);
+// seg_off[row][seg]: matches of a row of an L2 list (within a double excitation) in
+// the segments before seg.
+void k1_seg_offsets(const uint64_t *dets, int n, int W, int32_t *seg_off, cudaStream_t s);
 void k1_count(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int W, int mode, int max_degree,
               int lower, int64_t *counts_plus1, cudaStream_t s);
 void k1_fill_pairs(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int W, int mode, int cont_spin,
@@ -81,30 +81,12 @@ void l2_mirror_fill(const int32_t *col, const int64_t *row_ptr, int n, const int
 
 // K5 Slater-Condon (k_slater.cu)
 void build_jk(const Ints &I, double *jk, cudaStream_t s);
-void l2_csr_fill(const Ints &I, const uint64_t *dets, int n, int W, const int64_t *row_ptr, int32_t *col,
-                 double *val, double e_core, cudaStream_t s);
-void pair_values(const Ints &I, const uint64_t *A, const uint64_t *B, int W, const hb_pair *pairs,
-                 int64_t n_pairs, double *val, cudaStream_t s);
 
 // K2 target side (k_target.cu)
-void sandwich_rows(const hb_pair *pairs, const int64_t *row_ptr, const double *val, int n_rows, const double *Cp,
-                   int nsp, double *Wout, cudaStream_t s);
 int tn_chunks(int n_rows);
-void gemm_tn_reduce(const double *C, const double *Wm, int n_rows, int ns, int nsp, double *partials,
-                    double *out, cudaStream_t s);
 void gamma_item_counts(const hb_pair *pairs, const int64_t *row_ptr, int n_rows, int n_elec,
                        int64_t *counts_plus1, cudaStream_t s);
-void gamma_item_fill(const hb_pair *pairs, const int64_t *row_ptr, int n_rows, const uint64_t *bra_dets, int W,
-                     int n_to, int n_elec, const int64_t *item_ptr, GammaItem *items, cudaStream_t s);
 int sort_chunks(int64_t n_items, int n_keys);
-void gamma_sort(const GammaItem *items, int64_t n_items, int n_keys, int64_t *offsets_plus1, int64_t *cursors,
-                int32_t *order, cudaStream_t s);
-void gamma_bins(const GammaItem *items, const int32_t *order, const int64_t *offsets, int n_keys,
-                int64_t n_items, const double *C, int ns, const double *Cp, int nsp, double *gamma,
-                cudaStream_t s);
-void assemble_coefficients(const double *gamma, const double *S, const double *E, const int32_t *nn, int n_nn,
-                           int ns, int nsp, int n_to, int cont_spin, double e_core, int Kpad, double *A,
-                           cudaStream_t s);
 
 // K3 expansion (k_expand.cu)
 void build_panel(const double *ttcc, const double *tctc, const double *h, int n_to, int n_co, int Kc,
@@ -113,10 +95,5 @@ void build_panel(const double *ttcc, const double *tctc, const double *h, int n_
 // is the class of label k, co_irrep the continuum orbitals' irreps)
 void check_panel_symmetry(const double *ttcc, const double *tctc, const double *h, int n_to, int n_co, int K,
                           const int32_t *label_cls, const int32_t *co_irrep, int *flag, cudaStream_t s);
-// K4 class 4 (k_class4.cu)
-// dfloat = 0: FP64 accumulation; 1: FP32 double-float accumulation (mixed path)
-void class4_build(const Ints &I, const hb_pair *pairs, const int64_t *row_ptr, int n_l2, const uint64_t *dets,
-                  const double *C, int ns, int cf, int cn, int W, int cont_spin, int64_t col_off, int64_t ld,
-                  double *Hlc, int dfloat, cudaStream_t s);
 
 }  // namespace hb

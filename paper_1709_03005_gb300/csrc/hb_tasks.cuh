@@ -269,7 +269,7 @@ struct L2MTask {        // classes 2 and 8: the entries below the diagonal from 
 // Each returns the number of kernel launches it made (0 for an empty stage).
 int g_classify(const Grouped<ClsTask> &g, int W, int mode, cudaStream_t s);
 int g_pair_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s);
-// the diagonal records (m, m) of same-group tasks, one thread per row
+// the diagonal records (m, m) of same-group tasks, a warp per row
 int g_diag_values(const Grouped<PVTask> &g, int W, int dfloat, cudaStream_t s);
 int64_t blocks_diag_values(int n_rows);
 int g_l2_csr(const Grouped<L2Task> &g, int W, cudaStream_t s);
@@ -304,7 +304,8 @@ size_t smem_gdiag(int ns);
 // shard_r, shard_n: only the blocks shard_r, shard_r + shard_n, ... of the grid do their tile
 int g_expand_fp64(const Grouped<XTask> &g, const ExpCol *cols, cudaStream_t s, int shard_r = 0, int shard_n = 1);
 // dfloat = 0: FP64; 1: double-float; ns_tile states a pass (a multiple of 4 up
-// to 32, or in double-float of 8 up to 64) and jt threads a block (32, 64 or 128)
+// to 32, or in double-float of 8 up to 64) and jt threads a block (class4_shape: a
+// multiple of 32 up to 224; the tuner and hb_options also offer 32, 64 and 128)
 int g_class4(const Grouped<C4Task> &g, int W, int dfloat, int ns_tile, int jt, cudaStream_t s);
 void class4_shape(int ns, int cn, int *ns_tile, int *jt);
 

@@ -141,28 +141,26 @@ k1_count_kernel(const uint64_t *__restrict__ A, int n_a, const uint64_t *__restr
     if (lane == 0) counts_plus1[row + 1] = cnt;
 }
 
-// Matches of each row within each segment of kSeg columns (one warp per
+// Matches of each row of an L2 list within each segment of kSeg columns (one warp per
 // (row, segment)), turned into offsets from the row start by seg_scan_kernel.
-template <int W, int MODE>
+template <int W>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock)
-k1_seg_count_kernel(const uint64_t *__restrict__ A, int n_a, const uint64_t *__restrict__ B, int n_b,
-                    int max_degree, int lower, int nseg, int32_t *__restrict__ cnt) {
+k1_seg_count_kernel(const uint64_t *__restrict__ D, int n, int nseg, int32_t *__restrict__ cnt) {
     const int lane = threadIdx.x & 31;
     const int64_t wid = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (wid >= (int64_t)n_a * nseg) return;
+    if (wid >= (int64_t)n * nseg) return;
     const int row = (int)(wid / nseg), sg = (int)(wid % nseg);
     uint64_t a[2 * W];
-    load_det<W>(A + (int64_t)row * 2 * W, a);
-    const int limit = lower ? min(n_b, row + 1) : n_b;
-    const int c_end = min(limit, (sg + 1) * kSeg);
+    load_det<W>(D + (int64_t)row * 2 * W, a);
+    const int c_end = min(n, (sg + 1) * kSeg);
     int c_cnt = 0;
     for (int c0 = sg * kSeg; c0 < c_end; c0 += 32) {
         const int c = c0 + lane;
         bool ok = false;
         if (c < c_end) {
             uint64_t b[2 * W];
-            load_det<W>(B + (int64_t)c * 2 * W, b);
-            ok = degree_of<W, MODE>(a, b) <= max_degree;
+            load_det<W>(D + (int64_t)c * 2 * W, b);
+            ok = degree_of<W, 0>(a, b) <= 2;
         }
         c_cnt += __popc(__ballot_sync(0xffffffffu, ok));
     }
@@ -330,20 +328,18 @@ void k1_fill_pairs(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int W
 
 int seg_count(int n_b) { return n_b > 0 ? (n_b + kSeg - 1) / kSeg : 1; }
 
-void k1_seg_offsets(const uint64_t *a, int n_a, const uint64_t *b, int n_b, int W, int mode, int max_degree,
-                    int lower, int32_t *seg_off, cudaStream_t s) {
-    if (n_a <= 0) return;
-    const int nseg = seg_count(n_b);
-    const unsigned grid = (unsigned)(((int64_t)n_a * nseg + kWarpsPerBlock - 1) / kWarpsPerBlock);
+void k1_seg_offsets(const uint64_t *dets, int n, int W, int32_t *seg_off, cudaStream_t s) {
+    if (n <= 0) return;
+    const int nseg = seg_count(n);
+    const unsigned grid = (unsigned)(((int64_t)n * nseg + kWarpsPerBlock - 1) / kWarpsPerBlock);
     const dim3 block(32 * kWarpsPerBlock);
-#define HB_SEG(WW, MM) k1_seg_count_kernel<WW, MM><<<grid, block, 0, s>>>(a, n_a, b, n_b, max_degree, lower, nseg, seg_off)
-    if (mode == 0) {
-        switch (W) { case 1: HB_SEG(1, 0); break; case 2: HB_SEG(2, 0); break; case 3: HB_SEG(3, 0); break; default: HB_SEG(4, 0); break; }
-    } else {
-        switch (W) { case 1: HB_SEG(1, 1); break; case 2: HB_SEG(2, 1); break; case 3: HB_SEG(3, 1); break; default: HB_SEG(4, 1); break; }
+    switch (W) {
+        case 1: k1_seg_count_kernel<1><<<grid, block, 0, s>>>(dets, n, nseg, seg_off); break;
+        case 2: k1_seg_count_kernel<2><<<grid, block, 0, s>>>(dets, n, nseg, seg_off); break;
+        case 3: k1_seg_count_kernel<3><<<grid, block, 0, s>>>(dets, n, nseg, seg_off); break;
+        default: k1_seg_count_kernel<4><<<grid, block, 0, s>>>(dets, n, nseg, seg_off); break;
     }
-#undef HB_SEG
-    seg_scan_kernel<<<(n_a + 255) / 256, 256, 0, s>>>(seg_off, n_a, nseg);
+    seg_scan_kernel<<<(n + 255) / 256, 256, 0, s>>>(seg_off, n, nseg);
 }
 
 int64_t blocks_seg_rows8(int64_t rows, int n_b) { return ((rows + 7) / 8) * seg_count(n_b); }

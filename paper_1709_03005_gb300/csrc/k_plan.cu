@@ -162,8 +162,9 @@ struct Plan {
     // taking the SMs they leave
     cudaStream_t main = nullptr, side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, join_main = nullptr;
-    // the target side's independent chains: the diagonal H^N values and the
-    // gamma items (aux1), the diagonal gamma (aux2), beside the E, S chain
+    // the target side's independent chains beside the E, S chain: the gamma items
+    // (aux1), the diagonal gamma and the diagonal H^N values (aux2); then, beside the
+    // expansion, the FP64 build's magnitudes (aux1) and the rows j = j' (aux2)
     cudaStream_t aux1 = nullptr, aux2 = nullptr;
     cudaEvent_t k1_done = nullptr, items_done = nullptr, gd_done = nullptr, asm_done = nullptr, dr_done = nullptr;
     cudaEvent_t slices_done = nullptr, bits_done = nullptr;

@@ -387,7 +387,7 @@ __device__ __forceinline__ void drain_int(uint32_t taddr, long long (&acc)[2][NC
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             float x = __uint_as_float(v[i]);
-            if (SS <= 2) x *= to_int;
+            if constexpr (SS <= 2) x *= to_int;
             else x = x * (float)(1ull << 40) * (float)(1ull << (16 + 9 * SS - 40));
             acc[w][c0 + i] += (long long)__float2int_rn(x) * (1ll << lift);
         }

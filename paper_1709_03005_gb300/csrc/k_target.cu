@@ -602,43 +602,43 @@ __global__ void gamma_kernel(const GTask *__restrict__ tasks, const int64_t *__r
     double *cb = sm + kItemBatch * ns;        // [kItemBatch][nsp]
     // keys of this block: one, or several where most have no items
     for (int key = lb / T.ny * T.kpb; key < min(T.n_keys, (lb / T.ny + 1) * T.kpb); ++key) {
-    // with no items (nc == 0) both ends are off[0] = 0 and gamma is zero
-    const int64_t b = T.off[(int64_t)key * T.nc];
-    const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) continue;    // empty key: never written, the coefficient rows read it as zero
-    const int nout = ns * nsp;
-    // each thread keeps up to 4 outputs in registers
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t i0 = b; i0 < e; i0 += kItemBatch) {
-        const int cnt = (int)(e - i0 < kItemBatch ? e - i0 : kItemBatch);
-        __syncthreads();
-        for (int t = threadIdx.x; t < cnt * ns; t += blockDim.x) {
-            const int i = t / ns, a = t % ns;
-            const GammaItem it = T.items[T.order[i0 + i]];
-            ca[i * ns + a] = it.phase * T.C[(int64_t)it.m * ns + a];
+        // with no items (nc == 0) both ends are off[0] = 0 and gamma is zero
+        const int64_t b = T.off[(int64_t)key * T.nc];
+        const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
+        if (b == e) continue;    // empty key: never written, the coefficient rows read it as zero
+        const int nout = ns * nsp;
+        // each thread keeps up to 4 outputs in registers
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int64_t i0 = b; i0 < e; i0 += kItemBatch) {
+            const int cnt = (int)(e - i0 < kItemBatch ? e - i0 : kItemBatch);
+            __syncthreads();
+            for (int t = threadIdx.x; t < cnt * ns; t += blockDim.x) {
+                const int i = t / ns, a = t % ns;
+                const GammaItem it = T.items[T.order[i0 + i]];
+                ca[i * ns + a] = it.phase * T.C[(int64_t)it.m * ns + a];
+            }
+            for (int t = threadIdx.x; t < cnt * nsp; t += blockDim.x) {
+                const int i = t / nsp, a = t % nsp;
+                const GammaItem it = T.items[T.order[i0 + i]];
+                cb[i * nsp + a] = T.Cp[(int64_t)it.mp * nsp + a];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
+                if (t < nout) {
+                    const int a = t / nsp, c = t % nsp;
+                    double s = acc[u];
+                    for (int i = 0; i < cnt; ++i) s = fma(ca[i * ns + a], cb[i * nsp + c], s);
+                    acc[u] = s;
+                }
+            }
         }
-        for (int t = threadIdx.x; t < cnt * nsp; t += blockDim.x) {
-            const int i = t / nsp, a = t % nsp;
-            const GammaItem it = T.items[T.order[i0 + i]];
-            cb[i * nsp + a] = T.Cp[(int64_t)it.mp * nsp + a];
-        }
-        __syncthreads();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
-            if (t < nout) {
-                const int a = t / nsp, c = t % nsp;
-                double s = acc[u];
-                for (int i = 0; i < cnt; ++i) s = fma(ca[i * ns + a], cb[i * nsp + c], s);
-                acc[u] = s;
-            }
+            if (t < nout) T.gamma[(int64_t)key * nout + t] = acc[u];
         }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
-        if (t < nout) T.gamma[(int64_t)key * nout + t] = acc[u];
-    }
     }
 }
 
@@ -651,21 +651,21 @@ __global__ void gamma_warp_kernel(const GTask *__restrict__ tasks, const int64_t
     const int key0 = ((int)(blockIdx.x - blk[ti]) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * T.kpb;
     const int ns = T.ns, nsp = T.nsp, nout = ns * nsp;
     for (int key = key0; key < min(T.n_keys, key0 + T.kpb); ++key) {
-    const int64_t b = T.off[(int64_t)key * T.nc];
-    const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) continue;
-    double acc0 = 0.0, acc1 = 0.0;
-    const int t0 = lane, t1 = lane + 32;
-    const int a0 = t0 / nsp, c0 = t0 % nsp, a1 = t1 / nsp, c1 = t1 % nsp;
-    for (int64_t i = b; i < e; ++i) {
-        const GammaItem it = T.items[T.order[i]];
-        if (t0 < nout)
-            acc0 = fma(it.phase * __ldg(T.C + (int64_t)it.m * ns + a0), __ldg(T.Cp + (int64_t)it.mp * nsp + c0), acc0);
-        if (t1 < nout)
-            acc1 = fma(it.phase * __ldg(T.C + (int64_t)it.m * ns + a1), __ldg(T.Cp + (int64_t)it.mp * nsp + c1), acc1);
-    }
-    if (t0 < nout) T.gamma[(int64_t)key * nout + t0] = acc0;
-    if (t1 < nout) T.gamma[(int64_t)key * nout + t1] = acc1;
+        const int64_t b = T.off[(int64_t)key * T.nc];
+        const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
+        if (b == e) continue;
+        double acc0 = 0.0, acc1 = 0.0;
+        const int t0 = lane, t1 = lane + 32;
+        const int a0 = t0 / nsp, c0 = t0 % nsp, a1 = t1 / nsp, c1 = t1 % nsp;
+        for (int64_t i = b; i < e; ++i) {
+            const GammaItem it = T.items[T.order[i]];
+            if (t0 < nout)
+                acc0 = fma(it.phase * __ldg(T.C + (int64_t)it.m * ns + a0), __ldg(T.Cp + (int64_t)it.mp * nsp + c0), acc0);
+            if (t1 < nout)
+                acc1 = fma(it.phase * __ldg(T.C + (int64_t)it.m * ns + a1), __ldg(T.Cp + (int64_t)it.mp * nsp + c1), acc1);
+        }
+        if (t0 < nout) T.gamma[(int64_t)key * nout + t0] = acc0;
+        if (t1 < nout) T.gamma[(int64_t)key * nout + t1] = acc1;
     }
 }
 
@@ -917,47 +917,47 @@ __global__ void gamma_df_kernel(const GTask *__restrict__ tasks, const int64_t *
     float2 *cb = smf + kItemBatch * ns;       // [kItemBatch][nsp]
     // keys of this block: one, or several where most have no items
     for (int key = lb / T.ny * T.kpb; key < min(T.n_keys, (lb / T.ny + 1) * T.kpb); ++key) {
-    const int64_t b = T.off[(int64_t)key * T.nc];
-    const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
-    if (b == e) continue;
-    const int nout = ns * nsp;
-    float ah[4] = {0.0f, 0.0f, 0.0f, 0.0f}, al[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int64_t i0 = b; i0 < e; i0 += kItemBatch) {
-        const int cnt = (int)(e - i0 < kItemBatch ? e - i0 : kItemBatch);
-        __syncthreads();
-        for (int t = threadIdx.x; t < cnt * ns; t += blockDim.x) {
-            const int i = t / ns, a = t % ns;
-            const GammaItem it = T.items[T.order[i0 + i]];
-            float2 x = T.C_df[(int64_t)it.m * ns + a];
-            if (it.phase < 0) { x.x = -x.x; x.y = -x.y; }
-            ca[i * ns + a] = x;
+        const int64_t b = T.off[(int64_t)key * T.nc];
+        const int64_t e = T.off[(int64_t)(key + 1) * T.nc];
+        if (b == e) continue;
+        const int nout = ns * nsp;
+        float ah[4] = {0.0f, 0.0f, 0.0f, 0.0f}, al[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int64_t i0 = b; i0 < e; i0 += kItemBatch) {
+            const int cnt = (int)(e - i0 < kItemBatch ? e - i0 : kItemBatch);
+            __syncthreads();
+            for (int t = threadIdx.x; t < cnt * ns; t += blockDim.x) {
+                const int i = t / ns, a = t % ns;
+                const GammaItem it = T.items[T.order[i0 + i]];
+                float2 x = T.C_df[(int64_t)it.m * ns + a];
+                if (it.phase < 0) { x.x = -x.x; x.y = -x.y; }
+                ca[i * ns + a] = x;
+            }
+            for (int t = threadIdx.x; t < cnt * nsp; t += blockDim.x) {
+                const int i = t / nsp, a = t % nsp;
+                const GammaItem it = T.items[T.order[i0 + i]];
+                cb[i * nsp + a] = T.Cp_df[(int64_t)it.mp * nsp + a];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
+                if (t < nout) {
+                    const int a = t / nsp, c = t % nsp;
+                    for (int i = 0; i < cnt; ++i) {
+                        const float2 x = ca[i * ns + a], y = cb[i * nsp + c];
+                        df_fma(ah[u], al[u], x.x, x.y, y.x, y.y);
+                    }
+                }
+            }
+            // keep the low words small over long keys
+#pragma unroll
+            for (int u = 0; u < 4; ++u) df_norm(ah[u], al[u]);
         }
-        for (int t = threadIdx.x; t < cnt * nsp; t += blockDim.x) {
-            const int i = t / nsp, a = t % nsp;
-            const GammaItem it = T.items[T.order[i0 + i]];
-            cb[i * nsp + a] = T.Cp_df[(int64_t)it.mp * nsp + a];
-        }
-        __syncthreads();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
-            if (t < nout) {
-                const int a = t / nsp, c = t % nsp;
-                for (int i = 0; i < cnt; ++i) {
-                    const float2 x = ca[i * ns + a], y = cb[i * nsp + c];
-                    df_fma(ah[u], al[u], x.x, x.y, y.x, y.y);
-                }
-            }
+            if (t < nout) reinterpret_cast<float2 *>(T.gamma)[(int64_t)key * nout + t] = make_float2(ah[u], al[u]);
         }
-        // keep the low words small over long keys
-#pragma unroll
-        for (int u = 0; u < 4; ++u) df_norm(ah[u], al[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int t = by * 4 * blockDim.x + u * blockDim.x + threadIdx.x;
-        if (t < nout) reinterpret_cast<float2 *>(T.gamma)[(int64_t)key * nout + t] = make_float2(ah[u], al[u]);
-    }
     }
 }
 
@@ -1119,8 +1119,6 @@ int64_t blocks_gdiag_reduce(int n_to, int ns) { return (int64_t)2 * n_to * ((ns 
 size_t smem_gdiag(int ns) { return sizeof(double) * ns * gdiag_batch(ns); }
 
 int64_t blocks_scan(int64_t n) { return (n + kScanSeg - 1) / kScanSeg; }
-
-int64_t scan_one_limit() { return kScanOne; }
 
 int g_scan(const Grouped<ScanTask> &g, int64_t longest, cudaStream_t s) {
     if (g.n <= 0) return 0;
