@@ -287,7 +287,7 @@ int64_t hb_group_offset(const hb_ctx *ctx, int32_t g);
    largest entry of a row of labels, rounded once; elements whose terms are
    small beside those largest entries are summed in double.  The operand
    slices, 16 bytes for every 8 of the expansion panel, are made where they are
-   at most an eighth of the free device memory or within a workspace measured
+   at most a quarter of the free device memory or within a workspace measured
    with them, and given back where a mixed build or a solve of the context
    finds no room; without them all sums are in double) or HB_MIXED: the
    continuum-continuum
