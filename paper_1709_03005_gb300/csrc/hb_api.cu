@@ -395,6 +395,7 @@ static int setup_label_classes(hb_ctx *ctx, const hb_problem *p, cudaStream_t s)
         if ((p->orb_irrep != nullptr) != (B->n_cls > 1))
             return fail(ctx, HB_ERR_INVALID_ARG, "orb_irrep must be given for the base context and this one alike");
         ctx->n_cls = B->n_cls; ctx->Kc = B->Kc; ctx->cls_labels = B->cls_labels; ctx->cls_labels_h = B->cls_labels_h;
+        ctx->cls_by_lane = B->cls_by_lane;
         ctx->co_irrep = B->co_irrep; ctx->co_irrep_d = B->co_irrep_d; ctx->delta_pos = B->delta_pos;
     } else if (!p->orb_irrep) {
         ctx->n_cls = 1;
@@ -419,6 +420,22 @@ static int setup_label_classes(hb_ctx *ctx, const hb_problem *p, cudaStream_t s)
                 if (lists[x][i] == delta_label) ctx->delta_pos = (int)i;
             }
         ctx->co_irrep.assign(p->orb_irrep + p->n_to, p->orb_irrep + n_orb);
+        std::vector<int32_t> by_lane((size_t)8 * 33 + 2 * (size_t)8 * ctx->Kc, 0);
+        for (int x = 0; x < 8; ++x) {
+            int32_t *ptr = &by_lane[(size_t)x * 33], *out = &by_lane[(size_t)8 * 33 + 2 * (size_t)x * ctx->Kc];
+            int n = 0;
+            for (int r = 0; r < 32; ++r) {
+                ptr[r] = n;
+                for (size_t i = 0; i < lists[x].size(); ++i)
+                    if (lists[x][i] % 32 == r) {
+                        out[2 * n] = (int32_t)i;
+                        out[2 * n++ + 1] = lists[x][i];
+                    }
+            }
+            ptr[32] = n;
+        }
+        DALLOC(ctx->cls_by_lane, by_lane.size());
+        CK(cudaMemcpyAsync(ctx->cls_by_lane, by_lane.data(), sizeof(int32_t) * by_lane.size(), cudaMemcpyHostToDevice, s));
         DALLOC(ctx->cls_labels, (size_t)8 * ctx->Kc);
         DALLOC(ctx->co_irrep_d, std::max(p->n_co, 1));
         CK(cudaMemcpyAsync(ctx->cls_labels, ctx->cls_labels_h.data(), sizeof(int32_t) * ctx->cls_labels_h.size(),

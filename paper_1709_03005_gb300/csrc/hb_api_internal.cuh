@@ -137,6 +137,10 @@ struct hb_ctx {
     int n_cls = 1, Kc = 0;
     int32_t *cls_labels = nullptr;          // device [n_cls][Kc]: the labels of each class (-1 padding)
     std::vector<int32_t> cls_labels_h;
+    // with symmetry, for sums over a class's labels in 32 parts, label mod 32, as those
+    // over all labels have them: device int32 [8][33] first entries of the parts, then
+    // int2 [8][Kc] (column, label) part after part, labels ascending
+    int32_t *cls_by_lane = nullptr;
     std::vector<int32_t> co_irrep;          // irrep of every continuum orbital (empty without symmetry)
     int32_t *co_irrep_d = nullptr;
     int delta_pos = 0;                      // panel column of the delta label (in class 0)

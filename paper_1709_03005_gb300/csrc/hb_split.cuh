@@ -8,6 +8,15 @@
 #include "hb_api_internal.cuh"
 #include "hb_tasks.cuh"
 
+// Scale of a row of an FP64 build's operand: the exponent its slices are apart from,
+// and the line below which sums of magnitudes are weak.
+namespace hb {
+struct RowScale {
+    int32_t exp;
+    float line;
+};
+}  // namespace hb
+
 // Panel slices and tensor maps of a context (or of the context it borrows from)
 // for one precision.
 int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s);
@@ -23,9 +32,8 @@ int mixed_slices(const hb_ctx *ctx, int precision);
 const float2 *mixed_panel_diag(const hb_ctx *ctx);
 // Coefficient slices [S][Kpad/64][rows][64] bf16 and their tensor maps
 // tm[0..3]: 32-K stages at tile widths 32, 64, 128, and 64-K stages at 128.
-// exps (or null): the rows' exponents, kept apart from the slices (S then counts
-// the magnitudes too).
-int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int16_t **exps, CUtensorMap *tm,
+// scales (FP64, or null): those of the rows (S then counts the magnitudes too).
+int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, hb::RowScale **scales, CUtensorMap *tm,
                      std::string *err);
 int64_t blocks_split(int cn, int cnp, int N, int lg, int bn);
 int split_ntn(int N, int bn);
@@ -41,14 +49,14 @@ int split_tile_heuristic(int cn, int cnp);
 // coefficient rows of Kin labels into slices of Kout columns, column k being
 // label perm[k] (null: label k)
 int g_slice(const hb::Grouped<hb::SliceTask> &g, int64_t R, int Kin, int Kout, const int32_t *perm, int S,
-            int skip_col, void *out, int16_t *exps, cudaStream_t s);
+            int skip_col, void *out, hb::RowScale *scales, cudaStream_t s);
 // lg: tile arrangement (3..5, see SplitTask) and bn: tile width (32, 64,
 // 128); every task of g must use both.  tm_coef: the four coefficient maps.
 // kblocks: 64-wide K blocks of the panel rows; coef_planes: K blocks per
 // slice of the coefficient slices (the task's kc0 selects its label class)
 // shard_r, shard_n: the launch takes tiles shard_r, shard_r + shard_n, ... only
 int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef,
-            const int16_t *coef_exps, const hb::Grouped<hb::SplitTask> &g, int kblocks, int coef_planes,
+            const hb::RowScale *coef_scales, const hb::Grouped<hb::SplitTask> &g, int kblocks, int coef_planes,
             const hb::ExpCol *cols, int *err, cudaStream_t s, int shard_r = 0, int shard_n = 1);
 // FP64 build: a bit an element (SplitTask::weak0), set where the digits are not good
 // enough, from the magnitudes; g: the blocks of `digits` (g_split's) in tiles of
@@ -58,8 +66,8 @@ constexpr int kWeakCols = 128;
 int64_t blocks_weak_sums(int cn, int cnp, int N);
 int g_weak_sums(const hb_ctx *panel_ctx, const hb::Grouped<hb::SplitTask> &g, const hb::Grouped<hb::SplitTask> &digits,
                 const uint32_t *weak, int kblocks, const hb::ExpCol *cols, cudaStream_t s, int shard_r, int shard_n);
-int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const hb::Grouped<hb::SplitTask> &g,
-                uint32_t *weak, int kblocks, int coef_planes, const hb::ExpCol *cols, int *err, cudaStream_t s);
+int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const hb::RowScale *coef_scales,
+                const hb::Grouped<hb::SplitTask> &g, uint32_t *weak, int kblocks, int coef_planes, const hb::ExpCol *cols, int *err, cudaStream_t s);
 int64_t blocks_diag_rows(int j_lo, int j_hi, int n_nn);
 int diag_rows_ny(int n_nn);
 int g_diag_rows(const hb::Grouped<hb::DRTask> &g, int dfloat, cudaStream_t s);

@@ -142,7 +142,7 @@ struct Plan {
     bool upload_pending = false;
     // tensor-core operands
     void *coef = nullptr;
-    int16_t *coef_exps = nullptr;      // FP64 build: the coefficient rows' exponents
+    RowScale *coef_scales = nullptr;   // FP64 build: the coefficient rows' scales
     CUtensorMap tm_coef[4];            // coefficient slices: 32-K stages at widths 32, 64, 128; 64-K at 128
     int64_t coef_rows = 0;
     uint32_t *weak = nullptr;          // FP64: the bits of the elements summed in FP64
@@ -721,7 +721,7 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
     if (any_pairs && room && precision == HB_FP64) {
         const int S = mixed_slices(ctxs[0], precision);
         rc = f64_slices_fit(ctxs[0], 2 * (size_t)(S + 1) * rows * p->Kw)
-                 ? split_coef_alloc(ctxs[0], S + 1, rows, p->Kw, &p->coef, &p->coef_exps, p->tm_coef, err) : HB_ERR_OOM;
+                 ? split_coef_alloc(ctxs[0], S + 1, rows, p->Kw, &p->coef, &p->coef_scales, p->tm_coef, err) : HB_ERR_OOM;
         room = rc == HB_OK;
         if (rc == HB_ERR_OOM) rc = HB_OK;
         if (rc != HB_OK) { plan_destroy(p); return rc; }
@@ -745,9 +745,9 @@ int plan_create(hb_ctx *const *ctxs, int n, const hb_blocks *outs, int precision
         if (precision == HB_FP64 && rc == HB_ERR_OOM) {
             rc = HB_OK;
             dfree(ctxs[0], p->coef);
-            dfree(ctxs[0], p->coef_exps);
+            dfree(ctxs[0], p->coef_scales);
             p->coef = nullptr;
-            p->coef_exps = nullptr;
+            p->coef_scales = nullptr;
         }
         if (rc != HB_OK) { plan_destroy(p); return rc; }
         p->delta_col = ctxs[0]->delta_pos;   // the delta label's column (class 0 comes first)
@@ -933,7 +933,7 @@ int plan_autotune(Plan *p, cudaStream_t s, std::string *err) {
                     }
                     if (ts.empty()) continue;
                     ms += time_tasks(p->ctxs[0], ts, nb, [&](const Grouped<SplitTask> &g) {
-                        g_split(pc, p->precision, lg, bn, p->tm_coef, p->coef_exps, g, p->Kc / 64,
+                        g_split(pc, p->precision, lg, bn, p->tm_coef, p->coef_scales, g, p->Kc / 64,
                                 p->Kw / 64, p->d_cols, p->err, s);
                     }, s);
                 }
@@ -1159,7 +1159,7 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
                 L += g_diag_rows(p->drows.g, DF, sb);
                 cudaEventRecord(p->dr_done, sb);
             }
-            L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, p->coef_exps,
+            L += g_slice(p->slc.g, p->coef_rows, p->Kpad, p->Kw, p->perm, p->S, p->delta_col, p->coef, p->coef_scales,
                          s);
             // FP64: the bits of the elements that the digits are not good enough for,
             // in CTAs that fit beside class 4's
@@ -1167,14 +1167,14 @@ int plan_run(Plan *p, cudaStream_t s, bool timing, bool capture, int *launches, 
                 cudaEventRecord(p->slices_done, s);
                 cudaStreamWaitEvent(sa, p->slices_done, 0);
                 for (auto &g : p->split)
-                    L += g_weak_bits(g.panel_ctx, g.lg, p->tm_coef, g.weak.g, p->weak, p->Kc / 64, p->Kw / 64, p->d_cols,
-                                     p->err, sa);
+                    L += g_weak_bits(g.panel_ctx, g.lg, p->tm_coef, p->coef_scales, g.weak.g, p->weak, p->Kc / 64, p->Kw / 64,
+                                     p->d_cols, p->err, sa);
                 cudaEventRecord(p->bits_done, sa);
             }
             if (after_c4 && !DF) cudaStreamWaitEvent(s, p->c4_done, 0);
             for (size_t i = 0; i < p->split.size(); ++i) {
                 rec(p->ev_split[2 * i]);
-                LX += g_split(p->split[i].panel_ctx, p->precision, p->split[i].lg, p->split[i].bn, p->tm_coef, p->coef_exps,
+                LX += g_split(p->split[i].panel_ctx, p->precision, p->split[i].lg, p->split[i].bn, p->tm_coef, p->coef_scales,
                               p->split[i].st.g, p->Kc / 64, p->Kw / 64,
                               p->d_cols, p->err, s, p->shard_r, p->shard_n);
                 rec(p->ev_split[2 * i + 1]);
@@ -1352,7 +1352,7 @@ void plan_destroy(Plan *p) {
     if (mem) {
         dfree(mem, p->dev);
         dfree(mem, p->coef);
-        dfree(mem, p->coef_exps);
+        dfree(mem, p->coef_scales);
         dfree(mem, p->weak);
         dfree(mem, p->err);
     }

@@ -37,12 +37,15 @@
 // the one row meet zeros or tiny entries of the other (h_jj' of 50 and S = 0
 // between groups, beside integrals of 1e-6) M can be so small that FP64 is closer.
 // So the FP64 build carries an eighth slice, the magnitudes to 8 bits rounded down,
-// whose product is a lower bound of M: an element with 0 < M < sqrt(K) 2^-9 of the
-// scales (there the typical errors are alike; at least 2^-7, where the bounds are)
+// whose product is a lower bound of M: an element with 0 < M < sqrt(K') 2^-9 of the
+// scales (K' nonzero entries in the row that has fewer; there the typical errors are
+// alike; at least 2^-7, where the bounds are)
 // is summed in FP64 (fp64_elements_kernel).  Magnitudes below 2^-9 count as 2^-40,
 // so M = 0 means that no two entries meet, and the sum is exactly zero; a row with a
-// value that is not finite is all 2^-40.  Molecular integrals and target densities stay far above the line
-// (the lowest 1e-3 of M lies at 0.05 to 0.6 of the scales, the line at 0.03 to 0.08).
+// value that is not finite is all 2^-40.  Molecular integrals with dense target
+// densities lie above the line (the lowest 1e-3 of M at 0.05 to 0.6 of the scales, the
+// line at 0.01 to 0.08); densities of a few entries, between small groups of a batch
+// over symmetries, leave 0.1 % of the elements below it.
 // The magnitudes are multiplied by a launch of their own (this kernel with one
 // slice and 128-wide tiles), which leaves a bit an element, beside what comes before
 // the digits: an eighth pair of tiles in every stage of those made them 22 % slower
@@ -85,7 +88,7 @@ namespace hb {
 struct PanelSlices {
     int slices = 0;
     __nv_bfloat16 *buf = nullptr;            // [S][Kpad/64][n_co*n_co][64] (FP64: S + 1, the last the magnitudes)
-    int16_t *exps = nullptr;                 // FP64: row exponents [n_co*n_co]
+    RowScale *scales = nullptr;              // FP64: those of the rows [n_co*n_co]
     // [stage width 32, 64][box of 8 x 16, 16 x 8, 32 x 4 continuum pairs (j' x j)]
     CUtensorMap tm[2][3];
     bool ready = false, borrowed = false;
@@ -394,9 +397,9 @@ __device__ __forceinline__ void drain_int(uint32_t taddr, long long (&acc)[2][NC
     }
 }
 
-// The magnitude sums of 32 columns: bit c set where the digits of column c are
-// not good enough (see the head of this file).
-__device__ __forceinline__ uint32_t drain_weak(uint32_t taddr, float line) {
+// The magnitude sums of 32 columns, of which n exist: bit c set where the digits of
+// column c are not good enough (see the head of this file).
+__device__ __forceinline__ uint32_t drain_weak(uint32_t taddr, float line, const RowScale *__restrict__ cols, int n) {
     uint32_t weak = 0;
 #pragma unroll
     for (int c0 = 0; c0 < 32; c0 += 16) {
@@ -407,14 +410,14 @@ __device__ __forceinline__ uint32_t drain_weak(uint32_t taddr, float line) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const float x = __uint_as_float(v[i]);
-            if (x > 0.0f && x < line) weak |= 1u << (c0 + i);
+            if (c0 + i < n && x > 0.0f && x < fminf(line, __ldg(&cols[c0 + i].line))) weak |= 1u << (c0 + i);
         }
     }
     return weak;
 }
 
 // The FP64 element of the two words and the row and column exponents.
-constexpr int kExpNaN = 32767;               // exponent of a row with a value that is not finite
+constexpr int kExpNaN = 1 << 20;               // exponent of a row with a value that is not finite
 __device__ __forceinline__ double int_words_to_double(long long a, long long b, int ea, int eb) {
     if (ea == kExpNaN || eb == kExpNaN) return __longlong_as_double(0x7FF8000000000000ll);
     const double v = fma((double)b, 0x1p-36, (double)a);
@@ -485,16 +488,16 @@ __device__ __forceinline__ TilePos tile_pos(const SplitTask *__restrict__ tasks,
 // The slot ring, the accumulator hand-over and their barrier phases run on
 // across tiles, so the loads and MMAs of the next tile start while the
 // epilogue warps still write the last one out from registers.  kF64Sums: the FP64
-// build's kernel (integer sums, exponents apart: pexp of the panel's rows,
-// n_co x n_co, cexp of the coefficient rows).  kWeakBits: a bit an element in `weak`,
-// set where the sum of the magnitudes (plane `plane0` of the slices) is below `line`.
+// build's kernel (integer sums, exponents apart: pscale of the panel's rows,
+// n_co x n_co, cscale of the coefficient rows).  kWeakBits: a bit an element in `weak`,
+// set where the sum of the magnitudes (plane `plane0` of the slices) is below the
+// lines of its rows.
 template <int S, int TBN, int KS, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_constant__ CUtensorMap tm_coef,
                     const SplitTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int n_tiles,
-                    int kblocks, int coef_planes, const ExpCol *__restrict__ cols, const int16_t *__restrict__ pexp,
-                    const int16_t *__restrict__ cexp, uint32_t *__restrict__ weak, int plane0, float line, int n_co,
-                    int *err, int shard_r, int shard_n) {
+                    int kblocks, int coef_planes, const ExpCol *__restrict__ cols, const RowScale *__restrict__ pscale,
+                    const RowScale *__restrict__ cscale, uint32_t *__restrict__ weak, int plane0, int n_co, int *err, int shard_r, int shard_n) {
     // this launch's tiles: shard_r, shard_r + shard_n, ... (all of them unless
     // sharded), numbered t = 0, 1, ... so that every role walks the same list
     const int n_local = n_tiles > shard_r ? (n_tiles - shard_r + shard_n - 1) / shard_n : 0;
@@ -653,7 +656,13 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                     if (!ok) continue;
                     tc_fence_after();
                     if constexpr (WEAK) {
-                        for (int w = 0; w < 2; ++w) bits[w] = drain_weak(tq + 32 * w, line);
+                        const int jj = tp[buf].jj0 + (row >> a.bjp_log2), jjp = tp[buf].jjp0 + (row & ((1 << a.bjp_log2) - 1));
+                        const float line = jj < a.cn && jjp < a.cnp
+                                               ? __ldg(&pscale[(int64_t)(a.cf + jj) * n_co + a.cfp + jjp].line) : 0.0f;
+                        const int n0 = tp[buf].n0 + col0;
+#pragma unroll
+                        for (int w = 0; w < 2; ++w)
+                            bits[w] = drain_weak(tq + 32 * w, line, cscale + a.coef_row0 + n0 + 32 * w, a.N - n0 - 32 * w);
                     } else if constexpr (F64) {
                         if (b == 0) drain_int<0>(tq, wd);
                         else if (b == 1) drain_int<1>(tq + TBN, wd);
@@ -690,7 +699,7 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                 const int n0 = tp[buf].n0 + col0;
                 const int4 *__restrict__ cm = reinterpret_cast<const int4 *>(cols + a.col0 + n0);
                 int ea = 0;
-                if constexpr (F64) ea = __ldg(pexp + (int64_t)(a.cf + jj) * n_co + a.cfp + jjp);
+                if constexpr (F64) ea = __ldg(&pscale[(int64_t)(a.cf + jj) * n_co + a.cfp + jjp].exp);
                 // two columns' destinations are fetched together
 #pragma unroll
                 for (int c0 = 0; c0 < ECOLS; c0 += 2) {
@@ -701,7 +710,7 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
                         if (n0 + c0 + u < a.N) {
                             d0[u] = __ldg(cm + 2 * (c0 + u));
                             d1[u] = __ldg(cm + 2 * (c0 + u) + 1);
-                            if constexpr (F64) eb[u] = __ldg(cexp + a.coef_row0 + n0 + c0 + u);
+                            if constexpr (F64) eb[u] = __ldg(&cscale[a.coef_row0 + n0 + c0 + u].exp);
                         }
                     float vh[2] = {}, vl[2] = {};
                     if constexpr (!F64) {
@@ -745,7 +754,7 @@ split_expand_kernel(const __grid_constant__ CUtensorMap tm_panel, const __grid_c
 __global__ void __launch_bounds__(256)
 fp64_elements_kernel(const SplitTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks,
                      const int64_t *__restrict__ digit_blk, const uint32_t *__restrict__ weak,
-                     const double *__restrict__ panel, int n_co, int Kc, int K, const int32_t *__restrict__ labels,
+                     const double *__restrict__ panel, int n_co, int Kc, int K, const int32_t *__restrict__ by_lane,
                      const ExpCol *__restrict__ all_cols, int shard_r, int shard_n) {
     constexpr unsigned full = 0xffffffffu;
     const int ti = task_of(blk, n_tasks, blockIdx.x), lane = threadIdx.x & 31;
@@ -763,7 +772,13 @@ fp64_elements_kernel(const SplitTask *__restrict__ tasks, const int64_t *__restr
     if (any == 0) return;
     const int tile_m = (jj / (BM >> T.bjp_log2)) * T.jpt_tiles + (jjp >> T.bjp_log2);
     const unsigned long long mine = (unsigned long long)(panel + ((int64_t)(T.cf + jj) * n_co + T.cfp + jjp) * Kc);
-    const int32_t *__restrict__ lab = labels ? labels + T.kc0 * 64 : nullptr;
+    // this lane's labels (and their panel columns): every 32nd, or those of them that
+    // the block's class holds
+    const int cls = T.kc0 * 64 / Kc;
+    const int l0 = by_lane ? __ldg(by_lane + cls * 33 + lane) : 0;
+    const int n_lab = by_lane ? __ldg(by_lane + cls * 33 + lane + 1) - l0 : (K - lane + 31) / 32;
+    const int2 *__restrict__ mine_lab =
+        by_lane ? reinterpret_cast<const int2 *>(by_lane + 8 * 33) + (int64_t)cls * Kc + l0 : nullptr;
     while (any) {
         const int c = 32 * w + __ffs(any) - 1;
         unsigned left = __ballot_sync(full, ((todo >> (__ffs(any) - 1)) & 1u) &&
@@ -781,22 +796,22 @@ fp64_elements_kernel(const SplitTask *__restrict__ tasks, const int64_t *__restr
                 p[u] = (const double *)__shfl_sync(full, mine, src[u]);
             }
             double v[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int l = lane; l < K; l += 32) {
-                int k = l;                        // the label's panel column
-                if (lab) {
-                    int b = 0, t = Kc;            // (padding columns, label -1, come last)
-                    while (b < t) {
-                        const int m = (b + t) / 2, x = __ldg(lab + m);
-                        if (x >= 0 && x < l) b = m + 1;
-                        else t = m;
-                    }
-                    if (b == Kc || __ldg(lab + b) != l) continue;
-                    k = b;
-                }
-                const double a = __ldg(e.arow + l);
+            // the loads of four labels are in flight together
+            for (int i0 = 0; i0 < n_lab; i0 += 4) {
+                double a[4], x[4][4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (u < n) v[u] = fma(__ldg(p[u] + k), a, v[u]);
+                for (int t = 0; t < 4; ++t) {
+                    const int i = i0 + t;
+                    const int2 kl = i >= n_lab ? make_int2(0, 0) : (mine_lab ? __ldg(mine_lab + i) : make_int2(lane + 32 * i, lane + 32 * i));
+                    a[t] = i < n_lab ? __ldg(e.arow + kl.y) : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[t][u] = i < n_lab && u < n ? __ldg(p[u] + kl.x) : 0.0;
+                }
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (u < n && i0 + t < n_lab) v[u] = fma(x[t][u], a[t], v[u]);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -1018,31 +1033,48 @@ __device__ __forceinline__ uint32_t magnitude_bits(double x, int emax) {
     return top ? slice_bits((float)top, -8) : (127 - 40) << 7;
 }
 
+// The scale of a row with exponent emax and nz entries that are not zero.  The line is
+// half-way between two sums of magnitudes, which are multiples of 2^-16 but for the
+// 2^-40 ones, so that the order in which they are added does not matter.
+__device__ __forceinline__ RowScale row_scale(int emax, int nz) {
+    const float at = fmaxf(sqrtf((float)nz) / 512.0f, 1.0f / 128.0f);
+    return {emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0), (floorf(at * 65536.0f) + 0.5f) / 65536.0f};
+}
+
 // One row into its S bf16 slices by a whole block: every thread reads its
 // share of the row, the row exponent is reduced through shared memory, then
 // each thread writes the digits of its elements, two neighbours to a store.
-// at(k) gives element k (0 beyond the row's data).  With `exps` the row exponent
-// goes there, the slices are those of x / 2^e, and slice S holds the magnitudes.
+// at(k) gives element k (0 beyond the row's data).  With `scales` the row's goes
+// there, the slices are those of x / 2^e, and slice S holds the magnitudes.
 template <class At>
 __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S, int first, int step,
-                                                __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps = nullptr) {
-    __shared__ int red[32];
-    int emax = -2000;
+                                                __nv_bfloat16 *__restrict__ out, RowScale *__restrict__ scales = nullptr) {
+    __shared__ int red[32], count[32];
+    int emax = -2000, nz = 0;
     for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
         const double x0 = at(k), x1 = at(k + 1);
         emax = max(emax, max(fp64_exponent((unsigned long long)__double_as_longlong(x0)),
                              fp64_exponent((unsigned long long)__double_as_longlong(x1))));
+        nz += (x0 != 0.0) + (x1 != 0.0);
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
+    nz = __reduce_add_sync(0xffffffffu, nz);
     const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if ((threadIdx.x & 31) == 0) red[warp] = emax;
+    if ((threadIdx.x & 31) == 0) {
+        red[warp] = emax;
+        count[warp] = nz;
+    }
     __syncthreads();
     emax = -2000;
-    for (int w = 0; w < nw; ++w) emax = max(emax, red[w]);
-    if (exps && threadIdx.x == 0) exps[dest] = (int16_t)(emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0));
+    nz = 0;
+    for (int w = 0; w < nw; ++w) {
+        emax = max(emax, red[w]);
+        nz += count[w];
+    }
+    if (scales && threadIdx.x == 0) scales[dest] = row_scale(emax, nz);
     const int64_t plane = (int64_t)(Kpad / BKB) * R * BKB;
-    const int e0 = exps ? 0 : emax;
+    const int e0 = scales ? 0 : emax;
     for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
         uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(k / BKB) * R + dest) * BKB + k % BKB);
         uint32_t lo[MAXS + 1];
@@ -1050,7 +1082,7 @@ __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, 
         digits(at(k + 1), emax, S, first, step, [&](int i, float d) {
             o[i * (plane / 2)] = lo[i] | slice_bits(d, e0 - first - step * i) << 16;
         });
-        if (exps) o[S * (plane / 2)] = magnitude_bits(at(k), emax) | magnitude_bits(at(k + 1), emax) << 16;
+        if (scales) o[S * (plane / 2)] = magnitude_bits(at(k), emax) | magnitude_bits(at(k + 1), emax) << 16;
     }
 }
 
@@ -1071,7 +1103,7 @@ slice_rows2_kernel(const double *__restrict__ X1, int64_t ld1, int K1, const dou
 // in all), so a 64-wide K block of consecutive rows is contiguous.  Column
 // skip_col is zero.
 __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t dest, int64_t R, int Kpad, int S,
-                                          int skip_col, __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps,
+                                          int skip_col, __nv_bfloat16 *__restrict__ out, RowScale *__restrict__ scales,
                                           int lane) {
     const int KB = Kpad / BKB;
     // exponent of the row maximum from the bit patterns (no FP64 arithmetic)
@@ -1080,15 +1112,20 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
         if (k != skip_col) emax = max(emax, fp64_exponent((unsigned long long)__double_as_longlong(x[k])));
 #pragma unroll
     for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
-    if (exps && lane == 0) exps[dest] = (int16_t)(emax > 1024 ? kExpNaN : (emax > -2000 ? emax : 0));
-    const int e0 = exps ? 0 : emax;
+    if (scales) {
+        int nz = 0;
+        for (int k = lane; k < Kpad; k += 32) nz += k != skip_col && x[k] != 0.0;
+        nz = __reduce_add_sync(0xffffffffu, nz);
+        if (lane == 0) scales[dest] = row_scale(emax, nz);
+    }
+    const int e0 = scales ? 0 : emax;
     for (int k = lane; k < Kpad; k += 32) {
         const int kb = k / BKB, kk = k % BKB;
         digits(k != skip_col ? x[k] : 0.0, emax, S, kXFirst, kXStep, [&](int i, float d) {
             out[(((int64_t)i * KB + kb) * R + dest) * BKB + kk] =
                 __ushort_as_bfloat16((unsigned short)slice_bits(d, e0 - kXFirst - kXStep * i));
         });
-        if (exps)
+        if (scales)
             out[(((int64_t)S * KB + kb) * R + dest) * BKB + kk] =
                 __ushort_as_bfloat16((unsigned short)(k != skip_col ? magnitude_bits(x[k], emax) : 0));
     }
@@ -1098,11 +1135,11 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
 // zeroed on the rows with j == j' (elsewhere that label is zero, or, with
 // orbital symmetry, the column holds another label).
 __global__ void slice_rows_kernel(const double *__restrict__ X, int64_t rows, int Kpad, int S, int skip_col,
-                                  int n_co, __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps) {
+                                  int n_co, __nv_bfloat16 *__restrict__ out, RowScale *__restrict__ scales) {
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     const bool diag = row / n_co == row % n_co;
-    slice_row(X + row * Kpad, row, rows, Kpad, S, diag ? skip_col : -1, out, exps, threadIdx.x & 31);
+    slice_row(X + row * Kpad, row, rows, Kpad, S, diag ? skip_col : -1, out, scales, threadIdx.x & 31);
 }
 
 // Coefficient rows (Kin entries each) into slices of Kout columns: column k
@@ -1112,7 +1149,7 @@ __global__ void slice_rows_kernel(const double *__restrict__ X, int64_t rows, in
 __global__ void __launch_bounds__(256)
 slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int64_t R,
                    int Kin, int Kout, const int32_t *__restrict__ perm, int S, int skip_col,
-                   __nv_bfloat16 *__restrict__ out, int16_t *__restrict__ exps) {
+                   __nv_bfloat16 *__restrict__ out, RowScale *__restrict__ scales) {
     const int ti = task_of(blk, n_tasks, blockIdx.x);
     const SliceTask &T = tasks[ti];
     const int64_t row = blockIdx.x - blk[ti];
@@ -1121,7 +1158,7 @@ slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restric
         if (k == skip_col) return 0.0;
         const int lab = perm ? __ldg(perm + k) : k;
         return (lab >= 0 && lab < Kin) ? __ldg(x + lab) : 0.0;
-    }, T.row0 + row, R, Kout, S, kXFirst, kXStep, out, exps);
+    }, T.row0 + row, R, Kout, S, kXFirst, kXStep, out, scales);
 }
 
 // Rows with j == j' (both ranges): H[(n,j),(n',j)] over all K, incl. delta,
@@ -1377,13 +1414,13 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)planes * rows * Kc;
     if (precision == HB_FP64 && !f64_slices_fit(ctx, bytes))
         return mixed_fail(ctx, HB_ERR_OOM, "panel slices: more than an FP64 build may take");
-    const size_t extra = precision == HB_MIXED ? sizeof(float2) * (size_t)ctx->n_co * Kc : sizeof(int16_t) * (size_t)rows;
+    const size_t extra = precision == HB_MIXED ? sizeof(float2) * (size_t)ctx->n_co * Kc : sizeof(RowScale) * (size_t)rows;
     // everything that can fail comes before the kernels; a failure leaves nothing behind
     auto undo = [&](int code, const std::string &m) {
         dfree(ctx, PS.buf);
-        dfree(ctx, PS.exps);
+        dfree(ctx, PS.scales);
         PS.buf = nullptr;
-        PS.exps = nullptr;
+        PS.scales = nullptr;
         if (precision == HB_MIXED) {
             dfree(ctx, M.pdiag);
             M.pdiag = nullptr;
@@ -1391,7 +1428,7 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
         return mixed_fail(ctx, code, m);
     };
     cudaError_t e = dmalloc(ctx, (void **)&PS.buf, bytes);
-    if (e == cudaSuccess) e = precision == HB_MIXED ? dmalloc(ctx, (void **)&M.pdiag, extra) : dmalloc(ctx, (void **)&PS.exps, extra);
+    if (e == cudaSuccess) e = precision == HB_MIXED ? dmalloc(ctx, (void **)&M.pdiag, extra) : dmalloc(ctx, (void **)&PS.scales, extra);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return undo(HB_ERR_OOM, std::string("panel slices: ") + cudaGetErrorString(e));
@@ -1420,7 +1457,7 @@ int mixed_prepare(hb_ctx *ctx, int precision, cudaStream_t s) {
     ctx->dev_bytes += bytes + extra;
     if (precision == HB_MIXED) panel_diag_df_kernel<<<ctx->n_co, 256, 0, s>>>(ctx->panel, ctx->n_co, Kc, M.pdiag);
     slice_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ctx->panel, rows, Kc, PS.slices, ctx->delta_pos,
-                                                                 ctx->n_co, PS.buf, PS.exps);
+                                                                 ctx->n_co, PS.buf, PS.scales);
     PS.ready = true;
     return HB_OK;
 }
@@ -1437,15 +1474,15 @@ int mixed_slices(const hb_ctx *ctx, int precision) {
 // four 3D maps: for 32-K stages one per tile width bn = 32, 64, 128 (box: bn
 // rows x half a K block of one slice plane, 64-byte swizzle), and for 64-K
 // stages one of 128 rows x a whole K block (128-byte swizzle).
-// exps (FP64 build, or null): the rows' exponents.
-int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int16_t **exps, CUtensorMap *tm,
+// scales (FP64 build, or null): those of the rows.
+int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, RowScale **scales, CUtensorMap *tm,
                      std::string *err) {
     *buf = nullptr;
-    if (exps) *exps = nullptr;
+    if (scales) *scales = nullptr;
     if (!encode_fn()) { *err = "cuTensorMapEncodeTiled is not available"; return HB_ERR_CUDA; }
     if (rows < 1) rows = 1;
     cudaError_t e = dmalloc(mem, buf, sizeof(__nv_bfloat16) * (size_t)S * rows * Kpad);
-    if (e == cudaSuccess && exps) e = dmalloc_n(mem, exps, (size_t)rows);
+    if (e == cudaSuccess && scales) e = dmalloc_n(mem, scales, (size_t)rows);
     if (e != cudaSuccess) {
         cudaGetLastError();
         dfree(mem, *buf);
@@ -1467,7 +1504,7 @@ int split_coef_alloc(hb_ctx *mem, int S, int64_t rows, int Kpad, void **buf, int
     if (r != CUDA_SUCCESS) {
         dfree(mem, *buf);
         *buf = nullptr;
-        if (exps) { dfree(mem, *exps); *exps = nullptr; }
+        if (scales) { dfree(mem, *scales); *scales = nullptr; }
         *err = "coefficient tensor map: error " + std::to_string((int)r);
         return HB_ERR_CUDA;
     }
@@ -1511,10 +1548,10 @@ int split_tile_heuristic(int cn, int cnp) {
 }
 
 int g_slice(const Grouped<SliceTask> &g, int64_t R, int Kin, int Kout, const int32_t *perm, int S, int skip_col,
-            void *out, int16_t *exps, cudaStream_t s) {
+            void *out, RowScale *scales, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
     slice_rows_grouped<<<(unsigned)g.blocks, 256, 0, s>>>(g.tasks, g.blk, g.n, R, Kin, Kout, perm, S, skip_col,
-                                                          (__nv_bfloat16 *)out, exps);
+                                                          (__nv_bfloat16 *)out, scales);
     return 1;
 }
 
@@ -1524,22 +1561,14 @@ int split_kstage_choice(int bn, int kblocks, int force) {
     return kblocks >= kK64Blocks ? 64 : 32;
 }
 
-// The line of a panel's weak elements (see the head of this file): half-way between
-// two sums of magnitudes, which are multiples of 2^-16 but for the 2^-40 ones, so
-// that the order in which they are added does not matter.
-static float weak_line(int K) {
-    const double at = std::max(std::sqrt((double)K) / 512.0, 1.0 / 128.0);
-    return (float)((std::floor(at * 65536.0) + 0.5) / 65536.0);
-}
-
-int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const Grouped<SplitTask> &g,
-                uint32_t *weak, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s) {
+int g_weak_bits(const hb_ctx *panel_ctx, int lg, const CUtensorMap *tm_coef, const RowScale *coef_scales,
+                const Grouped<SplitTask> &g, uint32_t *weak, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
     const PanelSlices &PS = panel_ctx->mixed->panel[0];
     const unsigned grid = (unsigned)std::min((int)g.blocks, sm_count());
     split_expand_kernel<1, kWeakCols, 64, kWeakBits><<<grid, NTHREADS, split_smem_bytes(kWeakCols, 64, kWeakSlots), s>>>(
-        PS.tm[1][lg - 3], tm_coef[3], g.tasks, g.blk, g.n, (int)g.blocks, kblocks, coef_planes, cols, nullptr, nullptr,
-        weak, kF64Slices, weak_line(panel_ctx->K), panel_ctx->n_co, err, 0, 1);
+        PS.tm[1][lg - 3], tm_coef[3], g.tasks, g.blk, g.n, (int)g.blocks, kblocks, coef_planes, cols, PS.scales, coef_scales,
+        weak, kF64Slices, panel_ctx->n_co, err, 0, 1);
     return 1;
 }
 
@@ -1551,11 +1580,11 @@ int g_weak_sums(const hb_ctx *panel_ctx, const Grouped<SplitTask> &g, const Grou
     if (g.blocks <= 0) return 0;
     fp64_elements_kernel<<<(unsigned)g.blocks, 256, 0, s>>>(
         g.tasks, g.blk, g.n, digits.blk, weak, panel_ctx->panel, panel_ctx->n_co, kblocks * 64, panel_ctx->K,
-        panel_ctx->n_cls > 1 ? panel_ctx->cls_labels : nullptr, cols, shard_r, shard_n);
+        panel_ctx->cls_by_lane, cols, shard_r, shard_n);
     return 1;
 }
 
-int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef, const int16_t *coef_exps,
+int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtensorMap *tm_coef, const RowScale *coef_scales,
             const Grouped<SplitTask> &g, int kblocks, int coef_planes, const ExpCol *cols, int *err, cudaStream_t s,
             int shard_r, int shard_n) {
     if (g.blocks <= 0) return 0;
@@ -1573,8 +1602,8 @@ int g_split(const hb_ctx *panel_ctx, int precision, int lg, int bn, const CUtens
     const unsigned grid = (unsigned)std::min(n_local, sm_count());
 #define HB_SPLIT(SS, BB, KK, MM)                                                                                   \
     split_expand_kernel<SS, BB, KK, MM><<<grid, NTHREADS, smem, s>>>(tm_panel, tm_c, g.tasks, g.blk, g.n, n_tiles, \
-                                                                     kblocks, coef_planes, cols, PS.exps, coef_exps, \
-                                                                     nullptr, 0, 0.0f, panel_ctx->n_co, err, shard_r, \
+                                                                     kblocks, coef_planes, cols, PS.scales, coef_scales, \
+                                                                     nullptr, 0, panel_ctx->n_co, err, shard_r, \
                                                                      shard_n)
 #define HB_SPLIT_S(SS)                                       \
     do {                                                     \
@@ -1708,7 +1737,7 @@ bool release_f64_slices(hb_ctx *ctx) {
             }
     PanelSlices &PS = owner->mixed->panel[0];
     dfree(owner, PS.buf);
-    dfree(owner, PS.exps);
+    dfree(owner, PS.scales);
     PS = PanelSlices();
     if (ctx != owner && ctx->mixed) ctx->mixed->panel[0] = PanelSlices();
     ++owner->tables_gen;          // other borrowing contexts let go of them before their next build
@@ -1720,7 +1749,7 @@ void release_mixed(hb_ctx *ctx) {
     for (PanelSlices &P : ctx->mixed->panel)
         if (!P.borrowed) {
             dfree(ctx, P.buf);
-            dfree(ctx, P.exps);
+            dfree(ctx, P.scales);
         }
     if (!ctx->mixed->panel[1].borrowed) dfree(ctx, ctx->mixed->pdiag);
     delete ctx->mixed;
