@@ -1033,6 +1033,9 @@ __device__ __forceinline__ uint32_t magnitude_bits(double x, int emax) {
     return top ? slice_bits((float)top, -8) : (127 - 40) << 7;
 }
 
+// Whether x is not zero, without FP64 arithmetic.
+__device__ __forceinline__ int nonzero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) != 0; }
+
 // The scale of a row with exponent emax and nz entries that are not zero.  The line is
 // half-way between two sums of magnitudes, which are multiples of 2^-16 but for the
 // 2^-40 ones, so that the order in which they are added does not matter.
@@ -1044,37 +1047,40 @@ __device__ __forceinline__ RowScale row_scale(int emax, int nz) {
 // One row into its S bf16 slices by a whole block: every thread reads its
 // share of the row, the row exponent is reduced through shared memory, then
 // each thread writes the digits of its elements, two neighbours to a store.
-// at(k) gives element k (0 beyond the row's data).  With `scales` the row's goes
-// there, the slices are those of x / 2^e, and slice S holds the magnitudes.
-template <class At>
+// at(k) gives element k (0 beyond the row's data).  With SCALES the row's goes to
+// `scales`, the slices are those of x / 2^e, and slice S holds the magnitudes.
+// (Decided at compile time: left to the pointer, the count of the entries and the
+// magnitudes, which mixed builds have not, made theirs slower too: a batch of 12
+// over 8 symmetries 3.71 ms, 3.62 without.)
+template <bool SCALES, class At>
 __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, int Kpad, int S, int first, int step,
                                                 __nv_bfloat16 *__restrict__ out, RowScale *__restrict__ scales = nullptr) {
-    __shared__ int red[32], count[32];
+    __shared__ int red[32], count[SCALES ? 32 : 1];
     int emax = -2000, nz = 0;
     for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
         const double x0 = at(k), x1 = at(k + 1);
         emax = max(emax, max(fp64_exponent((unsigned long long)__double_as_longlong(x0)),
                              fp64_exponent((unsigned long long)__double_as_longlong(x1))));
-        nz += (x0 != 0.0) + (x1 != 0.0);
+        if (SCALES) nz += nonzero(x0) + nonzero(x1);
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
-    nz = __reduce_add_sync(0xffffffffu, nz);
+    if (SCALES) nz = __reduce_add_sync(0xffffffffu, nz);
     const int warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     if ((threadIdx.x & 31) == 0) {
         red[warp] = emax;
-        count[warp] = nz;
+        if (SCALES) count[warp] = nz;
     }
     __syncthreads();
     emax = -2000;
     nz = 0;
     for (int w = 0; w < nw; ++w) {
         emax = max(emax, red[w]);
-        nz += count[w];
+        if (SCALES) nz += count[w];
     }
-    if (scales && threadIdx.x == 0) scales[dest] = row_scale(emax, nz);
+    if (SCALES && threadIdx.x == 0) scales[dest] = row_scale(emax, nz);
     const int64_t plane = (int64_t)(Kpad / BKB) * R * BKB;
-    const int e0 = scales ? 0 : emax;
+    const int e0 = SCALES ? 0 : emax;
     for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
         uint32_t *o = reinterpret_cast<uint32_t *>(out + ((int64_t)(k / BKB) * R + dest) * BKB + k % BKB);
         uint32_t lo[MAXS + 1];
@@ -1082,7 +1088,7 @@ __device__ __forceinline__ void slice_row_block(At at, int64_t dest, int64_t R, 
         digits(at(k + 1), emax, S, first, step, [&](int i, float d) {
             o[i * (plane / 2)] = lo[i] | slice_bits(d, e0 - first - step * i) << 16;
         });
-        if (scales) o[S * (plane / 2)] = magnitude_bits(at(k), emax) | magnitude_bits(at(k + 1), emax) << 16;
+        if (SCALES) o[S * (plane / 2)] = magnitude_bits(at(k), emax) | magnitude_bits(at(k + 1), emax) << 16;
     }
 }
 
@@ -1094,7 +1100,7 @@ slice_rows2_kernel(const double *__restrict__ X1, int64_t ld1, int K1, const dou
     const int64_t row = blockIdx.x;
     const double *x1 = X1 + row * ld1;
     const double *x2 = X2 ? X2 + row * ld2 : nullptr;
-    slice_row_block([&](int k) -> double { return k < K1 ? __ldg(x1 + k) : ((x2 && k < K1 + K2) ? __ldg(x2 + k - K1) : 0.0); },
+    slice_row_block<false>([&](int k) -> double { return k < K1 ? __ldg(x1 + k) : ((x2 && k < K1 + K2) ? __ldg(x2 + k - K1) : 0.0); },
                     row, R, Kpad, S, kDFirst, kDStep, out);
 }
 
@@ -1114,7 +1120,7 @@ __device__ __forceinline__ void slice_row(const double *__restrict__ x, int64_t 
     for (int off = 16; off; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
     if (scales) {
         int nz = 0;
-        for (int k = lane; k < Kpad; k += 32) nz += k != skip_col && x[k] != 0.0;
+        for (int k = lane; k < Kpad; k += 32) nz += k != skip_col && nonzero(x[k]);
         nz = __reduce_add_sync(0xffffffffu, nz);
         if (lane == 0) scales[dest] = row_scale(emax, nz);
     }
@@ -1146,6 +1152,7 @@ __global__ void slice_rows_kernel(const double *__restrict__ X, int64_t rows, in
 // holds label perm[k] (the labels class by class, with orbital symmetry; -1
 // padding), or label k without a permutation; column skip_col (the delta
 // label) is zero.
+template <bool SCALES>
 __global__ void __launch_bounds__(256)
 slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restrict__ blk, int n_tasks, int64_t R,
                    int Kin, int Kout, const int32_t *__restrict__ perm, int S, int skip_col,
@@ -1154,7 +1161,7 @@ slice_rows_grouped(const SliceTask *__restrict__ tasks, const int64_t *__restric
     const SliceTask &T = tasks[ti];
     const int64_t row = blockIdx.x - blk[ti];
     const double *x = T.X + row * Kin;
-    slice_row_block([&](int k) -> double {
+    slice_row_block<SCALES>([&](int k) -> double {
         if (k == skip_col) return 0.0;
         const int lab = perm ? __ldg(perm + k) : k;
         return (lab >= 0 && lab < Kin) ? __ldg(x + lab) : 0.0;
@@ -1550,8 +1557,9 @@ int split_tile_heuristic(int cn, int cnp) {
 int g_slice(const Grouped<SliceTask> &g, int64_t R, int Kin, int Kout, const int32_t *perm, int S, int skip_col,
             void *out, RowScale *scales, cudaStream_t s) {
     if (g.blocks <= 0) return 0;
-    slice_rows_grouped<<<(unsigned)g.blocks, 256, 0, s>>>(g.tasks, g.blk, g.n, R, Kin, Kout, perm, S, skip_col,
-                                                          (__nv_bfloat16 *)out, scales);
+    auto *kernel = scales ? slice_rows_grouped<true> : slice_rows_grouped<false>;
+    kernel<<<(unsigned)g.blocks, 256, 0, s>>>(g.tasks, g.blk, g.n, R, Kin, Kout, perm, S, skip_col, (__nv_bfloat16 *)out,
+                                              scales);
     return 1;
 }
 
